@@ -622,17 +622,19 @@ cudaError_t launch_vjp_warp(lj_ctx *c, const VjpCoef &kd, double scale, double *
 
 }  // namespace
 
-cudaError_t launch_vjp(lj_ctx *c, const double *g, double scale, double *dx, double *dparam)
+static cudaError_t launch_vjp_terms(lj_ctx *c, const double *g, double scale, double *dx, double *dparam, double *lam,
+                                    double dt_axpy, bool *lam_done)
 {
     const int n = (int)c->p.n;
-    if (n == 0) return cudaSuccess;
     const bool fp64 = c->p.precision == LJ_PREC_FP64;
     const unsigned gb = (unsigned)((n + 255) / 256);
-    if (fp64)
+    if (c->slots_open == 1)
+        ;   // the slotted binning has copied the cotangents
+    else if (fp64)
         k_gather_cotangent<double4_16a><<<gb, 256, 0, c->stream>>>(g, c->perm, n, (double4_16a *)c->g4);
     else
         k_gather_cotangent<float4><<<gb, 256, 0, c->stream>>>(g, c->perm, n, (float4 *)c->g4);
-    c->kernel_launches++;
+    if (c->slots_open != 1) c->kernel_launches++;
     VjpCoef k;
     const double sg = c->p.sigma, rc = c->p.rc;
     const double s6 = sg * sg * sg * sg * sg * sg, s12 = s6 * s6;
@@ -646,12 +648,8 @@ cudaError_t launch_vjp(lj_ctx *c, const double *g, double scale, double *dx, dou
     if (!fp64 && uses_vjp_n3(c) && c->f_sorted) {
         // each pair once (lj_vjp_n3.cu); f_sorted is its float4 accumulator
         const double coef[7] = {k.rc2, k.a1, k.b1, k.fc1, k.dfc1, k.eps, k.inv_sigma};
-        int grid = 0;
-        cudaError_t e = launch_vjp_n3(c, coef, scale, dx, (float4 *)c->f_sorted, &grid);
-        if (e != cudaSuccess) return e;
-        k_accum_params<<<1, kReduceThreads, 0, c->stream>>>(c->partial, grid, scale, dparam);
-        c->kernel_launches++;
-        return cudaGetLastError();
+        *lam_done = true;
+        return launch_vjp_n3(c, coef, scale, dx, (float4 *)c->f_sorted, dparam, lam, dt_axpy);
     }
     if (!fp64) return launch_vjp_warp(c, k, scale, dx, dparam);
     if (c->p.cell_subdiv != 2 && c->wcap > 0 && c->w64_lcap > 0) {
@@ -679,6 +677,16 @@ cudaError_t launch_vjp(lj_ctx *c, const double *g, double scale, double *dx, dou
     k_accum_params<<<1, kReduceThreads, 0, c->stream>>>(c->partial, grid, scale, dparam);
     c->kernel_launches += 2;
     return cudaGetLastError();
+}
+
+cudaError_t launch_vjp(lj_ctx *c, const double *g, double scale, double *dx, double *dparam, double *lam,
+                       double dt_axpy)
+{
+    if (c->p.n == 0) return cudaSuccess;
+    bool lam_done = false;
+    const cudaError_t e = launch_vjp_terms(c, g, scale, dx, dparam, lam, dt_axpy, &lam_done);
+    if (e != cudaSuccess || !lam || lam_done) return e;
+    return launch_axpy(c, lam, dx, dt_axpy);
 }
 
 cudaError_t launch_axpy(lj_ctx *c, double *y, const double *x, double a)

@@ -90,6 +90,7 @@ void free_ctx(lj_ctx *c)
     cudaFree(c->scan_status);
     cudaFree(c->scan_ctl);
     cudaFree(c->centre);
+    cudaFree(c->centre2);
     cudaFree(c->work);
     cudaFree(c->thb);
     cudaFree(c->partial);
@@ -100,6 +101,7 @@ void free_ctx(lj_ctx *c)
     cudaFree(c->vs);
     cudaFree(c->fs);
     cudaFree(c->g4);
+    slots_free(c);
     cudaFree(c->n2_scratch);
     cudaFree(c->f_sorted);
     if (c->copy_stream) cudaStreamDestroy(c->copy_stream);
@@ -162,10 +164,28 @@ int skin_restart(lj_ctx *c)
 
 int do_bin(lj_ctx *c, const double *x, bool wrap_in_scatter)
 {
+    if (c->slots_open == 1) c->slots_open = 2;   // a slotted binning that no kernel read
+    c->slots_last = 0;
     LJ_CK(launch_bin_count(c, x));
     LJ_CK(launch_scan(c));
     LJ_CK(launch_scatter(c, x, wrap_in_scatter));
     return skin_restart(c);
+}
+
+// Bin x for a force evaluation into f (zeroed here with slotted cells).
+int bin_for_force(lj_ctx *c, const double *x, void *f)
+{
+    if (!uses_slots(c)) return do_bin(c, x, true);
+    LJ_CK(launch_bin_slots(c, x, (float4 *)f, nullptr));
+    return LJ_OK;
+}
+
+// Bin x for a VJP of the cotangents g.
+int bin_for_vjp(lj_ctx *c, const double *x, const double *g)
+{
+    if (!uses_slots(c)) return do_bin(c, x, true);
+    LJ_CK(launch_bin_slots(c, x, (float4 *)c->f_sorted, g));
+    return LJ_OK;
 }
 
 // Cell lists with a skin: the cells are rebuilt only when the device-side
@@ -178,6 +198,17 @@ bool fused_mode(const lj_ctx *c) { return !c->use_run_kernel && c->fuse_update &
 // graph replay captures.
 int one_step(lj_ctx *c, double *x, double *v, void *f, int s, int nsteps, cudaEvent_t x_final = nullptr)
 {
+    if (uses_slots(c)) {
+        // slotted cells: one pass over the particles, then the forces
+        if (s == 0 && c->kdb_done)
+            c->kdb_done = 0;
+        else
+            LJ_CK(launch_kick_drift_slots(c, x, v, (float4 *)f, s == 0 ? 1 : 2));
+        if (x_final) LJ_CK(cudaEventRecord(x_final, c->stream));   // x holds its final value
+        LJ_CK(launch_force(c, f, false));
+        return LJ_OK;
+    }
+    c->slots_last = 0;
     if (c->skin > 0.0) {
         // cell lists with a skin: the cells are rebuilt only when the
         // device-side decision (k_skin_decide) asks for it; otherwise the
@@ -241,7 +272,8 @@ int ensure_zero_stream(lj_ctx *c)
     return LJ_OK;
 }
 
-// Capture the launches of one middle step for (x, v, f) into c->gexec.
+// Capture the launches of a middle step for (x, v, f) into c->gexec; of two
+// with slotted cells, whose count buffers alternate.
 int capture_middle_step(lj_ctx *c, double *x, double *v, void *f)
 {
     if (c->gexec) {
@@ -261,7 +293,9 @@ int capture_middle_step(lj_ctx *c, double *x, double *v, void *f)
     if (e == cudaSuccess) {
         cudaStream_t keep = c->stream;
         c->stream = cs;
-        r = one_step(c, x, v, f, 1, 3);
+        c->gsteps = uses_slots(c) ? 2 : 1;
+        c->gpar = c->slot_par;
+        for (int k = 0; k < c->gsteps && r == LJ_OK; k++) r = one_step(c, x, v, f, 1, 3);
         c->stream = keep;
         e = cudaStreamEndCapture(cs, &g);
     }
@@ -332,21 +366,25 @@ int do_steps(lj_ctx *c, double *x, double *v, void *f, int nsteps, cudaEvent_t x
     if (nsteps <= 0) return LJ_OK;
     if (persistent_mode(c)) return persistent_steps(c, x, v, f, nsteps, x_final);
     if (fused_mode(c)) LJ_CK(launch_kick_drift_bin(c, x, v, f, 1));
-    if (c->skin <= 0.0 && !fused_mode(c) && uses_force_n3(c)) {
+    if (c->skin <= 0.0 && !fused_mode(c) && uses_force_n3(c) && !uses_slots(c)) {
         int r = ensure_zero_stream(c);
         if (r) return r;
     }
     const bool graph = c->use_graph && !c->timing && nsteps >= 3;
+    const int gs = uses_slots(c) ? 2 : 1;   // steps per replay
     for (int s = 0; s < nsteps; s++) {
         // after step 0 (which does any lazy set-up outside the capture and
         // settles a pending skin rebuild) the middle steps are graph replays
-        if (graph && s > 0 && s < nsteps - 1 && !c->skin_dirty) {
-            if (!c->gexec || c->gx != x || c->gv != v || c->gf != f || c->ggen != c->gen) {
+        const bool have = c->gexec && c->gx == x && c->gv == v && c->gf == f && c->ggen == c->gen && c->gsteps == gs;
+        if (graph && s > 0 && s + gs <= nsteps - 1 && !c->skin_dirty &&
+            !(have && gs == 2 && c->gpar != c->slot_par)) {
+            if (!have) {
                 int r = capture_middle_step(c, x, v, f);
                 if (r) return r;
             }
             LJ_CK(cudaGraphLaunch(c->gexec, c->stream));
             c->kernel_launches += c->glaunches;
+            s += gs - 1;
         } else {
             int r = one_step(c, x, v, f, s, nsteps, s == nsteps - 1 && !fused_mode(c) ? x_final : nullptr);
             if (r) return r;
@@ -365,6 +403,7 @@ int ensure_vjp_buffers(lj_ctx *c)
     if (!c->g4) LJ_CK(cudaMalloc(&c->g4, (size_t)c->p.n * force_vsize(c)));
     if (c->p.precision == LJ_PREC_MIXED && uses_vjp_n3(c) && !c->f_sorted)
         LJ_CK(cudaMalloc(&c->f_sorted, (size_t)c->p.n * sizeof(float4)));
+    if (uses_slots(c) && !c->sg4) LJ_CK(cudaMalloc(&c->sg4, ((size_t)c->nslots + (size_t)c->p.n) * sizeof(float4)));
     return LJ_OK;
 }
 
@@ -413,6 +452,7 @@ int setup_grid(lj_ctx *c, int nc)
     cudaFree(c->count);
     cudaFree(c->start);
     cudaFree(c->centre);
+    cudaFree(c->centre2);
     cudaFree(c->thb);
     cudaFree(c->tile_sum);
     cudaFree(c->scan_status);
@@ -422,6 +462,7 @@ int setup_grid(lj_ctx *c, int nc)
     c->scan_status = nullptr;
     c->scan_ctl = nullptr;
     c->centre = nullptr;
+    c->centre2 = nullptr;
     c->thb = nullptr;
     c->partial = nullptr;
     c->nc = nc;
@@ -442,6 +483,18 @@ int setup_grid(lj_ctx *c, int nc)
         for (int k = 0; k < nc; k++) h[k] = ((double)k + 0.5) * c->cw;
         cudaError_t e = cudaMalloc(&c->centre, sizeof(double) * (size_t)nc);
         if (e == cudaSuccess) e = cudaMemcpy(c->centre, h, sizeof(double) * (size_t)nc, cudaMemcpyHostToDevice);
+        float2 *h2 = (float2 *)malloc(sizeof(float2) * (size_t)nc);
+        if (!h2 && e == cudaSuccess) e = cudaErrorMemoryAllocation;
+        if (h2) {
+            for (int k = 0; k < nc; k++) {
+                h2[k].x = (float)h[k];
+                h2[k].y = (float)(h[k] - (double)h2[k].x);
+            }
+            if (e == cudaSuccess) e = cudaMalloc(&c->centre2, sizeof(float2) * (size_t)nc);
+            if (e == cudaSuccess)
+                e = cudaMemcpy(c->centre2, h2, sizeof(float2) * (size_t)nc, cudaMemcpyHostToDevice);
+            free(h2);
+        }
         free(h);
         long long *tb = (long long *)malloc(sizeof(long long) * (size_t)(nc + 1));
         if (!tb && e == cudaSuccess) e = cudaErrorMemoryAllocation;
@@ -470,6 +523,7 @@ int setup_grid(lj_ctx *c, int nc)
     c->pipe_grid = 0;
     if (c->p.precision == LJ_PREC_MIXED && c->p.cell_subdiv != 2) LJ_GRID_CK(pipe_force_configure(c));
     if (c->p.precision == LJ_PREC_MIXED && c->p.cell_subdiv != 2) LJ_GRID_CK(n3_force_configure(c));
+    LJ_GRID_CK(slots_setup(c));
     if (c->p.precision == LJ_PREC_FP64 && !c->f_sorted && c->p.n > 0)   // the FP64 pair-once sums, in cell order
         LJ_GRID_CK(cudaMalloc(&c->f_sorted, (size_t)c->p.n * 4 * sizeof(double)));
     {
@@ -575,6 +629,7 @@ extern "C" int lj_get_cells(lj_ctx *c, int32_t *cell_of, int32_t *count, int32_t
 {
     if (!c) return LJ_EINVAL;
     const size_t n = (size_t)c->p.n;
+    if (c->slots_last) LJ_CK(launch_slots_to_lists(c));   // the last binning was a slotted one
     if (cell_of && n) {
         int r = check_dev_ptr(cell_of, 4);
         if (r) return r;
@@ -608,7 +663,7 @@ extern "C" int lj_forces(lj_ctx *c, const double *x, void *f, double *e_pot, dou
         r = check_dev_ptr(f, 16);
         if (r) return r;
     }
-    int r = do_bin(c, x, true);
+    int r = bin_for_force(c, x, f);
     if (r) return r;
     const bool energy = e_pot || virial;
     LJ_CK(launch_force(c, f, energy));
@@ -668,10 +723,14 @@ extern "C" int lj_langevin_step(lj_ctx *c, double *x, double *v, void *f, int32_
     if (r) return r;
     r = check_dev_ptr(f, 16);
     if (r) return r;
+    const bool slots = uses_slots(c);
+    if (!slots) c->slots_last = 0;
     for (int s = 0; s < nsteps; s++) {
         LJ_CK(launch_langevin_bin(c, x, v, f, s == 0 ? 1 : 2, gamma, kT));
-        LJ_CK(launch_scan(c));
-        LJ_CK(launch_scatter(c, x, false));
+        if (!slots) {
+            LJ_CK(launch_scan(c));
+            LJ_CK(launch_scatter(c, x, false));
+        }
         LJ_CK(launch_force(c, f, false));
     }
     LJ_CK(launch_kick(c, v, f));
@@ -745,7 +804,10 @@ extern "C" int lj_step_host(lj_ctx *c, double *x, double *v, void *f, int32_t ns
                                   cudaMemcpyHostToDevice, c->copy_stream));
             LJ_CK(cudaEventRecord(c->ev_chunk[k], c->copy_stream));
             LJ_CK(cudaStreamWaitEvent(c->stream, c->ev_chunk[k], 0));
-            LJ_CK(launch_kick_drift_bin(c, c->xs, c->vs, c->fs, 1, (int64_t)i0, (int64_t)i1));
+            if (uses_slots(c))
+                LJ_CK(launch_kick_drift_slots(c, c->xs, c->vs, (float4 *)c->fs, 1, (int64_t)i0, (int64_t)i1));
+            else
+                LJ_CK(launch_kick_drift_bin(c, c->xs, c->vs, c->fs, 1, (int64_t)i0, (int64_t)i1));
         }
         c->kdb_done = 1;
     } else if (n > 0) {
@@ -787,7 +849,7 @@ extern "C" int lj_energy(lj_ctx *c, const double *x, const double *v, double *ou
     LJ_CK(cudaMemsetAsync(c->scalars, 0, 4 * sizeof(double), c->stream));
     if (c->p.n > 0) {
         LJ_CK(launch_ekin(c, v));
-        r = do_bin(c, x, true);
+        r = bin_for_force(c, x, c->fs);
         if (r) return r;
         LJ_CK(launch_force(c, c->fs, true));
         LJ_CK(launch_energy_reduce(c));
@@ -815,7 +877,7 @@ extern "C" int lj_observables(lj_ctx *c, const double *x, const double *v, doubl
     LJ_CK(cudaMemsetAsync(c->scalars, 0, 8 * sizeof(double), c->stream));
     if (c->p.n > 0) {
         LJ_CK(launch_ekin(c, v));
-        r = do_bin(c, x, true);
+        r = bin_for_force(c, x, c->fs);
         if (r) return r;
         LJ_CK(launch_force(c, c->fs, true));
         LJ_CK(launch_energy_reduce(c));
@@ -863,7 +925,7 @@ extern "C" int lj_forces_vjp(lj_ctx *c, const double *x, const double *g, double
     if ((r = check_dev_ptr(g, 8)) != LJ_OK) return r;
     if ((r = check_dev_ptr(dx, 8)) != LJ_OK) return r;
     if ((r = ensure_vjp_buffers(c)) != LJ_OK) return r;
-    if ((r = do_bin(c, x, true)) != LJ_OK) return r;
+    if ((r = bin_for_vjp(c, x, g)) != LJ_OK) return r;
     LJ_CK(launch_vjp(c, g, scale, dx, dparam));
     return LJ_OK;
 }
@@ -882,12 +944,11 @@ extern "C" int lj_vv_adjoint_step(lj_ctx *c, const double *x_n, const double *x_
     if ((r = ensure_vjp_buffers(c)) != LJ_OK) return r;
     const double h = 0.5 * c->p.dt / c->p.mass;
     // v_{n+1} = v_half + h F(x_{n+1})
-    if ((r = do_bin(c, x_n1, true)) != LJ_OK) return r;
-    LJ_CK(launch_vjp(c, lam_v, h, lam_x, dparam));
-    // x_{n+1} = x_n + dt v_half
-    LJ_CK(launch_axpy(c, lam_v, lam_x, c->p.dt));
+    // and x_{n+1} = x_n + dt v_half
+    if ((r = bin_for_vjp(c, x_n1, lam_v)) != LJ_OK) return r;
+    LJ_CK(launch_vjp(c, lam_v, h, lam_x, dparam, lam_v, c->p.dt));
     // v_half = v_n + h F(x_n)
-    if ((r = do_bin(c, x_n, true)) != LJ_OK) return r;
+    if ((r = bin_for_vjp(c, x_n, lam_v)) != LJ_OK) return r;
     LJ_CK(launch_vjp(c, lam_v, h, lam_x, dparam));
     return LJ_OK;
 }

@@ -360,7 +360,7 @@ __device__ void phase_force_n3(const BatchDev &b, const WarpParams &k, float4 *_
         for (int c = (int)c0; c < c1; c++) {
             const HalfLoad cur = nxt;
             if (c + 1 < c1) nxt = load(c + 1);
-            n3_cell<MODE, ENERGY, false>(k, b.pos, f, cur, (float)b.cw[b.rep_of_cell[c]], S, stab, spre, H, eacc,
+            n3_cell<MODE, ENERGY, false, false>(k, b.pos, f, cur, c, (float)b.cw[b.rep_of_cell[c]], S, stab, spre, H, eacc,
                                          wacc);
         }
     }
@@ -805,6 +805,7 @@ extern "C" int lj_batch_create(lj_batch **out, int32_t nrep, const int64_t *n, c
     WarpParams &k = b->k;
     k.gw = 0;
     k.n = (int)ntot;
+    k.last = k.n - 1;
     k.nc = 0;
     k.ncell = ncell;
     k.cw = 0.f;

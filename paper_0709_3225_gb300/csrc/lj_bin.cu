@@ -23,7 +23,7 @@ __global__ void k_bin_count(const double *__restrict__ x, int n, double L, doubl
     int c = 0;
     if (valid) {
         double px = x[3 * (int64_t)i + 0], py = x[3 * (int64_t)i + 1], pz = x[3 * (int64_t)i + 2];
-        if (isfinite(px) && isfinite(py) && isfinite(pz)) {
+        if (finite64(px) && finite64(py) && finite64(pz)) {
             int cx = lj_cell1(lj_wrap_fast(px, L, whi, wlo), s, nc);
             int cy = lj_cell1(lj_wrap_fast(py, L, whi, wlo), s, nc);
             int cz = lj_cell1(lj_wrap_fast(pz, L, whi, wlo), s, nc);
@@ -272,7 +272,8 @@ constexpr int kScatterPer = 1;
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_scatter(const double *__restrict__ x, int n, double L, double whi,
-                                                 double wlo, const double *__restrict__ centre, int nc,
+                                                 double wlo, const double *__restrict__ centre,
+                                                 const float2 *__restrict__ centre2, int nc,
                                                  float inv_nc, bool wrap, const int32_t *__restrict__ cell_of,
                                                  const int32_t *__restrict__ rank, const int32_t *__restrict__ start,
                                                  int32_t *__restrict__ perm, typename Vec4<T>::type *__restrict__ pos)
@@ -307,9 +308,15 @@ __global__ void __launch_bounds__(256) k_scatter(const double *__restrict__ x, i
         if (c < nc * nc * nc) {
             int cx, cy, cz;
             lj_cell_decode(c, nc, inv_nc, cx, cy, cz);
-            q.x = (T)(px - __ldg(centre + cx));
-            q.y = (T)(py - __ldg(centre + cy));
-            q.z = (T)(pz - __ldg(centre + cz));
+            if constexpr (sizeof(T) == 4) {
+                q.x = rel_f32(px, __ldg(centre2 + cx));
+                q.y = rel_f32(py, __ldg(centre2 + cy));
+                q.z = rel_f32(pz, __ldg(centre2 + cz));
+            } else {
+                q.x = px - __ldg(centre + cx);
+                q.y = py - __ldg(centre + cy);
+                q.z = pz - __ldg(centre + cz);
+            }
         } else {   // the extra cell of non-finite particles (never read as a neighbour)
             q.x = q.y = q.z = (T)px;
         }
@@ -412,11 +419,13 @@ cudaError_t launch_scatter(lj_ctx *c, const double *x, bool wrap)
         const unsigned grid = blocks_for(n, kScatterPer * 256);
         // inv_nc_f is 0 in contexts that do not set it (integer division)
         if (c->p.precision == LJ_PREC_FP64)
-            k_scatter<double><<<grid, 256, 0, c->stream>>>(x, n, c->p.box, c->wrap_hi, c->wrap_lo, c->centre, c->nc,
+            k_scatter<double><<<grid, 256, 0, c->stream>>>(x, n, c->p.box, c->wrap_hi, c->wrap_lo, c->centre,
+                                                            c->centre2, c->nc,
                                                             c->inv_nc_f, wrap, c->cell_of, c->rank, c->start, c->perm,
                                                             (double4_16a *)c->pos);
         else
-            k_scatter<float><<<grid, 256, 0, c->stream>>>(x, n, c->p.box, c->wrap_hi, c->wrap_lo, c->centre, c->nc,
+            k_scatter<float><<<grid, 256, 0, c->stream>>>(x, n, c->p.box, c->wrap_hi, c->wrap_lo, c->centre,
+                                                            c->centre2, c->nc,
                                                            c->inv_nc_f, wrap, c->cell_of, c->rank, c->start, c->perm,
                                                            (float4 *)c->pos);
         c->kernel_launches++;

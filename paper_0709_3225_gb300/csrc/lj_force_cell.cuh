@@ -40,6 +40,13 @@ struct WarpParams {
     float cw;
     float rc2, rc, a12, b6, c12, c6, uc, fc;
     float inv_nc;                // 1 / nc (cell-id decoding of the pair-once kernel)
+    int last;                    // last index of the position array (the pair-once kernel's clamp)
+    // slotted cells (lj_slots.cuh; the pair-once kernel of single systems)
+    int scap, nslots;
+    const int2 *cellq;           // (count, overflow list head + 1) per cell
+    int2 *cellq_next;            // the next binning's, zeroed by this launch (ncell + 1 entries)
+    unsigned *octr_next;
+    const int32_t *onext;
 };
 
 __device__ __forceinline__ float rcp_approx(float x)
@@ -582,6 +589,7 @@ inline WarpParams warp_params_of(const lj_ctx *c)
     k.grab = c->grab;
     k.work = c->work;
     k.n = (int)c->p.n;
+    k.last = k.n - 1;
     k.nc = c->nc;
     k.cap = c->wcap;
     k.ncell = c->ncell;

@@ -6,7 +6,9 @@
 
 namespace {
 
-template <int MODE, bool ENERGY>
+// SLOTS: slotted cells (start unused); the launch also zeroes the next
+// binning's counts.
+template <int MODE, bool ENERGY, bool SLOTS>
 __global__ void __launch_bounds__(kN3Threads, 6) k_force_n3(WarpParams k, const float4 *__restrict__ pos,
                                                          const int32_t *__restrict__ start, float4 *__restrict__ fout,
                                                          double *__restrict__ partial)
@@ -20,8 +22,17 @@ __global__ void __launch_bounds__(kN3Threads, 6) k_force_n3(WarpParams k, const 
     float4 *H = reinterpret_cast<float4 *>(spre + 16);
     const int nc = k.nc;
     double eacc = 0.0, wacc = 0.0;
-    auto one_cell = [&](HalfLoad tl) {
-        n3_cell<MODE, ENERGY, true>(k, pos, fout, tl, k.cw, S, stab, spre, H, eacc, wacc);
+    if constexpr (SLOTS) {
+        start = reinterpret_cast<const int32_t *>(k.cellq);
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
+            k.cellq_next[k.ncell] = make_int2(0, 0);
+            *k.octr_next = 0u;
+        }
+    }
+    auto load = [&](int c) { return half_load<true, SLOTS>(start, c, nc, k.inv_nc, 0, k.scap); };
+    auto one_cell = [&](HalfLoad tl, int c) {
+        if (SLOTS && lane == 31) k.cellq_next[c] = make_int2(0, 0);
+        n3_cell<MODE, ENERGY, true, SLOTS>(k, pos, fout, tl, c, k.cw, S, stab, spre, H, eacc, wacc);
     };
     if (k.grab > 0) {
         // pulls of k.grab cells, then single cells over the last stretch (two
@@ -38,21 +49,21 @@ __global__ void __launch_bounds__(kN3Threads, 6) k_force_n3(WarpParams k, const 
             last = c0;
             const int c1 = (int)min((int64_t)c0 + g, k.ncell);
             // the next cell's table loads are issued before this cell's work
-            HalfLoad nxt = half_load<true>(start, (int)c0, nc, k.inv_nc);
+            HalfLoad nxt = load((int)c0);
             for (int c = (int)c0; c < c1; c++) {
                 const HalfLoad cur = nxt;
-                if (c + 1 < c1) nxt = half_load<true>(start, c + 1, nc, k.inv_nc);
-                one_cell(cur);
+                if (c + 1 < c1) nxt = load(c + 1);
+                one_cell(cur, c);
             }
         }
     } else {
         const int nwarps = gridDim.x * (kN3Threads / 32);
         int c = blockIdx.x * (kN3Threads / 32) + warp;
-        HalfLoad nxt = half_load<true>(start, c < k.ncell ? c : 0, nc, k.inv_nc);
+        HalfLoad nxt = load(c < k.ncell ? c : 0);
         for (; c < k.ncell; c += nwarps) {
             const HalfLoad cur = nxt;
-            if (c + nwarps < k.ncell) nxt = half_load<true>(start, c + nwarps, nc, k.inv_nc);
-            one_cell(cur);
+            if (c + nwarps < k.ncell) nxt = load(c + nwarps);
+            one_cell(cur, c);
         }
     }
     if constexpr (ENERGY) {
@@ -78,16 +89,22 @@ __global__ void __launch_bounds__(kN3Threads, 6) k_force_n3(WarpParams k, const 
     }
 }
 
-void *n3_kernel(int mode, bool energy)
+template <bool SLOTS>
+void *n3_kernel_of(int mode, bool energy)
 {
     switch (mode * 2 + (energy ? 1 : 0)) {
-        case 0: return (void *)k_force_n3<0, false>;
-        case 1: return (void *)k_force_n3<0, true>;
-        case 2: return (void *)k_force_n3<1, false>;
-        case 3: return (void *)k_force_n3<1, true>;
-        case 4: return (void *)k_force_n3<2, false>;
-        default: return (void *)k_force_n3<2, true>;
+        case 0: return (void *)k_force_n3<0, false, SLOTS>;
+        case 1: return (void *)k_force_n3<0, true, SLOTS>;
+        case 2: return (void *)k_force_n3<1, false, SLOTS>;
+        case 3: return (void *)k_force_n3<1, true, SLOTS>;
+        case 4: return (void *)k_force_n3<2, false, SLOTS>;
+        default: return (void *)k_force_n3<2, true, SLOTS>;
     }
+}
+
+void *n3_kernel(int mode, bool energy, bool slots)
+{
+    return slots ? n3_kernel_of<true>(mode, energy) : n3_kernel_of<false>(mode, energy);
 }
 
 }  // namespace
@@ -110,14 +127,14 @@ cudaError_t n3_force_configure(lj_ctx *c)
     c->n3_smem = (kN3Threads / 32) * n3_slice_words(cap) * (int)sizeof(float);
     int minblk = 1 << 30;
     for (int mode = 0; mode < 3; mode++)
-        for (int en = 0; en < 2; en++) {
-            void *kern = n3_kernel(mode, en != 0);
+        for (int en = 0; en < 4; en++) {
+            void *kern = n3_kernel(mode, (en & 1) != 0, en >= 2);
             cudaError_t e = raise_dyn_smem(kern, c->n3_smem);
             if (e != cudaSuccess) return e;
             int nb = 0;
             e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, kN3Threads, c->n3_smem);
             if (e != cudaSuccess) return e;
-            if (en == 0 && nb < minblk) minblk = nb;   // the energy kernels get the same grid
+            if ((en & 1) == 0 && nb < minblk) minblk = nb;   // the energy kernels get the same grid
         }
     if (minblk < 1) minblk = 1;
     int64_t need = (c->ncell + kN3Threads / 32 - 1) / (kN3Threads / 32);
@@ -134,18 +151,29 @@ cudaError_t launch_force_n3(lj_ctx *c, void *f, bool energy)
     WarpParams k = warp_params_of(c);
     k.cap = c->n3cap;
     k.inv_nc = c->inv_nc_f;
-    const float4 *pos = (const float4 *)c->pos;
+    // the slotted binning, when it was one, has zeroed f
+    const bool slots = c->slots_open == 1;
+    const float4 *pos = slots ? c->spos : (const float4 *)c->pos;
     const int32_t *start = c->start;
+    if (slots) {
+        k.last = c->nslots + k.n - 1;
+        k.scap = c->scap;
+        k.nslots = c->nslots;
+        k.cellq = c->cellq[c->slot_par];
+        k.cellq_next = c->cellq[c->slot_par ^ 1];
+        k.octr_next = c->octr + (c->slot_par ^ 1);
+        k.onext = c->onext;
+    }
     double *partial = c->partial;
     void *args[] = {&k, (void *)&pos, (void *)&start, &f, &partial};
     if (c->timing && c->ev_used + 2 <= c->nev) cudaEventRecord(c->ev[c->ev_used], c->stream);
     // f must start at zero: zeroed here, unless the step zeroed it already
     // on its side stream
     cudaError_t e = cudaSuccess;
-    if (!c->f_prezeroed) e = cudaMemsetAsync(f, 0, (size_t)c->p.n * sizeof(float4), c->stream);
+    if (!c->f_prezeroed && !slots) e = cudaMemsetAsync(f, 0, (size_t)c->p.n * sizeof(float4), c->stream);
     c->f_prezeroed = 0;
     if (e == cudaSuccess)
-        e = cudaLaunchKernel(n3_kernel(c->p.shift_mode, energy), dim3(c->n3_grid), dim3(kN3Threads), args, c->n3_smem,
+        e = cudaLaunchKernel(n3_kernel(c->p.shift_mode, energy, slots), dim3(c->n3_grid), dim3(kN3Threads), args, c->n3_smem,
                              c->stream);
     if (c->timing && c->ev_used + 2 <= c->nev) {
         cudaEventRecord(c->ev[c->ev_used + 1], c->stream);
@@ -154,5 +182,6 @@ cudaError_t launch_force_n3(lj_ctx *c, void *f, bool energy)
     c->npartial = c->n3_grid;
     c->kernel_launches++;
     if (e != cudaSuccess) return e;
+    if (slots) slots_consumed(c);
     return cudaGetLastError();
 }

@@ -87,30 +87,41 @@ __host__ __device__ constexpr int n3_slice_words(int cap) { return 4 * cap + kN3
 // exclusive prefix sums of the counts, and returns the total.  Both are
 // called by all 32 lanes.  c is the cell's id in its grid of nc^3 cells,
 // whose ids start at cell_base in start[] (0 for a single system; the
-// replica's first cell in a batch); inv_nc as lj_cell_decode.
+// replica's first cell in a batch); inv_nc as lj_cell_decode.  scap > 0
+// (SLOTS): slotted cells of scap slots (lj_slots.cuh), `start` then being
+// the (count, list head) pairs; a count beyond scap shows in e - s.
 struct HalfLoad {
     int s, e;
 };
 
-template <bool NC>
+// Linear id of entry e of cell c's half stencil in a grid of nc^3 cells.
+__device__ __forceinline__ int half_cell(int c, int e, int nc, float inv_nc)
+{
+    int cx, cy, cz, dx, dy, dz;
+    lj_cell_decode(c, nc, inv_nc, cx, cy, cz);
+    half_delta(e, dx, dy, dz);
+    int ux = cx + dx, uy = cy + dy, uz = cz + dz;
+    ux += ux < 0 ? nc : 0;
+    ux -= ux >= nc ? nc : 0;
+    uy += uy < 0 ? nc : 0;
+    uy -= uy >= nc ? nc : 0;
+    uz += uz < 0 ? nc : 0;
+    uz -= uz >= nc ? nc : 0;
+    return ux + nc * (uy + nc * uz);   // < 2^31
+}
+
+template <bool NC, bool SLOTS = false>
 __device__ __forceinline__ HalfLoad half_load(const int32_t *__restrict__ start, int c, int nc, float inv_nc,
-                                              int cell_base = 0)
+                                              int cell_base = 0, int scap = 0)
 {
     const int lane = threadIdx.x & 31;
     HalfLoad t{0, 0};
     if (lane < kN3Half) {
-        int cx, cy, cz, dx, dy, dz;
-        lj_cell_decode(c, nc, inv_nc, cx, cy, cz);
-        half_delta(lane, dx, dy, dz);
-        int ux = cx + dx, uy = cy + dy, uz = cz + dz;
-        ux += ux < 0 ? nc : 0;
-        ux -= ux >= nc ? nc : 0;
-        uy += uy < 0 ? nc : 0;
-        uy -= uy >= nc ? nc : 0;
-        uz += uz < 0 ? nc : 0;
-        uz -= uz >= nc ? nc : 0;
-        const int cn = cell_base + ux + nc * (uy + nc * uz);   // < 2^31
-        if constexpr (NC) {
+        const int cn = cell_base + half_cell(c, lane, nc, inv_nc);
+        if constexpr (SLOTS) {
+            t.s = cn * scap;
+            t.e = t.s + __ldg(reinterpret_cast<const int2 *>(start) + cn).x;
+        } else if constexpr (NC) {
             t.s = __ldg(start + cn);
             t.e = __ldg(start + cn + 1);
         } else {
@@ -433,7 +444,7 @@ __device__ __forceinline__ bool n3_stage(const WarpParams &k, const float4 *__re
     const int j_entry = lane < __popc(nem) ? tmp[lane] : 0;
     __syncwarp();
     const unsigned le = (2u << lane) - 1u;
-    const int last = k.n - 1;
+    const int last = k.last;
     int T = 0;
     for (int t0 = 0; t0 < Ttot; t0 += 32 * kN3Batch) {
         float4 q[kN3Batch], sh[kN3Batch];
@@ -495,26 +506,39 @@ __device__ __forceinline__ bool n3_stage(const WarpParams &k, const float4 *__re
     return true;
 }
 
-// Plain path for a cell whose pruned half stencil overflows the slice: lane
-// = home particle, candidates read from global memory (all lanes the same
-// one), reactions summed over the warp.
-template <int MODE, bool ENERGY, bool NC>
+// Plain path for a cell whose pruned half stencil overflows the slice, or
+// that has a cell beyond its slots in the half stencil (SLOTS): lane = home
+// particle, candidates read from global memory (all lanes the same one; the
+// slots, then the cell's overflow list), reactions summed over the warp.
+template <int MODE, bool ENERGY, bool NC, bool SLOTS>
 __device__ void n3_plain(const WarpParams &k, const float4 *__restrict__ pos, float4 *__restrict__ fout,
-                         const float4 *stab, const int *spre, int s_home, int n_home, double &eacc, double &wacc)
+                         const float4 *stab, const int *spre, int c, int s_home, int n_home, double &eacc, double &wacc)
 {
     const int lane = threadIdx.x & 31;
     for (int p0 = 0; p0 < n_home; p0 += 32) {
         const int i = p0 + lane;
         const bool vi = i < n_home;
-        const float4 pi = load_pos<NC>(pos + s_home + (vi ? i : 0));
+        int si = s_home + (vi ? i : 0);
+        if (SLOTS && vi && i >= k.scap) {   // the (i - scap)-th of the home cell's overflow list
+            int o = __ldg(&k.cellq[c].y);
+            for (int m = k.scap; m < i; m++) o = __ldg(k.onext + o - 1);
+            si = k.nslots + o - 1;
+        }
+        const float4 pi = load_pos<NC>(pos + si);
         float fx = 0.f, fy = 0.f, fz = 0.f, e = 0.f, w = 0.f;
         for (int kk = 0; kk < kN3Half; kk++) {
             const float4 sh = stab[kk];
             const int s = __float_as_int(sh.w);
             const int nn = spre[kk + 1] - spre[kk];
             const float xs = pi.x - sh.x, ys = pi.y - sh.y, zs = pi.z - sh.z;
-            for (int j = (kk == 0 ? p0 + 1 : 0); j < nn; j++) {
-                const float4 q = load_pos<NC>(pos + s + j);
+            int o = 0;   // cursor of the overflow list: index + 1
+            for (int j = (kk == 0 && !SLOTS ? p0 + 1 : 0); j < nn; j++) {
+                int sj = s + j;
+                if (SLOTS && j >= k.scap) {
+                    o = j == k.scap ? __ldg(&k.cellq[half_cell(c, kk, k.nc, k.inv_nc)].y) : __ldg(k.onext + o - 1);
+                    sj = k.nslots + o - 1;
+                }
+                const float4 q = load_pos<NC>(pos + sj);
                 const float dx = xs - q.x, dy = ys - q.y, dz = zs - q.z;
                 const float r2 = dx * dx + dy * dy + dz * dz;
                 const bool in = vi && r2 < k.rc2 && (kk != 0 || j > i);
@@ -567,9 +591,10 @@ __device__ void n3_plain(const WarpParams &k, const float4 *__restrict__ pos, fl
 // spre, H: the warp's slice).  cw: the
 // cell side of the cell's grid.  NC: read-only loads of the sorted
 // positions (not when an earlier phase of the same launch writes them).
-template <int MODE, bool ENERGY, bool NC>
+// SLOTS: slotted cells; c: the cell's id.
+template <int MODE, bool ENERGY, bool NC, bool SLOTS>
 __device__ __forceinline__ void n3_cell(const WarpParams &k, const float4 *__restrict__ pos, float4 *__restrict__ fout,
-                                        HalfLoad tl, float cw, float4 *S, float4 *stab, int *spre, float4 *H,
+                                        HalfLoad tl, int c, float cw, float4 *S, float4 *stab, int *spre, float4 *H,
                                         double &eacc, double &wacc)
 {
     __syncwarp();   // the slice still holds the previous cell's data
@@ -578,10 +603,11 @@ __device__ __forceinline__ void n3_cell(const WarpParams &k, const float4 *__res
     if (n_home == 0) return;
     const int s_home = __float_as_int(stab[0].w);
     int T = 0;
-    if (n_home <= 32 && tot <= 2 * k.cap && n3_stage<NC>(k, pos, S, stab, spre, tot, s_home, n_home, T))
+    const bool over = SLOTS && __any_sync(0xffffffffu, tl.e - tl.s > k.scap);
+    if (!over && n_home <= 32 && tot <= 2 * k.cap && n3_stage<NC>(k, pos, S, stab, spre, tot, s_home, n_home, T))
         n3_compute<MODE, ENERGY>(k, fout, S, H, T, n_home, eacc, wacc);
     else
-        n3_plain<MODE, ENERGY, NC>(k, pos, fout, stab, spre, s_home, n_home, eacc, wacc);
+        n3_plain<MODE, ENERGY, NC, SLOTS>(k, pos, fout, stab, spre, c, s_home, n_home, eacc, wacc);
 }
 
 }  // namespace

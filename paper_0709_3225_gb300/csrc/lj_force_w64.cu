@@ -108,20 +108,6 @@ struct W64Layout {
     }
 };
 
-// FP32 value of a double by truncation of its IEEE-754 fields (relative
-// error below 2^-23; |x| < 2^-126 gives 0).  Exponent bias 1023 -> 127 is a
-// subtraction of 896 << 20 from the high word; the 23-bit mantissa is the
-// high word's 20 bits and the top 3 bits of the low word.  Integer
-// operations only: the filters never touch the FP64 pipe.
-__device__ __forceinline__ float f32_trunc(double x)
-{
-    const unsigned hi = (unsigned)__double2hiint(x);
-    const unsigned lo = (unsigned)__double2loint(x);
-    const unsigned mag = hi & 0x7fffffffu;
-    const unsigned b = mag >= (897u << 20) ? (((mag - (896u << 20)) << 3) | (lo >> 29)) : 0u;
-    return __uint_as_float(b | (hi & 0x80000000u));
-}
-
 __device__ __forceinline__ double3 load_xyz(const double4_16a *__restrict__ pos, int i)
 {
     const double2 *p2 = reinterpret_cast<const double2 *>(pos + i);

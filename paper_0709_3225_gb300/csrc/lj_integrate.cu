@@ -11,9 +11,15 @@ template <typename F4>
 __device__ __forceinline__ void load_f(const F4 *__restrict__ f, int i, double &fx, double &fy, double &fz)
 {
     F4 q = f[i];
-    fx = (double)q.x;
-    fy = (double)q.y;
-    fz = (double)q.z;
+    if constexpr (sizeof(q.x) == 4) {
+        fx = f64_of_f32(q.x);
+        fy = f64_of_f32(q.y);
+        fz = f64_of_f32(q.z);
+    } else {
+        fx = q.x;
+        fy = q.y;
+        fz = q.z;
+    }
 }
 
 // nkick half kicks v += h f (1 on the first step of a call, 2 when the
@@ -74,7 +80,7 @@ __global__ void __launch_bounds__(256) k_kick_drift_bin(double *__restrict__ x, 
             x[b] = px;
             x[b + 1] = py;
             x[b + 2] = pz;
-            if (isfinite(px) && isfinite(py) && isfinite(pz)) {
+            if (finite64(px) && finite64(py) && finite64(pz)) {
                 int ox, oy, oz;
                 lj_cell_decode(old[u], nc, inv_nc, ox, oy, oz);
                 c = lj_cell_from_guess(px, ox, thb, s, nc) +
@@ -119,7 +125,7 @@ __global__ void k_kick_drift_skin(double *__restrict__ x, double *__restrict__ v
         x[b] = px;
         x[b + 1] = py;
         x[b + 2] = pz;
-        if (!(isfinite(px) && isfinite(py) && isfinite(pz))) atomicOr(err, LJ_ERRBIT_NONFINITE);
+        if (!(finite64(px) && finite64(py) && finite64(pz))) atomicOr(err, LJ_ERRBIT_NONFINITE);
         float4 d = disp[i];
         d.x += (float)(dt * vx);
         d.y += (float)(dt * vy);

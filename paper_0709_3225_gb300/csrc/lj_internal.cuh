@@ -51,6 +51,7 @@ struct lj_ctx {
     int32_t *cell_of, *rank, *count, *start, *perm;
     void *pos;           // float4 or double4_16a [n], sorted, cell-centred coordinates
     double *centre;      // [nc] cell-centre coordinate (k + 1/2) L / nc
+    float2 *centre2;     // [nc] the same as two floats (rel_f32)
     long long *thb;      // [nc + 1] bits of the cell thresholds (lj_cell_from_guess)
     double wrap_hi, wrap_lo;  // lj_wrap_fast bounds
     int32_t *tile_sum;
@@ -121,9 +122,22 @@ struct lj_ctx {
     cudaStream_t zero_stream;
     cudaEvent_t ev_zfork, ev_zjoin;
     int f_prezeroed;
+    // slotted cells (lj_slots.cuh; see uses_slots): scap = slots per cell
+    // (0: not set up).  cellq[2]: (count, overflow list head) per cell, in
+    // two buffers: the binning fills slot_par's, which is zero by then, and
+    // the force (VJP) kernel after it zeroes the other one.
+    int scap, nslots;        // nslots = ncell * scap; spos holds nslots + n
+    int2 *cellq[2];
+    unsigned *octr;          // [2] overflow particles per buffer
+    float4 *spos, *sg4;      // slotted positions; cotangents (lazily allocated)
+    int32_t *onext;          // overflow lists: index + 1 of the next, 0 = end
+    int slot_par;            // buffer of the next binning
+    int slots_open;          // 1: a slotted binning waits for its kernel, 2: the buffers are not known to be zero
+    int slots_last;          // the last binning was a slotted one
     // graph replay of the middle steps of lj_step (lj_set_graph)
     int use_graph;
-    cudaGraphExec_t gexec;   // one captured middle step
+    cudaGraphExec_t gexec;   // captured middle steps: two with slotted cells (one per buffer), else one
+    int gsteps, gpar;        // how many; slot_par at their start
     const void *gx, *gv, *gf;
     int gen, ggen;       // configuration generation; the one captured
     int64_t glaunches;   // kernel launches in one captured step
@@ -218,14 +232,15 @@ __device__ __forceinline__ void lj_cell_decode(int c, int nc, float inv_nc, int 
 // the warp: lanes holding the same cell id are grouped with match.any, the
 // lowest lane adds the group size, and ranks follow lane order inside the
 // group.  All 32 lanes must call it (valid = false lanes get no rank).
-__device__ __forceinline__ int lj_warp_rank(int32_t *count, int c, bool valid)
+// Cell c's counter is count[stride c].
+__device__ __forceinline__ int lj_warp_rank(int32_t *count, int c, bool valid, int stride = 1)
 {
     const unsigned key = valid ? (unsigned)c : 0xffffffffu;
     const unsigned peers = __match_any_sync(0xffffffffu, key);
     const int lane = threadIdx.x & 31;
     const int leader = __ffs(peers) - 1;
     int base = 0;
-    if (valid && lane == leader) base = atomicAdd(count + c, __popc(peers));
+    if (valid && lane == leader) base = atomicAdd(count + (int64_t)stride * c, __popc(peers));
     base = __shfl_sync(0xffffffffu, base, leader);
     return base + __popc(peers & ((1u << lane) - 1u));
 }
@@ -269,6 +284,62 @@ __device__ __forceinline__ int lj_cell_from_guess(double w, int g, const long lo
         if (g >= nc || b >= __ldg(thb + g + 1)) return lj_cell1(w, s, nc);
     }
     return g;
+}
+
+// FP32 value of a double by truncation of its IEEE-754 fields (relative
+// error below 2^-23; |x| < 2^-126 gives 0).  Exponent bias 1023 -> 127 is a
+// subtraction of 896 << 20 from the high word; the 23-bit mantissa is the
+// high word's 20 bits and the top 3 bits of the low word.  Integer
+// operations only: the filters never touch the FP64 pipe.
+__device__ __forceinline__ float f32_trunc(double x)
+{
+    const unsigned hi = (unsigned)__double2hiint(x);
+    const unsigned lo = (unsigned)__double2loint(x);
+    const unsigned mag = hi & 0x7fffffffu;
+    const unsigned b = mag >= (897u << 20) ? (((mag - (896u << 20)) << 3) | (lo >> 29)) : 0u;
+    return __uint_as_float(b | (hi & 0x80000000u));
+}
+
+// A float as a double by integer operations, exactly: this GPU converts and
+// adds doubles at 2 per clock per SM (1/64 of FP32), and in the update and
+// scatter kernels those conversions and subtractions, not memory, set the
+// time (measured: 18 FP64-pipe instructions per particle held the slotted
+// update at 4M particles to 207 us; the 6 FMAs that remain take 38 us of the
+// pipe).  Zeros, denormals, infinities and NaN take the conversion.
+__device__ __forceinline__ double f64_of_f32(float f)
+{
+    const unsigned u = __float_as_uint(f);
+    const unsigned e = u & 0x7f800000u;
+    if ((u << 1) == 0u) return __hiloint2double((int)u, 0);
+    if (e == 0u || e == 0x7f800000u) return (double)f;
+    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20))), (int)(u << 29));
+}
+
+__device__ __forceinline__ bool finite64(double x)
+{
+    return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000;
+}
+
+// (float)(x - c) for a wrapped x in [0, L) and a cell centre c given as two
+// floats (c = c.x + c.y, c.x its nearest float), without the FP64 pipe: x =
+// h + l with h its leading 24 bits and l the other 29 (as a float, rounded
+// to 2^-48 x); h - c.x with its rounding error (a two-sum), then the low
+// parts.  Rounded to nearest but for an absolute error of 2^-48 x, at most
+// 2^-37 cell sides (x <= 1290 of them), far below the 2^-25 of the rounding:
+// 3 in 10^5 results differ from (float)(x - c) in their last place at L = 168.
+__device__ __forceinline__ float rel_f32(double x, float2 c)
+{
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    const float h = f32_trunc(x);
+    // 2^(e - 1075), the weight of the mantissa's last bit, as a float; 0
+    // where it is below 2^-126 (x < 2^-74)
+    const int ew = (int)((hi >> 20) & 0x7ffu) - 1075 + 127;
+    const float w = __uint_as_float(ew > 0 ? (unsigned)ew << 23 : 0u);
+    const float s = __fsub_rn(h, c.x);
+    const float bb = __fsub_rn(s, h);
+    const float e = __fsub_rn(__fsub_rn(h, __fsub_rn(s, bb)), __fadd_rn(c.x, bb));
+    const float l = __fmaf_rn(__uint2float_rn(lo & 0x1fffffffu), w, -c.y);
+    return __fadd_rn(s, __fadd_rn(l, e));
 }
 
 template <typename T> struct Vec4;
@@ -315,7 +386,9 @@ int check_dev_ptr(const void *ptr, size_t align);
 cudaError_t warp_force_configure(lj_ctx *c);
 // Staged-candidate capacity per warp of the warp kernels (lj_force_warp.cu).
 int warp_stencil_cap(double mean_occupancy, int subdiv, int threads, int static_bytes);
-cudaError_t launch_vjp(lj_ctx *c, const double *g, double scale, double *dx, double *dparam);
+// lam (NULL: not): then also lam += dt_axpy * dx, with the updated dx.
+cudaError_t launch_vjp(lj_ctx *c, const double *g, double scale, double *dx, double *dparam, double *lam = nullptr,
+                       double dt_axpy = 0.0);
 cudaError_t launch_axpy(lj_ctx *c, double *y, const double *x, double a);
 cudaError_t launch_force_warp(lj_ctx *c, void *f, bool energy);
 // FP64 warp kernel with compacted pair lists (lj_force_w64.cu); it uses the
@@ -332,7 +405,8 @@ cudaError_t pipe_force_configure(lj_ctx *c);
 cudaError_t launch_force_pipe(lj_ctx *c, void *f, bool energy);
 // rand48 streams and the Langevin update (lj_rand48.cu).
 cudaError_t launch_r48_seed(uint64_t *state, int64_t S, uint64_t x0, cudaStream_t stream);
-cudaError_t launch_langevin_bin(lj_ctx *c, double *x, double *v, const void *f, int nkick, double gamma, double kT);
+// (f zeroed with slotted cells.)
+cudaError_t launch_langevin_bin(lj_ctx *c, double *x, double *v, void *f, int nkick, double gamma, double kT);
 
 // One bounded mbarrier wait that cannot complete (lj_force.cu).
 cudaError_t launch_wait_selftest(lj_ctx *c);
@@ -352,5 +426,21 @@ bool uses_force_n3(const lj_ctx *c);   // launch_force dispatches to the pair-on
 // eps = 1, its sigma-derivative, eps, 1 / sigma); sums into acc (float4
 // [n], zeroed there), parameter partials into c->partial (*grid_out).
 bool uses_vjp_n3(const lj_ctx *c);
-cudaError_t launch_vjp_n3(lj_ctx *c, const double *coef, double scale, double *dx, float4 *acc, int *grid_out);
+// lam: also lam += dt_axpy * dx (NULL: not); dparam += scale * the sums.
+cudaError_t launch_vjp_n3(lj_ctx *c, const double *coef, double scale, double *dx, float4 *acc, double *dparam,
+                          double *lam, double dt_axpy);
+// Slotted cells (lj_slots.cu): set up for the context's grid (scap stays 0
+// where they do not apply), whether force evaluations take them, and the
+// binning: bin x (any coordinates), zero `zero` (float4 [n]), and with g
+// copy the cotangents beside the positions.
+cudaError_t slots_setup(lj_ctx *c);
+void slots_free(lj_ctx *c);
+bool uses_slots(const lj_ctx *c);
+cudaError_t launch_bin_slots(lj_ctx *c, const double *x, float4 *zero, const double *g);
+cudaError_t launch_kick_drift_slots(lj_ctx *c, double *x, double *v, float4 *f, int nkick, int64_t i_begin = 0,
+                                    int64_t i_end = -1);
+cudaError_t slots_begin(lj_ctx *c, int64_t i_begin);   // before a slotted binning launch
+void slots_consumed(lj_ctx *c);                        // after the launch that reads it
+// Rebuild cell_of, start and perm from the last slotted binning.
+cudaError_t launch_slots_to_lists(lj_ctx *c);
 cudaError_t launch_force_n3(lj_ctx *c, void *f, bool energy);

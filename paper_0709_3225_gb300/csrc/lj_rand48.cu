@@ -16,7 +16,7 @@
 // A x += (dt/2) v, wrap, bin; after the force the closing B.  xi from
 // Box-Muller on four uniforms per particle and step: stream i is particle
 // i, S = n, and step s uses series elements (4 s + k) n + i + 1, k = 0..3.
-#include "lj_internal.cuh"
+#include "lj_slots.cuh"
 
 namespace {
 
@@ -116,6 +116,55 @@ __device__ __forceinline__ void box_muller(uint64_t a, uint64_t b, T &z0, T &z1)
     }
 }
 
+// One BAOAB update of particle i, random numbers included: x, v and the
+// stream advance, the wrapped position is returned in p.
+template <typename F4, typename T>
+__device__ __forceinline__ void baoab(double *__restrict__ x, double *__restrict__ v, F4 q, int i, double hk, double hdt,
+                                      double c1, double c2s, double L, double whi, double wlo,
+                                      uint64_t *__restrict__ state, uint64_t A, uint64_t C, double *p)
+{
+    // four series elements of this particle for this step
+    const uint64_t u0 = state[i];
+    const uint64_t u1 = r48_next(u0, A, C);
+    const uint64_t u2 = r48_next(u1, A, C);
+    const uint64_t u3 = r48_next(u2, A, C);
+    state[i] = r48_next(u3, A, C);
+    T z0, z1, z2, z3;
+    box_muller<T>(u0, u1, z0, z1);
+    box_muller<T>(u2, u3, z2, z3);
+    (void)z3;
+    const int64_t b = 3 * (int64_t)i;
+    double xi[3], fq[3];
+    if constexpr (sizeof(T) == 4) {
+        xi[0] = f64_of_f32(z0);
+        xi[1] = f64_of_f32(z1);
+        xi[2] = f64_of_f32(z2);
+    } else {
+        xi[0] = z0;
+        xi[1] = z1;
+        xi[2] = z2;
+    }
+    if constexpr (sizeof(q.x) == 4) {
+        fq[0] = f64_of_f32(q.x);
+        fq[1] = f64_of_f32(q.y);
+        fq[2] = f64_of_f32(q.z);
+    } else {
+        fq[0] = q.x;
+        fq[1] = q.y;
+        fq[2] = q.z;
+    }
+#pragma unroll
+    for (int d = 0; d < 3; d++) {
+        double vv = __fma_rn(hk, fq[d], v[b + d]);
+        double xx = __fma_rn(hdt, vv, x[b + d]);
+        vv = __fma_rn(c2s, xi[d], c1 * vv);
+        xx = __fma_rn(hdt, vv, xx);
+        p[d] = lj_wrap_fast(xx, L, whi, wlo);
+        v[b + d] = vv;
+        x[b + d] = p[d];
+    }
+}
+
 template <typename F4, typename T>
 __global__ void k_langevin_bin(double *__restrict__ x, double *__restrict__ v, const F4 *__restrict__ f, int n,
                                double hk, double hdt, double c1, double c2s, double L, double whi, double wlo,
@@ -127,31 +176,9 @@ __global__ void k_langevin_bin(double *__restrict__ x, double *__restrict__ v, c
     const bool valid = i < n;
     int c = 0;
     if (valid) {
-        // four series elements of this particle for this step
-        const uint64_t u0 = state[i];
-        const uint64_t u1 = r48_next(u0, A, C);
-        const uint64_t u2 = r48_next(u1, A, C);
-        const uint64_t u3 = r48_next(u2, A, C);
-        state[i] = r48_next(u3, A, C);
-        T z0, z1, z2, z3;
-        box_muller<T>(u0, u1, z0, z1);
-        box_muller<T>(u2, u3, z2, z3);
-        (void)z3;
-        const double xi[3] = {(double)z0, (double)z1, (double)z2};
-        const int64_t b = 3 * (int64_t)i;
-        const F4 q = f[i];
-        const double fq[3] = {(double)q.x, (double)q.y, (double)q.z};
         double p[3];
-        for (int d = 0; d < 3; d++) {
-            double vv = __fma_rn(hk, fq[d], v[b + d]);
-            double xx = __fma_rn(hdt, vv, x[b + d]);
-            vv = __fma_rn(c2s, xi[d], c1 * vv);
-            xx = __fma_rn(hdt, vv, xx);
-            p[d] = lj_wrap_fast(xx, L, whi, wlo);
-            v[b + d] = vv;
-            x[b + d] = p[d];
-        }
-        if (isfinite(p[0]) && isfinite(p[1]) && isfinite(p[2])) {
+        baoab<F4, T>(x, v, f[i], i, hk, hdt, c1, c2s, L, whi, wlo, state, A, C, p);
+        if (finite64(p[0]) && finite64(p[1]) && finite64(p[2])) {
             const int old = cell_of[i];
             const int ox = old % nc, oy = (old / nc) % nc, oz = old / (nc * nc);
             c = lj_cell_from_guess(p[0], ox, thb, s, nc) +
@@ -168,11 +195,30 @@ __global__ void k_langevin_bin(double *__restrict__ x, double *__restrict__ v, c
     }
 }
 
+// The same update with the slotted binning (lj_slots.cuh); f is zeroed for
+// the force kernel, which adds into it.
+__global__ void __launch_bounds__(256) k_langevin_slots(SlotBin b, double *__restrict__ x, double *__restrict__ v,
+                                                        float4 *__restrict__ f, int n, double hk, double hdt, double c1,
+                                                        double c2s, uint64_t *__restrict__ state, uint64_t A, uint64_t C,
+                                                        int32_t *__restrict__ err)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i == 0) *b.work = 0u;
+    const bool valid = i < n;
+    double p[3] = {0.0, 0.0, 0.0};
+    if (valid) {
+        const float4 q = f[i];
+        f[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        baoab<float4, float>(x, v, q, i, hk, hdt, c1, c2s, b.L, b.whi, b.wlo, state, A, C, p);
+    }
+    slot_place(b, valid, i, p[0], p[1], p[2], err);
+}
+
 inline unsigned grid_for(int64_t n, int threads) { return (unsigned)((n + threads - 1) / threads); }
 
 }  // namespace
 
-cudaError_t launch_langevin_bin(lj_ctx *c, double *x, double *v, const void *f, int nkick, double gamma, double kT)
+cudaError_t launch_langevin_bin(lj_ctx *c, double *x, double *v, void *f, int nkick, double gamma, double kT)
 {
     const int n = (int)c->p.n;
     if (n == 0) return cudaSuccess;
@@ -182,6 +228,14 @@ cudaError_t launch_langevin_bin(lj_ctx *c, double *x, double *v, const void *f, 
     const double c2s = sqrt(1.0 - c1 * c1) * sqrt(kT / m);
     uint64_t A, C;
     r48_jump((uint64_t)n, A, C);
+    if (uses_slots(c)) {
+        const cudaError_t e = slots_begin(c, 0);
+        if (e != cudaSuccess) return e;
+        k_langevin_slots<<<grid_for(n, 256), 256, 0, c->stream>>>(slot_bin_of(c), x, v, (float4 *)f, n, hk, 0.5 * dt, c1,
+                                                                  c2s, c->r48_state, A, C, c->err);
+        c->kernel_launches++;
+        return cudaGetLastError();
+    }
     if (c->p.precision == LJ_PREC_FP64)
         k_langevin_bin<double4_16a, double><<<grid_for(n, 256), 256, 0, c->stream>>>(
             x, v, (const double4_16a *)f, n, hk, 0.5 * dt, c1, c2s, c->p.box, c->wrap_hi, c->wrap_lo, c->inv_cw,

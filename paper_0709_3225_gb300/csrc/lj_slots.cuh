@@ -1,0 +1,82 @@
+// Slotted cells: the cell lists of the FP32-mixed pair-once kernels, built in
+// one pass over the particles.
+//
+// Section 3.1 of the paper keeps a cell's particles physically together in
+// a fixed number of placeholders.  Here cell c owns `cap` slots of the
+// sorted-position array, [c cap, (c + 1) cap), and a particle's slot is its
+// rank in the cell, which the binning's atomic count returns anyway: the
+// position goes straight to its slot, with no scan over the counts, no
+// second pass over x, and no cell-id and rank arrays in between.  Particles
+// beyond a cell's slots are not dropped: they go to an overflow region after
+// the slots, chained per cell (a lock-free push on the cell's list head),
+// which the kernels' plain path reads.  Non-finite particles are counted
+// in the extra cell ncell and get no slot.
+//
+// The counts must be zero when a binning starts.  They are held twice; the
+// force (or VJP) kernel that reads one buffer zeroes the other for the
+// next binning.
+#pragma once
+
+#include "lj_internal.cuh"
+
+struct SlotBin {
+    int2 *cellq;            // this binning's (count, list head + 1) per cell, zero before it
+    float4 *pos;            // [nslots + n]
+    int32_t *onext;
+    unsigned *octr, *work;  // overflow counter of this buffer; the force kernel's work counter, zeroed here
+    const float2 *centre;   // cell centres as two floats
+    const long long *thb;
+    double L, whi, wlo, s;
+    float sf;               // (float)s
+    int nc, ncell, cap, nslots;
+};
+
+#ifdef __CUDACC__
+namespace {
+
+// Cell of the wrapped position (px, py, pz); the guess comes from the FP32
+// truncated coordinates (integer work: no FP64-pipe multiply or conversion)
+// and lj_cell_from_guess makes it exact.
+__device__ __forceinline__ int3 slot_cell(const SlotBin &b, double px, double py, double pz)
+{
+    int3 c;
+    c.x = lj_cell_from_guess(px, __float2int_rz(f32_trunc(px) * b.sf), b.thb, b.s, b.nc);
+    c.y = lj_cell_from_guess(py, __float2int_rz(f32_trunc(py) * b.sf), b.thb, b.s, b.nc);
+    c.z = lj_cell_from_guess(pz, __float2int_rz(f32_trunc(pz) * b.sf), b.thb, b.s, b.nc);
+    return c;
+}
+
+// Rank particle i in its cell and store its position relative to the cell
+// centre.  All 32 lanes call it; lanes with valid = false do nothing.
+// Returns the slot, or -1 when none was taken.
+__device__ __forceinline__ int slot_place(const SlotBin &b, bool valid, int i, double px, double py, double pz,
+                                          int32_t *err)
+{
+    int c = 0;
+    int3 cc = make_int3(0, 0, 0);
+    if (valid) {
+        if (finite64(px) && finite64(py) && finite64(pz)) {
+            cc = slot_cell(b, px, py, pz);
+            c = cc.x + b.nc * (cc.y + b.nc * cc.z);
+        } else {
+            atomicOr(err, LJ_ERRBIT_NONFINITE);
+            c = b.ncell;
+        }
+    }
+    const int r = lj_warp_rank(reinterpret_cast<int32_t *>(b.cellq), c, valid, 2);
+    if (!valid || c >= b.ncell) return -1;
+    int slot = c * b.cap + r;
+    if (r >= b.cap) {   // overflow: the next free entry, pushed on the cell's list
+        const int k = (int)atomicAdd(b.octr, 1u);
+        slot = b.nslots + k;
+        b.onext[k] = atomicExch(&b.cellq[c].y, k + 1);
+    }
+    b.pos[slot] = make_float4(rel_f32(px, __ldg(b.centre + cc.x)), rel_f32(py, __ldg(b.centre + cc.y)),
+                              rel_f32(pz, __ldg(b.centre + cc.z)), __int_as_float(i));
+    return slot;
+}
+
+}  // namespace
+#endif
+
+SlotBin slot_bin_of(const lj_ctx *c);

@@ -39,9 +39,15 @@ constexpr int kVn3HomeStride = 2 * (4 + 2) + 1;   // float4 per lane group in th
 
 struct VjpN3Coef {
     float rc2, a1, b1, c8, c14, s12, s6, fc1, dfc1, eps, cw, inv_nc;
-    int n, nc, cap, grab;
+    int last, nc, cap, grab;   // last: last index of the position array
     int64_t ncell;
     unsigned *work;
+    // slotted cells, as WarpParams
+    int scap, nslots;
+    const int2 *cellq;
+    int2 *cellq_next;
+    unsigned *octr_next;
+    const int32_t *onext;
 };
 
 // Words of a warp's slice: S and SG (cap float4 each), the half-stencil
@@ -70,7 +76,7 @@ __device__ __forceinline__ bool vn3_stage(const VjpN3Coef &k, const float4 *__re
     const int j_entry = lane < __popc(nem) ? tmp[lane] : 0;
     __syncwarp();
     const unsigned le = (2u << lane) - 1u;
-    const int last = k.n - 1;
+    const int last = k.last;
     int T = 0;
     for (int t0 = 0; t0 < Ttot; t0 += 32 * kN3Batch) {
         float4 q[kN3Batch], qg[kN3Batch], sh[kN3Batch];
@@ -344,27 +350,39 @@ __device__ __forceinline__ void vn3_compute(const VjpN3Coef &k, float4 *__restri
 }
 
 // Plain path: lane = home particle, the half stencil's candidates read
-// from global memory (all lanes the same one), reactions summed over the
-// warp.
-template <int MODE>
+// from global memory (all lanes the same one; with SLOTS the slots, then the
+// cell's overflow list, as n3_plain), reactions summed over the warp.
+template <int MODE, bool SLOTS>
 __device__ void vn3_plain(const VjpN3Coef &k, const float4 *__restrict__ pos, const float4 *__restrict__ g4,
-                          float4 *__restrict__ acc, const float4 *stab, const int *spre, int s_home, int n_home,
+                          float4 *__restrict__ acc, const float4 *stab, const int *spre, int c, int s_home, int n_home,
                           double &acc_e, double &acc_s)
 {
     const int lane = threadIdx.x & 31;
     for (int p0 = 0; p0 < n_home; p0 += 32) {
         const int i = p0 + lane;
         const bool vi = i < n_home;
-        const float4 pi = __ldg(pos + s_home + (vi ? i : 0));
-        const float4 gi = __ldg(g4 + s_home + (vi ? i : 0));
+        int si = s_home + (vi ? i : 0);
+        if (SLOTS && vi && i >= k.scap) {
+            int o = __ldg(&k.cellq[c].y);
+            for (int m = k.scap; m < i; m++) o = __ldg(k.onext + o - 1);
+            si = k.nslots + o - 1;
+        }
+        const float4 pi = __ldg(pos + si);
+        const float4 gi = __ldg(g4 + si);
         float2 ax = f2(0.f), ay = f2(0.f), az = f2(0.f), te = f2(0.f), ts = f2(0.f);
         for (int kk = 0; kk < kN3Half; kk++) {
             const float4 sh = stab[kk];
             const int s = __float_as_int(sh.w);
             const int nn = spre[kk + 1] - spre[kk];
-            for (int j = (kk == 0 ? p0 + 1 : 0); j < nn; j++) {
-                const float4 q = __ldg(pos + s + j);
-                const float4 h = __ldg(g4 + s + j);
+            int o = 0;
+            for (int j = (kk == 0 && !SLOTS ? p0 + 1 : 0); j < nn; j++) {
+                int sj = s + j;
+                if (SLOTS && j >= k.scap) {
+                    o = j == k.scap ? __ldg(&k.cellq[half_cell(c, kk, k.nc, k.inv_nc)].y) : __ldg(k.onext + o - 1);
+                    sj = k.nslots + o - 1;
+                }
+                const float4 q = __ldg(pos + sj);
+                const float4 h = __ldg(g4 + sj);
                 float2 rx = f2(0.f), ry = f2(0.f), rz = f2(0.f);
                 // slot y is a far dummy; home pairs count for j > i only
                 vn3_pair2<MODE, true>(make_float2(pi.x, -kFar), make_float2(pi.y, -kFar), make_float2(pi.z, -kFar),
@@ -389,7 +407,7 @@ __device__ void vn3_plain(const VjpN3Coef &k, const float4 *__restrict__ pos, co
     }
 }
 
-template <int MODE>
+template <int MODE, bool SLOTS>
 __global__ void __launch_bounds__(kVn3Threads, 4) k_vjp_n3(VjpN3Coef k, const float4 *__restrict__ pos,
                                                          const float4 *__restrict__ g4,
                                                          const int32_t *__restrict__ start, float4 *__restrict__ acc,
@@ -404,6 +422,14 @@ __global__ void __launch_bounds__(kVn3Threads, 4) k_vjp_n3(VjpN3Coef k, const fl
     int *spre = reinterpret_cast<int *>(stab + kN3Half);
     float4 *H = reinterpret_cast<float4 *>(spre + 16);
     double acc_e = 0.0, acc_s = 0.0;
+    if constexpr (SLOTS) {   // as k_force_n3
+        start = reinterpret_cast<const int32_t *>(k.cellq);
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
+            k.cellq_next[k.ncell] = make_int2(0, 0);
+            *k.octr_next = 0u;
+        }
+    }
+    auto load = [&](int c) { return half_load<true, SLOTS>(start, c, k.nc, k.inv_nc, 0, k.scap); };
     // pulls of k.grab cells, single cells over the last stretch (as k_force_n3)
     const int64_t tail = 2 * (int64_t)k.grab * gridDim.x * (kVn3Threads / 32);
     unsigned last = 0;
@@ -415,19 +441,22 @@ __global__ void __launch_bounds__(kVn3Threads, 4) k_vjp_n3(VjpN3Coef k, const fl
         if ((int64_t)c0 >= k.ncell) break;
         last = c0;
         const int c1 = (int)min((int64_t)c0 + gr, k.ncell);
-        HalfLoad nxt = half_load<true>(start, (int)c0, k.nc, k.inv_nc);
+        HalfLoad nxt = load((int)c0);
         for (int c = (int)c0; c < c1; c++) {
             const HalfLoad cur = nxt;
-            if (c + 1 < c1) nxt = half_load<true>(start, c + 1, k.nc, k.inv_nc);
+            if (c + 1 < c1) nxt = load(c + 1);
+            if (SLOTS && lane == 31) k.cellq_next[c] = make_int2(0, 0);
             __syncwarp();   // the slice still holds the previous cell's data
             const int tot = half_finish(cur, k.cw, stab, spre);
             const int n_home = spre[1];
             if (n_home == 0) continue;
             int T = 0;
-            if (n_home <= 32 && tot <= 2 * k.cap && vn3_stage(k, pos, g4, S, SG, stab, spre, tot, n_home, T))
+            const bool over = SLOTS && __any_sync(0xffffffffu, cur.e - cur.s > k.scap);
+            if (!over && n_home <= 32 && tot <= 2 * k.cap && vn3_stage(k, pos, g4, S, SG, stab, spre, tot, n_home, T))
                 vn3_compute<MODE>(k, acc, S, SG, H, T, n_home, acc_e, acc_s);
             else
-                vn3_plain<MODE>(k, pos, g4, acc, stab, spre, __float_as_int(stab[0].w), n_home, acc_e, acc_s);
+                vn3_plain<MODE, SLOTS>(k, pos, g4, acc, stab, spre, c, __float_as_int(stab[0].w), n_home, acc_e,
+                                       acc_s);
         }
     }
     __shared__ double red[2 * (kVn3Threads / 32)];
@@ -451,22 +480,60 @@ __global__ void __launch_bounds__(kVn3Threads, 4) k_vjp_n3(VjpN3Coef k, const fl
     }
 }
 
-// dx[i] += scale * acc[i] (FP64), particle order.
-__global__ void k_add_scaled_acc(const float4 *__restrict__ acc, int n, double scale, double *__restrict__ dx)
+// dx[i] += scale * acc[i] (FP64), particle order, then with lam also lam += a
+// dx (the drift of the velocity-Verlet adjoint); block 0 adds scale times the
+// sum of the parameter partials to dparam instead (fixed order).  One launch
+// for what were three: at 32,000 particles each took 3 to 6 us.
+__global__ void __launch_bounds__(kReduceThreads) k_vjp_finish(const float4 *__restrict__ acc, int n, double scale,
+                                                               double *__restrict__ dx, double *__restrict__ lam,
+                                                               double a, const double *__restrict__ partial, int np,
+                                                               double *__restrict__ dparam)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (blockIdx.x == 0) {
+        __shared__ double se[kReduceThreads], ss[kReduceThreads];
+        double e = 0.0, s = 0.0;
+        for (int k = threadIdx.x; k < np; k += kReduceThreads) {
+            e += partial[2 * k];
+            s += partial[2 * k + 1];
+        }
+        se[threadIdx.x] = e;
+        ss[threadIdx.x] = s;
+        __syncthreads();
+        for (int w = kReduceThreads / 2; w > 0; w >>= 1) {
+            if (threadIdx.x < w) {
+                se[threadIdx.x] += se[threadIdx.x + w];
+                ss[threadIdx.x] += ss[threadIdx.x + w];
+            }
+            __syncthreads();
+        }
+        if (threadIdx.x == 0) {
+            dparam[0] += scale * se[0];
+            dparam[1] += scale * ss[0];
+        }
+        return;
+    }
+    const int i = (blockIdx.x - 1) * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const float4 q = acc[i];
     const int64_t b = 3 * (int64_t)i;
-    dx[b] = __fma_rn(scale, (double)q.x, dx[b]);
-    dx[b + 1] = __fma_rn(scale, (double)q.y, dx[b + 1]);
-    dx[b + 2] = __fma_rn(scale, (double)q.z, dx[b + 2]);
+    const double d0 = __fma_rn(scale, (double)q.x, dx[b]);
+    const double d1 = __fma_rn(scale, (double)q.y, dx[b + 1]);
+    const double d2 = __fma_rn(scale, (double)q.z, dx[b + 2]);
+    dx[b] = d0;
+    dx[b + 1] = d1;
+    dx[b + 2] = d2;
+    if (lam) {
+        lam[b] = __fma_rn(a, d0, lam[b]);
+        lam[b + 1] = __fma_rn(a, d1, lam[b + 1]);
+        lam[b + 2] = __fma_rn(a, d2, lam[b + 2]);
+    }
 }
 
-void *vn3_kernel(int mode)
+void *vn3_kernel(int mode, bool slots)
 {
     // modes 0 and 1 have the same force
-    return mode == 2 ? (void *)k_vjp_n3<2> : (void *)k_vjp_n3<0>;
+    if (slots) return mode == 2 ? (void *)k_vjp_n3<2, true> : (void *)k_vjp_n3<0, true>;
+    return mode == 2 ? (void *)k_vjp_n3<2, false> : (void *)k_vjp_n3<0, false>;
 }
 
 }  // namespace
@@ -474,11 +541,13 @@ void *vn3_kernel(int mode)
 bool uses_vjp_n3(const lj_ctx *c) { return uses_force_n3(c); }
 
 // The pair-once FP32-mixed VJP: the sums go to acc (float4 [n], particle
-// order, zeroed here), the parameter partials to c->partial (*grid_out of
-// them), and dx += scale acc.  The work counter must be zero (the scan of
-// the binning before it zeroes it).
-cudaError_t launch_vjp_n3(lj_ctx *c, const double *coef, double scale, double *dx, float4 *acc, int *grid_out)
+// order, zeroed here or by the slotted binning), the parameter partials to
+// c->partial, then dx += scale acc (and what k_vjp_finish does besides).  The
+// work counter must be zero (the binning before it zeroes it).
+cudaError_t launch_vjp_n3(lj_ctx *c, const double *coef, double scale, double *dx, float4 *acc, double *dparam,
+                          double *lam, double dt_axpy)
 {
+    const bool slots = c->slots_open == 1;
     const double *q = coef;
     const double mean = c->ncell > 0 ? (double)c->p.n / (double)c->ncell : 0.0;
     const double m = kN3Half * mean;
@@ -488,7 +557,7 @@ cudaError_t launch_vjp_n3(lj_ctx *c, const double *coef, double scale, double *d
     const int warps = kVn3Threads / 32;
     while (cap > kN3Home * 32 && warps * vn3_slice_words(cap) * (int)sizeof(float) > 227 * 1024 - 256) cap -= 32;
     const int smem = warps * vn3_slice_words(cap) * (int)sizeof(float);
-    void *kern = vn3_kernel(c->p.shift_mode);
+    void *kern = vn3_kernel(c->p.shift_mode, slots);
     cudaError_t e = raise_dyn_smem(kern, smem);
     if (e != cudaSuccess) return e;
     int nb = 0;
@@ -512,24 +581,33 @@ cudaError_t launch_vjp_n3(lj_ctx *c, const double *coef, double scale, double *d
     k.eps = (float)q[5];
     k.cw = (float)c->cw;
     k.inv_nc = c->inv_nc_f;
-    k.n = (int)c->p.n;
+    k.last = (slots ? c->nslots : 0) + (int)c->p.n - 1;
+    k.scap = c->scap;
+    k.nslots = c->nslots;
+    k.cellq = c->cellq[c->slot_par];
+    k.cellq_next = c->cellq[c->slot_par ^ 1];
+    k.octr_next = slots ? c->octr + (c->slot_par ^ 1) : nullptr;
+    k.onext = c->onext;
     k.nc = c->nc;
     k.cap = cap;
     k.grab = 4;
     k.ncell = c->ncell;
     k.work = c->work;
-    const float4 *pos = (const float4 *)c->pos;
-    const float4 *g4 = (const float4 *)c->g4;
+    const float4 *pos = slots ? c->spos : (const float4 *)c->pos;
+    const float4 *g4 = slots ? c->sg4 : (const float4 *)c->g4;
     const int32_t *start = c->start;
     double *partial = c->partial;
-    e = cudaMemsetAsync(acc, 0, (size_t)c->p.n * sizeof(float4), c->stream);
-    if (e != cudaSuccess) return e;
+    if (!slots) {
+        e = cudaMemsetAsync(acc, 0, (size_t)c->p.n * sizeof(float4), c->stream);
+        if (e != cudaSuccess) return e;
+    }
     void *args[] = {&k, (void *)&pos, (void *)&g4, (void *)&start, &acc, &partial};
     e = cudaLaunchKernel(kern, dim3((unsigned)grid), dim3(kVn3Threads), args, smem, c->stream);
     if (e != cudaSuccess) return e;
+    if (slots) slots_consumed(c);
     const int n = (int)c->p.n;
-    k_add_scaled_acc<<<(unsigned)((n + 255) / 256), 256, 0, c->stream>>>(acc, n, scale, dx);
+    k_vjp_finish<<<(unsigned)((n + kReduceThreads - 1) / kReduceThreads) + 1, kReduceThreads, 0, c->stream>>>(
+        acc, n, scale, dx, lam, dt_axpy, partial, (int)grid, dparam);
     c->kernel_launches += 2;
-    *grid_out = (int)grid;
     return cudaGetLastError();
 }
