@@ -203,7 +203,7 @@ int one_step(lj_ctx *c, double *x, double *v, void *f, int s, int nsteps, cudaEv
         if (s == 0 && c->kdb_done)
             c->kdb_done = 0;
         else
-            LJ_CK(launch_kick_drift_slots(c, x, v, (float4 *)f, s == 0 ? 1 : 2));
+            LJ_CK(launch_kick_drift_slots(c, x, v, (float4 *)f, s == 0 ? 1 : 2, 0, -1, s > 0 && !c->timing));
         if (x_final) LJ_CK(cudaEventRecord(x_final, c->stream));   // x holds its final value
         LJ_CK(launch_force(c, f, false));
         return LJ_OK;
@@ -390,7 +390,7 @@ int do_steps(lj_ctx *c, double *x, double *v, void *f, int nsteps, cudaEvent_t x
             if (r) return r;
         }
     }
-    if (!fused_mode(c)) LJ_CK(launch_kick(c, v, f));
+    if (!fused_mode(c)) LJ_CK(launch_kick(c, v, f, uses_slots(c) && !c->timing));
     if (x_final && fused_mode(c)) LJ_CK(cudaEventRecord(x_final, c->stream));
     return LJ_OK;
 }
@@ -726,14 +726,14 @@ extern "C" int lj_langevin_step(lj_ctx *c, double *x, double *v, void *f, int32_
     const bool slots = uses_slots(c);
     if (!slots) c->slots_last = 0;
     for (int s = 0; s < nsteps; s++) {
-        LJ_CK(launch_langevin_bin(c, x, v, f, s == 0 ? 1 : 2, gamma, kT));
+        LJ_CK(launch_langevin_bin(c, x, v, f, s == 0 ? 1 : 2, gamma, kT, slots && s > 0 && !c->timing));
         if (!slots) {
             LJ_CK(launch_scan(c));
             LJ_CK(launch_scatter(c, x, false));
         }
         LJ_CK(launch_force(c, f, false));
     }
-    LJ_CK(launch_kick(c, v, f));
+    LJ_CK(launch_kick(c, v, f, slots && !c->timing));
     return LJ_OK;
 }
 

@@ -360,8 +360,8 @@ __device__ void phase_force_n3(const BatchDev &b, const WarpParams &k, float4 *_
         for (int c = (int)c0; c < c1; c++) {
             const HalfLoad cur = nxt;
             if (c + 1 < c1) nxt = load(c + 1);
-            n3_cell<MODE, ENERGY, false, false>(k, b.pos, f, cur, c, (float)b.cw[b.rep_of_cell[c]], S, stab, spre, H, eacc,
-                                         wacc);
+            n3_cell<MODE, ENERGY, false, false, false>(k, b.pos, f, cur, c, 0, 0, (float)b.cw[b.rep_of_cell[c]], S, stab, spre, H,
+                                                eacc, wacc);
         }
     }
 }

@@ -41,6 +41,7 @@ struct WarpParams {
     float rc2, rc, a12, b6, c12, c6, uc, fc;
     float inv_nc;                // 1 / nc (cell-id decoding of the pair-once kernel)
     int last;                    // last index of the position array (the pair-once kernel's clamp)
+    int lgw;                     // pair-once kernel: a cell's candidates are split over 2^lgw warps
     // slotted cells (lj_slots.cuh; the pair-once kernel of single systems)
     int scap, nslots;
     const int2 *cellq;           // (count, overflow list head + 1) per cell

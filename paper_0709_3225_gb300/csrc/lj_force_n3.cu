@@ -7,9 +7,9 @@
 namespace {
 
 // SLOTS: slotted cells (start unused); the launch also zeroes the next
-// binning's counts.
-template <int MODE, bool ENERGY, bool SLOTS>
-__global__ void __launch_bounds__(kN3Threads, 6) k_force_n3(WarpParams k, const float4 *__restrict__ pos,
+// binning's counts.  SPLIT: each cell is 2^k.lgw items.
+template <int MODE, bool ENERGY, bool SLOTS, bool SPLIT>
+__global__ void __launch_bounds__(kN3Threads, ENERGY ? 4 : 6) k_force_n3(WarpParams k, const float4 *__restrict__ pos,
                                                          const int32_t *__restrict__ start, float4 *__restrict__ fout,
                                                          double *__restrict__ partial)
 {
@@ -23,6 +23,7 @@ __global__ void __launch_bounds__(kN3Threads, 6) k_force_n3(WarpParams k, const 
     const int nc = k.nc;
     double eacc = 0.0, wacc = 0.0;
     if constexpr (SLOTS) {
+        pdl_wait();
         start = reinterpret_cast<const int32_t *>(k.cellq);
         if (blockIdx.x == 0 && threadIdx.x == 0) {
             k.cellq_next[k.ncell] = make_int2(0, 0);
@@ -30,11 +31,16 @@ __global__ void __launch_bounds__(kN3Threads, 6) k_force_n3(WarpParams k, const 
         }
     }
     auto load = [&](int c) { return half_load<true, SLOTS>(start, c, nc, k.inv_nc, 0, k.scap); };
-    auto one_cell = [&](HalfLoad tl, int c) {
-        if (SLOTS && lane == 31) k.cellq_next[c] = make_int2(0, 0);
-        n3_cell<MODE, ENERGY, true, SLOTS>(k, pos, fout, tl, c, k.cw, S, stab, spre, H, eacc, wacc);
+    auto one_cell = [&](HalfLoad tl, int c, int part) {
+        if (SLOTS && lane == 31 && part == 0) k.cellq_next[c] = make_int2(0, 0);
+        n3_cell<MODE, ENERGY, true, SLOTS, SPLIT>(k, pos, fout, tl, c, part, k.lgw, k.cw, S, stab, spre, H, eacc, wacc);
     };
-    if (k.grab > 0) {
+    if constexpr (SPLIT) {
+        // at most one item per resident warp: no pulls
+        const int it = blockIdx.x * (kN3Threads / 32) + warp;
+        const int c = it >> k.lgw;
+        if (c < k.ncell) one_cell(load(c), c, it & ((1 << k.lgw) - 1));
+    } else if (k.grab > 0) {
         // pulls of k.grab cells, then single cells over the last stretch (two
         // rounds of pulls of the whole grid), so that the warps finish closer
         // together
@@ -53,7 +59,7 @@ __global__ void __launch_bounds__(kN3Threads, 6) k_force_n3(WarpParams k, const 
             for (int c = (int)c0; c < c1; c++) {
                 const HalfLoad cur = nxt;
                 if (c + 1 < c1) nxt = load(c + 1);
-                one_cell(cur, c);
+                one_cell(cur, c, 0);
             }
         }
     } else {
@@ -63,7 +69,7 @@ __global__ void __launch_bounds__(kN3Threads, 6) k_force_n3(WarpParams k, const 
         for (; c < k.ncell; c += nwarps) {
             const HalfLoad cur = nxt;
             if (c + nwarps < k.ncell) nxt = load(c + nwarps);
-            one_cell(cur, c);
+            one_cell(cur, c, 0);
         }
     }
     if constexpr (ENERGY) {
@@ -89,22 +95,24 @@ __global__ void __launch_bounds__(kN3Threads, 6) k_force_n3(WarpParams k, const 
     }
 }
 
-template <bool SLOTS>
+template <bool SLOTS, bool SPLIT>
 void *n3_kernel_of(int mode, bool energy)
 {
     switch (mode * 2 + (energy ? 1 : 0)) {
-        case 0: return (void *)k_force_n3<0, false, SLOTS>;
-        case 1: return (void *)k_force_n3<0, true, SLOTS>;
-        case 2: return (void *)k_force_n3<1, false, SLOTS>;
-        case 3: return (void *)k_force_n3<1, true, SLOTS>;
-        case 4: return (void *)k_force_n3<2, false, SLOTS>;
-        default: return (void *)k_force_n3<2, true, SLOTS>;
+        case 0: return (void *)k_force_n3<0, false, SLOTS, SPLIT>;
+        case 1: return (void *)k_force_n3<0, true, SLOTS, SPLIT>;
+        case 2: return (void *)k_force_n3<1, false, SLOTS, SPLIT>;
+        case 3: return (void *)k_force_n3<1, true, SLOTS, SPLIT>;
+        case 4: return (void *)k_force_n3<2, false, SLOTS, SPLIT>;
+        default: return (void *)k_force_n3<2, true, SLOTS, SPLIT>;
     }
 }
 
-void *n3_kernel(int mode, bool energy, bool slots)
+// form: 0 sorted lists, 1 slotted cells, 2 slotted and split
+void *n3_kernel(int mode, bool energy, int form)
 {
-    return slots ? n3_kernel_of<true>(mode, energy) : n3_kernel_of<false>(mode, energy);
+    return form == 2 ? n3_kernel_of<true, true>(mode, energy)
+                     : form == 1 ? n3_kernel_of<true, false>(mode, energy) : n3_kernel_of<false, false>(mode, energy);
 }
 
 }  // namespace
@@ -127,8 +135,8 @@ cudaError_t n3_force_configure(lj_ctx *c)
     c->n3_smem = (kN3Threads / 32) * n3_slice_words(cap) * (int)sizeof(float);
     int minblk = 1 << 30;
     for (int mode = 0; mode < 3; mode++)
-        for (int en = 0; en < 4; en++) {
-            void *kern = n3_kernel(mode, (en & 1) != 0, en >= 2);
+        for (int en = 0; en < 6; en++) {
+            void *kern = n3_kernel(mode, (en & 1) != 0, en >> 1);
             cudaError_t e = raise_dyn_smem(kern, c->n3_smem);
             if (e != cudaSuccess) return e;
             int nb = 0;
@@ -137,8 +145,16 @@ cudaError_t n3_force_configure(lj_ctx *c)
             if ((en & 1) == 0 && nb < minblk) minblk = nb;   // the energy kernels get the same grid
         }
     if (minblk < 1) minblk = 1;
-    int64_t need = (c->ncell + kN3Threads / 32 - 1) / (kN3Threads / 32);
     int64_t grid = (int64_t)minblk * c->nsm;
+    // Cells so few that warps would stand idle are split over 2 or 4 warps
+    // each, while that still gives every item a resident warp of its own: one
+    // warp takes a cell's chain of loads, staging and compute in 6 us alone,
+    // a share of it in 3 (step at 2,048 particles 16.5 -> 14.4 us, 10,007
+    // 17.2 -> 16.2; from two cells per warp up the shares' common work, the
+    // home particles' staging and the final sums, costs more than it gains).
+    c->n3_lgw = 0;
+    while (c->n3_lgw < 2 && (c->ncell << (c->n3_lgw + 1)) <= grid * (kN3Threads / 32)) c->n3_lgw++;
+    const int64_t need = ((c->ncell << c->n3_lgw) + kN3Threads / 32 - 1) / (kN3Threads / 32);
     if (grid > need) grid = need;
     if (grid < 1) grid = 1;
     c->n3_grid = (int)grid;
@@ -151,6 +167,7 @@ cudaError_t launch_force_n3(lj_ctx *c, void *f, bool energy)
     WarpParams k = warp_params_of(c);
     k.cap = c->n3cap;
     k.inv_nc = c->inv_nc_f;
+    k.lgw = c->n3_lgw;
     // the slotted binning, when it was one, has zeroed f
     const bool slots = c->slots_open == 1;
     const float4 *pos = slots ? c->spos : (const float4 *)c->pos;
@@ -173,8 +190,8 @@ cudaError_t launch_force_n3(lj_ctx *c, void *f, bool energy)
     if (!c->f_prezeroed && !slots) e = cudaMemsetAsync(f, 0, (size_t)c->p.n * sizeof(float4), c->stream);
     c->f_prezeroed = 0;
     if (e == cudaSuccess)
-        e = cudaLaunchKernel(n3_kernel(c->p.shift_mode, energy, slots), dim3(c->n3_grid), dim3(kN3Threads), args, c->n3_smem,
-                             c->stream);
+        e = launch_pdl(n3_kernel(c->p.shift_mode, energy, !slots ? 0 : c->n3_lgw > 0 ? 2 : 1), c->n3_grid, kN3Threads,
+                       args, c->n3_smem, c->stream, slots && !c->timing);
     if (c->timing && c->ev_used + 2 <= c->nev) {
         cudaEventRecord(c->ev[c->ev_used + 1], c->stream);
         c->ev_used += 2;

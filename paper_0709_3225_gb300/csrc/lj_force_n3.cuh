@@ -258,7 +258,7 @@ __device__ __forceinline__ float4 n3_ld4(const float4 *p)
     return q;
 }
 
-// One candidate block: lane (a, b) takes candidate blk B + b against its NH
+// One candidate block: lane (a, b) takes candidate j0 + b against its NH
 // home pairs (pairs past its home particles sit far away and add nothing),
 // then the candidate's reaction is added to f in two parts (see the file
 // header).
@@ -266,12 +266,11 @@ __device__ __forceinline__ float4 n3_ld4(const float4 *p)
 // pairs (0, 1) and (2, 3), one float4 each, then a float4 of padding so
 // that the groups' simultaneous reads fall in different banks.
 template <int NH, int LGB, int MODE, bool ENERGY, bool SELF>
-__device__ __forceinline__ void n3_block1(const WarpParams &k, float4 *__restrict__ fout, const float4 *S, int T, int blk,
+__device__ __forceinline__ void n3_block1(const WarpParams &k, float4 *__restrict__ fout, const float4 *S, int T, int j0,
                                           int a, int b, int A, const float4 *H, float2 *fx, float2 *fy, float2 *fz,
                                           float2 *fe, float2 &fw)
 {
-    constexpr int B = 1 << LGB;
-    const int j = (blk << LGB) + b;
+    const int j = j0 + b;
     const float4 c = S[j];
     const float2 cx = f2(c.x), cy = f2(c.y), cz = f2(c.z);
     float2 rx = f2(0.0f), ry = f2(0.0f), rz = f2(0.0f), re = f2(0.0f);
@@ -304,17 +303,17 @@ __device__ __forceinline__ void n3_block1(const WarpParams &k, float4 *__restric
 
 template <int NH, int LGB, int MODE, bool ENERGY>
 __device__ __forceinline__ void n3_blocks(const WarpParams &k, float4 *__restrict__ fout, const float4 *S, int T,
-                                          int n_home, int a, int b, int A, const float4 *H, float2 *fx, float2 *fy,
+                                          int jbeg, int n_home, int a, int b, int A, const float4 *H, float2 *fx, float2 *fy,
                                           float2 *fz, float2 *fe, float2 &fw)
 {
     constexpr int B = 1 << LGB;
-    const int nblk = (T + B - 1) >> LGB;
-    const int nself = min(nblk, (n_home + B - 1) >> LGB);   // blocks holding home particles
+    const int nblk = (T - jbeg + B - 1) >> LGB;
+    const int nself = min(nblk, (n_home - jbeg + B - 1) >> LGB);   // blocks holding home particles
     int blk = 0;
     for (; blk < nself; blk++)
-        n3_block1<NH, LGB, MODE, ENERGY, true>(k, fout, S, T, blk, a, b, A, H, fx, fy, fz, fe, fw);
+        n3_block1<NH, LGB, MODE, ENERGY, true>(k, fout, S, T, jbeg + (blk << LGB), a, b, A, H, fx, fy, fz, fe, fw);
     for (; blk < nblk; blk++)
-        n3_block1<NH, LGB, MODE, ENERGY, false>(k, fout, S, T, blk, a, b, A, H, fx, fy, fz, fe, fw);
+        n3_block1<NH, LGB, MODE, ENERGY, false>(k, fout, S, T, jbeg + (blk << LGB), a, b, A, H, fx, fy, fz, fe, fw);
 }
 
 // Compute phase of a cell of n_home <= 32 home particles staged in S (home
@@ -324,9 +323,10 @@ __device__ __forceinline__ void n3_blocks(const WarpParams &k, float4 *__restric
 // block against the home particles u A + a, u = 0..7, in FP32x2 pairs read
 // from the table H (kN3HomeStride float4 per group).  The home forces' transpose
 // reuses S once the candidate blocks are done (S holds >= kN3Home * 32).
+// jbeg: the first candidate, 0, or n_home for a part without the home pairs.
 template <int MODE, bool ENERGY>
 __device__ __forceinline__ void n3_compute(const WarpParams &k, float4 *__restrict__ fout, float4 *S, float4 *H,
-                                           int T, int n_home, double &eacc, double &wacc)
+                                           int T, int jbeg, int n_home, double &eacc, double &wacc)
 {
     const int lane = threadIdx.x & 31;
     const int hp = n_home;
@@ -354,18 +354,18 @@ __device__ __forceinline__ void n3_compute(const WarpParams &k, float4 *__restri
     const int nh = (nu + 1) >> 1;
     if (lgB == 4) {
         if (nh >= 4)
-            n3_blocks<4, 4, MODE, ENERGY>(k, fout, S, T, n_home, a, b, A, H, fx, fy, fz, fe, fw);
+            n3_blocks<4, 4, MODE, ENERGY>(k, fout, S, T, jbeg, n_home, a, b, A, H, fx, fy, fz, fe, fw);
         else if (nh == 3)
-            n3_blocks<3, 4, MODE, ENERGY>(k, fout, S, T, n_home, a, b, A, H, fx, fy, fz, fe, fw);
+            n3_blocks<3, 4, MODE, ENERGY>(k, fout, S, T, jbeg, n_home, a, b, A, H, fx, fy, fz, fe, fw);
         else
-            n3_blocks<2, 4, MODE, ENERGY>(k, fout, S, T, n_home, a, b, A, H, fx, fy, fz, fe, fw);
+            n3_blocks<2, 4, MODE, ENERGY>(k, fout, S, T, jbeg, n_home, a, b, A, H, fx, fy, fz, fe, fw);
     } else {
         if (nh >= 4)
-            n3_blocks<4, 3, MODE, ENERGY>(k, fout, S, T, n_home, a, b, A, H, fx, fy, fz, fe, fw);
+            n3_blocks<4, 3, MODE, ENERGY>(k, fout, S, T, jbeg, n_home, a, b, A, H, fx, fy, fz, fe, fw);
         else if (nh == 3)
-            n3_blocks<3, 3, MODE, ENERGY>(k, fout, S, T, n_home, a, b, A, H, fx, fy, fz, fe, fw);
+            n3_blocks<3, 3, MODE, ENERGY>(k, fout, S, T, jbeg, n_home, a, b, A, H, fx, fy, fz, fe, fw);
         else
-            n3_blocks<2, 3, MODE, ENERGY>(k, fout, S, T, n_home, a, b, A, H, fx, fy, fz, fe, fw);
+            n3_blocks<2, 3, MODE, ENERGY>(k, fout, S, T, jbeg, n_home, a, b, A, H, fx, fy, fz, fe, fw);
     }
     const int p = A == 2 ? lane >> 1 : lane;            // home particle of this lane
     const int bh = A == 2 ? (lane & 1) * 8 : 0;         // its half of the B columns
@@ -406,28 +406,17 @@ __device__ __forceinline__ void n3_compute(const WarpParams &k, float4 *__restri
     __syncwarp();
 }
 
-// Staging of the half stencil (see the file header) into S.  Returns false,
-// having computed nothing, when the kept candidates would not fit the slice.
-template <bool NC>
+// Staging of the half stencil (see the file header) into S: candidates
+// ta .. tb - 1 of it (ta = 0, or ta >= n_home and then the home particles
+// too, first).  n_home <= 32.  Returns false, having computed nothing, when
+// the kept candidates would not fit the slice.  SPLIT: ta may be above 0.
+template <bool NC, bool SPLIT>
 __device__ __forceinline__ bool n3_stage(const WarpParams &k, const float4 *__restrict__ pos, float4 *S,
-                                         const float4 *stab, const int *spre, int Ttot, int s_home, int n_home,
-                                         int &T_out)
+                                         const float4 *stab, const int *spre, int ta, int tb_end, int s_home,
+                                         int n_home, int &T_out)
 {
     const int lane = threadIdx.x & 31;
     float bxl = 3.4e38f, byl = 3.4e38f, bzl = 3.4e38f, bxh = -3.4e38f, byh = -3.4e38f, bzh = -3.4e38f;
-    if (n_home > 32) {   // bounding box from a pass of its own; else from the first staging round
-        for (int p0 = 0; p0 < n_home; p0 += 32) {
-            if (p0 + lane < n_home) {
-                const float4 q = load_pos<NC>(pos + s_home + p0 + lane);
-                bxl = fminf(bxl, q.x);
-                byl = fminf(byl, q.y);
-                bzl = fminf(bzl, q.z);
-                bxh = fmaxf(bxh, q.x);
-                byh = fmaxf(byh, q.y);
-                bzh = fmaxf(bzh, q.z);
-            }
-        }
-    }
     // the margin of the box test (0.01 % of rc^2) covers the FP32 rounding of
     // the centre and half extents (~1e-7 relative)
     const float rcut2 = k.rc2 * 1.0001f;
@@ -446,7 +435,16 @@ __device__ __forceinline__ bool n3_stage(const WarpParams &k, const float4 *__re
     const unsigned le = (2u << lane) - 1u;
     const int last = k.last;
     int T = 0;
-    for (int t0 = 0; t0 < Ttot; t0 += 32 * kN3Batch) {
+    if (!SPLIT) ta = 0;
+    float4 home = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (SPLIT && ta > 0) {   // a later part: the home particles by themselves
+        if (lane < n_home) {
+            home = load_pos<NC>(pos + s_home + lane);
+            S[lane] = home;
+        }
+        T = n_home;
+    }
+    for (int t0 = ta; t0 < tb_end; t0 += 32 * kN3Batch) {
         float4 q[kN3Batch], sh[kN3Batch];
 #pragma unroll
         for (int u = 0; u < kN3Batch; u++) {
@@ -458,26 +456,26 @@ __device__ __forceinline__ bool n3_stage(const WarpParams &k, const float4 *__re
             const int kc = __shfl_sync(0xffffffffu, j_entry, jc & 31);
             const int kb = __shfl_sync(0xffffffffu, s_e, kc);
             sh[u] = stab[kc];
-            // past the stencil (t >= Ttot) the index is clamped into the array
+            // past the end (t >= tb_end) the index is clamped into the array
             // and the candidate is not kept
             q[u] = load_pos<NC>(pos + min(__float_as_int(sh[u].w) + (t - kb), last));
         }
-        if (t0 == 0 && n_home <= 32) {
+        if (t0 == ta) {
             // the home particles are candidates 0 .. n_home-1 of the first round
-            if (lane < n_home) {
+            if (SPLIT && ta > 0) {
+                if (lane < n_home) { bxl = bxh = home.x; byl = byh = home.y; bzl = bzh = home.z; }
+            } else if (lane < n_home) {
                 bxl = bxh = q[0].x;
                 byl = byh = q[0].y;
                 bzl = bzh = q[0].z;
             }
-            box_reduce(bxl, byl, bzl, bxh, byh, bzh);
-        } else if (t0 == 0) {
             box_reduce(bxl, byl, bzl, bxh, byh, bzh);
         }
         if (T + 32 * kN3Batch + 32 > k.cap) {   // this batch plus the padding might not fit
             __syncwarp();
             return false;
         }
-        if (t0 == 0) {   // the box as centre and half extents
+        if (t0 == ta) {   // the box as centre and half extents
             bcx = 0.5f * (bxl + bxh);
             bcy = 0.5f * (byl + byh);
             bcz = 0.5f * (bzl + bzh);
@@ -494,7 +492,7 @@ __device__ __forceinline__ bool n3_stage(const WarpParams &k, const float4 *__re
             const float dx = fmaxf(fabsf(cx - bcx) - bhx, 0.f);
             const float dy = fmaxf(fabsf(cy - bcy) - bhy, 0.f);
             const float dz = fmaxf(fabsf(cz - bcz) - bhz, 0.f);
-            const bool keep = t < Ttot && dx * dx + dy * dy + dz * dz < rcut2;
+            const bool keep = t < tb_end && dx * dx + dy * dy + dz * dz < rcut2;
             const unsigned kept = __ballot_sync(0xffffffffu, keep);
             if (keep) S[T + __popc(kept & lt)] = make_float4(cx, cy, cz, q[u].w);
             T += __popc(kept);
@@ -508,11 +506,13 @@ __device__ __forceinline__ bool n3_stage(const WarpParams &k, const float4 *__re
 
 // Plain path for a cell whose pruned half stencil overflows the slice, or
 // that has a cell beyond its slots in the half stencil (SLOTS): lane = home
-// particle, candidates read from global memory (all lanes the same one; the
-// slots, then the cell's overflow list), reactions summed over the warp.
-template <int MODE, bool ENERGY, bool NC, bool SLOTS>
+// particle, candidates ta .. tb_end - 1 of the half stencil read from global
+// memory (all lanes the same one; the slots, then the cell's overflow list),
+// reactions summed over the warp.
+template <int MODE, bool ENERGY, bool NC, bool SLOTS, bool SPLIT>
 __device__ void n3_plain(const WarpParams &k, const float4 *__restrict__ pos, float4 *__restrict__ fout,
-                         const float4 *stab, const int *spre, int c, int s_home, int n_home, double &eacc, double &wacc)
+                         const float4 *stab, const int *spre, int c, int ta, int tb_end, int s_home, int n_home,
+                         double &eacc, double &wacc)
 {
     const int lane = threadIdx.x & 31;
     for (int p0 = 0; p0 < n_home; p0 += 32) {
@@ -538,6 +538,7 @@ __device__ void n3_plain(const WarpParams &k, const float4 *__restrict__ pos, fl
                     o = j == k.scap ? __ldg(&k.cellq[half_cell(c, kk, k.nc, k.inv_nc)].y) : __ldg(k.onext + o - 1);
                     sj = k.nslots + o - 1;
                 }
+                if (SPLIT && (spre[kk] + j < ta || spre[kk] + j >= tb_end)) continue;   // another part's
                 const float4 q = load_pos<NC>(pos + sj);
                 const float dx = xs - q.x, dy = ys - q.y, dz = zs - q.z;
                 const float r2 = dx * dx + dy * dy + dz * dz;
@@ -591,23 +592,34 @@ __device__ void n3_plain(const WarpParams &k, const float4 *__restrict__ pos, fl
 // spre, H: the warp's slice).  cw: the
 // cell side of the cell's grid.  NC: read-only loads of the sorted
 // positions (not when an earlier phase of the same launch writes them).
-// SLOTS: slotted cells; c: the cell's id.
-template <int MODE, bool ENERGY, bool NC, bool SLOTS>
+// SLOTS: slotted cells; c: the cell's id.  part of 2^lgw: the cell's
+// candidates are split evenly over 2^lgw warps (0 of 1: the whole cell),
+// part 0 with the home pairs; every part stages the home particles and adds
+// its share of their forces (SPLIT; otherwise whole cells only).
+template <int MODE, bool ENERGY, bool NC, bool SLOTS, bool SPLIT>
 __device__ __forceinline__ void n3_cell(const WarpParams &k, const float4 *__restrict__ pos, float4 *__restrict__ fout,
-                                        HalfLoad tl, int c, float cw, float4 *S, float4 *stab, int *spre, float4 *H,
-                                        double &eacc, double &wacc)
+                                        HalfLoad tl, int c, int part, int lgw, float cw, float4 *S, float4 *stab,
+                                        int *spre, float4 *H, double &eacc, double &wacc)
 {
     __syncwarp();   // the slice still holds the previous cell's data
     const int tot = half_finish(tl, cw, stab, spre);
     const int n_home = spre[1];
     if (n_home == 0) return;
+    int ta = 0, tb_end = tot;
+    if constexpr (SPLIT) {
+        const int nn = tot - n_home;   // at most 32-bit counts of particles: products below 2^34
+        ta = part == 0 ? 0 : n_home + (int)(((int64_t)nn * part) >> lgw);
+        tb_end = n_home + (int)(((int64_t)nn * (part + 1)) >> lgw);
+        if (ta >= tb_end) return;
+    }
     const int s_home = __float_as_int(stab[0].w);
     int T = 0;
     const bool over = SLOTS && __any_sync(0xffffffffu, tl.e - tl.s > k.scap);
-    if (!over && n_home <= 32 && tot <= 2 * k.cap && n3_stage<NC>(k, pos, S, stab, spre, tot, s_home, n_home, T))
-        n3_compute<MODE, ENERGY>(k, fout, S, H, T, n_home, eacc, wacc);
+    if (!over && n_home <= 32 && tot <= 2 * k.cap &&
+        n3_stage<NC, SPLIT>(k, pos, S, stab, spre, ta, tb_end, s_home, n_home, T))
+        n3_compute<MODE, ENERGY>(k, fout, S, H, T, SPLIT && ta > 0 ? n_home : 0, n_home, eacc, wacc);
     else
-        n3_plain<MODE, ENERGY, NC, SLOTS>(k, pos, fout, stab, spre, c, s_home, n_home, eacc, wacc);
+        n3_plain<MODE, ENERGY, NC, SLOTS, SPLIT>(k, pos, fout, stab, spre, c, ta, tb_end, s_home, n_home, eacc, wacc);
 }
 
 }  // namespace

@@ -159,6 +159,7 @@ __global__ void k_skin_decide(int32_t *flags, long long *counts, float thr2, int
 template <typename F4>
 __global__ void k_kick(double *__restrict__ v, const F4 *__restrict__ f, int n, double h)
 {
+    pdl_wait();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const int64_t b = 3 * (int64_t)i;
@@ -263,7 +264,7 @@ cudaError_t launch_kick_drift_skin(lj_ctx *c, double *x, double *v, const void *
     return cudaGetLastError();
 }
 
-cudaError_t launch_kick(lj_ctx *c, double *v, const void *f)
+cudaError_t launch_kick(lj_ctx *c, double *v, const void *f, bool after_force)
 {
     int n = (int)c->p.n;
     if (n == 0) return cudaSuccess;
@@ -271,7 +272,13 @@ cudaError_t launch_kick(lj_ctx *c, double *v, const void *f)
     if (c->p.precision == LJ_PREC_FP64)
         k_kick<double4_16a><<<blocks_for(n, 256), 256, 0, c->stream>>>(v, (const double4_16a *)f, n, h);
     else
-        k_kick<float4><<<blocks_for(n, 256), 256, 0, c->stream>>>(v, (const float4 *)f, n, h);
+    {
+        double hh = h;
+        void *args[] = {&v, &f, &n, &hh};
+        const cudaError_t e = launch_pdl((const void *)k_kick<float4>, (int)blocks_for(n, 256), 256, args, 0, c->stream,
+                                         after_force);
+        if (e != cudaSuccess) return e;
+    }
     c->kernel_launches++;
     return cudaGetLastError();
 }

@@ -202,6 +202,7 @@ __global__ void __launch_bounds__(256) k_langevin_slots(SlotBin b, double *__res
                                                         double c2s, uint64_t *__restrict__ state, uint64_t A, uint64_t C,
                                                         int32_t *__restrict__ err)
 {
+    pdl_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i == 0) *b.work = 0u;
     const bool valid = i < n;
@@ -218,7 +219,8 @@ inline unsigned grid_for(int64_t n, int threads) { return (unsigned)((n + thread
 
 }  // namespace
 
-cudaError_t launch_langevin_bin(lj_ctx *c, double *x, double *v, void *f, int nkick, double gamma, double kT)
+cudaError_t launch_langevin_bin(lj_ctx *c, double *x, double *v, void *f, int nkick, double gamma, double kT,
+                                bool after_force)
 {
     const int n = (int)c->p.n;
     if (n == 0) return cudaSuccess;
@@ -229,12 +231,16 @@ cudaError_t launch_langevin_bin(lj_ctx *c, double *x, double *v, void *f, int nk
     uint64_t A, C;
     r48_jump((uint64_t)n, A, C);
     if (uses_slots(c)) {
-        const cudaError_t e = slots_begin(c, 0);
+        cudaError_t e = slots_begin(c, 0);
         if (e != cudaSuccess) return e;
-        k_langevin_slots<<<grid_for(n, 256), 256, 0, c->stream>>>(slot_bin_of(c), x, v, (float4 *)f, n, hk, 0.5 * dt, c1,
-                                                                  c2s, c->r48_state, A, C, c->err);
+        SlotBin b = slot_bin_of(c);
+        float4 *fo = (float4 *)f;
+        int np = n;
+        double h = hk, hd = 0.5 * dt, k1 = c1, k2 = c2s;
+        void *args[] = {&b, &x, &v, &fo, &np, &h, &hd, &k1, &k2, &c->r48_state, &A, &C, &c->err};
+        e = launch_pdl((const void *)k_langevin_slots, (int)grid_for(n, 256), 256, args, 0, c->stream, after_force);
         c->kernel_launches++;
-        return cudaGetLastError();
+        return e != cudaSuccess ? e : cudaGetLastError();
     }
     if (c->p.precision == LJ_PREC_FP64)
         k_langevin_bin<double4_16a, double><<<grid_for(n, 256), 256, 0, c->stream>>>(

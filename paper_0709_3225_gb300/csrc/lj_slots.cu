@@ -48,7 +48,10 @@ __global__ void __launch_bounds__(256) k_kick_drift_slots(SlotBin b, double *__r
                                                           float4 *__restrict__ f, int i_begin, int n, double hk,
                                                           double dt, int32_t *__restrict__ err)
 {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    pdl_wait();
+    // the last particles first: what this kernel wrote last, and the force
+    // kernel reads (adds into) first, is then still in L2
+    const int t = (gridDim.x - 1 - blockIdx.x) * blockDim.x + threadIdx.x;
     if (t == 0) *b.work = 0u;
     const int i = i_begin + t;
     const bool valid = i < n;
@@ -237,17 +240,21 @@ cudaError_t launch_bin_slots(lj_ctx *c, const double *x, float4 *zero, const dou
 }
 
 cudaError_t launch_kick_drift_slots(lj_ctx *c, double *x, double *v, float4 *f, int nkick, int64_t i_begin,
-                                    int64_t i_end)
+                                    int64_t i_end, bool after_force)
 {
     const int n = (int)(i_end < 0 ? c->p.n : i_end);
     if (n <= (int)i_begin) return cudaSuccess;
     cudaError_t e = slots_begin(c, i_begin);
     if (e != cudaSuccess) return e;
     const double hk = nkick * (0.5 * c->p.dt / c->p.mass);
-    k_kick_drift_slots<<<blocks_for(n - i_begin, 256), 256, 0, c->stream>>>(slot_bin_of(c), x, v, f, (int)i_begin, n,
-                                                                            hk, c->p.dt, c->err);
+    SlotBin b = slot_bin_of(c);
+    int i0 = (int)i_begin, i1 = n;
+    double h = hk, dt = c->p.dt;
+    int32_t *err = c->err;
+    void *args[] = {&b, &x, &v, &f, &i0, &i1, &h, &dt, &err};
+    e = launch_pdl((const void *)k_kick_drift_slots, (int)blocks_for(n - i_begin, 256), 256, args, 0, c->stream, after_force);
     c->kernel_launches++;
-    return cudaGetLastError();
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 cudaError_t launch_slots_to_lists(lj_ctx *c)

@@ -423,6 +423,7 @@ __global__ void __launch_bounds__(kVn3Threads, 4) k_vjp_n3(VjpN3Coef k, const fl
     float4 *H = reinterpret_cast<float4 *>(spre + 16);
     double acc_e = 0.0, acc_s = 0.0;
     if constexpr (SLOTS) {   // as k_force_n3
+        pdl_wait();
         start = reinterpret_cast<const int32_t *>(k.cellq);
         if (blockIdx.x == 0 && threadIdx.x == 0) {
             k.cellq_next[k.ncell] = make_int2(0, 0);
@@ -489,6 +490,7 @@ __global__ void __launch_bounds__(kReduceThreads) k_vjp_finish(const float4 *__r
                                                                double a, const double *__restrict__ partial, int np,
                                                                double *__restrict__ dparam)
 {
+    pdl_wait();
     if (blockIdx.x == 0) {
         __shared__ double se[kReduceThreads], ss[kReduceThreads];
         double e = 0.0, s = 0.0;
@@ -602,12 +604,13 @@ cudaError_t launch_vjp_n3(lj_ctx *c, const double *coef, double scale, double *d
         if (e != cudaSuccess) return e;
     }
     void *args[] = {&k, (void *)&pos, (void *)&g4, (void *)&start, &acc, &partial};
-    e = cudaLaunchKernel(kern, dim3((unsigned)grid), dim3(kVn3Threads), args, smem, c->stream);
+    e = launch_pdl(kern, (int)grid, kVn3Threads, args, (size_t)smem, c->stream, slots);
     if (e != cudaSuccess) return e;
     if (slots) slots_consumed(c);
-    const int n = (int)c->p.n;
-    k_vjp_finish<<<(unsigned)((n + kReduceThreads - 1) / kReduceThreads) + 1, kReduceThreads, 0, c->stream>>>(
-        acc, n, scale, dx, lam, dt_axpy, partial, (int)grid, dparam);
+    int n = (int)c->p.n, np = (int)grid;
+    void *fargs[] = {&acc, &n, &scale, &dx, &lam, &dt_axpy, &partial, &np, &dparam};
+    e = launch_pdl((const void *)k_vjp_finish, (n + kReduceThreads - 1) / kReduceThreads + 1, kReduceThreads, fargs, 0,
+                   c->stream, true);
     c->kernel_launches += 2;
-    return cudaGetLastError();
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
