@@ -360,11 +360,11 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 
 // ------------------------------------------------------------------ host --
 
-inline cudaError_t launch_pdl(const void *kern, int grid, int block, void **args, size_t smem, cudaStream_t stream,
+inline cudaError_t launch_pdl(const void *kern, dim3 grid, int block, void **args, size_t smem, cudaStream_t stream,
                               bool pdl)
 {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
+    cfg.gridDim = grid;
     cfg.blockDim = dim3((unsigned)block);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
