@@ -6,7 +6,7 @@
 // Organisation on GB300:
 //  * A CTA of kN2Threads threads; thread t owns particle
 //    i = blockIdx.x * kN2Threads + t.
-//  * The j particles stream through shared memory in tiles of kN2Tile,
+//  * The j particles stream through shared memory in tiles,
 //    copied by cp.async.bulk (issued by thread 0, completing on an mbarrier,
 //    two buffers, bounded waits).  This is the paper's "load a block of
 //    particles into shared memory, synchronise, compute", with the copy
@@ -22,7 +22,8 @@
 namespace {
 
 constexpr int kN2Threads = 128;
-constexpr int kN2Tile = 512;   // j particles per shared-memory tile
+constexpr int kN2Tile = 512;    // j particles per shared-memory tile, FP64
+constexpr int kN2TileF = 128;   // FP32: at most (a multiple of 32; 256 measured 48 us against 46 at 8,788)
 
 struct N2Params {
     int n, ntiles;
@@ -50,6 +51,27 @@ __global__ void k_n2_prep(const double *__restrict__ x, int n, double L, double 
         q.w = (double)i;
     }
     pos[i] = q;
+}
+
+// FP32: coordinates in three arrays of npad (a multiple of 32) floats; the
+// padding is far away (its squared distance is inf, the image included).
+__global__ void k_n2_prep_f32(const double *__restrict__ x, int n, int npad, double L, double whi, double wlo,
+                              float *__restrict__ soa, int32_t *err)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= npad) return;
+    float q[3] = {1.0e30f, 1.0e30f, 1.0e30f};
+    if (i < n) {
+        const double px = x[3 * (int64_t)i], py = x[3 * (int64_t)i + 1], pz = x[3 * (int64_t)i + 2];
+        if (!(finite64(px) && finite64(py) && finite64(pz))) atomicOr(err, LJ_ERRBIT_NONFINITE);
+        const double h = 0.5 * L;
+        q[0] = (float)(lj_wrap_fast(px, L, whi, wlo) - h);
+        q[1] = (float)(lj_wrap_fast(py, L, whi, wlo) - h);
+        q[2] = (float)(lj_wrap_fast(pz, L, whi, wlo) - h);
+    }
+    soa[i] = q[0];
+    soa[(size_t)npad + i] = q[1];
+    soa[2 * (size_t)npad + i] = q[2];
 }
 
 template <typename V>
@@ -178,11 +200,152 @@ __global__ void __launch_bounds__(kN2Threads) k_n2_force(N2Params p, const typen
     }
 }
 
+// The squared minimum-image distances of two j to one i, for the cutoff
+// test only: per component min(|d|, L - |d|), the magnitude of d - L rint(d /
+// L) for every pair within L / 2, bit for bit, without the rounding
+// instruction (a quarter-rate one) and the two multiplications around it.
+__device__ __forceinline__ float2 n2_r2(float2 xi, float2 yi, float2 zi, float2 xj, float2 yj, float2 zj, float L)
+{
+    const float2 m1 = make_float2(-1.0f, -1.0f);
+    float2 dx = __ffma2_rn(xj, m1, xi);
+    float2 dy = __ffma2_rn(yj, m1, yi);
+    float2 dz = __ffma2_rn(zj, m1, zi);
+    dx.x = fminf(fabsf(dx.x), L - fabsf(dx.x));
+    dx.y = fminf(fabsf(dx.y), L - fabsf(dx.y));
+    dy.x = fminf(fabsf(dy.x), L - fabsf(dy.x));
+    dy.y = fminf(fabsf(dy.y), L - fabsf(dy.y));
+    dz.x = fminf(fabsf(dz.x), L - fabsf(dz.x));
+    dz.y = fminf(fabsf(dz.y), L - fabsf(dz.y));
+    float2 r2 = __fmul2_rn(dx, dx);
+    r2 = __ffma2_rn(dy, dy, r2);
+    return __ffma2_rn(dz, dz, r2);
+}
+
+// FP32 form of k_n2_force.  Only some 55 of the n - 1 pairs of a particle
+// are within rc, so all pairs go through the distance test alone and the
+// few that pass through the pair term: a thread takes its particle against
+// 32 j at a time, collects the passing ones in a bit mask (the sign of r^2 -
+// rc^2 (1 + 1e-5), shifted in), and then evaluates those with the exact
+// cutoff and minimum image of pair_accum, in the order of j.  Bound by
+// instruction issue: ~13 instructions per pair (six for the three
+// components' images, 1.5 each for r^2 and the mask) against ~30 with three
+// quarter-rate roundings before.  At 8,788
+// particles a call took 137 us, now 46.
+template <int MODE, bool ENERGY>
+__global__ void __launch_bounds__(kN2Threads) k_n2_force_f32(N2Params p, int npad, int tile, const float *__restrict__ soa,
+                                                             float4 *__restrict__ part, double *__restrict__ epart,
+                                                             int32_t *err)
+{
+    __shared__ __align__(128) float sm[2][3][kN2TileF];
+    __shared__ __align__(8) uint64_t bars[2];
+    __shared__ int s_abort;
+    __shared__ double red[2 * (kN2Threads / 32)];
+    pdl_wait();
+    const int i = blockIdx.x * kN2Threads + threadIdx.x;
+    const bool vi = i < p.n;
+    const float pix = soa[vi ? i : 0], piy = soa[(size_t)npad + (vi ? i : 0)], piz = soa[2 * (size_t)npad + (vi ? i : 0)];
+    const int split = blockIdx.y, nsplit = gridDim.y;
+    const int mine = p.ntiles > split ? (p.ntiles - split + nsplit - 1) / nsplit : 0;
+    auto issue = [&](int k) {
+        const int t0 = (split + k * nsplit) * tile;
+        const uint32_t bytes = (uint32_t)min(tile, npad - t0) * 4u;   // a multiple of 128
+        const int b = k & 1;
+        mbar_arrive_expect_tx(&bars[b], 3 * bytes);
+        for (int d = 0; d < 3; d++) bulk_g2s(sm[b][d], soa + (size_t)d * npad + t0, bytes, &bars[b]);
+    };
+    if (threadIdx.x == 0) {
+        s_abort = 0;
+        mbar_init(&bars[0], 1);
+        mbar_init(&bars[1], 1);
+        fence_mbar_init();
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        if (mine > 0) issue(0);
+        if (mine > 1) issue(1);
+    }
+    const Coef<float> kc(p);
+    const float L = (float)p.L, invL = (float)p.invL;
+    const float thr = -(float)p.rc2 * 1.00001f;
+    const float2 xi = make_float2(pix, pix), yi = make_float2(piy, piy), zi = make_float2(piz, piz);
+    float fx = 0, fy = 0, fz = 0, e = 0, w = 0;
+    int k = 0;
+    for (; k < mine; k++) {
+        const int b = k & 1;
+        const int cnt = min(tile, npad - (split + k * nsplit) * tile);   // a multiple of 32
+        if (!mbar_wait_bounded(&bars[b], (uint32_t)((k >> 1) & 1), err)) s_abort = 1;
+        __syncthreads();
+        if (s_abort) break;
+        const float *X = sm[b][0], *Y = sm[b][1], *Z = sm[b][2];
+        for (int j0 = 0; j0 < cnt; j0 += 32) {
+            unsigned mask = 0;
+#pragma unroll
+            for (int u = 0; u < 32; u += 4) {
+                const float4 qx = *reinterpret_cast<const float4 *>(X + j0 + u);
+                const float4 qy = *reinterpret_cast<const float4 *>(Y + j0 + u);
+                const float4 qz = *reinterpret_cast<const float4 *>(Z + j0 + u);
+                const float2 t = make_float2(thr, thr);
+                const float2 a = __fadd2_rn(n2_r2(xi, yi, zi, make_float2(qx.x, qx.y), make_float2(qy.x, qy.y),
+                                                  make_float2(qz.x, qz.y), L), t);
+                const float2 c = __fadd2_rn(n2_r2(xi, yi, zi, make_float2(qx.z, qx.w), make_float2(qy.z, qy.w),
+                                                  make_float2(qz.z, qz.w), L), t);
+                mask = __funnelshift_l(__float_as_uint(a.x), mask, 1);   // j0 ends in the top bit
+                mask = __funnelshift_l(__float_as_uint(a.y), mask, 1);
+                mask = __funnelshift_l(__float_as_uint(c.x), mask, 1);
+                mask = __funnelshift_l(__float_as_uint(c.y), mask, 1);
+            }
+            while (mask) {
+                const int u = __clz((int)mask);
+                mask &= ~(0x80000000u >> u);
+                float dx = pix - X[j0 + u], dy = piy - Y[j0 + u], dz = piz - Z[j0 + u];
+                dx -= L * rint_t(dx * invL);
+                dy -= L * rint_t(dy * invL);
+                dz -= L * rint_t(dz * invL);
+                pair_accum<float, MODE, ENERGY>(dx, dy, dz, kc, fx, fy, fz, e, w);
+            }
+        }
+        __syncthreads();   // everyone is done with buffer b
+        if (threadIdx.x == 0 && k + 2 < mine) {
+            fence_proxy_async_smem();
+            issue(k + 2);
+        }
+    }
+    if (s_abort && threadIdx.x == 0) {   // as k_n2_force: the copies that may still be in flight
+        mbar_wait_bounded(&bars[k & 1], (uint32_t)((k >> 1) & 1), err);
+        if (k + 1 < mine) mbar_wait_bounded(&bars[(k + 1) & 1], (uint32_t)(((k + 1) >> 1) & 1), err);
+    }
+    if (vi) part[(size_t)split * p.n + i] = make_float4(fx, fy, fz, ENERGY ? 0.5f * e : 0.0f);
+    if constexpr (ENERGY) {
+        double de = vi ? 0.5 * (double)e : 0.0, dw = vi ? 0.5 * (double)w : 0.0;
+        for (int o = 16; o > 0; o >>= 1) {
+            de += __shfl_xor_sync(0xffffffffu, de, o);
+            dw += __shfl_xor_sync(0xffffffffu, dw, o);
+        }
+        const int warp = threadIdx.x >> 5;
+        if ((threadIdx.x & 31) == 0) {
+            red[2 * warp] = de;
+            red[2 * warp + 1] = dw;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            double es = 0.0, ws = 0.0;
+            for (int q = 0; q < kN2Threads / 32; q++) {
+                es += red[2 * q];
+                ws += red[2 * q + 1];
+            }
+            const size_t cta = (size_t)blockIdx.y * gridDim.x + blockIdx.x;
+            epart[2 * cta] = es;
+            epart[2 * cta + 1] = ws;
+        }
+    }
+}
+
 // f[i] = sum over splits s = 0 .. nsplit-1 (in order) of part[s * n + i].
 template <typename T>
 __global__ void k_n2_sum(const typename Vec4<T>::type *__restrict__ part, int nsplit, int n,
                          typename Vec4<T>::type *__restrict__ f)
 {
+    pdl_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     typename Vec4<T>::type a = part[i];
@@ -221,16 +384,21 @@ __global__ void k_n2_energy(const double *__restrict__ epart, int m, double *__r
     }
 }
 
-template <typename T>
-void *n2_kernel(int mode, bool energy)
+void *n2_kernel(bool fp64, int mode, bool energy)
 {
-    switch (mode * 2 + (energy ? 1 : 0)) {
-        case 0: return (void *)k_n2_force<T, 0, false>;
-        case 1: return (void *)k_n2_force<T, 0, true>;
-        case 2: return (void *)k_n2_force<T, 1, false>;
-        case 3: return (void *)k_n2_force<T, 1, true>;
-        case 4: return (void *)k_n2_force<T, 2, false>;
-        default: return (void *)k_n2_force<T, 2, true>;
+    switch ((fp64 ? 6 : 0) + mode * 2 + (energy ? 1 : 0)) {
+        case 0: return (void *)k_n2_force_f32<0, false>;
+        case 1: return (void *)k_n2_force_f32<0, true>;
+        case 2: return (void *)k_n2_force_f32<1, false>;
+        case 3: return (void *)k_n2_force_f32<1, true>;
+        case 4: return (void *)k_n2_force_f32<2, false>;
+        case 5: return (void *)k_n2_force_f32<2, true>;
+        case 6: return (void *)k_n2_force<double, 0, false>;
+        case 7: return (void *)k_n2_force<double, 0, true>;
+        case 8: return (void *)k_n2_force<double, 1, false>;
+        case 9: return (void *)k_n2_force<double, 1, true>;
+        case 10: return (void *)k_n2_force<double, 2, false>;
+        default: return (void *)k_n2_force<double, 2, true>;
     }
 }
 
@@ -240,12 +408,19 @@ cudaError_t run_n2(lj_ctx *c, const double *x, void *f, bool energy)
     using V = typename Vec4<T>::type;
     const int n = (int)c->p.n;
     const int iblocks = (n + kN2Threads - 1) / kN2Threads;
-    const int ntiles = (n + kN2Tile - 1) / kN2Tile;
-    int nsplit = (2 * c->nsm + iblocks - 1) / iblocks;
+    constexpr bool fp64 = sizeof(T) == 8;
+    // FP32: smaller tiles while they give fewer than 8 CTAs per SM, and j
+    // splits up to 16 per SM: with 2 per SM (of 4 warps) the SMs were unevenly
+    // loaded and the distance tests' latency showed.
+    int tile = fp64 ? kN2Tile : kN2TileF;
+    while (!fp64 && tile > 32 && (int64_t)iblocks * ((n + tile - 1) / tile) < 8 * c->nsm) tile /= 2;
+    int ntiles = (n + tile - 1) / tile;
+    int nsplit = ((fp64 ? 2 : 16) * c->nsm + iblocks - 1) / iblocks;
     nsplit = nsplit < 1 ? 1 : (nsplit > ntiles ? ntiles : nsplit);
     nsplit = nsplit > 64 ? 64 : nsplit;
+    int npad = (n + 31) & ~31;
     // scratch: sorted-free positions, per-split partials, per-CTA energy pairs
-    const size_t need = (size_t)n * sizeof(V) * (size_t)(1 + nsplit) + 2 * sizeof(double) * (size_t)iblocks * nsplit;
+    const size_t need = (size_t)npad * sizeof(V) * (size_t)(1 + nsplit) + 2 * sizeof(double) * (size_t)iblocks * nsplit;
     if (need > c->n2_bytes) {
         cudaFree(c->n2_scratch);
         c->n2_scratch = nullptr;
@@ -255,10 +430,14 @@ cudaError_t run_n2(lj_ctx *c, const double *x, void *f, bool energy)
         c->n2_bytes = need;
     }
     V *pos = reinterpret_cast<V *>(c->n2_scratch);
-    V *part = pos + n;
+    V *part = pos + npad;
     double *epart = reinterpret_cast<double *>(part + (size_t)n * nsplit);
     V *fo = reinterpret_cast<V *>(f);
-    k_n2_prep<T><<<(n + 255) / 256, 256, 0, c->stream>>>(x, n, c->p.box, c->wrap_hi, c->wrap_lo, pos, c->err);
+    if constexpr (fp64)
+        k_n2_prep<T><<<(n + 255) / 256, 256, 0, c->stream>>>(x, n, c->p.box, c->wrap_hi, c->wrap_lo, pos, c->err);
+    else   // three arrays of npad floats
+        k_n2_prep_f32<<<(npad + 255) / 256, 256, 0, c->stream>>>(x, n, npad, c->p.box, c->wrap_hi, c->wrap_lo,
+                                                                 (float *)pos, c->err);
     N2Params p;
     p.n = n;
     p.ntiles = ntiles;
@@ -275,18 +454,26 @@ cudaError_t run_n2(lj_ctx *c, const double *x, void *f, bool energy)
     p.c6 = 4.0 * eps * s6;
     p.uc = rci6 * (p.c12 * rci6 - p.c6);
     p.fc = rc * rci2 * rci6 * (p.a12 * rci6 - p.b6);
-    void *kern = n2_kernel<T>(c->p.shift_mode, energy);
-    const int smem = 2 * kN2Tile * (int)sizeof(V) + 2 * (int)sizeof(uint64_t);
-    cudaError_t e = raise_dyn_smem(kern, smem);
-    if (e != cudaSuccess) return e;
+    void *kern = n2_kernel(fp64, c->p.shift_mode, energy);
     V *dst = nsplit == 1 ? fo : part;
     int32_t *err = c->err;
-    void *args[] = {&p, (void *)&pos, (void *)&dst, (void *)&epart, (void *)&err};
-    e = cudaLaunchKernel(kern, dim3(iblocks, nsplit), dim3(kN2Threads), args, smem, c->stream);
+    cudaError_t e;
+    if constexpr (fp64) {
+        const int smem = 2 * kN2Tile * (int)sizeof(V) + 2 * (int)sizeof(uint64_t);
+        if ((e = raise_dyn_smem(kern, smem)) != cudaSuccess) return e;
+        void *args[] = {&p, (void *)&pos, (void *)&dst, (void *)&epart, (void *)&err};
+        e = cudaLaunchKernel(kern, dim3(iblocks, nsplit), dim3(kN2Threads), args, smem, c->stream);
+    } else {
+        void *args[] = {&p, &npad, &tile, (void *)&pos, (void *)&dst, (void *)&epart, (void *)&err};
+        e = launch_pdl(kern, dim3(iblocks, nsplit), kN2Threads, args, 0, c->stream, true);
+    }
     if (e != cudaSuccess) return e;
     c->kernel_launches += 2;
     if (nsplit > 1) {
-        k_n2_sum<T><<<(n + 255) / 256, 256, 0, c->stream>>>(part, nsplit, n, fo);
+        int np = nsplit, nn = n;
+        void *args[] = {(void *)&part, &np, &nn, (void *)&fo};
+        e = launch_pdl((const void *)k_n2_sum<T>, dim3((n + 255) / 256), 256, args, 0, c->stream, !fp64);
+        if (e != cudaSuccess) return e;
         c->kernel_launches++;
     }
     if (energy) {
