@@ -65,7 +65,8 @@ typedef enum lj_shift {
 typedef enum lj_precision {
     LJ_PREC_MIXED = 0,   /* FP32 pair arithmetic and per-particle sums,
                             FP64 positions, integrator, energy and virial */
-    LJ_PREC_FP64 = 1     /* FP64 throughout */
+    LJ_PREC_FP64 = 1     /* FP64 throughout; pair forces and their sums in
+                            64-bit fixed point where its error is smaller */
 } lj_precision;
 
 /* Simulation parameters (Section 2 and 3: N, box, eps, sigma, rc, dt). */

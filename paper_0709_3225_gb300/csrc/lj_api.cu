@@ -198,6 +198,15 @@ bool fused_mode(const lj_ctx *c) { return !c->use_run_kernel && c->fuse_update &
 // graph replay captures.
 int one_step(lj_ctx *c, double *x, double *v, void *f, int s, int nsteps, cudaEvent_t x_final = nullptr)
 {
+    if (uses_fx(c)) {   // the same in FP64; the sums of the step before are in f and fx_acc
+        if (s == 0 && c->kdb_done)
+            c->kdb_done = 0;
+        else
+            LJ_CK(launch_kick_drift_fx(c, x, v, (double4_16a *)f, s == 0 ? 1 : 2, s > 0, 0, -1, s > 0 && !c->timing));
+        if (x_final) LJ_CK(cudaEventRecord(x_final, c->stream));
+        LJ_CK(launch_force_fx(c, (double4_16a *)f));
+        return LJ_OK;
+    }
     if (uses_slots(c)) {
         // slotted cells: one pass over the particles, then the forces
         if (s == 0 && c->kdb_done)
@@ -293,7 +302,7 @@ int capture_middle_step(lj_ctx *c, double *x, double *v, void *f)
     if (e == cudaSuccess) {
         cudaStream_t keep = c->stream;
         c->stream = cs;
-        c->gsteps = uses_slots(c) ? 2 : 1;
+        c->gsteps = uses_slots(c) || uses_fx(c) ? 2 : 1;
         c->gpar = c->slot_par;
         for (int k = 0; k < c->gsteps && r == LJ_OK; k++) r = one_step(c, x, v, f, 1, 3);
         c->stream = keep;
@@ -371,7 +380,7 @@ int do_steps(lj_ctx *c, double *x, double *v, void *f, int nsteps, cudaEvent_t x
         if (r) return r;
     }
     const bool graph = c->use_graph && !c->timing && nsteps >= 3;
-    const int gs = uses_slots(c) ? 2 : 1;   // steps per replay
+    const int gs = uses_slots(c) || uses_fx(c) ? 2 : 1;   // steps per replay
     for (int s = 0; s < nsteps; s++) {
         // after step 0 (which does any lazy set-up outside the capture and
         // settles a pending skin rebuild) the middle steps are graph replays
@@ -390,7 +399,8 @@ int do_steps(lj_ctx *c, double *x, double *v, void *f, int nsteps, cudaEvent_t x
             if (r) return r;
         }
     }
-    if (!fused_mode(c)) LJ_CK(launch_kick(c, v, f, uses_slots(c) && !c->timing));
+    if (uses_fx(c)) LJ_CK(launch_fx_finish(c, v, (double4_16a *)f));
+    else if (!fused_mode(c)) LJ_CK(launch_kick(c, v, f, uses_slots(c) && !c->timing));
     if (x_final && fused_mode(c)) LJ_CK(cudaEventRecord(x_final, c->stream));
     return LJ_OK;
 }
@@ -663,9 +673,15 @@ extern "C" int lj_forces(lj_ctx *c, const double *x, void *f, double *e_pot, dou
         r = check_dev_ptr(f, 16);
         if (r) return r;
     }
+    const bool energy = e_pot || virial;
+    if (!energy && uses_fx(c)) {
+        LJ_CK(launch_bin_fx(c, x, (double4_16a *)f));
+        LJ_CK(launch_force_fx(c, (double4_16a *)f));
+        LJ_CK(launch_fx_finish(c, nullptr, (double4_16a *)f));
+        return LJ_OK;
+    }
     int r = bin_for_force(c, x, f);
     if (r) return r;
-    const bool energy = e_pot || virial;
     LJ_CK(launch_force(c, f, energy));
     if (!energy) return LJ_OK;
     LJ_CK(cudaMemsetAsync(c->scalars, 0, 2 * sizeof(double), c->stream));
@@ -806,6 +822,8 @@ extern "C" int lj_step_host(lj_ctx *c, double *x, double *v, void *f, int32_t ns
             LJ_CK(cudaStreamWaitEvent(c->stream, c->ev_chunk[k], 0));
             if (uses_slots(c))
                 LJ_CK(launch_kick_drift_slots(c, c->xs, c->vs, (float4 *)c->fs, 1, (int64_t)i0, (int64_t)i1));
+            else if (uses_fx(c))
+                LJ_CK(launch_kick_drift_fx(c, c->xs, c->vs, (double4_16a *)c->fs, 1, false, (int64_t)i0, (int64_t)i1));
             else
                 LJ_CK(launch_kick_drift_bin(c, c->xs, c->vs, c->fs, 1, (int64_t)i0, (int64_t)i1));
         }

@@ -1,0 +1,509 @@
+// The FP64 pair-once force kernel in 64-bit fixed point (forces without
+// energies, plain or energy-shifted truncation; slotted cells, lj_slots.cuh).
+//
+// The method is that of lj_force_w64.cu: a warp per home cell stages its
+// half stencil, lists the pairs within rc by FP32 filters (Phase A), and
+// evaluates the listed pairs at full precision, each once (Phase B).  What
+// differs is Phase B's arithmetic.  GB300's FP64 pipe takes a warp
+// instruction every 16 cycles per SM, and the pair term needs 20 of them:
+// 320 cycles, in which the SM could issue 1,280 other instructions.  The
+// same term in integers takes about 200.
+//
+//  * Coordinates are x 2^S mod 2^64, 2^-S being 2^-63 of 1.5 cell sides (the
+//    reach of the half stencil from the home cell's centre): exact for x >=
+//    2^(53-S) (a double has 53 bits), and so are the differences of particles
+//    within rc, whatever the box; a periodic image adds +-L 2^S, an integer.  So d = x_i - x_j carries no
+//    rounding at all; FP64 coordinates relative to cell centres carried the
+//    centres' (the forces' error at N = 131,072 was 2.5e-14 of their norm).
+//  * r^2: the upper 64 bits of the squares, 2^-57 relative at r = 0.4 rc.
+//  * u = sigma^2 / r^2: a float reciprocal of the normalised r^2 (error e <
+//    2^-22, formed exactly in integers) and the series 1 + e + e^2 (e^3 <
+//    2^-66), then u^2, u^3, u^4 by high products; F(r) / r = 24 eps / sigma^2
+//    u^4 (2 u^3 - 1), in units of 2^-56, and its products with d.
+//  * The sums are 64-bit integers, added by integer atomics: exact, so they
+//    do not depend on the order (the forces repeat from run to run).  Their
+//    unit, 2^-52 24 eps / sigma at most, leaves a range of 300 times the
+//    largest pair force taken here, for the net force of a particle (sums
+//    that leave the range on the way come back): eight cells' slots hold 256.
+//  * Pairs closer than sqrt(0.8) sigma, where u > 1.25 and the force has no
+//    bound, and cells that take the plain path are evaluated in FP64 as
+//    before (pair64_nf) and added to f itself; the readers of the sums add
+//    the two (fx_force, lj_slots.cu).
+// Bound by instruction issue and the latencies that 14 to 18 warps per SM
+// leave (52 % of issue slots; ALU pipe 40 %).  Step in FP64: 257 -> 96 us at
+// 131,072 particles (the force kernel 220 -> 92), 174 -> 34 at 32,000, 1,309
+// -> 646 at 10^6.  Forces against an FP64 evaluation: 6.7e-15 of their norm at
+// 131,072 particles (2.5e-14 before), 5.5e-15 at 2,048 (8.3e-15), 1.3e-14 for
+// a gas of 100,003 at density 0.3 (3.9e-14).
+#include <math.h>
+#include <string.h>
+
+#include "lj_force_n3.cuh"
+#include "lj_slots.cuh"
+
+namespace {
+
+constexpr int kFxThreads = 32;    // one warp per CTA, as the FP64 kernel
+constexpr int kFxPMax = 32;       // home particles of a staged cell
+constexpr int kFxList = 1024;     // list entries per batch
+
+struct FxParams {
+    int nc, cap, scap, nslots, last;
+    float inv_nc, to_f;                    // to_f = 2^(32 - S)
+    float rc2_box, rc2_pair;
+    unsigned *work;
+    int64_t ncell;
+    const int2 *cellq;
+    int2 *cellq_next;
+    unsigned *octr_next;
+    const int32_t *onext;
+    const double *centre;
+    int S, kappa_e, tsh;                        // u = K / 2^63 2^kappa_e 2^lz RI 2^-62
+    long long Lfix;
+    unsigned long long K, r2c, r2min;
+    // FP64 pairs
+    double to_d;                           // 2^-S
+    double rc2, a12, b6;
+};
+
+// Byte layout of a warp's slice (cap a multiple of 2).
+struct FxLayout {
+    int x64, x32, iw, sh, spre, off, list, bytes;
+    __host__ __device__ explicit FxLayout(int cap)
+    {
+        x64 = 0;                                   // int64[3][cap]
+        sh = x64 + 24 * cap;                       // int64[3][kN3Half], then int start[kN3Half]
+        x32 = (sh + 28 * kN3Half + 15) & ~15;      // float[3][cap]
+        iw = x32 + 12 * cap;                       // int[cap] particle index
+        spre = (iw + 4 * cap + 15) & ~15;          // int[16]
+        off = spre + 64;                           // int[kFxPMax + 4]
+        list = off + 4 * (kFxPMax + 4);            // uint16[kFxList]
+        bytes = (list + 2 * kFxList + 15) & ~15;
+    }
+};
+
+// The FP64 pair term of lj_force_w64.cu (pair64_nf) for truncation without a
+// force shift: -F(r) / r, 0 outside rc or for r = 0.
+__device__ __forceinline__ double fx_pair64(double dx, double dy, double dz, const FxParams &k)
+{
+    const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
+    const bool in = r2 < k.rc2 && r2 != 0.0;
+    const double ri = in ? 1.0 / r2 : 0.0;
+    const double r6 = ri * ri * ri;
+    return ri * r6 * fma(-k.a12, r6, k.b6);
+}
+
+__device__ __forceinline__ void fx_add64(double4_16a *f, int i, double x, double y, double z)
+{
+    atomicAdd(&f[i].x, x);
+    atomicAdd(&f[i].y, y);
+    atomicAdd(&f[i].z, z);
+}
+
+__device__ __forceinline__ void fx_add(long long *acc, int i, long long x, long long y, long long z)
+{
+    unsigned long long *o = reinterpret_cast<unsigned long long *>(acc) + 4 * (int64_t)i;
+    atomicAdd(o, (unsigned long long)x);
+    atomicAdd(o + 1, (unsigned long long)y);
+    atomicAdd(o + 2, (unsigned long long)z);
+}
+
+__device__ __forceinline__ unsigned long long fx_sq(long long d)
+{
+    const unsigned long long a = (unsigned long long)(d < 0 ? -d : d);
+    return __umul64hi(a, a);
+}
+
+// F(r) / r in units of 24 eps / sigma^2 2^-56 for r2min <= R2 < r2c.
+__device__ __forceinline__ long long fx_term(unsigned long long R2, const FxParams &k)
+{
+    const int lz = __clzll((long long)R2);
+    const unsigned long long M = R2 << lz;   // m = M 2^-64 in [1/2, 1)
+    const float y = rcp_approx(__uint_as_float(0x3f000000u | ((unsigned)(M >> 40) & 0x7fffffu)));
+    const unsigned y0 = __float_as_uint(y) - 0x3f800000u + 0x800000u;   // y 2^23, in (2^23, 2^24]
+    // e = 1 - m y in units of 2^-63
+    const unsigned long long plo = (unsigned long long)(unsigned)M * y0;
+    const unsigned long long phi = (M >> 32) * y0;
+    const long long E = (long long)(0x8000000000000000ull - ((phi << 8) + (plo >> 24)));
+    const int eh = (int)(E >> 11);
+    const long long G = E + (((long long)eh * eh) >> 41);
+    // 1 / m in units of 2^-62
+    const unsigned long long RI = ((unsigned long long)y0 << 39) + (unsigned long long)(((long long)y0 * (G >> 3)) >> 21);
+    const unsigned long long h = __umul64hi(RI, k.K);
+    const int s = k.kappa_e + lz + 2;
+    const unsigned long long U = s >= 0 ? h << s : (s > -64 ? h >> -s : 0ull);   // u 2^63
+    const unsigned long long U2 = __umul64hi(U, U);                              // 2^62
+    const unsigned long long U3 = __umul64hi(U2, U);                             // 2^61
+    const unsigned long long U4 = __umul64hi(U2, U2);                            // 2^60
+    const long long T = (long long)U3 - (1ll << 60);                             // (2 u^3 - 1) 2^60
+    return __mul64hi((long long)U4, T);
+}
+
+// The product's upper 64 bits, rounded towards zero: the same magnitude for d
+// and -d, so that a pair's force does not depend on which of the two is home.
+__device__ __forceinline__ long long fx_mul(long long t, long long d)
+{
+    const long long h = __mul64hi(t, d);
+    return h + (long long)((unsigned long long)h >> 63);
+}
+
+// Plain path: lanes own home particles, FP64 over the half stencil's slots
+// and overflow lists.
+__device__ void fx_plain(const FxParams &k, const longlong4_16a *__restrict__ pos, double4_16a *__restrict__ f,
+                         const long long *sh, const int *st, const int *spre, int c, int n_home)
+{
+    const int lane = threadIdx.x & 31;
+    for (int p0 = 0; p0 < n_home; p0 += 32) {
+        const int i = p0 + lane;
+        const bool vi = i < n_home;
+        int si = st[0] + (vi ? i : 0);
+        if (vi && i >= k.scap) {
+            int o = __ldg(&k.cellq[c].y);
+            for (int m = k.scap; m < i; m++) o = __ldg(k.onext + o - 1);
+            si = k.nslots + o - 1;
+        }
+        const longlong4_16a pi = pos[si];
+        // coordinates relative to the home cell's centre (their differences
+        // may leave the range of 64 bits here: formed in FP64)
+        const double xi = (double)(pi.x + sh[0]), yi = (double)(pi.y + sh[kN3Half]), zi = (double)(pi.z + sh[2 * kN3Half]);
+        double fx = 0.0, fy = 0.0, fz = 0.0;
+        for (int kk = 0; kk < kN3Half; kk++) {
+            const int nn = spre[kk + 1] - spre[kk];
+            int o = 0;
+            for (int j = 0; j < nn; j++) {
+                int sj = st[kk] + j;
+                if (j >= k.scap) {
+                    o = j == k.scap ? __ldg(&k.cellq[half_cell(c, kk, k.nc, k.inv_nc)].y) : __ldg(k.onext + o - 1);
+                    sj = k.nslots + o - 1;
+                }
+                if (!vi || (kk == 0 && j <= i)) continue;
+                const longlong4_16a q = pos[sj];
+                const double dx = (xi - (double)(q.x + sh[kk])) * k.to_d,
+                             dy = (yi - (double)(q.y + sh[kN3Half + kk])) * k.to_d,
+                             dz = (zi - (double)(q.z + sh[2 * kN3Half + kk])) * k.to_d;
+                const double nf = fx_pair64(dx, dy, dz, k);
+                if (nf == 0.0) continue;
+                fx -= nf * dx;
+                fy -= nf * dy;
+                fz -= nf * dz;
+                fx_add64(f, (int)q.w, nf * dx, nf * dy, nf * dz);
+            }
+        }
+        if (vi) fx_add64(f, (int)pi.w, fx, fy, fz);
+    }
+}
+
+// Staging: the half stencil's candidates within rc of the home box, home
+// particles first; returns their number, or -1 when they and 64 entries of
+// padding would not fit.
+__device__ __forceinline__ int fx_stage(const FxParams &k, const longlong4_16a *__restrict__ pos, long long *X64,
+                                        float *X, int *iw, const long long *sh, const int *st, const int *spre, int tot,
+                                        int n_home)
+{
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u, le = (2u << lane) - 1u;
+    float bxl = 3.4e38f, byl = 3.4e38f, bzl = 3.4e38f, bxh = -3.4e38f, byh = -3.4e38f, bzh = -3.4e38f;
+    // warp-vote entry lookup, as n3_stage
+    const int s_e = lane < kN3Half ? spre[lane] : 0x7fffffff;
+    const bool ne = lane < kN3Half && spre[lane + 1] > s_e;
+    const unsigned nem = __ballot_sync(0xffffffffu, ne);
+    if (ne) iw[__popc(nem & lt)] = lane;
+    __syncwarp();
+    const int j_entry = lane < __popc(nem) ? iw[lane] : 0;
+    __syncwarp();
+    int T = 0;
+    constexpr int kB = 2;   // rounds whose loads are in flight together
+    for (int t0 = 0; t0 < tot; t0 += 32 * kB) {
+        longlong2 qa[kB], qb[kB];
+        int kcs[kB];
+#pragma unroll
+        for (int u = 0; u < kB; u++) {
+            const int tb = t0 + 32 * u, t = tb + lane;
+            const int o = s_e - tb;
+            const unsigned inside = __reduce_or_sync(0xffffffffu, (ne && o >= 1 && o <= 31) ? (1u << o) : 0u);
+            const int jc = __popc(__ballot_sync(0xffffffffu, ne && o <= 0)) - 1 + __popc(inside & le);
+            const int kc = __shfl_sync(0xffffffffu, j_entry, jc & 31);
+            const int kb = __shfl_sync(0xffffffffu, s_e, kc);
+            kcs[u] = kc;
+            const longlong2 *p = reinterpret_cast<const longlong2 *>(pos + min(st[kc] + (t - kb), k.last));
+            qa[u] = __ldg(p);
+            qb[u] = __ldg(p + 1);
+        }
+#pragma unroll
+        for (int u = 0; u < kB; u++) {
+            const int t = t0 + 32 * u + lane;
+            const int kc = kcs[u];
+            const long long x = qa[u].x + sh[kc], y = qa[u].y + sh[kN3Half + kc], z = qb[u].x + sh[2 * kN3Half + kc];
+            const float cx = (float)(int)(x >> 32) * k.to_f, cy = (float)(int)(y >> 32) * k.to_f,
+                        cz = (float)(int)(z >> 32) * k.to_f;
+            if (u == 0 && t0 == 0) {   // the home particles are the first n_home <= 32 candidates
+                if (lane < n_home) {
+                    bxl = bxh = cx;
+                    byl = byh = cy;
+                    bzl = bzh = cz;
+                }
+                box_reduce(bxl, byl, bzl, bxh, byh, bzh);
+            }
+            const float dx = fmaxf(fmaxf(bxl - cx, cx - bxh), 0.f);
+            const float dy = fmaxf(fmaxf(byl - cy, cy - byh), 0.f);
+            const float dz = fmaxf(fmaxf(bzl - cz, cz - bzh), 0.f);
+            const bool keep = t < tot && dx * dx + dy * dy + dz * dz < k.rc2_box;
+            const unsigned kept = __ballot_sync(0xffffffffu, keep);
+            if (T + __popc(kept) + 64 > k.cap) {   // the padding must fit too
+                __syncwarp();
+                return -1;
+            }
+            if (keep) {
+                const int s = T + __popc(kept & lt);
+                X[s] = cx;
+                X[k.cap + s] = cy;
+                X[2 * k.cap + s] = cz;
+                X64[s] = x;
+                X64[k.cap + s] = y;
+                X64[2 * k.cap + s] = z;
+                iw[s] = (int)qb[u].y;
+            }
+            T += __popc(kept);
+        }
+    }
+    for (int u = 0; u < 64; u += 32) X[T + u + lane] = X[k.cap + T + u + lane] = X[2 * k.cap + T + u + lane] = kFar;
+    __syncwarp();
+    return T;
+}
+
+// Phase B over one batch: the entries [0, E) of the list, home particles pb
+// .. pb + P - 1; every lane takes an equal contiguous range.
+__device__ __forceinline__ void fx_pairs(const FxParams &k, long long *__restrict__ acc, double4_16a *__restrict__ f,
+                                         const long long *X64, const int *iw, const uint16_t *list, const int *off,
+                                         int E, int P, int pb)
+{
+    const int lane = threadIdx.x & 31;
+    const int lo = (lane * E) >> 5, hi = ((lane + 1) * E) >> 5;
+    const long long *Y64 = X64 + k.cap, *Z64 = Y64 + k.cap;
+    if (lo < hi) {
+        int q = 0;
+#pragma unroll
+        for (int step = kFxPMax / 2; step > 0; step >>= 1)
+            if (q + step < P && off[q + step] <= lo) q += step;
+        int nxt = off[q + 1];
+        long long xp = X64[pb + q], yp = Y64[pb + q], zp = Z64[pb + q];
+        long long ax = 0, ay = 0, az = 0;
+        for (int e = lo; e < hi; e++) {
+            if (e == nxt) {
+                fx_add(acc, iw[pb + q], ax, ay, az);
+                do {
+                    q++;
+                    nxt = off[q + 1];
+                } while (nxt == e);
+                xp = X64[pb + q];
+                yp = Y64[pb + q];
+                zp = Z64[pb + q];
+                ax = ay = az = 0;
+            }
+            const int j = list[e];
+            const long long dx = xp - X64[j], dy = yp - Y64[j], dz = zp - Z64[j];
+            const unsigned long long R2 = fx_sq(dx) + fx_sq(dy) + fx_sq(dz);
+            if (R2 >= k.r2c) continue;
+            if (R2 < k.r2min) {   // too close for the fixed-point range
+                const double ex = (double)dx * k.to_d, ey = (double)dy * k.to_d, ez = (double)dz * k.to_d;
+                const double nf = fx_pair64(ex, ey, ez, k);
+                fx_add64(f, iw[pb + q], -nf * ex, -nf * ey, -nf * ez);
+                fx_add64(f, iw[j], nf * ex, nf * ey, nf * ez);
+                continue;
+            }
+            const long long t = fx_term(R2, k) >> k.tsh;
+            const long long gx = fx_mul(t, dx), gy = fx_mul(t, dy), gz = fx_mul(t, dz);
+            ax += gx;
+            ay += gy;
+            az += gz;
+            fx_add(acc, iw[j], -gx, -gy, -gz);
+        }
+        fx_add(acc, iw[pb + q], ax, ay, az);
+    }
+    __syncwarp();   // list and off are rewritten by the next batch
+}
+
+__global__ void __launch_bounds__(kFxThreads) k_force_fx(FxParams k, const longlong4_16a *__restrict__ pos,
+                                                         long long *__restrict__ acc, double4_16a *__restrict__ f)
+{
+    extern __shared__ __align__(16) unsigned char fxsmem[];
+    const int lane = threadIdx.x & 31;
+    const FxLayout L(k.cap);
+    long long *X64 = reinterpret_cast<long long *>(fxsmem + L.x64);
+    long long *sh = reinterpret_cast<long long *>(fxsmem + L.sh);
+    int *st = reinterpret_cast<int *>(sh + 3 * kN3Half);
+    float *X = reinterpret_cast<float *>(fxsmem + L.x32);
+    int *iw = reinterpret_cast<int *>(fxsmem + L.iw);
+    int *spre = reinterpret_cast<int *>(fxsmem + L.spre);
+    int *off = reinterpret_cast<int *>(fxsmem + L.off);
+    uint16_t *list = reinterpret_cast<uint16_t *>(fxsmem + L.list);
+    const unsigned lt = (1u << lane) - 1u;
+    pdl_wait();
+    if (blockIdx.x == 0 && lane == 0) {
+        k.cellq_next[k.ncell] = make_int2(0, 0);
+        *k.octr_next = 0u;
+    }
+    const float2 *X2 = reinterpret_cast<const float2 *>(X);
+    const float2 *Y2 = reinterpret_cast<const float2 *>(X + k.cap);
+    const float2 *Z2 = reinterpret_cast<const float2 *>(X + 2 * k.cap);
+    for (int c = blockIdx.x; c < k.ncell;) {
+        if (lane == 31) k.cellq_next[c] = make_int2(0, 0);
+        __syncwarp();   // the slice still holds the previous cell's data
+        // half-stencil table: first slot, prefix sums, image shift minus the
+        // home cell's centre
+        const HalfLoad tl = half_load<true, true>(reinterpret_cast<const int32_t *>(k.cellq), c, k.nc, k.inv_nc, 0, k.scap);
+        const int nn = tl.e - tl.s;
+        if (lane < kN3Half) {
+            int cx, cy, cz, dx, dy, dz;
+            lj_cell_decode(c, k.nc, k.inv_nc, cx, cy, cz);
+            half_delta(lane, dx, dy, dz);
+            const int ux = cx + dx, uy = cy + dy, uz = cz + dz;
+            sh[lane] = (ux < 0 ? -k.Lfix : ux >= k.nc ? k.Lfix : 0ll) - lj_fix64(__ldg(k.centre + cx), k.S);
+            sh[kN3Half + lane] = (uy < 0 ? -k.Lfix : uy >= k.nc ? k.Lfix : 0ll) - lj_fix64(__ldg(k.centre + cy), k.S);
+            sh[2 * kN3Half + lane] = (uz < 0 ? -k.Lfix : uz >= k.nc ? k.Lfix : 0ll) - lj_fix64(__ldg(k.centre + cz), k.S);
+            st[lane] = tl.s;
+        }
+        int Pf = nn;
+#pragma unroll
+        for (int o = 1; o < 16; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, Pf, o);
+            if (lane >= o) Pf += y;
+        }
+        if (lane < kN3Half) spre[lane] = Pf - nn;
+        if (lane == kN3Half - 1) spre[kN3Half] = Pf;
+        __syncwarp();
+        const int tot = spre[kN3Half], n_home = spre[1];
+        if (n_home > 0) {
+            const bool over = __any_sync(0xffffffffu, nn > k.scap);
+            const int T = over || n_home > 32 || tot > 4 * k.cap ? -1 : fx_stage(k, pos, X64, X, iw, sh, st, spre, tot, n_home);
+            if (T < 0) fx_plain(k, pos, f, sh, st, spre, c, n_home);
+            int p = T < 0 ? n_home : 0;
+            while (p < n_home) {
+                // Phase A: the lists of the batch's particles (candidates j > p)
+                const int pb = p;
+                int E = 0;
+                if (lane == 0) off[0] = 0;
+                while (p < n_home && E + T <= kFxList) {
+                    const float2 xs = f2(X[p]), ys = f2(X[k.cap + p]), zs = f2(X[2 * k.cap + p]);
+                    for (int j0 = p & ~63; j0 < T; j0 += 64) {
+                        const int jx = j0 + 2 * lane;
+                        const float2 qx = X2[(j0 >> 1) + lane], qy = Y2[(j0 >> 1) + lane], qz = Z2[(j0 >> 1) + lane];
+                        const float2 dx = __ffma2_rn(qx, f2(-1.0f), xs);
+                        const float2 dy = __ffma2_rn(qy, f2(-1.0f), ys);
+                        const float2 dz = __ffma2_rn(qz, f2(-1.0f), zs);
+                        float2 r2 = __fmul2_rn(dx, dx);
+                        r2 = __ffma2_rn(dy, dy, r2);
+                        r2 = __ffma2_rn(dz, dz, r2);
+                        const bool ina = r2.x < k.rc2_pair && jx > p;
+                        const bool inb = r2.y < k.rc2_pair && jx + 1 > p;
+                        const unsigned ba = __ballot_sync(0xffffffffu, ina);
+                        const unsigned bb = __ballot_sync(0xffffffffu, inb);
+                        if (ina) list[E + __popc(ba & lt)] = (uint16_t)jx;
+                        if (inb) list[E + __popc(ba) + __popc(bb & lt)] = (uint16_t)(jx + 1);
+                        E += __popc(ba) + __popc(bb);
+                    }
+                    if (lane == 0) off[p - pb + 1] = E;
+                    p++;
+                }
+                __syncwarp();
+                fx_pairs(k, acc, f, X64, iw, list, off, E, p - pb, pb);
+            }
+        }
+        unsigned nx = 0;   // the next cell (asked for when this one is done, as k_force_n3's single pulls)
+        if (lane == 0) nx = gridDim.x + atomicAdd(k.work, 1u);
+        c = (int)__shfl_sync(0xffffffffu, nx, 0);
+    }
+}
+
+}  // namespace
+
+int fx_shift(const lj_ctx *c) { return (int)floor(62.95 - log2(1.5 * c->cw)); }
+
+// acc counts 24 eps / sigma^2 2^-(S - 8 - tsh); tsh makes that 2^-52 / sigma
+// or more (the file header's range).
+static int fx_tsh(const lj_ctx *c)
+{
+    const int fb = (int)floor(63.0 - log2(1900.0 * c->p.sigma));
+    const int t = fx_shift(c) - 8 - fb;
+    return t > 0 ? t : 0;
+}
+
+double fx_scale(const lj_ctx *c)
+{
+    return ldexp(24.0 * c->p.eps / (c->p.sigma * c->p.sigma), 8 + fx_tsh(c) - fx_shift(c));
+}
+
+cudaError_t fx_configure(lj_ctx *c)
+{
+    const double mean = (double)c->p.n / (double)c->ncell;
+    // ~0.63 m of the m = 14 n_cell raw candidates survive the box test; room
+    // for 2.5 sqrt(m) more and the padding.  Slots cost resident warps (12 KB
+    // a warp at liquid density, 18 warps per SM): with 4 sqrt(m) + 96 the step
+    // at 10^6 particles took 688 us, with 2.5 sqrt(m) + 96 669, now 646.
+    const double m = kN3Half * mean;
+    int cap = ((int)(0.65 * m + 2.5 * sqrt(m)) + 64 + 7) & ~7;
+    cap = cap < 128 ? 128 : (cap > kFxList ? kFxList : cap);
+    c->fx_cap = cap;
+    c->fx_smem = FxLayout(cap).bytes;
+    cudaError_t e = raise_dyn_smem((const void *)k_force_fx, c->fx_smem);
+    if (e != cudaSuccess) return e;
+    int nb = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_force_fx, kFxThreads, c->fx_smem);
+    if (e != cudaSuccess) return e;
+    const int64_t grid = (int64_t)(nb > 0 ? nb : 1) * c->nsm;
+    c->fx_grid = (int)(grid < c->ncell ? grid : c->ncell);
+    return cudaSuccess;
+}
+
+cudaError_t launch_force_fx(lj_ctx *c, double4_16a *f)
+{
+    FxParams k;
+    memset(&k, 0, sizeof(k));
+    const double rc = c->p.rc, sg = c->p.sigma;
+    const int S = fx_shift(c);
+    k.nc = c->nc;
+    k.cap = c->fx_cap;
+    k.scap = c->scap;
+    k.nslots = c->nslots;
+    k.last = c->nslots + (int)c->p.n - 1;
+    k.inv_nc = c->inv_nc_f;
+    k.to_f = (float)ldexp(1.0, 32 - S);
+    k.rc2_box = (float)(rc * rc) * 1.0001f;
+    k.rc2_pair = (float)(rc * rc * (1.0 + 1e-4));
+    k.work = c->work;
+    k.ncell = c->ncell;
+    k.cellq = c->cellq[c->slot_par];
+    k.cellq_next = c->cellq[c->slot_par ^ 1];
+    k.octr_next = c->octr + (c->slot_par ^ 1);
+    k.onext = c->onext;
+    k.centre = c->centre;
+    k.S = S;
+    k.tsh = fx_tsh(c);
+    k.Lfix = lj_fix64(c->p.box, S);
+    int ex = 0;
+    const double mant = frexp(sg * sg, &ex);
+    k.K = (unsigned long long)ldexp(mant, 64);
+    k.kappa_e = ex + 2 * S - 129;
+    k.r2c = (unsigned long long)ldexp(rc * rc, 2 * S - 64);
+    const double rmin = ldexp(0.8 * sg * sg, 2 * S - 64);
+    k.r2min = rmin < (double)k.r2c ? (unsigned long long)rmin : k.r2c;
+    k.to_d = ldexp(1.0, -S);
+    const double s6 = sg * sg * sg * sg * sg * sg;
+    k.rc2 = rc * rc;
+    k.a12 = 48.0 * c->p.eps * s6 * s6;
+    k.b6 = 24.0 * c->p.eps * s6;
+    const longlong4_16a *pos = (const longlong4_16a *)c->spos;
+    long long *acc = c->fx_acc;
+    void *args[] = {&k, (void *)&pos, &acc, &f};
+    if (c->timing && c->ev_used + 2 <= c->nev) cudaEventRecord(c->ev[c->ev_used], c->stream);
+    const cudaError_t e = launch_pdl((const void *)k_force_fx, c->fx_grid, kFxThreads, args, (size_t)c->fx_smem, c->stream,
+                                     !c->timing);
+    if (c->timing && c->ev_used + 2 <= c->nev) {
+        cudaEventRecord(c->ev[c->ev_used + 1], c->stream);
+        c->ev_used += 2;
+    }
+    c->kernel_launches++;
+    if (e != cudaSuccess) return e;
+    slots_consumed(c);
+    return cudaGetLastError();
+}

@@ -170,7 +170,7 @@ cudaError_t launch_force_n3(lj_ctx *c, void *f, bool energy)
     k.lgw = c->n3_lgw;
     // the slotted binning, when it was one, has zeroed f
     const bool slots = c->slots_open == 1;
-    const float4 *pos = slots ? c->spos : (const float4 *)c->pos;
+    const float4 *pos = (const float4 *)(slots ? c->spos : c->pos);
     const int32_t *start = c->start;
     if (slots) {
         k.last = c->nslots + k.n - 1;

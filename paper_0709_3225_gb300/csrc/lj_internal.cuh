@@ -130,8 +130,13 @@ struct lj_ctx {
     int scap, nslots;        // nslots = ncell * scap; spos holds nslots + n
     int2 *cellq[2];
     unsigned *octr;          // [2] overflow particles per buffer
-    float4 *spos, *sg4;      // slotted positions; cotangents (lazily allocated)
+    void *spos;              // slotted positions: float4 (FP64: longlong4)
+    float4 *sg4;             // cotangents (lazily allocated)
     int32_t *onext;          // overflow lists: index + 1 of the next, 0 = end
+    // FP64 contexts (lj_force_fx.cu): spos holds longlong4 (fixed-point
+    // coordinates, particle index), fx_acc the force sums, int64[4] per particle
+    long long *fx_acc;
+    int fx_cap, fx_smem, fx_grid;
     int slot_par;            // buffer of the next binning
     int slots_open;          // 1: a slotted binning waits for its kernel, 2: the buffers are not known to be zero
     int slots_last;          // the last binning was a slotted one
@@ -157,6 +162,22 @@ struct lj_ctx {
     int64_t force_launches;
     int64_t kernel_launches;
 };
+
+// x 2^S mod 2^64 for x >= 0, truncated (exact when x >= 2^(53-S)).
+__host__ __device__ __forceinline__ long long lj_fix64(double x, int S)
+{
+#ifdef __CUDA_ARCH__
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+#else
+    unsigned long long b;
+    __builtin_memcpy(&b, &x, sizeof(b));
+#endif
+    const int e = (int)(b >> 52) & 0x7ff;
+    const unsigned long long m = (b & 0xfffffffffffffull) | (e ? 1ull << 52 : 0ull);
+    const int s = e - 1075 + S;
+    if (s >= 0) return s < 64 ? (long long)(m << s) : 0ll;
+    return s > -64 ? (long long)(m >> -s) : 0ll;
+}
 
 // ---------------------------------------------------------------- device --
 
@@ -472,6 +493,19 @@ cudaError_t launch_kick_drift_slots(lj_ctx *c, double *x, double *v, float4 *f, 
                                     int64_t i_end = -1, bool after_force = false);
 cudaError_t slots_begin(lj_ctx *c, int64_t i_begin);   // before a slotted binning launch
 void slots_consumed(lj_ctx *c);                        // after the launch that reads it
+// FP64 contexts: the fixed-point kernel (lj_force_fx.cu) over slotted cells.
+// Its forces are f (the pairs taken in FP64) plus fx_scale times fx_acc:
+// launch_kick_drift_fx reads both (with_acc) or f alone and zeroes them,
+// launch_fx_finish leaves the sum in f and with v adds the half kick.
+bool uses_fx(const lj_ctx *c);
+int fx_shift(const lj_ctx *c);
+double fx_scale(const lj_ctx *c);
+cudaError_t fx_configure(lj_ctx *c);
+cudaError_t launch_force_fx(lj_ctx *c, double4_16a *f);
+cudaError_t launch_bin_fx(lj_ctx *c, const double *x, double4_16a *f);
+cudaError_t launch_kick_drift_fx(lj_ctx *c, double *x, double *v, double4_16a *f, int nkick, bool with_acc,
+                                 int64_t i_begin = 0, int64_t i_end = -1, bool after_force = false);
+cudaError_t launch_fx_finish(lj_ctx *c, double *v, double4_16a *f);
 // Rebuild cell_of, start and perm from the last slotted binning.
 cudaError_t launch_slots_to_lists(lj_ctx *c);
 cudaError_t launch_force_n3(lj_ctx *c, void *f, bool energy);

@@ -78,6 +78,111 @@ __global__ void __launch_bounds__(256) k_kick_drift_slots(SlotBin b, double *__r
     slot_place(b, valid, i, px, py, pz, err);
 }
 
+// The FP64 forms (lj_force_fx.cu): fixed-point coordinates; f holds the
+// forces of the pairs taken in FP64 and acc, in units of 1 / scale, those of
+// all others.
+__device__ __forceinline__ void fx_force(const double4_16a *f, const longlong2 *acc, int i, double scale, double &fx,
+                                         double &fy, double &fz)
+{
+    const double4_16a q = f[i];
+    const longlong2 a = acc[2 * (int64_t)i], b = acc[2 * (int64_t)i + 1];
+    fx = fma((double)a.x, scale, q.x);
+    fy = fma((double)a.y, scale, q.y);
+    fz = fma((double)b.x, scale, q.z);
+}
+
+__device__ __forceinline__ void fx_zero(double4_16a *f, longlong2 *acc, int i)
+{
+    double4_16a z;
+    z.x = z.y = z.z = z.w = 0.0;
+    f[i] = z;
+    acc[2 * (int64_t)i] = acc[2 * (int64_t)i + 1] = make_longlong2(0, 0);
+}
+
+__global__ void __launch_bounds__(256) k_bin_fx(SlotBin b, const double *__restrict__ x, int n, double4_16a *__restrict__ f,
+                                                longlong2 *__restrict__ acc, int32_t *__restrict__ err)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i == 0) *b.work = 0u;
+    const bool valid = i < n;
+    double px = 0.0, py = 0.0, pz = 0.0;
+    if (valid) {
+        const int64_t o = 3 * (int64_t)i;
+        px = lj_wrap_fast(x[o], b.L, b.whi, b.wlo);
+        py = lj_wrap_fast(x[o + 1], b.L, b.whi, b.wlo);
+        pz = lj_wrap_fast(x[o + 2], b.L, b.whi, b.wlo);
+        fx_zero(f, acc, i);
+    }
+    slot_place<true>(b, valid, i, px, py, pz, err);
+}
+
+// k_kick_drift_slots in FP64; with_acc: f alone is not yet the force.
+__global__ void __launch_bounds__(256) k_kick_drift_fx(SlotBin b, double *__restrict__ x, double *__restrict__ v,
+                                                       double4_16a *__restrict__ f, longlong2 *__restrict__ acc,
+                                                       int with_acc, double scale, int i_begin, int n, double hk,
+                                                       double dt, int32_t *__restrict__ err)
+{
+    pdl_wait();
+    const int t = (gridDim.x - 1 - blockIdx.x) * blockDim.x + threadIdx.x;
+    if (t == 0) *b.work = 0u;
+    const int i = i_begin + t;
+    const bool valid = i < n;
+    double px = 0.0, py = 0.0, pz = 0.0;
+    if (valid) {
+        const int64_t o = 3 * (int64_t)i;
+        double fx, fy, fz;
+        if (with_acc) {
+            fx_force(f, acc, i, scale, fx, fy, fz);
+        } else {
+            const double4_16a q = f[i];
+            fx = q.x;
+            fy = q.y;
+            fz = q.z;
+        }
+        fx_zero(f, acc, i);
+        const double vx = __fma_rn(hk, fx, v[o]);
+        const double vy = __fma_rn(hk, fy, v[o + 1]);
+        const double vz = __fma_rn(hk, fz, v[o + 2]);
+        px = lj_wrap_fast(__fma_rn(dt, vx, x[o]), b.L, b.whi, b.wlo);
+        py = lj_wrap_fast(__fma_rn(dt, vy, x[o + 1]), b.L, b.whi, b.wlo);
+        pz = lj_wrap_fast(__fma_rn(dt, vz, x[o + 2]), b.L, b.whi, b.wlo);
+        v[o] = vx;
+        v[o + 1] = vy;
+        v[o + 2] = vz;
+        x[o] = px;
+        x[o + 1] = py;
+        x[o + 2] = pz;
+    }
+    slot_place<true>(b, valid, i, px, py, pz, err);
+}
+
+// f := the force; with v also the closing half kick v += h f.
+__global__ void __launch_bounds__(256) k_fx_finish(double *__restrict__ v, double4_16a *__restrict__ f,
+                                                   const longlong2 *__restrict__ acc, int n, double scale, double h)
+{
+    pdl_wait();
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    double4_16a q;
+    fx_force(f, acc, i, scale, q.x, q.y, q.z);
+    q.w = 0.0;
+    f[i] = q;
+    if (v) {
+        const int64_t o = 3 * (int64_t)i;
+        v[o] = __fma_rn(h, q.x, v[o]);
+        v[o + 1] = __fma_rn(h, q.y, v[o + 1]);
+        v[o + 2] = __fma_rn(h, q.z, v[o + 2]);
+    }
+}
+
+// Particle index of a slot.
+template <bool FX>
+__device__ __forceinline__ int slot_index(const void *pos, int64_t s)
+{
+    if constexpr (FX) return (int)reinterpret_cast<const longlong2 *>(pos)[2 * s + 1].y;
+    return __float_as_int(reinterpret_cast<const float4 *>(pos)[s].w);
+}
+
 // Counts of every cell (the extra one included) for the scan of
 // launch_slots_to_lists; cell_of starts as the extra cell everywhere.
 __global__ void k_slot_counts(const int2 *__restrict__ cellq, int ncell1, int32_t *__restrict__ count, int n,
@@ -90,7 +195,8 @@ __global__ void k_slot_counts(const int2 *__restrict__ cellq, int ncell1, int32_
 
 // perm and cell_of of the particles in slots and overflow lists, one thread
 // per cell.
-__global__ void k_slot_lists(const int2 *__restrict__ cellq, const float4 *__restrict__ pos,
+template <bool FX>
+__global__ void k_slot_lists(const int2 *__restrict__ cellq, const void *__restrict__ pos,
                              const int32_t *__restrict__ onext, int ncell, int cap, int nslots,
                              const int32_t *__restrict__ start, int32_t *__restrict__ perm,
                              int32_t *__restrict__ cell_of)
@@ -101,12 +207,12 @@ __global__ void k_slot_lists(const int2 *__restrict__ cellq, const float4 *__res
     const int s = start[c];
     int r = 0;
     for (; r < min(q.x, cap); r++) {
-        const int i = __float_as_int(pos[(int64_t)c * cap + r].w);
+        const int i = slot_index<FX>(pos, (int64_t)c * cap + r);
         perm[s + r] = i;
         cell_of[i] = c;
     }
     for (int o = q.y; o > 0; o = onext[o - 1], r++) {
-        const int i = __float_as_int(pos[(int64_t)nslots + o - 1].w);
+        const int i = slot_index<FX>(pos, (int64_t)nslots + o - 1);
         perm[s + r] = i;
         cell_of[i] = c;
     }
@@ -144,6 +250,7 @@ SlotBin slot_bin_of(const lj_ctx *c)
     b.ncell = (int)c->ncell;
     b.cap = c->scap;
     b.nslots = c->nslots;
+    b.S = c->p.precision == LJ_PREC_FP64 ? fx_shift(c) : 0;
     return b;
 }
 
@@ -155,10 +262,13 @@ void slots_free(lj_ctx *c)
     cudaFree(c->spos);
     cudaFree(c->sg4);
     cudaFree(c->onext);
+    cudaFree(c->fx_acc);
     c->cellq[0] = c->cellq[1] = nullptr;
     c->octr = nullptr;
-    c->spos = c->sg4 = nullptr;
+    c->spos = nullptr;
+    c->sg4 = nullptr;
     c->onext = nullptr;
+    c->fx_acc = nullptr;
     c->scap = c->nslots = 0;
     c->slot_par = c->slots_open = c->slots_last = 0;
 }
@@ -166,7 +276,9 @@ void slots_free(lj_ctx *c)
 cudaError_t slots_setup(lj_ctx *c)
 {
     slots_free(c);
-    if (c->p.precision != LJ_PREC_MIXED || c->p.cell_subdiv == 2 || c->p.n == 0) return cudaSuccess;
+    // (FP64: the fixed-point kernel has no force-shifted form)
+    const bool fp64 = c->p.precision == LJ_PREC_FP64;
+    if (c->p.cell_subdiv == 2 || c->p.n == 0 || (fp64 && c->p.shift_mode == LJ_SHIFT_FORCE)) return cudaSuccess;
     // Slots per cell: the mean occupancy plus 7 standard deviations of a
     // random gas, a multiple of 8 (128 bytes), at most the 32 home particles
     // that the kernels' fast path takes.
@@ -182,7 +294,9 @@ cudaError_t slots_setup(lj_ctx *c)
     const size_t qb = (size_t)(c->ncell + 1) * sizeof(int2);
     for (int k = 0; k < 2 && e == cudaSuccess; k++) e = cudaMalloc(&c->cellq[k], qb);
     if (e == cudaSuccess) e = cudaMalloc(&c->octr, 2 * sizeof(unsigned));
-    if (e == cudaSuccess) e = cudaMalloc(&c->spos, (size_t)(nslots + c->p.n) * sizeof(float4));
+    if (e == cudaSuccess)
+        e = cudaMalloc(&c->spos, (size_t)(nslots + c->p.n) * (fp64 ? sizeof(longlong4_16a) : sizeof(float4)));
+    if (e == cudaSuccess && fp64) e = cudaMalloc(&c->fx_acc, (size_t)c->p.n * 4 * sizeof(long long));
     if (e == cudaSuccess) e = cudaMalloc(&c->onext, (size_t)c->p.n * sizeof(int32_t));
     if (e == cudaErrorMemoryAllocation) {   // the sorted lists need less
         cudaGetLastError();
@@ -193,19 +307,71 @@ cudaError_t slots_setup(lj_ctx *c)
     c->scap = cap;
     c->nslots = (int)nslots;
     c->slots_open = 2;
-    return cudaSuccess;
+    return fp64 ? fx_configure(c) : cudaSuccess;
 }
 
 // Force evaluations take the slotted cells where the pair-once kernel runs
 // and a cell beyond its slots is rare: cells so thinly filled that even a
 // random gas overflows one in some 10^5, or a dense fluid (n sigma^3 / L^3
 // >= 0.5), whose excluded volume keeps the occupancy near its mean.
-bool uses_slots(const lj_ctx *c)
+static bool slots_suit(const lj_ctx *c)
 {
-    if (c->scap == 0 || c->skin > 0.0 || c->fuse_update || !uses_force_n3(c)) return false;
     const double mean = (double)c->p.n / (double)c->ncell;
     const double sg = c->p.sigma / c->p.box;
     return mean + 4.5 * sqrt(mean) <= kSlotMax || (double)c->p.n * sg * sg * sg >= 0.5;
+}
+
+bool uses_slots(const lj_ctx *c)
+{
+    return c->scap > 0 && c->skin <= 0.0 && !c->fuse_update && uses_force_n3(c) && slots_suit(c);
+}
+
+// The fixed-point term's error is below FP64's while rc <= 5 sigma (measured
+// against 113 bits: 2.7e-15 against 1.4e-14, in units of 24 eps / sigma^2, at
+// 2.5 and 3, 1.1e-14 against 1.3e-14 at 5, 4.2e-14 against 1.2e-14 at 10:
+// r^2 is held in units of rc^2 2^-60).
+bool uses_fx(const lj_ctx *c)
+{
+    return c->scap > 0 && c->p.rc <= 4.0 * c->p.sigma && c->skin <= 0.0 && c->p.precision == LJ_PREC_FP64 && c->n3 && !c->deterministic &&
+           !c->use_run_kernel && !c->use_aop && slots_suit(c);
+}
+
+cudaError_t launch_bin_fx(lj_ctx *c, const double *x, double4_16a *f)
+{
+    cudaError_t e = slots_begin(c, 0);
+    if (e != cudaSuccess) return e;
+    const int n = (int)c->p.n;
+    k_bin_fx<<<blocks_for(n, 256), 256, 0, c->stream>>>(slot_bin_of(c), x, n, f, (longlong2 *)c->fx_acc, c->err);
+    c->kernel_launches++;
+    return cudaGetLastError();
+}
+
+cudaError_t launch_kick_drift_fx(lj_ctx *c, double *x, double *v, double4_16a *f, int nkick, bool with_acc,
+                                 int64_t i_begin, int64_t i_end, bool after_force)
+{
+    const int n = (int)(i_end < 0 ? c->p.n : i_end);
+    if (n <= (int)i_begin) return cudaSuccess;
+    cudaError_t e = slots_begin(c, i_begin);
+    if (e != cudaSuccess) return e;
+    SlotBin b = slot_bin_of(c);
+    int i0 = (int)i_begin, i1 = n, wa = with_acc ? 1 : 0;
+    double h = nkick * (0.5 * c->p.dt / c->p.mass), dt = c->p.dt, scale = fx_scale(c);
+    int32_t *err = c->err;
+    void *args[] = {&b, &x, &v, &f, &c->fx_acc, &wa, &scale, &i0, &i1, &h, &dt, &err};
+    e = launch_pdl((const void *)k_kick_drift_fx, (int)blocks_for(n - i_begin, 256), 256, args, 0, c->stream, after_force);
+    c->kernel_launches++;
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+cudaError_t launch_fx_finish(lj_ctx *c, double *v, double4_16a *f)
+{
+    int n = (int)c->p.n;
+    double scale = fx_scale(c), h = 0.5 * c->p.dt / c->p.mass;
+    void *args[] = {&v, &f, &c->fx_acc, &n, &scale, &h};
+    const cudaError_t e = launch_pdl((const void *)k_fx_finish, (int)blocks_for(n, 256), 256, args, 0, c->stream,
+                                     !c->timing);
+    c->kernel_launches++;
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 cudaError_t slots_begin(lj_ctx *c, int64_t i_begin)
@@ -267,8 +433,12 @@ cudaError_t launch_slots_to_lists(lj_ctx *c)
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = launch_scan(c);   // start from the counts, which it zeroes
     if (e != cudaSuccess) return e;
-    k_slot_lists<<<blocks_for(ncell, 256), 256, 0, c->stream>>>(q, c->spos, c->onext, ncell, c->scap, c->nslots,
-                                                                c->start, c->perm, c->cell_of);
+    if (c->p.precision == LJ_PREC_FP64)
+        k_slot_lists<true><<<blocks_for(ncell, 256), 256, 0, c->stream>>>(q, c->spos, c->onext, ncell, c->scap, c->nslots,
+                                                                          c->start, c->perm, c->cell_of);
+    else
+        k_slot_lists<false><<<blocks_for(ncell, 256), 256, 0, c->stream>>>(q, c->spos, c->onext, ncell, c->scap,
+                                                                           c->nslots, c->start, c->perm, c->cell_of);
     k_slot_extra<<<blocks_for(n, 256), 256, 0, c->stream>>>(c->cell_of, n, ncell, c->start, c->perm, c->count + ncell);
     c->kernel_launches += 2;
     e = cudaMemsetAsync(c->count + ncell, 0, sizeof(int32_t), c->stream);

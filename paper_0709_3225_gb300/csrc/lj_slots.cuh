@@ -21,14 +21,14 @@
 
 struct SlotBin {
     int2 *cellq;            // this binning's (count, list head + 1) per cell, zero before it
-    float4 *pos;            // [nslots + n]
+    void *pos;              // [nslots + n] float4, or longlong4 in FP64 contexts
     int32_t *onext;
     unsigned *octr, *work;  // overflow counter of this buffer; the force kernel's work counter, zeroed here
     const float2 *centre;   // cell centres as two floats
     const long long *thb;
     double L, whi, wlo, s;
     float sf;               // (float)s
-    int nc, ncell, cap, nslots;
+    int nc, ncell, cap, nslots, S;   // S: scale of the fixed-point coordinates (FP64)
 };
 
 #ifdef __CUDACC__
@@ -46,9 +46,10 @@ __device__ __forceinline__ int3 slot_cell(const SlotBin &b, double px, double py
     return c;
 }
 
-// Rank particle i in its cell and store its position relative to the cell
-// centre.  All 32 lanes call it; lanes with valid = false do nothing.
-// Returns the slot, or -1 when none was taken.
+// Rank particle i in its cell and store its position, relative to the cell
+// centre (FX: in fixed point, lj_force_fx.cu).  All 32 lanes call it; lanes
+// with valid = false do nothing.  Returns the slot, or -1 when none was taken.
+template <bool FX = false>
 __device__ __forceinline__ int slot_place(const SlotBin &b, bool valid, int i, double px, double py, double pz,
                                           int32_t *err)
 {
@@ -71,8 +72,15 @@ __device__ __forceinline__ int slot_place(const SlotBin &b, bool valid, int i, d
         slot = b.nslots + k;
         b.onext[k] = atomicExch(&b.cellq[c].y, k + 1);
     }
-    b.pos[slot] = make_float4(rel_f32(px, __ldg(b.centre + cc.x)), rel_f32(py, __ldg(b.centre + cc.y)),
-                              rel_f32(pz, __ldg(b.centre + cc.z)), __int_as_float(i));
+    if constexpr (FX) {
+        longlong2 *o = reinterpret_cast<longlong2 *>(b.pos) + 2 * (int64_t)slot;
+        o[0] = make_longlong2(lj_fix64(px, b.S), lj_fix64(py, b.S));
+        o[1] = make_longlong2(lj_fix64(pz, b.S), (long long)i);
+    } else {
+        reinterpret_cast<float4 *>(b.pos)[slot] =
+            make_float4(rel_f32(px, __ldg(b.centre + cc.x)), rel_f32(py, __ldg(b.centre + cc.y)),
+                        rel_f32(pz, __ldg(b.centre + cc.z)), __int_as_float(i));
+    }
     return slot;
 }
 

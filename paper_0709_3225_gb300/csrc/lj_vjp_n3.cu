@@ -595,7 +595,7 @@ cudaError_t launch_vjp_n3(lj_ctx *c, const double *coef, double scale, double *d
     k.grab = 4;
     k.ncell = c->ncell;
     k.work = c->work;
-    const float4 *pos = slots ? c->spos : (const float4 *)c->pos;
+    const float4 *pos = (const float4 *)(slots ? c->spos : c->pos);
     const float4 *g4 = slots ? c->sg4 : (const float4 *)c->g4;
     const int32_t *start = c->start;
     double *partial = c->partial;
