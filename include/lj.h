@@ -308,6 +308,19 @@ int lj_forces_vjp(lj_ctx *ctx, const double *x, const double *g, double scale, d
 int lj_vv_adjoint_step(lj_ctx *ctx, const double *x_n, const double *x_n1, double *lam_x, double *lam_v,
                        double *dparam);
 
+/* nsteps velocity-Verlet steps (Section 2) that keep every state's positions:
+ * traj (device (nsteps + 1, n, 3) double) holds the start positions in
+ * traj[0], f (as lj_step's) the forces there; afterwards traj[s] holds the
+ * positions after s steps, v and f those of the last.  Asynchronous. */
+int lj_step_record(lj_ctx *ctx, double *traj, double *v, void *f, int32_t nsteps);
+
+/* The adjoint of nsteps steps, from the positions lj_step_record kept: what
+ * lj_vv_adjoint_step over (traj[s], traj[s + 1]), s = nsteps - 1 .. 0, gives
+ * up to rounding, with one VJP per state (the last VJP of a step and the
+ * first of the one after it are of the same cotangents).  Asynchronous. */
+int lj_vv_adjoint_segment(lj_ctx *ctx, const double *traj, int32_t nsteps, double *lam_x, double *lam_v,
+                          double *dparam);
+
 /* Cell lists with a skin (Section 3.1: cells wider than the interaction
  * range plus a skin lambda stay valid while particles move, so they need not
  * be rebuilt every step; the paper's one-step-lagged update is the case of a

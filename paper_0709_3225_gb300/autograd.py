@@ -10,7 +10,7 @@ The paper has no adjoint; these differentiate its force (Eq. n2_force with the
 Section 2 pair force, rc held fixed) and its velocity-Verlet integration.
 The cell list is piecewise constant and contributes no derivative.  Every
 arithmetic step runs in the library's kernels (lj_forces, lj_step,
-lj_forces_vjp, lj_vv_adjoint_step); this module only sequences the calls and
+lj_forces_vjp, lj_step_record, lj_vv_adjoint_segment); this module only sequences the calls and
 keeps checkpoints.  Use the force-shifted potential (shift_mode 2) when the
 trajectory derivative must match finite differences: with the energy shift
 the force jumps at rc and the trajectory is not differentiable there.
@@ -80,15 +80,12 @@ class _Trajectory(torch.autograd.Function):
         f = torch.empty((ctx.n, 4), dtype=ctx.force_dtype, device=ref.device)
         for xs, vs, k in reversed(fctx.ckpts):
             # recompute the segment's states from its checkpoint
-            x = xs.clone()
+            traj = torch.empty((k + 1, ctx.n, 3), dtype=torch.float64, device=xs.device)
+            traj[0].copy_(xs)
             v = vs.clone()
-            lj.lj_forces(ctx, x, f)
-            states = [x.clone()]
-            for _ in range(k):
-                lj.lj_step(ctx, x, v, f, 1)
-                states.append(x.clone())
-            for s in range(k - 1, -1, -1):
-                lj.lj_vv_adjoint_step(ctx, states[s], states[s + 1], lam_x, lam_v, dp)
+            lj.lj_forces(ctx, traj[0], f)
+            lj.lj_step_record(ctx, traj, v, f, k)
+            lj.lj_vv_adjoint_segment(ctx, traj, k, lam_x, lam_v, dp)
         fctx.ckpts = None
         return lam_x, lam_v, dp.to(theta.device, theta.dtype), None, None, None
 

@@ -623,7 +623,7 @@ cudaError_t launch_vjp_warp(lj_ctx *c, const VjpCoef &kd, double scale, double *
 }  // namespace
 
 static cudaError_t launch_vjp_terms(lj_ctx *c, const double *g, double scale, double *dx, double *dparam, double *lam,
-                                    double dt_axpy, bool *lam_done)
+                                    double dt_axpy, const double *next, bool *lam_done)
 {
     const int n = (int)c->p.n;
     const bool fp64 = c->p.precision == LJ_PREC_FP64;
@@ -649,7 +649,7 @@ static cudaError_t launch_vjp_terms(lj_ctx *c, const double *g, double scale, do
         // each pair once (lj_vjp_n3.cu); f_sorted is its float4 accumulator
         const double coef[7] = {k.rc2, k.a1, k.b1, k.fc1, k.dfc1, k.eps, k.inv_sigma};
         *lam_done = true;
-        return launch_vjp_n3(c, coef, scale, dx, (float4 *)c->f_sorted, dparam, lam, dt_axpy);
+        return launch_vjp_n3(c, coef, scale, dx, (float4 *)c->f_sorted, dparam, lam, dt_axpy, next);
     }
     if (!fp64) return launch_vjp_warp(c, k, scale, dx, dparam);
     if (c->p.cell_subdiv != 2 && c->wcap > 0 && c->w64_lcap > 0) {
@@ -680,11 +680,11 @@ static cudaError_t launch_vjp_terms(lj_ctx *c, const double *g, double scale, do
 }
 
 cudaError_t launch_vjp(lj_ctx *c, const double *g, double scale, double *dx, double *dparam, double *lam,
-                       double dt_axpy)
+                       double dt_axpy, const double *next)
 {
     if (c->p.n == 0) return cudaSuccess;
     bool lam_done = false;
-    const cudaError_t e = launch_vjp_terms(c, g, scale, dx, dparam, lam, dt_axpy, &lam_done);
+    const cudaError_t e = launch_vjp_terms(c, g, scale, dx, dparam, lam, dt_axpy, next, &lam_done);
     if (e != cudaSuccess || !lam || lam_done) return e;
     return launch_axpy(c, lam, dx, dt_axpy);
 }

@@ -436,8 +436,9 @@ cudaError_t warp_force_configure(lj_ctx *c);
 // Staged-candidate capacity per warp of the warp kernels (lj_force_warp.cu).
 int warp_stencil_cap(double mean_occupancy, int subdiv, int threads, int static_bytes);
 // lam (NULL: not): then also lam += dt_axpy * dx, with the updated dx.
+// next (slotted cells, with lam): the positions of the VJP of lam that follows, which are binned here too.
 cudaError_t launch_vjp(lj_ctx *c, const double *g, double scale, double *dx, double *dparam, double *lam = nullptr,
-                       double dt_axpy = 0.0);
+                       double dt_axpy = 0.0, const double *next = nullptr);
 cudaError_t launch_axpy(lj_ctx *c, double *y, const double *x, double a);
 cudaError_t launch_force_warp(lj_ctx *c, void *f, bool energy);
 // FP64 warp kernel with compacted pair lists (lj_force_w64.cu); it uses the
@@ -478,7 +479,7 @@ bool uses_force_n3(const lj_ctx *c);   // launch_force dispatches to the pair-on
 bool uses_vjp_n3(const lj_ctx *c);
 // lam: also lam += dt_axpy * dx (NULL: not); dparam += scale * the sums.
 cudaError_t launch_vjp_n3(lj_ctx *c, const double *coef, double scale, double *dx, float4 *acc, double *dparam,
-                          double *lam, double dt_axpy);
+                          double *lam, double dt_axpy, const double *next);
 // Slotted cells (lj_slots.cu): set up for the context's grid (scap stays 0
 // where they do not apply), whether force evaluations take them, and the
 // binning: bin x (any coordinates), zero `zero` (float4 [n]), and with g
@@ -489,8 +490,9 @@ bool uses_slots(const lj_ctx *c);
 cudaError_t launch_bin_slots(lj_ctx *c, const double *x, float4 *zero, const double *g);
 // after_force: the launch before it in the stream is this context's force
 // kernel (then they overlap, pdl_wait).
-cudaError_t launch_kick_drift_slots(lj_ctx *c, double *x, double *v, float4 *f, int nkick, int64_t i_begin = 0,
-                                    int64_t i_end = -1, bool after_force = false);
+// xo: where the new positions go (x, or another state).
+cudaError_t launch_kick_drift_slots(lj_ctx *c, const double *x, double *xo, double *v, float4 *f, int nkick,
+                                    int64_t i_begin = 0, int64_t i_end = -1, bool after_force = false);
 cudaError_t slots_begin(lj_ctx *c, int64_t i_begin);   // before a slotted binning launch
 void slots_consumed(lj_ctx *c);                        // after the launch that reads it
 // FP64 contexts: the fixed-point kernel (lj_force_fx.cu) over slotted cells.

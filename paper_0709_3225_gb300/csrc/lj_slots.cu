@@ -44,9 +44,10 @@ __global__ void __launch_bounds__(256) k_bin_slots(SlotBin b, const double *__re
 // the scan of the counts (11 us, and 10 us of latency at 131,072 particles
 // too), k_scatter (49 us) and the zeroing of f.  Per step: 815 -> 763 us at
 // 4M, 57 -> 40 at 131,072, 26 -> 16.5 at 2,048.
-__global__ void __launch_bounds__(256) k_kick_drift_slots(SlotBin b, double *__restrict__ x, double *__restrict__ v,
-                                                          float4 *__restrict__ f, int i_begin, int n, double hk,
-                                                          double dt, int32_t *__restrict__ err)
+// xo: where the new positions go, x itself or the next state of a trajectory.
+__global__ void __launch_bounds__(256) k_kick_drift_slots(SlotBin b, const double *x, double *xo,
+                                                          double *__restrict__ v, float4 *__restrict__ f, int i_begin,
+                                                          int n, double hk, double dt, int32_t *__restrict__ err)
 {
     pdl_wait();
     // the last particles first: what this kernel wrote last, and the force
@@ -71,9 +72,9 @@ __global__ void __launch_bounds__(256) k_kick_drift_slots(SlotBin b, double *__r
         v[o] = vx;
         v[o + 1] = vy;
         v[o + 2] = vz;
-        x[o] = px;
-        x[o + 1] = py;
-        x[o + 2] = pz;
+        xo[o] = px;
+        xo[o + 1] = py;
+        xo[o + 2] = pz;
     }
     slot_place(b, valid, i, px, py, pz, err);
 }
@@ -405,8 +406,8 @@ cudaError_t launch_bin_slots(lj_ctx *c, const double *x, float4 *zero, const dou
     return cudaGetLastError();
 }
 
-cudaError_t launch_kick_drift_slots(lj_ctx *c, double *x, double *v, float4 *f, int nkick, int64_t i_begin,
-                                    int64_t i_end, bool after_force)
+cudaError_t launch_kick_drift_slots(lj_ctx *c, const double *x, double *xo, double *v, float4 *f, int nkick,
+                                    int64_t i_begin, int64_t i_end, bool after_force)
 {
     const int n = (int)(i_end < 0 ? c->p.n : i_end);
     if (n <= (int)i_begin) return cudaSuccess;
@@ -417,7 +418,7 @@ cudaError_t launch_kick_drift_slots(lj_ctx *c, double *x, double *v, float4 *f, 
     int i0 = (int)i_begin, i1 = n;
     double h = hk, dt = c->p.dt;
     int32_t *err = c->err;
-    void *args[] = {&b, &x, &v, &f, &i0, &i1, &h, &dt, &err};
+    void *args[] = {&b, (void *)&x, &xo, &v, &f, &i0, &i1, &h, &dt, &err};
     e = launch_pdl((const void *)k_kick_drift_slots, (int)blocks_for(n - i_begin, 256), 256, args, 0, c->stream, after_force);
     c->kernel_launches++;
     return e != cudaSuccess ? e : cudaGetLastError();

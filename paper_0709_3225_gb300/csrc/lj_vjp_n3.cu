@@ -31,6 +31,7 @@
 #include <math.h>
 
 #include "lj_force_n3.cuh"
+#include "lj_slots.cuh"
 
 namespace {
 
@@ -484,11 +485,15 @@ __global__ void __launch_bounds__(kVn3Threads, 4) k_vjp_n3(VjpN3Coef k, const fl
 // dx[i] += scale * acc[i] (FP64), particle order, then with lam also lam += a
 // dx (the drift of the velocity-Verlet adjoint); block 0 adds scale times the
 // sum of the parameter partials to dparam instead (fixed order).  One launch
-// for what were three: at 32,000 particles each took 3 to 6 us.
-__global__ void __launch_bounds__(kReduceThreads) k_vjp_finish(const float4 *__restrict__ acc, int n, double scale,
+// for what were three: at 32,000 particles each took 3 to 6 us.  BIN: the
+// binning of x, for the VJP of lam that follows (k_bin_slots), as well.
+template <bool BIN>
+__global__ void __launch_bounds__(kReduceThreads) k_vjp_finish(float4 *__restrict__ acc, int n, double scale,
                                                                double *__restrict__ dx, double *__restrict__ lam,
                                                                double a, const double *__restrict__ partial, int np,
-                                                               double *__restrict__ dparam)
+                                                               double *__restrict__ dparam, SlotBin b,
+                                                               const double *__restrict__ x, float4 *__restrict__ g4,
+                                                               int32_t *__restrict__ err)
 {
     pdl_wait();
     if (blockIdx.x == 0) {
@@ -511,23 +516,46 @@ __global__ void __launch_bounds__(kReduceThreads) k_vjp_finish(const float4 *__r
         if (threadIdx.x == 0) {
             dparam[0] += scale * se[0];
             dparam[1] += scale * ss[0];
+            if (BIN) *b.work = 0u;
         }
         return;
     }
     const int i = (blockIdx.x - 1) * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float4 q = acc[i];
-    const int64_t b = 3 * (int64_t)i;
-    const double d0 = __fma_rn(scale, (double)q.x, dx[b]);
-    const double d1 = __fma_rn(scale, (double)q.y, dx[b + 1]);
-    const double d2 = __fma_rn(scale, (double)q.z, dx[b + 2]);
-    dx[b] = d0;
-    dx[b + 1] = d1;
-    dx[b + 2] = d2;
-    if (lam) {
-        lam[b] = __fma_rn(a, d0, lam[b]);
-        lam[b + 1] = __fma_rn(a, d1, lam[b + 1]);
-        lam[b + 2] = __fma_rn(a, d2, lam[b + 2]);
+    const bool valid = i < n;
+    if (!BIN && !valid) return;
+    const int64_t o = 3 * (int64_t)i;
+    double px = 0.0, py = 0.0, pz = 0.0, l0 = 0.0, l1 = 0.0, l2 = 0.0;
+    if (valid) {
+        const float4 q = acc[i];
+        if (BIN) {
+            px = x[o];
+            py = x[o + 1];
+            pz = x[o + 2];
+            acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+        const double d0 = __fma_rn(scale, (double)q.x, dx[o]);
+        const double d1 = __fma_rn(scale, (double)q.y, dx[o + 1]);
+        const double d2 = __fma_rn(scale, (double)q.z, dx[o + 2]);
+        dx[o] = d0;
+        dx[o + 1] = d1;
+        dx[o + 2] = d2;
+        if (lam) {
+            l0 = __fma_rn(a, d0, lam[o]);
+            l1 = __fma_rn(a, d1, lam[o + 1]);
+            l2 = __fma_rn(a, d2, lam[o + 2]);
+            lam[o] = l0;
+            lam[o + 1] = l1;
+            lam[o + 2] = l2;
+        }
+    }
+    if constexpr (BIN) {
+        if (valid) {
+            px = lj_wrap_fast(px, b.L, b.whi, b.wlo);
+            py = lj_wrap_fast(py, b.L, b.whi, b.wlo);
+            pz = lj_wrap_fast(pz, b.L, b.whi, b.wlo);
+        }
+        const int slot = slot_place(b, valid, i, px, py, pz, err);
+        if (slot >= 0) g4[slot] = make_float4((float)l0, (float)l1, (float)l2, 0.f);
     }
 }
 
@@ -544,10 +572,11 @@ bool uses_vjp_n3(const lj_ctx *c) { return uses_force_n3(c); }
 
 // The pair-once FP32-mixed VJP: the sums go to acc (float4 [n], particle
 // order, zeroed here or by the slotted binning), the parameter partials to
-// c->partial, then dx += scale acc (and what k_vjp_finish does besides).  The
+// c->partial, then dx += scale acc (and what k_vjp_finish does besides; next:
+// the positions it bins).  The
 // work counter must be zero (the binning before it zeroes it).
 cudaError_t launch_vjp_n3(lj_ctx *c, const double *coef, double scale, double *dx, float4 *acc, double *dparam,
-                          double *lam, double dt_axpy)
+                          double *lam, double dt_axpy, const double *next)
 {
     const bool slots = c->slots_open == 1;
     const double *q = coef;
@@ -608,9 +637,14 @@ cudaError_t launch_vjp_n3(lj_ctx *c, const double *coef, double scale, double *d
     if (e != cudaSuccess) return e;
     if (slots) slots_consumed(c);
     int n = (int)c->p.n, np = (int)grid;
-    void *fargs[] = {&acc, &n, &scale, &dx, &lam, &dt_axpy, &partial, &np, &dparam};
-    e = launch_pdl((const void *)k_vjp_finish, (n + kReduceThreads - 1) / kReduceThreads + 1, kReduceThreads, fargs, 0,
-                   c->stream, true);
+    const bool bin = next && slots;
+    if (bin && (e = slots_begin(c, 0)) != cudaSuccess) return e;
+    SlotBin b = slot_bin_of(c);
+    float4 *sg4 = c->sg4;
+    int32_t *err = c->err;
+    void *fargs[] = {&acc, &n, &scale, &dx, &lam, &dt_axpy, &partial, &np, &dparam, &b, (void *)&next, &sg4, &err};
+    e = launch_pdl(bin ? (const void *)k_vjp_finish<true> : (const void *)k_vjp_finish<false>,
+                   (n + kReduceThreads - 1) / kReduceThreads + 1, kReduceThreads, fargs, 0, c->stream, true);
     c->kernel_launches += 2;
     return e != cudaSuccess ? e : cudaGetLastError();
 }

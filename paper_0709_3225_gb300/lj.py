@@ -105,6 +105,8 @@ _SIGS = {
     "lj_batch_launches": ([_P, ctypes.POINTER(ctypes.c_int64), ctypes.POINTER(ctypes.c_int32)], ctypes.c_int),
     "lj_forces_vjp": ([_P, _P, _P, ctypes.c_double, _P, _P], ctypes.c_int),
     "lj_vv_adjoint_step": ([_P, _P, _P, _P, _P, _P], ctypes.c_int),
+    "lj_step_record": ([_P, _P, _P, _P, ctypes.c_int32], ctypes.c_int),
+    "lj_vv_adjoint_segment": ([_P, _P, ctypes.c_int32, _P, _P, _P], ctypes.c_int),
     "lj_forces_static": ([ctypes.POINTER(lj_params), _P, _P, _P], ctypes.c_int),
     "lj_measure_peak": ([ctypes.c_int32, ctypes.POINTER(ctypes.c_double), ctypes.POINTER(ctypes.c_double),
                          ctypes.POINTER(ctypes.c_int32)], ctypes.c_int),
@@ -433,6 +435,24 @@ def lj_vv_adjoint_step(ctx: Context, x_n, x_n1, lam_x, lam_v, dparam) -> None:
                                   _dev(lam_x, torch.float64, (ctx.n, 3), "lam_x"),
                                   _dev(lam_v, torch.float64, (ctx.n, 3), "lam_v"),
                                   _dev(dparam, torch.float64, (2,), "dparam")), "lj_vv_adjoint_step")
+
+
+def lj_step_record(ctx: Context, traj, v, f, nsteps: int) -> None:
+    """nsteps steps from traj[0], whose states' positions go to traj[1:] (see
+    include/lj.h); v and f in place."""
+    import torch
+    _ck(load().lj_step_record(ctx.handle, _dev(traj, torch.float64, (nsteps + 1, ctx.n, 3), "traj"),
+                              _dev(v, torch.float64, (ctx.n, 3), "v"), _dev(f, ctx.force_dtype, (ctx.n, 4), "f"),
+                              int(nsteps)), "lj_step_record")
+
+
+def lj_vv_adjoint_segment(ctx: Context, traj, nsteps: int, lam_x, lam_v, dparam) -> None:
+    """The adjoint of the nsteps steps of traj (see include/lj.h), in place."""
+    import torch
+    _ck(load().lj_vv_adjoint_segment(ctx.handle, _dev(traj, torch.float64, (nsteps + 1, ctx.n, 3), "traj"),
+                                     int(nsteps), _dev(lam_x, torch.float64, (ctx.n, 3), "lam_x"),
+                                     _dev(lam_v, torch.float64, (ctx.n, 3), "lam_v"),
+                                     _dev(dparam, torch.float64, (2,), "dparam")), "lj_vv_adjoint_segment")
 
 
 def lj_set_tuning(ctx: Context, kernel: int, group_width: int = 0, cells_per_grab: int = 4) -> None:
