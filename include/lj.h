@@ -444,11 +444,13 @@ int lj_batch_set_tuning(lj_batch *b, int32_t cells_per_grab, int32_t use_graph, 
 /* Force kernel of the batch's step launch: 3 = the 27-cell warp-per-cell
  * code (the default, and the only choice for cell subdivision 2), 7 = each
  * pair once over the half stencil (the pair-once device code of
- * lj_set_tuning kernel 7, with f zeroed in the scatter phase and the
- * reactions added with atomics; FP32 sums not bitwise reproducible between
- * runs; its 128 registers leave fewer resident warps for the other phases
- * of the launch).  LJ_EINVAL for other values, or 7 with subdivision 2.
- * Host only; a captured step graph is captured again. */
+ * lj_set_tuning kernel 7, with the reactions added with atomics into f zeroed
+ * before; FP32 sums not bitwise reproducible between runs).  With 7 a step is
+ * two launches, the update, which also bins, and the forces (one cooperative
+ * launch, as with 3, where a replica's cells are too sparse or too full for
+ * slotted cells); a call of three steps or more replays them in pairs.
+ * LJ_EINVAL for other values, or 7 with subdivision 2.  Allocates the slots
+ * when 7 is first chosen; a captured step graph is captured again. */
 int lj_batch_set_kernel(lj_batch *b, int32_t kernel);
 
 /* Forces of every replica at x into f (device arrays as above); with

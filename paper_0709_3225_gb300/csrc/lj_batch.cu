@@ -22,10 +22,12 @@
 
 #include "lj_force_cell.cuh"
 #include "lj_force_n3.cuh"
+#include "lj_slots.cuh"
 
 namespace {
 
 constexpr int kBatchThreads = kWarpForceThreads;
+constexpr int kBatchSlotMax = 64;   // slots per cell at most
 
 struct BatchDev {
     int64_t ntot, ncell;
@@ -360,8 +362,8 @@ __device__ void phase_force_n3(const BatchDev &b, const WarpParams &k, float4 *_
         for (int c = (int)c0; c < c1; c++) {
             const HalfLoad cur = nxt;
             if (c + 1 < c1) nxt = load(c + 1);
-            n3_cell<MODE, ENERGY, false, false, false>(k, b.pos, f, cur, c, 0, 0, (float)b.cw[b.rep_of_cell[c]], S, stab, spre, H,
-                                                eacc, wacc);
+            n3_cell<MODE, ENERGY, false, false, false>(k, b.pos, f, cur, c, 0, 0, 0.f, 0, 0, (float)b.cw[b.rep_of_cell[c]],
+                                                       S, stab, spre, H, eacc, wacc);
         }
     }
 }
@@ -386,9 +388,156 @@ __global__ void __launch_bounds__(kBatchThreads, 3) k_batch_step_n3(BatchDev b, 
     phase_force_n3<MODE, ENERGY>(b, k, f);
 }
 
+// The pair-once kernel (lj_batch_set_kernel 7) on slotted cells (lj_slots.cuh):
+// a step is one pass over the particles that bins them too, and the force
+// launch, which starts as its dependent.  The cooperative launch ran the
+// update, two scan phases and the scatter at the force phase's occupancy,
+// with four grid barriers between them, and kept the FP64 pipe busy with
+// conversions (64 replicas, 1.6 million particles, per step:
+// 382 -> 319 us).
+struct BatchRep {   // one replica's grid, 64 bytes
+    double L, whi, wlo, s;
+    float cw, inv_nc, sf;
+    int nc, cell0, thoff, ceoff, pad;
+};
+
+struct BatchSlots {
+    SlotBin bin;                // thb, centre: all replicas' tables; the replica's fields are filled per particle
+    const BatchRep *rep;
+    const int32_t *rep_of, *rep_of_cell;
+};
+
+// op 0: kicks, drift and wrap, then bin; op 1: bin the given positions.
+template <int OP>
+__global__ void __launch_bounds__(256) k_batch_slots(BatchSlots a, double *__restrict__ x, double *__restrict__ v,
+                                                     float4 *__restrict__ f, int n, double hk, double dt,
+                                                     int32_t *__restrict__ err)
+{
+    pdl_wait();
+    const int i = (gridDim.x - 1 - blockIdx.x) * blockDim.x + threadIdx.x;   // as k_kick_drift_slots
+    if (i == 0) *a.bin.work = 0u;
+    const bool valid = i < n;
+    double px = 0.0, py = 0.0, pz = 0.0;
+    SlotBin b = a.bin;
+    if (valid) {
+        const int64_t o = 3 * (int64_t)i;
+        const BatchRep *r = a.rep + __ldg(a.rep_of + i);
+        px = x[o];
+        py = x[o + 1];
+        pz = x[o + 2];
+        double v0 = 0.0, v1 = 0.0, v2 = 0.0;
+        float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (OP == 0) {
+            q = f[i];
+            v0 = v[o];
+            v1 = v[o + 1];
+            v2 = v[o + 2];
+        }
+        b.L = r->L;
+        b.whi = r->whi;
+        b.wlo = r->wlo;
+        b.s = r->s;
+        b.sf = r->sf;
+        b.nc = r->nc;
+        b.cell0 = r->cell0;
+        b.thb += r->thoff;
+        b.centre += r->ceoff;
+        f[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (OP == 0) {
+            v0 = __fma_rn(hk, f64_of_f32(q.x), v0);
+            v1 = __fma_rn(hk, f64_of_f32(q.y), v1);
+            v2 = __fma_rn(hk, f64_of_f32(q.z), v2);
+            px = __fma_rn(dt, v0, px);
+            py = __fma_rn(dt, v1, py);
+            pz = __fma_rn(dt, v2, pz);
+        }
+        px = lj_wrap_fast(px, b.L, b.whi, b.wlo);
+        py = lj_wrap_fast(py, b.L, b.whi, b.wlo);
+        pz = lj_wrap_fast(pz, b.L, b.whi, b.wlo);
+        if (OP == 0) {
+            v[o] = v0;
+            v[o + 1] = v1;
+            v[o + 2] = v2;
+            x[o] = px;
+            x[o + 1] = py;
+            x[o + 2] = pz;
+        }
+    }
+    slot_place(b, valid, i, px, py, pz, err);
+}
+
+// k_force_n3 with each cell's replica looked up (one cell ahead, as the
+// cell's own table loads).  The energies go to f.w alone.
+template <int MODE, bool ENERGY>
+__global__ void __launch_bounds__(kN3Threads, ENERGY ? 4 : 6) k_batch_force_n3(WarpParams k, BatchSlots a, float4 *__restrict__ f)
+{
+    extern __shared__ __align__(16) float nsmem[];
+    const int lane = threadIdx.x & 31;
+    const int warp = threadIdx.x >> 5;
+    float4 *S = reinterpret_cast<float4 *>(nsmem + (size_t)warp * n3_slice_words(k.cap));
+    float4 *stab = S + k.cap;
+    int *spre = reinterpret_cast<int *>(stab + kN3Half);
+    float4 *H = reinterpret_cast<float4 *>(spre + 16);
+    const float4 *pos = reinterpret_cast<const float4 *>(a.bin.pos);
+    double eacc = 0.0, wacc = 0.0;
+    pdl_wait();
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        k.cellq_next[k.ncell] = make_int2(0, 0);
+        *k.octr_next = 0u;
+    }
+    struct Cell {
+        HalfLoad t;
+        float4 g;   // cw, 1 / nc, sf, nc of the replica
+        int cell0;
+    };
+    auto load = [&](int c) {
+        const BatchRep *r = a.rep + __ldg(a.rep_of_cell + c);
+        Cell q;
+        q.g = __ldg(reinterpret_cast<const float4 *>(&r->cw));
+        q.cell0 = __ldg(&r->cell0);
+        q.t = half_load<true, true>(reinterpret_cast<const int32_t *>(k.cellq), c - q.cell0, __float_as_int(q.g.w), q.g.y,
+                                    q.cell0, k.scap);
+        return q;
+    };
+    // pulls of k.grab cells, single cells over the last stretch (as k_force_n3)
+    const int64_t tail = 2 * (int64_t)k.grab * gridDim.x * (kN3Threads / 32);
+    unsigned last = 0;
+    for (;;) {
+        const unsigned gr = (int64_t)last + tail >= k.ncell ? 1u : (unsigned)k.grab;
+        unsigned c0 = 0;
+        if (lane == 0) c0 = atomicAdd(k.work, gr);
+        c0 = __shfl_sync(0xffffffffu, c0, 0);
+        if ((int64_t)c0 >= k.ncell) break;
+        last = c0;
+        const int c1 = (int)min((int64_t)c0 + gr, k.ncell);
+        Cell nxt = load((int)c0);
+        for (int c = (int)c0; c < c1; c++) {
+            const Cell cur = nxt;
+            if (c + 1 < c1) nxt = load(c + 1);
+            if (lane == 31) k.cellq_next[c] = make_int2(0, 0);
+            n3_cell<MODE, ENERGY, true, true, false>(k, pos, f, cur.t, c - cur.cell0, cur.cell0,
+                                                     __float_as_int(cur.g.w), cur.g.y, 0, 0, cur.g.x, S, stab, spre, H,
+                                                     eacc, wacc);
+        }
+    }
+}
+
+void *batch_slots_kernel(int mode, bool energy)
+{
+    switch (mode * 2 + (energy ? 1 : 0)) {
+        case 0: return (void *)k_batch_force_n3<0, false>;
+        case 1: return (void *)k_batch_force_n3<0, true>;
+        case 2: return (void *)k_batch_force_n3<1, false>;
+        case 3: return (void *)k_batch_force_n3<1, true>;
+        case 4: return (void *)k_batch_force_n3<2, false>;
+        default: return (void *)k_batch_force_n3<2, true>;
+    }
+}
+
 // Closing half kick of the last step: v += h f.
 __global__ void k_batch_kick(double *__restrict__ v, const float4 *__restrict__ f, int64_t n, double h)
 {
+    pdl_wait();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const float4 q = f[i];
@@ -522,6 +671,21 @@ struct lj_batch {
     // its own staging capacity), grid and shared memory; n3: it is selected
     WarpParams kn3;
     int grid_n3, smem_n3, n3;
+    // its slotted form (scap > 0): launch shape, slots, the double-buffered
+    // (count, list head) pairs, of which the next binning fills par's, zero
+    // by then; dirty: not known to be zero
+    int sgrid, ssmem, scap, nslots, par, dirty;
+    int2 *cellq[2];
+    unsigned *octr;
+    float4 *spos;
+    int32_t *onext;
+    const BatchRep *rep;
+    const float2 *centre2;
+    WarpParams ks;
+    int gpar;             // par where the captured pair of steps starts
+    int slots_ok;         // cells beyond their slots are rare in every replica
+    std::vector<BatchRep> hrep;
+    std::vector<float2> hcentre2;
     double max_mean_occ;
     double *rep_out, *host_out;
     int32_t *host_err;
@@ -604,8 +768,123 @@ cudaError_t configure(lj_batch *b)
     return cudaSuccess;
 }
 
+// Slotted cells for the pair-once kernel, as slots_setup and slots_suit
+// (lj_slots.cu) take them for one system, with slots per cell by the fullest
+// replica's mean, up to kBatchSlotMax: a replica of 3 cells a side can have
+// cells of (4/3 rc)^3, beyond the 32 home particles of the kernel's fast path,
+// and as neighbours they still need their slots.  Set up when kernel 7 is
+// chosen; without them (sparse boxes, no memory) the cooperative launch serves.
+cudaError_t batch_slots_setup(lj_batch *b)
+{
+    const std::vector<BatchRep> &rep = b->hrep;
+    const std::vector<float2> &centre2 = b->hcentre2;
+    const double mean = b->max_mean_occ;
+    int cap = ((int)ceil(mean + 7.0 * sqrt(mean) + 3.0) + 7) & ~7;
+    cap = cap > kBatchSlotMax ? kBatchSlotMax : cap;
+    const int64_t nslots = b->ncell * cap;
+    if (b->grid_n3 == 0 || b->ntot == 0 || !b->slots_ok || nslots + b->ntot >= ((int64_t)1 << 31) ||
+        nslots > 12 * b->ntot + ((int64_t)1 << 16))
+        return cudaSuccess;
+    cudaError_t e = cudaSuccess;
+    BatchRep *rd = nullptr;
+    float2 *cd = nullptr;
+    const size_t mark = b->allocs.size();
+    for (int k = 0; k < 2 && e == cudaSuccess; k++) e = balloc(b, &b->cellq[k], (size_t)b->ncell + 1);
+    if (e == cudaSuccess) e = balloc(b, &b->octr, 2);
+    if (e == cudaSuccess) e = balloc(b, &b->spos, (size_t)(nslots + b->ntot));
+    if (e == cudaSuccess) e = balloc(b, &b->onext, (size_t)b->ntot);
+    if (e == cudaSuccess) e = balloc(b, &rd, rep.size());
+    if (e == cudaSuccess) e = balloc(b, &cd, centre2.size());
+    if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        while (b->allocs.size() > mark) {
+            cudaFree(b->allocs.back());
+            b->allocs.pop_back();
+        }
+        return cudaSuccess;
+    }
+    if (e == cudaSuccess) e = cudaMemcpy(rd, rep.data(), rep.size() * sizeof(BatchRep), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(cd, centre2.data(), centre2.size() * sizeof(float2), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) return e;
+    b->rep = rd;
+    b->centre2 = cd;
+    b->ssmem = (kN3Threads / 32) * n3_slice_words(b->kn3.cap) * (int)sizeof(float);
+    int nblk = 1 << 30;
+    for (int q = 0; q < 6; q++) {
+        void *kern = batch_slots_kernel(q >> 1, (q & 1) != 0);
+        int nb = 0;
+        if ((e = raise_dyn_smem(kern, b->ssmem)) != cudaSuccess) return e;
+        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, kN3Threads, b->ssmem)) != cudaSuccess) return e;
+        if ((q & 1) == 0 && nb < nblk) nblk = nb;   // (the energy kernels get the same grid)
+    }
+    int64_t grid = (int64_t)(nblk < 1 ? 1 : nblk) * b->nsm;
+    const int64_t need = (b->ncell + kN3Threads / 32 - 1) / (kN3Threads / 32);
+    b->sgrid = (int)(grid > need ? need : grid);
+    b->scap = cap;
+    b->nslots = (int)nslots;
+    b->dirty = 1;
+    b->ks = b->kn3;
+    b->ks.last = b->nslots + (int)b->ntot - 1;
+    b->ks.scap = cap;
+    b->ks.nslots = b->nslots;
+    b->ks.onext = b->onext;
+    b->ks.work = b->d.work;
+    b->ks.ncell = b->ncell;
+    return cudaSuccess;
+}
+
+bool batch_slots(const lj_batch *b) { return b->n3 && b->scap > 0; }
+
+// One evaluation on slotted cells.  nkick: half kicks of the update (op 0);
+// after: the launch before it in the stream is this batch's force kernel.
+cudaError_t launch_slots_step(lj_batch *b, bool energy, int op, double *x, double *v, float4 *f, int nkick, bool after)
+{
+    cudaError_t e = cudaSuccess;
+    if (b->dirty) {
+        for (int k = 0; k < 2 && e == cudaSuccess; k++)
+            e = cudaMemsetAsync(b->cellq[k], 0, ((size_t)b->ncell + 1) * sizeof(int2), b->stream);
+        if (e == cudaSuccess) e = cudaMemsetAsync(b->octr, 0, 2 * sizeof(unsigned), b->stream);
+        if (e != cudaSuccess) return e;
+    }
+    b->dirty = 1;
+    BatchSlots a = {};
+    a.bin.cellq = b->cellq[b->par];
+    a.bin.pos = b->spos;
+    a.bin.onext = b->onext;
+    a.bin.octr = b->octr + b->par;
+    a.bin.work = b->d.work;
+    a.bin.centre = b->centre2;
+    a.bin.thb = b->d.thb;
+    a.bin.ncell = (int)b->ncell;
+    a.bin.cap = b->scap;
+    a.bin.nslots = b->nslots;
+    a.rep = b->rep;
+    a.rep_of = b->d.rep_of;
+    a.rep_of_cell = b->d.rep_of_cell;
+    int n = (int)b->ntot;
+    double hk = nkick * b->d.h, dt = b->d.dt;
+    int32_t *err = b->d.err;
+    void *args[] = {&a, &x, &v, &f, &n, &hk, &dt, &err};
+    e = launch_pdl(op == 0 ? (const void *)k_batch_slots<0> : (const void *)k_batch_slots<1>, (unsigned)((n + 255) / 256),
+                   256, args, 0, b->stream, after);
+    if (e != cudaSuccess) return e;
+    b->ks.grab = b->d.cells_per_grab;
+    b->ks.cellq = b->cellq[b->par];
+    b->ks.cellq_next = b->cellq[b->par ^ 1];
+    b->ks.octr_next = b->octr + (b->par ^ 1);
+    void *fargs[] = {&b->ks, &a, &f};
+    e = launch_pdl(batch_slots_kernel(b->p.shift_mode, energy), b->sgrid, kN3Threads, fargs, (size_t)b->ssmem, b->stream,
+                   true);
+    if (e != cudaSuccess) return e;
+    b->launches += 2;
+    b->par ^= 1;
+    b->dirty = 0;
+    return cudaSuccess;
+}
+
 cudaError_t launch_step_kernel(lj_batch *b, bool energy, int op, double *x, double *v, float4 *f)
 {
+    if (batch_slots(b)) return launch_slots_step(b, energy, op, x, v, f, 1, false);
     b->launches++;
     if (b->n3) {
         void *kern = batch_kernel_n3(b->p.shift_mode, energy);
@@ -615,6 +894,73 @@ cudaError_t launch_step_kernel(lj_batch *b, bool energy, int op, double *x, doub
     void *kern = batch_kernel(b->p.cell_subdiv, b->p.shift_mode, energy, b->k.gw);
     void *args[] = {&b->d, &b->k, &op, &x, &v, &f};
     return cudaLaunchCooperativeKernel(kern, dim3(b->grid), dim3(kBatchThreads), args, b->smem, b->stream);
+}
+
+// Capture two middle steps (the count buffers alternate) into gexec.
+cudaError_t capture_slots_pair(lj_batch *b, double *x, double *v, float4 *f)
+{
+    if (b->gexec) cudaGraphExecDestroy(b->gexec);
+    b->gexec = nullptr;
+    cudaStream_t cs = b->stream, keep = b->stream;
+    cudaError_t e = cudaSuccess;
+    if (!keep && (e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking)) != cudaSuccess) return e;
+    cudaGraph_t g = nullptr;
+    const int64_t k0 = b->launches;
+    const int par = b->par;
+    if ((e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal)) == cudaSuccess) {
+        b->stream = cs;
+        cudaError_t el = launch_slots_step(b, false, 0, x, v, f, 2, false);
+        if (el == cudaSuccess) el = launch_slots_step(b, false, 0, x, v, f, 2, true);
+        b->stream = keep;
+        e = cudaStreamEndCapture(cs, &g);
+        if (el != cudaSuccess) e = el;
+    }
+    b->launches = k0;
+    b->par = par;   // nothing has run
+    b->dirty = 0;
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&b->gexec, g, 0);
+    if (g) cudaGraphDestroy(g);
+    if (!keep) cudaStreamDestroy(cs);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        b->gexec = nullptr;
+        return e;
+    }
+    b->gx = x;
+    b->gv = v;
+    b->gf = f;
+    b->gpar = par;
+    return cudaSuccess;
+}
+
+// nsteps >= 1 steps: the first with one half kick, the others with two, in
+// replayed pairs where a pair is left and the buffers stand as captured.
+cudaError_t slots_steps(lj_batch *b, double *x, double *v, float4 *f, int nsteps)
+{
+    cudaError_t e = launch_slots_step(b, false, 0, x, v, f, 1, false);
+    for (int s = 1; s < nsteps && e == cudaSuccess;) {
+        const bool have = b->gexec && b->gx == x && b->gv == v && b->gf == f;
+        bool graph = b->use_graph && s + 2 <= nsteps && !(have && b->gpar != b->par);
+        if (graph && !have && capture_slots_pair(b, x, v, f) != cudaSuccess) {
+            b->use_graph = 0;   // capture unsupported here: launch directly
+            graph = false;
+        }
+        if (graph) {
+            e = cudaGraphLaunch(b->gexec, b->stream);
+            b->launches += 4;
+            s += 2;
+        } else {
+            e = launch_slots_step(b, false, 0, x, v, f, 2, true);
+            s++;
+        }
+    }
+    if (e != cudaSuccess) return e;
+    const float4 *fc = f;
+    int64_t n = b->ntot;
+    double h = b->d.h;
+    void *args[] = {&v, (void *)&fc, &n, &h};
+    b->launches++;
+    return launch_pdl((const void *)k_batch_kick, (unsigned)((n + 255) / 256), 256, args, 0, b->stream, true);
 }
 
 int sync_check(lj_batch *b)
@@ -687,6 +1033,7 @@ extern "C" int lj_batch_create(lj_batch **out, int32_t nrep, const int64_t *n, c
     b->stream = (cudaStream_t)stream;
     b->use_graph = 1;
     b->max_mean_occ = max_occ;
+    b->slots_ok = 1;
 #define LJ_BCK(call)                 \
     do {                             \
         cudaError_t e_ = (call);     \
@@ -723,6 +1070,29 @@ extern "C" int lj_batch_create(lj_batch **out, int32_t nrep, const int64_t *n, c
         }
         thb[thoff[r] + nc] = INT64_MAX;
         for (int64_t i = poff[r]; i < poff[r + 1]; i++) rep_of[i] = r;
+        BatchRep q = {};
+        q.L = L[r];
+        q.whi = whi[r];
+        q.wlo = wlo[r];
+        q.s = s[r];
+        q.cw = (float)cw[r];
+        q.sf = (float)s[r];
+        q.nc = nc;
+        q.cell0 = coff[r];
+        q.thoff = thoff[r];
+        q.ceoff = ceoff[r];
+        const int64_t nr = (int64_t)nc * nc * nc;
+        q.inv_nc = nr + 1 < (1 << 24) ? 1.0f / (float)nc : 0.0f;
+        b->hrep.push_back(q);
+        for (int k = 0; k < nc; k++) {
+            const double ce = centre[ceoff[r] + k];
+            b->hcentre2.push_back(make_float2((float)ce, (float)(ce - (double)(float)ce)));
+        }
+        // as slots_suit (lj_slots.cu)
+        const double mean = (double)n[r] / (double)nr, sl = common->sigma / box[r];
+        if (!(mean + 4.5 * sqrt(mean) <= kBatchSlotMax ||
+              (mean <= 45.0 && (double)n[r] * sl * sl * sl >= 0.5)))
+            b->slots_ok = 0;
         for (int64_t c = coff[r]; c < coff[r + 1]; c++) rep_of_cell[c] = r;
     }
 
@@ -842,7 +1212,7 @@ extern "C" int lj_batch_info(const lj_batch *b, int64_t *ntot, int64_t *ncell, i
     if (!b) return LJ_EINVAL;
     if (ntot) *ntot = b->ntot;
     if (ncell) *ncell = b->ncell;
-    if (grid) *grid = b->n3 ? b->grid_n3 : b->grid;
+    if (grid) *grid = batch_slots(b) ? b->sgrid : b->n3 ? b->grid_n3 : b->grid;
     if (cap) *cap = b->n3 ? b->kn3.cap : b->k.cap;
     return LJ_OK;
 }
@@ -873,6 +1243,10 @@ extern "C" int lj_batch_set_kernel(lj_batch *b, int32_t kernel)
         cudaGraphExecDestroy(b->gexec);
         b->gexec = nullptr;
     }
+    if (b->n3 && b->scap == 0) {
+        const cudaError_t e = batch_slots_setup(b);
+        if (e != cudaSuccess) return map_err(e);
+    }
     return LJ_OK;
 }
 
@@ -895,6 +1269,10 @@ extern "C" int lj_batch_step(lj_batch *b, double *x, double *v, void *f, int32_t
     if ((r = check_ptr(x, 8)) != LJ_OK) return r;
     if ((r = check_ptr(v, 8)) != LJ_OK) return r;
     if ((r = check_ptr(f, 16)) != LJ_OK) return r;
+    if (batch_slots(b)) {
+        const cudaError_t es = slots_steps(b, x, v, (float4 *)f, nsteps);
+        return es == cudaSuccess ? LJ_OK : map_err(es);
+    }
     cudaError_t e = cudaMemsetAsync(b->d.first, 1, 1, b->stream);
     if (e != cudaSuccess) return map_err(e);
     bool graph = b->use_graph != 0;

@@ -33,7 +33,8 @@ __global__ void __launch_bounds__(kN3Threads, ENERGY ? 4 : 6) k_force_n3(WarpPar
     auto load = [&](int c) { return half_load<true, SLOTS>(start, c, nc, k.inv_nc, 0, k.scap); };
     auto one_cell = [&](HalfLoad tl, int c, int part) {
         if (SLOTS && lane == 31 && part == 0) k.cellq_next[c] = make_int2(0, 0);
-        n3_cell<MODE, ENERGY, true, SLOTS, SPLIT>(k, pos, fout, tl, c, part, k.lgw, k.cw, S, stab, spre, H, eacc, wacc);
+        n3_cell<MODE, ENERGY, true, SLOTS, SPLIT>(k, pos, fout, tl, c, 0, nc, k.inv_nc, part, k.lgw, k.cw, S, stab, spre, H,
+                                                  eacc, wacc);
     };
     if constexpr (SPLIT) {
         // at most one item per resident warp: no pulls

@@ -511,8 +511,8 @@ __device__ __forceinline__ bool n3_stage(const WarpParams &k, const float4 *__re
 // reactions summed over the warp.
 template <int MODE, bool ENERGY, bool NC, bool SLOTS, bool SPLIT>
 __device__ void n3_plain(const WarpParams &k, const float4 *__restrict__ pos, float4 *__restrict__ fout,
-                         const float4 *stab, const int *spre, int c, int ta, int tb_end, int s_home, int n_home,
-                         double &eacc, double &wacc)
+                         const float4 *stab, const int *spre, int c, int cell0, int nc, float inv_nc, int ta,
+                         int tb_end, int s_home, int n_home, double &eacc, double &wacc)
 {
     const int lane = threadIdx.x & 31;
     for (int p0 = 0; p0 < n_home; p0 += 32) {
@@ -520,7 +520,7 @@ __device__ void n3_plain(const WarpParams &k, const float4 *__restrict__ pos, fl
         const bool vi = i < n_home;
         int si = s_home + (vi ? i : 0);
         if (SLOTS && vi && i >= k.scap) {   // the (i - scap)-th of the home cell's overflow list
-            int o = __ldg(&k.cellq[c].y);
+            int o = __ldg(&k.cellq[cell0 + c].y);
             for (int m = k.scap; m < i; m++) o = __ldg(k.onext + o - 1);
             si = k.nslots + o - 1;
         }
@@ -535,7 +535,7 @@ __device__ void n3_plain(const WarpParams &k, const float4 *__restrict__ pos, fl
             for (int j = (kk == 0 && !SLOTS ? p0 + 1 : 0); j < nn; j++) {
                 int sj = s + j;
                 if (SLOTS && j >= k.scap) {
-                    o = j == k.scap ? __ldg(&k.cellq[half_cell(c, kk, k.nc, k.inv_nc)].y) : __ldg(k.onext + o - 1);
+                    o = j == k.scap ? __ldg(&k.cellq[cell0 + half_cell(c, kk, nc, inv_nc)].y) : __ldg(k.onext + o - 1);
                     sj = k.nslots + o - 1;
                 }
                 if (SPLIT && (spre[kk] + j < ta || spre[kk] + j >= tb_end)) continue;   // another part's
@@ -592,14 +592,16 @@ __device__ void n3_plain(const WarpParams &k, const float4 *__restrict__ pos, fl
 // spre, H: the warp's slice).  cw: the
 // cell side of the cell's grid.  NC: read-only loads of the sorted
 // positions (not when an earlier phase of the same launch writes them).
-// SLOTS: slotted cells; c: the cell's id.  part of 2^lgw: the cell's
+// SLOTS: slotted cells; c: the cell's id in its grid of nc^3 cells, whose ids
+// start at cell0.  part of 2^lgw: the cell's
 // candidates are split evenly over 2^lgw warps (0 of 1: the whole cell),
 // part 0 with the home pairs; every part stages the home particles and adds
 // its share of their forces (SPLIT; otherwise whole cells only).
 template <int MODE, bool ENERGY, bool NC, bool SLOTS, bool SPLIT>
 __device__ __forceinline__ void n3_cell(const WarpParams &k, const float4 *__restrict__ pos, float4 *__restrict__ fout,
-                                        HalfLoad tl, int c, int part, int lgw, float cw, float4 *S, float4 *stab,
-                                        int *spre, float4 *H, double &eacc, double &wacc)
+                                        HalfLoad tl, int c, int cell0, int nc, float inv_nc, int part, int lgw,
+                                        float cw, float4 *S, float4 *stab, int *spre, float4 *H, double &eacc,
+                                        double &wacc)
 {
     __syncwarp();   // the slice still holds the previous cell's data
     const int tot = half_finish(tl, cw, stab, spre);
@@ -619,7 +621,8 @@ __device__ __forceinline__ void n3_cell(const WarpParams &k, const float4 *__res
         n3_stage<NC, SPLIT>(k, pos, S, stab, spre, ta, tb_end, s_home, n_home, T))
         n3_compute<MODE, ENERGY>(k, fout, S, H, T, SPLIT && ta > 0 ? n_home : 0, n_home, eacc, wacc);
     else
-        n3_plain<MODE, ENERGY, NC, SLOTS, SPLIT>(k, pos, fout, stab, spre, c, ta, tb_end, s_home, n_home, eacc, wacc);
+        n3_plain<MODE, ENERGY, NC, SLOTS, SPLIT>(k, pos, fout, stab, spre, c, cell0, nc, inv_nc, ta, tb_end, s_home,
+                                                 n_home, eacc, wacc);
 }
 
 }  // namespace

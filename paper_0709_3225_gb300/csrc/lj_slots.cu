@@ -251,6 +251,7 @@ SlotBin slot_bin_of(const lj_ctx *c)
     b.ncell = (int)c->ncell;
     b.cap = c->scap;
     b.nslots = c->nslots;
+    b.cell0 = 0;
     b.S = c->p.precision == LJ_PREC_FP64 ? fx_shift(c) : 0;
     return b;
 }

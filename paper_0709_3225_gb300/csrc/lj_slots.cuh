@@ -29,6 +29,7 @@ struct SlotBin {
     double L, whi, wlo, s;
     float sf;               // (float)s
     int nc, ncell, cap, nslots, S;   // S: scale of the fixed-point coordinates (FP64)
+    int cell0;              // id of the grid's first cell (a batch's replica; else 0); ncell counts all grids' cells
 };
 
 #ifdef __CUDACC__
@@ -58,7 +59,7 @@ __device__ __forceinline__ int slot_place(const SlotBin &b, bool valid, int i, d
     if (valid) {
         if (finite64(px) && finite64(py) && finite64(pz)) {
             cc = slot_cell(b, px, py, pz);
-            c = cc.x + b.nc * (cc.y + b.nc * cc.z);
+            c = b.cell0 + cc.x + b.nc * (cc.y + b.nc * cc.z);
         } else {
             atomicOr(err, LJ_ERRBIT_NONFINITE);
             c = b.ncell;
