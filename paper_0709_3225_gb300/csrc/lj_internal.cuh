@@ -404,6 +404,8 @@ cudaError_t launch_scan(lj_ctx *c, bool gated = false);
 cudaError_t launch_scatter(lj_ctx *c, const double *x, bool wrap);
 cudaError_t launch_force(lj_ctx *c, void *f, bool energy);
 cudaError_t launch_energy_reduce(lj_ctx *c);
+// The same straight into the pinned host_scalars, with the latched errors in host_err.
+cudaError_t launch_energy_publish(lj_ctx *c);
 // Particles [i_begin, i_end) (i_end < 0: to n).
 cudaError_t launch_kick_drift_bin(lj_ctx *c, double *x, double *v, const void *f, int nkick, int64_t i_begin = 0,
                                   int64_t i_end = -1);
