@@ -371,7 +371,33 @@ int persistent_steps(lj_ctx *c, double *x, double *v, void *f, int nsteps, cudaE
 
 constexpr int kHostChunks = 4;   // parts of lj_step_host's copies in
 
-int do_steps(lj_ctx *c, double *x, double *v, void *f, int nsteps, cudaEvent_t x_final = nullptr)
+// Pinned host memory from p on, readable and writable by kernels in 16-byte
+// accesses.
+bool mapped_host(const void *p, size_t bytes)
+{
+    if (((uintptr_t)p) % 16 != 0) return false;
+    const char *ends[2] = {(const char *)p, (const char *)p + bytes - 1};
+    for (const char *q : ends) {
+        cudaPointerAttributes a;
+        unsigned flags = 0;
+        if (cudaPointerGetAttributes(&a, q) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        if (a.type != cudaMemoryTypeHost || a.devicePointer != (void *)q) return false;
+        if (cudaHostGetFlags(&flags, (void *)q) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        if (flags & cudaHostRegisterReadOnly) return false;
+    }
+    return true;
+}
+
+constexpr int kHostSmall = 32768;   // below it x goes back in k_host_out too: 4 us of the link, less than a copy's set-up
+
+// close: the closing half kick (not where launch_host_out takes it).
+int do_steps(lj_ctx *c, double *x, double *v, void *f, int nsteps, cudaEvent_t x_final = nullptr, bool close = true)
 {
     if (nsteps <= 0) return LJ_OK;
     if (persistent_mode(c)) return persistent_steps(c, x, v, f, nsteps, x_final);
@@ -400,6 +426,7 @@ int do_steps(lj_ctx *c, double *x, double *v, void *f, int nsteps, cudaEvent_t x
             if (r) return r;
         }
     }
+    if (!close) return LJ_OK;
     if (uses_fx(c)) LJ_CK(launch_fx_finish(c, v, (double4_16a *)f));
     else if (!fused_mode(c)) LJ_CK(launch_kick(c, v, f, uses_slots(c) && !c->timing));
     if (x_final && fused_mode(c)) LJ_CK(cudaEventRecord(x_final, c->stream));
@@ -801,6 +828,22 @@ extern "C" int lj_step_host(lj_ctx *c, double *x, double *v, void *f, int32_t ns
     if (!c->ev_entry) LJ_CK(cudaEventCreateWithFlags(&c->ev_entry, cudaEventDisableTiming));
     for (int k = 0; k < kHostChunks; k++)
         if (!c->ev_chunk[k]) LJ_CK(cudaEventCreateWithFlags(&c->ev_chunk[k], cudaEventDisableTiming));
+    if (n > 0 && nsteps > 0 && uses_slots(c) && !persistent_mode(c) && mapped_host(x, bx) && mapped_host(v, bx) &&
+        mapped_host(f, bf)) {
+        const bool copy_x = n > kHostSmall;
+        LJ_CK(launch_host_in(c, x, v, (const float4 *)f, c->xs, c->vs, (float4 *)c->fs));
+        c->kdb_done = 1;
+        r = do_steps(c, c->xs, c->vs, c->fs, nsteps, copy_x ? c->ev_xfinal : nullptr, false);
+        c->kdb_done = 0;
+        if (r) return r;
+        if (copy_x) {   // beside the last force evaluation
+            LJ_CK(cudaStreamWaitEvent(c->copy_stream, c->ev_xfinal, 0));
+            LJ_CK(cudaMemcpyAsync(x, c->xs, bx, cudaMemcpyDeviceToHost, c->copy_stream));
+        }
+        LJ_CK(launch_host_out(c, c->xs, c->vs, (const float4 *)c->fs, copy_x ? nullptr : x, v, (float4 *)f));
+        if (copy_x) LJ_CK(cudaStreamSynchronize(c->copy_stream));
+        return sync_and_check(c, true);
+    }
     // The regular step's first kernel (kick, drift, bin) works on each part
     // of x, v, f as soon as its copy has arrived on the second stream; the
     // other update paths take the whole arrays first.

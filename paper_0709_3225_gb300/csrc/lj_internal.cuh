@@ -495,6 +495,12 @@ cudaError_t launch_bin_slots(lj_ctx *c, const double *x, float4 *zero, const dou
 // xo: where the new positions go (x, or another state).
 cudaError_t launch_kick_drift_slots(lj_ctx *c, const double *x, double *xo, double *v, float4 *f, int nkick,
                                     int64_t i_begin = 0, int64_t i_end = -1, bool after_force = false);
+// The first update from, and the closing half kick to, pinned host arrays
+// (hx: NULL where x is copied back otherwise); the latter publishes the
+// latched errors in host_err.
+cudaError_t launch_host_in(lj_ctx *c, const double *hx, const double *hv, const float4 *hf, double *x, double *v, float4 *f);
+cudaError_t launch_host_out(lj_ctx *c, const double *x, const double *v, const float4 *f, double *hx, double *hv,
+                            float4 *hf);
 cudaError_t slots_begin(lj_ctx *c, int64_t i_begin);   // before a slotted binning launch
 void slots_consumed(lj_ctx *c);                        // after the launch that reads it
 // FP64 contexts: the fixed-point kernel (lj_force_fx.cu) over slotted cells.

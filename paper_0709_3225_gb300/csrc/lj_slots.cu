@@ -79,6 +79,106 @@ __global__ void __launch_bounds__(256) k_kick_drift_slots(SlotBin b, const doubl
     slot_place(b, valid, i, px, py, pz, err);
 }
 
+// lj_step_host on pinned arrays: the first update reads x, v, f where they
+// are, over the link, and the last half kick writes v and f there (small
+// systems' x too).  The link is the bound, 205 GB/s in and 190 out here, by
+// copy engine or by loads alike; twelve chunked copies and an update per chunk
+// took 193 us for the 32 MB of 500,009 particles (156 at the link's rate), and
+// the closing kick ran before its copies: a call of one step there 437 -> 369
+// us.  The (n, 3) arrays go through shared memory, so that the link sees
+// whole 16-byte accesses in order.
+constexpr int kHostThreads = 256;
+
+// The block's 3 kHostThreads doubles of an (n, 3) array, from element e0.
+__device__ __forceinline__ void host_rows_in(const double *__restrict__ src, double2 *s, int64_t e0, int64_t end)
+{
+    for (int k = threadIdx.x; k < 3 * kHostThreads / 2; k += kHostThreads) {
+        const int64_t e = e0 + 2 * k;
+        double2 q = make_double2(0.0, 0.0);
+        if (e + 1 < end) q = __ldg(reinterpret_cast<const double2 *>(src + e));
+        else if (e < end) q.x = src[e];
+        s[k] = q;
+    }
+}
+
+__device__ __forceinline__ void host_rows_out(double *__restrict__ dst, const double2 *s, int64_t e0, int64_t end)
+{
+    for (int k = threadIdx.x; k < 3 * kHostThreads / 2; k += kHostThreads) {
+        const int64_t e = e0 + 2 * k;
+        if (e + 1 < end) *reinterpret_cast<double2 *>(dst + e) = s[k];
+        else if (e < end) dst[e] = s[k].x;
+    }
+}
+
+// k_kick_drift_slots from the host arrays hx, hv, hf to x, v and f (zeroed).
+__global__ void __launch_bounds__(kHostThreads) k_host_in(SlotBin b, const double *__restrict__ hx,
+                                                          const double *__restrict__ hv, const float4 *__restrict__ hf,
+                                                          double *__restrict__ x, double *__restrict__ v,
+                                                          float4 *__restrict__ f, int n, double hk, double dt,
+                                                          int32_t *__restrict__ err)
+{
+    __shared__ double2 sx[3 * kHostThreads / 2], sv[3 * kHostThreads / 2];
+    const int64_t i0 = (int64_t)blockIdx.x * kHostThreads;
+    const int i = (int)i0 + threadIdx.x;
+    if (i == 0) *b.work = 0u;
+    const bool valid = i < n;
+    float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (valid) q = __ldg(hf + i);
+    host_rows_in(hx, sx, 3 * i0, 3 * (int64_t)n);
+    host_rows_in(hv, sv, 3 * i0, 3 * (int64_t)n);
+    __syncthreads();
+    double *px3 = reinterpret_cast<double *>(sx) + 3 * threadIdx.x;
+    double *pv3 = reinterpret_cast<double *>(sv) + 3 * threadIdx.x;
+    double px = 0.0, py = 0.0, pz = 0.0;
+    if (valid) {
+        f[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        const double vx = __fma_rn(hk, f64_of_f32(q.x), pv3[0]);
+        const double vy = __fma_rn(hk, f64_of_f32(q.y), pv3[1]);
+        const double vz = __fma_rn(hk, f64_of_f32(q.z), pv3[2]);
+        px = lj_wrap_fast(__fma_rn(dt, vx, px3[0]), b.L, b.whi, b.wlo);
+        py = lj_wrap_fast(__fma_rn(dt, vy, px3[1]), b.L, b.whi, b.wlo);
+        pz = lj_wrap_fast(__fma_rn(dt, vz, px3[2]), b.L, b.whi, b.wlo);
+        const int64_t o = 3 * (int64_t)i;
+        v[o] = vx;
+        v[o + 1] = vy;
+        v[o + 2] = vz;
+        x[o] = px;
+        x[o + 1] = py;
+        x[o + 2] = pz;
+    }
+    slot_place(b, valid, i, px, py, pz, err);
+}
+
+// The closing half kick v += h f into the host arrays, with f (and x, if hx)
+// and the latched errors.
+__global__ void __launch_bounds__(kHostThreads) k_host_out(const double *__restrict__ x, const double *__restrict__ v,
+                                                           const float4 *__restrict__ f, int n, double h,
+                                                           double *__restrict__ hx, double *__restrict__ hv,
+                                                           float4 *__restrict__ hf, const int32_t *__restrict__ err,
+                                                           int32_t *__restrict__ host_err)
+{
+    __shared__ double2 s[3 * kHostThreads / 2];
+    pdl_wait();
+    const int64_t i0 = (int64_t)blockIdx.x * kHostThreads, end = 3 * (int64_t)n;
+    const int i = (int)i0 + threadIdx.x;
+    if (i == 0) *host_err = *err;
+    if (i < n) {
+        const int64_t o = 3 * (int64_t)i;
+        const float4 q = f[i];
+        double *d = reinterpret_cast<double *>(s) + 3 * threadIdx.x;
+        d[0] = __fma_rn(h, f64_of_f32(q.x), v[o]);
+        d[1] = __fma_rn(h, f64_of_f32(q.y), v[o + 1]);
+        d[2] = __fma_rn(h, f64_of_f32(q.z), v[o + 2]);
+        hf[i] = q;
+    }
+    __syncthreads();
+    host_rows_out(hv, s, 3 * i0, end);
+    if (hx) {
+        for (int k = threadIdx.x; k < 3 * kHostThreads; k += kHostThreads)
+            if (3 * i0 + k < end) hx[3 * i0 + k] = x[3 * i0 + k];
+    }
+}
+
 // The FP64 forms (lj_force_fx.cu): fixed-point coordinates; f holds the
 // forces of the pairs taken in FP64 and acc, in units of 1 / scale, those of
 // all others.
@@ -423,6 +523,28 @@ cudaError_t launch_kick_drift_slots(lj_ctx *c, const double *x, double *xo, doub
     e = launch_pdl((const void *)k_kick_drift_slots, (int)blocks_for(n - i_begin, 256), 256, args, 0, c->stream, after_force);
     c->kernel_launches++;
     return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+cudaError_t launch_host_in(lj_ctx *c, const double *hx, const double *hv, const float4 *hf, double *x, double *v, float4 *f)
+{
+    cudaError_t e = slots_begin(c, 0);
+    if (e != cudaSuccess) return e;
+    const int n = (int)c->p.n;
+    k_host_in<<<blocks_for(n, kHostThreads), kHostThreads, 0, c->stream>>>(
+        slot_bin_of(c), hx, hv, hf, x, v, f, n, 0.5 * c->p.dt / c->p.mass, c->p.dt, c->err);
+    c->kernel_launches++;
+    return cudaGetLastError();
+}
+
+cudaError_t launch_host_out(lj_ctx *c, const double *x, const double *v, const float4 *f, double *hx, double *hv,
+                            float4 *hf)
+{
+    int n = (int)c->p.n;
+    double h = 0.5 * c->p.dt / c->p.mass;
+    const int32_t *err = c->err;
+    void *args[] = {(void *)&x, (void *)&v, (void *)&f, &n, &h, &hx, &hv, &hf, (void *)&err, &c->host_err};
+    c->kernel_launches++;
+    return launch_pdl((const void *)k_host_out, blocks_for(n, kHostThreads), kHostThreads, args, 0, c->stream, !c->timing);
 }
 
 cudaError_t launch_slots_to_lists(lj_ctx *c)
