@@ -55,6 +55,9 @@ __global__ void k_n2_prep(const double *__restrict__ x, int n, double L, double 
 
 // FP32: coordinates in three arrays of npad (a multiple of 32) floats; the
 // padding is far away (its squared distance is inf, the image included).
+// After them, for each group of 32 consecutive particles, its bounding box as
+// two float4: the centre, and the half extents (with the rounding of both, and
+// 1e30 for a group with a non-finite coordinate, which is never left out).
 __global__ void k_n2_prep_f32(const double *__restrict__ x, int n, int npad, double L, double whi, double wlo,
                               float *__restrict__ soa, int32_t *err)
 {
@@ -72,6 +75,36 @@ __global__ void k_n2_prep_f32(const double *__restrict__ x, int n, int npad, dou
     soa[i] = q[0];
     soa[(size_t)npad + i] = q[1];
     soa[2 * (size_t)npad + i] = q[2];
+    const bool real = i < n;
+    const bool fin = !real || (fabsf(q[0]) < 1.0e30f && fabsf(q[1]) < 1.0e30f && fabsf(q[2]) < 1.0e30f);
+    const bool all = __all_sync(0xffffffffu, fin);
+    float c[3], h[3];
+#pragma unroll
+    for (int d = 0; d < 3; d++) {
+        float lo = real && fin ? q[d] : 3.0e38f, hi = real && fin ? q[d] : -3.0e38f;
+        for (int o = 16; o > 0; o >>= 1) {
+            lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+            hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+        }
+        c[d] = all ? 0.5f * (lo + hi) : 0.0f;
+        h[d] = all ? 0.5f * (hi - lo) + 1.0e-6f * (float)L : 1.0e30f;
+    }
+    if ((i & 31) == 0) {
+        float4 *box = reinterpret_cast<float4 *>(soa + 3 * (size_t)npad) + 2 * (i >> 5);
+        box[0] = make_float4(c[0], c[1], c[2], 0.0f);
+        box[1] = make_float4(h[0], h[1], h[2], 0.0f);
+    }
+}
+
+// A lower bound of the squared minimum-image distance between the particles
+// of two boxes.
+__device__ __forceinline__ float n2_gap2(float4 ca, float4 ha, float4 cb, float4 hb, float L)
+{
+    const float dx = fabsf(ca.x - cb.x), dy = fabsf(ca.y - cb.y), dz = fabsf(ca.z - cb.z);
+    const float gx = fmaxf(fminf(dx, L - dx) - (ha.x + hb.x), 0.0f);
+    const float gy = fmaxf(fminf(dy, L - dy) - (ha.y + hb.y), 0.0f);
+    const float gz = fmaxf(fminf(dz, L - dz) - (ha.z + hb.z), 0.0f);
+    return gx * gx + gy * gy + gz * gz;
 }
 
 template <typename V>
@@ -230,7 +263,13 @@ __device__ __forceinline__ float2 n2_r2(float2 xi, float2 yi, float2 zi, float2 
 // instruction issue: ~13 instructions per pair (six for the three
 // components' images, 1.5 each for r^2 and the mask) against ~30 with three
 // quarter-rate roundings before.  At 8,788
-// particles a call took 137 us, now 46.
+// particles a call took 137 us, then 46.
+// A warp's 32 particles leave out a group of 32 j whose bounding box is
+// further than rc from theirs: no pair of the two is in range, so the sums
+// stay the same bits.  Particles that are stored near their neighbours (grown
+// on a lattice, read from a file written by cells) leave out most groups (46
+// -> 28 us, 120 -> 40 at 16,000); where the order is random the boxes fill the
+// system and the test's cost does not show (46 us).
 template <int MODE, bool ENERGY>
 __global__ void __launch_bounds__(kN2Threads) k_n2_force_f32(N2Params p, int npad, int tile, const float *__restrict__ soa,
                                                              float4 *__restrict__ part, double *__restrict__ epart,
@@ -268,16 +307,28 @@ __global__ void __launch_bounds__(kN2Threads) k_n2_force_f32(N2Params p, int npa
     const float L = (float)p.L, invL = (float)p.invL;
     const float thr = -(float)p.rc2 * 1.00001f;
     const float2 xi = make_float2(pix, pix), yi = make_float2(piy, piy), zi = make_float2(piz, piz);
+    const float4 *box = reinterpret_cast<const float4 *>(soa + 3 * (size_t)npad);
+    const int lane = threadIdx.x & 31, gi = i >> 5;
+    const bool wi = 32 * gi < p.n;   // the warp has particles
+    const float4 ci = box[wi ? 2 * gi : 0], hi = box[wi ? 2 * gi + 1 : 1];
+    const float far2 = (float)p.rc2 * 1.0001f;
     float fx = 0, fy = 0, fz = 0, e = 0, w = 0;
     int k = 0;
     for (; k < mine; k++) {
         const int b = k & 1;
         const int cnt = min(tile, npad - (split + k * nsplit) * tile);   // a multiple of 32
+        bool near = false;   // group lane of the tile (cnt / 32 of at most 4)
+        if (wi && lane < cnt / 32) {
+            const int gj = (split + k * nsplit) * (tile / 32) + lane;
+            near = n2_gap2(ci, hi, box[2 * gj], box[2 * gj + 1], L) < far2;
+        }
+        const unsigned live = __ballot_sync(0xffffffffu, near);
         if (!mbar_wait_bounded(&bars[b], (uint32_t)((k >> 1) & 1), err)) s_abort = 1;
         __syncthreads();
         if (s_abort) break;
         const float *X = sm[b][0], *Y = sm[b][1], *Z = sm[b][2];
         for (int j0 = 0; j0 < cnt; j0 += 32) {
+            if (!((live >> (j0 / 32)) & 1u)) continue;
             unsigned mask = 0;
 #pragma unroll
             for (int u = 0; u < 32; u += 4) {
