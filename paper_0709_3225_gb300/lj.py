@@ -180,8 +180,9 @@ class Context:
         self.params = params
         self.nc = lj_grid(params)
         self.stream = stream
+        self.stream_ptr = _stream_ptr(stream)
         h = ctypes.c_void_p()
-        _ck(load().lj_create(ctypes.byref(h), ctypes.byref(params), _stream_ptr(stream)), "lj_create")
+        _ck(load().lj_create(ctypes.byref(h), ctypes.byref(params), self.stream_ptr), "lj_create")
         self.handle = h
 
     @property
