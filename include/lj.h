@@ -411,9 +411,10 @@ int lj_set_tuning(lj_ctx *ctx, int32_t kernel, int32_t group_width, int32_t cell
  * possibly different N and box, each the method above (Sections 2 and 3),
  * stored back to back: replica r owns particles [o_r, o_r + n[r]) of the
  * concatenated (sum n, 3) / (sum n, 4) arrays, o_r = n[0] + ... + n[r-1].
- * One velocity-Verlet step of every replica is ONE cooperative persistent
- * kernel launch (binning, scan, scatter and forces separated by bounded grid
- * barriers), captured once in a CUDA graph and replayed.  FP32-mixed only.
+ * With force kernel 3 one velocity-Verlet step of every replica is ONE
+ * cooperative persistent kernel launch (binning, scan, scatter and forces
+ * separated by bounded grid barriers), captured once in a CUDA graph and
+ * replayed; kernel 7: see lj_batch_set_kernel.  FP32-mixed only.
  * Batching is not in the paper; it serves many small systems at once.    */
 
 typedef struct lj_batch lj_batch;
