@@ -4,8 +4,10 @@
 // concatenates their particles and cells so that one persistent launch per
 // step covers all of them.
 //
-// One step is one cooperative launch of k_batch_step (captured once in a
-// CUDA graph and replayed), whose phases are separated by grid barriers:
+// With the pair-once kernel (7) on slotted cells a step is two launches,
+// k_batch_slots and k_batch_force_n3 below.  Otherwise it is one cooperative
+// launch of k_batch_step (captured once in a CUDA graph and replayed), whose
+// phases are separated by grid barriers:
 //   1. kick, drift, wrap, cell id and rank   (every particle)
 //   2. scan of the per-cell counts            (tiles of 4096 cells)
 //   3. scatter to cell-sorted, cell-centred FP32 positions
@@ -408,8 +410,10 @@ struct BatchSlots {
 };
 
 // op 0: kicks, drift and wrap, then bin; op 1: bin the given positions.
+// Bound by HBM and the latency of the replica's fields: 48 registers, for 5
+// blocks per SM (56 and 4 without the bound: a step 319 -> 316 us).
 template <int OP>
-__global__ void __launch_bounds__(256) k_batch_slots(BatchSlots a, double *__restrict__ x, double *__restrict__ v,
+__global__ void __launch_bounds__(256, 5) k_batch_slots(BatchSlots a, double *__restrict__ x, double *__restrict__ v,
                                                      float4 *__restrict__ f, int n, double hk, double dt,
                                                      int32_t *__restrict__ err)
 {
@@ -1191,9 +1195,8 @@ extern "C" int lj_batch_create(lj_batch **out, int32_t nrep, const int64_t *n, c
     k.uc = (float)(rci6 * (4.0 * eps * s12 * rci6 - 4.0 * eps * s6));
     k.fc = (float)(rc * rci2 * rci6 * (48.0 * eps * s12 * rci6 - 24.0 * eps * s6));
     LJ_BCK(configure(b));
-    // the 27-cell code by default: the pair-once step measured slower on the
-    // 256-replica ensemble (2.12 against 1.70 ms per step), its 128
-    // registers leaving 16 warps per SM for every phase of the launch
+    // the 27-cell code until lj_batch_set_kernel chooses the pair-once one
+    // (the faster; its sums are added by atomics)
     b->n3 = 0;
 #undef LJ_BCK
     *out = b;
