@@ -396,7 +396,7 @@ __global__ void __launch_bounds__(kBatchThreads, 3) k_batch_step_n3(BatchDev b, 
 // update, two scan phases and the scatter at the force phase's occupancy,
 // with four grid barriers between them, and kept the FP64 pipe busy with
 // conversions (64 replicas, 1.6 million particles, per step:
-// 382 -> 319 us).
+// 382 -> 316 us).
 struct BatchRep {   // one replica's grid, 64 bytes
     double L, whi, wlo, s;
     float cw, inv_nc, sf;

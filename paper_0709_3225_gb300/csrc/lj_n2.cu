@@ -268,7 +268,7 @@ __device__ __forceinline__ float2 n2_r2(float2 xi, float2 yi, float2 zi, float2 
 // further than rc from theirs: no pair of the two is in range, so the sums
 // stay the same bits.  Particles that are stored near their neighbours (grown
 // on a lattice, read from a file written by cells) leave out most groups (46
-// -> 28 us, 120 -> 40 at 16,000); where the order is random the boxes fill the
+// -> 27 us, 120 -> 40 at 16,000); where the order is random the boxes fill the
 // system and the test's cost does not show (46 us).
 template <int MODE, bool ENERGY>
 __global__ void __launch_bounds__(kN2Threads) k_n2_force_f32(N2Params p, int npad, int tile, const float *__restrict__ soa,
