@@ -166,7 +166,7 @@ int skin_restart(lj_ctx *c)
 int do_bin(lj_ctx *c, const double *x, bool wrap_in_scatter)
 {
     if (c->slots_open == 1) c->slots_open = 2;   // a slotted binning that no kernel read
-    c->slots_last = 0;
+    LJ_CK(lists_begin(c));
     LJ_CK(launch_bin_count(c, x));
     LJ_CK(launch_scan(c));
     LJ_CK(launch_scatter(c, x, wrap_in_scatter));
@@ -218,7 +218,7 @@ int one_step(lj_ctx *c, double *x, double *v, void *f, int s, int nsteps, cudaEv
         LJ_CK(launch_force(c, f, false));
         return LJ_OK;
     }
-    c->slots_last = 0;
+    LJ_CK(lists_begin(c));
     if (c->skin > 0.0) {
         // cell lists with a skin: the cells are rebuilt only when the
         // device-side decision (k_skin_decide) asks for it; otherwise the
@@ -305,7 +305,9 @@ int capture_middle_step(lj_ctx *c, double *x, double *v, void *f)
         c->stream = cs;
         c->gsteps = uses_slots(c) || uses_fx(c) ? 2 : 1;
         c->gpar = c->slot_par;
+        c->own_capture = 1;
         for (int k = 0; k < c->gsteps && r == LJ_OK; k++) r = one_step(c, x, v, f, 1, 3);
+        c->own_capture = 0;
         c->stream = keep;
         e = cudaStreamEndCapture(cs, &g);
     }
@@ -667,7 +669,7 @@ extern "C" int lj_get_cells(lj_ctx *c, int32_t *cell_of, int32_t *count, int32_t
 {
     if (!c) return LJ_EINVAL;
     const size_t n = (size_t)c->p.n;
-    if (c->slots_last) LJ_CK(launch_slots_to_lists(c));   // the last binning was a slotted one
+    LJ_CK(launch_slots_to_lists(c));   // if the last binning was a slotted one
     if (cell_of && n) {
         int r = check_dev_ptr(cell_of, 4);
         if (r) return r;
@@ -701,6 +703,7 @@ extern "C" int lj_forces(lj_ctx *c, const double *x, void *f, double *e_pot, dou
         r = check_dev_ptr(f, 16);
         if (r) return r;
     }
+    c->new_call = 1;
     const bool energy = e_pot || virial;
     if (!energy && uses_fx(c)) {
         LJ_CK(launch_bin_fx(c, x, (double4_16a *)f));
@@ -767,7 +770,8 @@ extern "C" int lj_langevin_step(lj_ctx *c, double *x, double *v, void *f, int32_
     r = check_dev_ptr(f, 16);
     if (r) return r;
     const bool slots = uses_slots(c);
-    if (!slots) c->slots_last = 0;
+    c->new_call = 1;
+    if (!slots) LJ_CK(lists_begin(c));
     for (int s = 0; s < nsteps; s++) {
         LJ_CK(launch_langevin_bin(c, x, v, f, s == 0 ? 1 : 2, gamma, kT, slots && s > 0 && !c->timing));
         if (!slots) {
@@ -812,6 +816,7 @@ extern "C" int lj_step(lj_ctx *c, double *x, double *v, void *f, int32_t nsteps)
         r = check_dev_ptr(f, 16);
         if (r) return r;
     }
+    c->new_call = 1;
     return do_steps(c, x, v, f, nsteps);
 }
 
@@ -820,6 +825,7 @@ extern "C" int lj_step_host(lj_ctx *c, double *x, double *v, void *f, int32_t ns
     if (!c || nsteps < 0) return LJ_EINVAL;
     const size_t n = (size_t)c->p.n;
     if (n > 0 && (!x || !v || !f)) return LJ_EINVAL;
+    c->new_call = 1;
     int r = ensure_staging(c);
     if (r) return r;
     const size_t bx = 3 * n * sizeof(double), bf = n * force_vsize(c);
@@ -910,6 +916,7 @@ extern "C" int lj_energy(lj_ctx *c, const double *x, const double *v, double *ou
     LJ_CK(cudaMemsetAsync(c->scalars, 0, 4 * sizeof(double), c->stream));
     if (c->p.n > 0) {
         LJ_CK(launch_ekin(c, v));
+        c->new_call = 1;
         r = bin_for_force(c, x, c->fs);
         if (r) return r;
         LJ_CK(launch_force(c, c->fs, true));
@@ -938,6 +945,7 @@ extern "C" int lj_observables(lj_ctx *c, const double *x, const double *v, doubl
     LJ_CK(cudaMemsetAsync(c->scalars, 0, 8 * sizeof(double), c->stream));
     if (c->p.n > 0) {
         LJ_CK(launch_ekin(c, v));
+        c->new_call = 1;
         r = bin_for_force(c, x, c->fs);
         if (r) return r;
         LJ_CK(launch_force(c, c->fs, true));
@@ -986,6 +994,7 @@ extern "C" int lj_forces_vjp(lj_ctx *c, const double *x, const double *g, double
     if ((r = check_dev_ptr(g, 8)) != LJ_OK) return r;
     if ((r = check_dev_ptr(dx, 8)) != LJ_OK) return r;
     if ((r = ensure_vjp_buffers(c)) != LJ_OK) return r;
+    c->new_call = 1;
     if ((r = bin_for_vjp(c, x, g)) != LJ_OK) return r;
     LJ_CK(launch_vjp(c, g, scale, dx, dparam));
     return LJ_OK;
@@ -1004,6 +1013,7 @@ extern "C" int lj_vv_adjoint_step(lj_ctx *c, const double *x_n, const double *x_
     if ((r = check_dev_ptr(lam_v, 8)) != LJ_OK) return r;
     if ((r = ensure_vjp_buffers(c)) != LJ_OK) return r;
     const double h = 0.5 * c->p.dt / c->p.mass;
+    c->new_call = 1;
     // v_{n+1} = v_half + h F(x_{n+1})
     // and x_{n+1} = x_n + dt v_half
     if ((r = bin_for_vjp(c, x_n1, lam_v)) != LJ_OK) return r;
@@ -1023,6 +1033,7 @@ extern "C" int lj_step_record(lj_ctx *c, double *traj, double *v, void *f, int32
     if ((r = check_dev_ptr(v, 8)) != LJ_OK) return r;
     if ((r = check_dev_ptr(f, 16)) != LJ_OK) return r;
     const size_t m = 3 * (size_t)c->p.n;
+    c->new_call = 1;
     if (!uses_slots(c) || persistent_mode(c)) {
         for (int s = 0; s < nsteps; s++) {
             LJ_CK(cudaMemcpyAsync(traj + (s + 1) * m, traj + s * m, m * sizeof(double), cudaMemcpyDeviceToDevice,
@@ -1058,6 +1069,7 @@ extern "C" int lj_vv_adjoint_segment(lj_ctx *c, const double *traj, int32_t nste
     if ((r = ensure_vjp_buffers(c)) != LJ_OK) return r;
     const double h = 0.5 * c->p.dt / c->p.mass;
     const size_t m = 3 * (size_t)c->p.n;
+    c->new_call = 1;
     const bool slots = uses_slots(c);   // then each VJP's last kernel bins the next state
     for (int s = nsteps; s >= 0; s--) {
         if (s == nsteps || !slots)

@@ -687,6 +687,9 @@ struct lj_batch {
     const float2 *centre2;
     WarpParams ks;
     int gpar;             // par where the captured pair of steps starts
+    // calls recorded into a caller's graph, as lj_ctx holds them (lj_internal.cuh)
+    unsigned long long cap_id;
+    int captured, new_call, own_capture;
     int slots_ok;         // cells beyond their slots are rare in every replica
     std::vector<BatchRep> hrep;
     std::vector<float2> hcentre2;
@@ -844,7 +847,19 @@ bool batch_slots(const lj_batch *b) { return b->n3 && b->scap > 0; }
 cudaError_t launch_slots_step(lj_batch *b, bool energy, int op, double *x, double *v, float4 *f, int nkick, bool after)
 {
     cudaError_t e = cudaSuccess;
-    if (b->dirty) {
+    bool zero = b->dirty != 0;
+    if (!b->own_capture) {   // as slots_begin (lj_slots.cu)
+        const unsigned long long id = capture_id(b->stream);
+        if (id) {
+            zero = zero || id != b->cap_id;
+            b->cap_id = id;
+            b->captured = 1;
+        } else if (b->captured && b->new_call) {
+            zero = true;
+        }
+        b->new_call = 0;
+    }
+    if (zero) {
         for (int k = 0; k < 2 && e == cudaSuccess; k++)
             e = cudaMemsetAsync(b->cellq[k], 0, ((size_t)b->ncell + 1) * sizeof(int2), b->stream);
         if (e == cudaSuccess) e = cudaMemsetAsync(b->octr, 0, 2 * sizeof(unsigned), b->stream);
@@ -862,6 +877,7 @@ cudaError_t launch_slots_step(lj_batch *b, bool energy, int op, double *x, doubl
     a.bin.ncell = (int)b->ncell;
     a.bin.cap = b->scap;
     a.bin.nslots = b->nslots;
+    a.bin.nover = (int)b->ntot;
     a.rep = b->rep;
     a.rep_of = b->d.rep_of;
     a.rep_of_cell = b->d.rep_of_cell;
@@ -913,8 +929,10 @@ cudaError_t capture_slots_pair(lj_batch *b, double *x, double *v, float4 *f)
     const int par = b->par;
     if ((e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal)) == cudaSuccess) {
         b->stream = cs;
+        b->own_capture = 1;
         cudaError_t el = launch_slots_step(b, false, 0, x, v, f, 2, false);
         if (el == cudaSuccess) el = launch_slots_step(b, false, 0, x, v, f, 2, true);
+        b->own_capture = 0;
         b->stream = keep;
         e = cudaStreamEndCapture(cs, &g);
         if (el != cudaSuccess) e = el;
@@ -942,9 +960,10 @@ cudaError_t capture_slots_pair(lj_batch *b, double *x, double *v, float4 *f)
 cudaError_t slots_steps(lj_batch *b, double *x, double *v, float4 *f, int nsteps)
 {
     cudaError_t e = launch_slots_step(b, false, 0, x, v, f, 1, false);
+    const bool replay = b->use_graph && !capture_id(b->stream);
     for (int s = 1; s < nsteps && e == cudaSuccess;) {
         const bool have = b->gexec && b->gx == x && b->gv == v && b->gf == f;
-        bool graph = b->use_graph && s + 2 <= nsteps && !(have && b->gpar != b->par);
+        bool graph = replay && b->use_graph && s + 2 <= nsteps && !(have && b->gpar != b->par);
         if (graph && !have && capture_slots_pair(b, x, v, f) != cudaSuccess) {
             b->use_graph = 0;   // capture unsupported here: launch directly
             graph = false;
@@ -985,6 +1004,7 @@ int sync_check(lj_batch *b)
     if (bits & LJ_ERRBIT_NONFINITE) return LJ_ENONFINITE;
     if (bits & LJ_ERRBIT_TIMEOUT) return LJ_ETIMEOUT;
     if (bits & LJ_ERRBIT_SCAN) return LJ_ECUDA;
+    if (bits & LJ_ERRBIT_OVERFLOW) return LJ_EOVERFLOW;
     return LJ_OK;
 }
 
@@ -1260,6 +1280,7 @@ extern "C" int lj_batch_forces(lj_batch *b, const double *x, void *f, int32_t en
     int r;
     if ((r = check_ptr(x, 8)) != LJ_OK) return r;
     if ((r = check_ptr(f, 16)) != LJ_OK) return r;
+    b->new_call = 1;
     cudaError_t e = launch_step_kernel(b, energy != 0, 1, (double *)x, nullptr, (float4 *)f);
     return e == cudaSuccess ? LJ_OK : map_err(e);
 }
@@ -1272,6 +1293,7 @@ extern "C" int lj_batch_step(lj_batch *b, double *x, double *v, void *f, int32_t
     if ((r = check_ptr(x, 8)) != LJ_OK) return r;
     if ((r = check_ptr(v, 8)) != LJ_OK) return r;
     if ((r = check_ptr(f, 16)) != LJ_OK) return r;
+    b->new_call = 1;
     if (batch_slots(b)) {
         const cudaError_t es = slots_steps(b, x, v, (float4 *)f, nsteps);
         return es == cudaSuccess ? LJ_OK : map_err(es);
@@ -1341,6 +1363,7 @@ extern "C" int lj_batch_energy(lj_batch *b, const double *x, const double *v, vo
         if ((r = check_ptr(x, 8)) != LJ_OK) return r;
         if ((r = check_ptr(v, 8)) != LJ_OK) return r;
         if ((r = check_ptr(f, 16)) != LJ_OK) return r;
+        b->new_call = 1;
         cudaError_t e = launch_step_kernel(b, true, 1, (double *)x, nullptr, (float4 *)f);
         if (e != cudaSuccess) return map_err(e);
     }
@@ -1363,6 +1386,7 @@ extern "C" int lj_batch_relax(lj_batch *b, double *x, void *f, int32_t nsteps, d
     int r;
     if ((r = check_ptr(x, 8)) != LJ_OK) return r;
     if ((r = check_ptr(f, 16)) != LJ_OK) return r;
+    b->new_call = 1;
     for (int s = 0; s < nsteps; s++) {
         cudaError_t e = launch_step_kernel(b, false, 1, x, nullptr, (float4 *)f);
         if (e != cudaSuccess) return map_err(e);

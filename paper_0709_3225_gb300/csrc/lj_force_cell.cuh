@@ -47,6 +47,8 @@ struct WarpParams {
     const int2 *cellq;           // (count, overflow list head + 1) per cell
     int2 *cellq_next;            // the next binning's, zeroed by this launch (ncell + 1 entries)
     unsigned *octr_next;
+    unsigned *last_par;          // the buffer this launch reads, par, is noted here
+    unsigned par;
     const int32_t *onext;
 };
 

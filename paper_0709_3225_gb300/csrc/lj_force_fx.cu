@@ -55,7 +55,8 @@ struct FxParams {
     int64_t ncell;
     const int2 *cellq;
     int2 *cellq_next;
-    unsigned *octr_next;
+    unsigned *octr_next, *last_par;
+    unsigned par;
     const int32_t *onext;
     const double *centre;
     int S, kappa_e, tsh;                        // u = K / 2^63 2^kappa_e 2^lz RI 2^-62
@@ -159,8 +160,8 @@ __device__ void fx_plain(const FxParams &k, const longlong4_16a *__restrict__ po
         int si = st[0] + (vi ? i : 0);
         if (vi && i >= k.scap) {
             int o = __ldg(&k.cellq[c].y);
-            for (int m = k.scap; m < i; m++) o = __ldg(k.onext + o - 1);
-            si = k.nslots + o - 1;
+            for (int m = k.scap; m < i && o > 0; m++) o = __ldg(k.onext + o - 1);
+            if (o > 0) si = k.nslots + o - 1;
         }
         const longlong4_16a pi = pos[si];
         // coordinates relative to the home cell's centre (their differences
@@ -174,6 +175,7 @@ __device__ void fx_plain(const FxParams &k, const longlong4_16a *__restrict__ po
                 int sj = st[kk] + j;
                 if (j >= k.scap) {
                     o = j == k.scap ? __ldg(&k.cellq[half_cell(c, kk, k.nc, k.inv_nc)].y) : __ldg(k.onext + o - 1);
+                    if (o <= 0) break;
                     sj = k.nslots + o - 1;
                 }
                 if (!vi || (kk == 0 && j <= i)) continue;
@@ -342,6 +344,7 @@ __global__ void __launch_bounds__(kFxThreads) k_force_fx(FxParams k, const longl
     if (blockIdx.x == 0 && lane == 0) {
         k.cellq_next[k.ncell] = make_int2(0, 0);
         *k.octr_next = 0u;
+        *k.last_par = k.par;
     }
     const float2 *X2 = reinterpret_cast<const float2 *>(X);
     const float2 *Y2 = reinterpret_cast<const float2 *>(X + k.cap);
@@ -475,6 +478,8 @@ cudaError_t launch_force_fx(lj_ctx *c, double4_16a *f)
     k.cellq = c->cellq[c->slot_par];
     k.cellq_next = c->cellq[c->slot_par ^ 1];
     k.octr_next = c->octr + (c->slot_par ^ 1);
+    k.last_par = c->octr + 2;
+    k.par = (unsigned)c->slot_par;
     k.onext = c->onext;
     k.centre = c->centre;
     k.S = S;

@@ -28,6 +28,7 @@ __global__ void __launch_bounds__(kN3Threads, ENERGY ? 4 : 6) k_force_n3(WarpPar
         if (blockIdx.x == 0 && threadIdx.x == 0) {
             k.cellq_next[k.ncell] = make_int2(0, 0);
             *k.octr_next = 0u;
+            *k.last_par = k.par;
         }
     }
     auto load = [&](int c) { return half_load<true, SLOTS>(start, c, nc, k.inv_nc, 0, k.scap); };
@@ -180,6 +181,8 @@ cudaError_t launch_force_n3(lj_ctx *c, void *f, bool energy)
         k.cellq = c->cellq[c->slot_par];
         k.cellq_next = c->cellq[c->slot_par ^ 1];
         k.octr_next = c->octr + (c->slot_par ^ 1);
+        k.last_par = c->octr + 2;
+        k.par = (unsigned)c->slot_par;
         k.onext = c->onext;
     }
     double *partial = c->partial;

@@ -521,8 +521,8 @@ __device__ void n3_plain(const WarpParams &k, const float4 *__restrict__ pos, fl
         int si = s_home + (vi ? i : 0);
         if (SLOTS && vi && i >= k.scap) {   // the (i - scap)-th of the home cell's overflow list
             int o = __ldg(&k.cellq[cell0 + c].y);
-            for (int m = k.scap; m < i; m++) o = __ldg(k.onext + o - 1);
-            si = k.nslots + o - 1;
+            for (int m = k.scap; m < i && o > 0; m++) o = __ldg(k.onext + o - 1);
+            if (o > 0) si = k.nslots + o - 1;   // (a list shorter than its count: only with its error latched)
         }
         const float4 pi = load_pos<NC>(pos + si);
         float fx = 0.f, fy = 0.f, fz = 0.f, e = 0.f, w = 0.f;
@@ -536,6 +536,7 @@ __device__ void n3_plain(const WarpParams &k, const float4 *__restrict__ pos, fl
                 int sj = s + j;
                 if (SLOTS && j >= k.scap) {
                     o = j == k.scap ? __ldg(&k.cellq[cell0 + half_cell(c, kk, nc, inv_nc)].y) : __ldg(k.onext + o - 1);
+                    if (o <= 0) break;
                     sj = k.nslots + o - 1;
                 }
                 if (SPLIT && (spre[kk] + j < ta || spre[kk] + j >= tb_end)) continue;   // another part's

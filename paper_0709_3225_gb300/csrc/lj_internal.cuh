@@ -129,7 +129,9 @@ struct lj_ctx {
     // the force (VJP) kernel after it zeroes the other one.
     int scap, nslots;        // nslots = ncell * scap; spos holds nslots + n
     int2 *cellq[2];
-    unsigned *octr;          // [2] overflow particles per buffer
+    // [0], [1] overflow particles per buffer; [2] the buffer of the last
+    // force (VJP) launch, -1 (as int) when the sorted lists are newer
+    unsigned *octr;
     void *spos;              // slotted positions: float4 (FP64: longlong4)
     float4 *sg4;             // cotangents (lazily allocated)
     int32_t *onext;          // overflow lists: index + 1 of the next, 0 = end
@@ -140,6 +142,14 @@ struct lj_ctx {
     int slot_par;            // buffer of the next binning
     int slots_open;          // 1: a slotted binning waits for its kernel, 2: the buffers are not known to be zero
     int slots_last;          // the last binning was a slotted one
+    // A caller may record calls into a graph of their own and replay it
+    // between direct calls: the state of the buffers is then not the host's
+    // to know.  cap_id: the capture whose first slotted binning has recorded
+    // their zeroing; captured: there has been one, and every direct call
+    // (new_call) zeroes them too; own_capture: the capture is the library's
+    // (lj_set_graph), whose replays the host follows.
+    unsigned long long cap_id;
+    int captured, new_call, own_capture;
     // graph replay of the middle steps of lj_step (lj_set_graph)
     int use_graph;
     cudaGraphExec_t gexec;   // captured middle steps: two with slotted cells (one per buffer), else one
@@ -397,6 +407,20 @@ inline cudaError_t launch_pdl(const void *kern, dim3 grid, int block, void **arg
     return cudaLaunchKernelExC(&cfg, kern, args);
 }
 
+// Id of the capture that stream s is in, 0 when it is in none (the legacy
+// stream cannot be).
+inline unsigned long long capture_id(cudaStream_t s)
+{
+    if (s == nullptr || s == cudaStreamLegacy) return 0;
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    unsigned long long id = 0;
+    if (cudaStreamGetCaptureInfo(s, &st, &id) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    return st == cudaStreamCaptureStatusActive ? id : 0;
+}
+
 // Kernel launchers (each returns cudaGetLastError()).
 // gated: skin mode, run only when the device-side rebuild flag is set
 cudaError_t launch_bin_count(lj_ctx *c, const double *x, bool gated = false);
@@ -502,6 +526,7 @@ cudaError_t launch_host_in(lj_ctx *c, const double *hx, const double *hv, const 
 cudaError_t launch_host_out(lj_ctx *c, const double *x, const double *v, const float4 *f, double *hx, double *hv,
                             float4 *hf);
 cudaError_t slots_begin(lj_ctx *c, int64_t i_begin);   // before a slotted binning launch
+cudaError_t lists_begin(lj_ctx *c);                    // before a binning into the sorted lists
 void slots_consumed(lj_ctx *c);                        // after the launch that reads it
 // FP64 contexts: the fixed-point kernel (lj_force_fx.cu) over slotted cells.
 // Its forces are f (the pairs taken in FP64) plus fx_scale times fx_acc:
@@ -516,6 +541,6 @@ cudaError_t launch_bin_fx(lj_ctx *c, const double *x, double4_16a *f);
 cudaError_t launch_kick_drift_fx(lj_ctx *c, double *x, double *v, double4_16a *f, int nkick, bool with_acc,
                                  int64_t i_begin = 0, int64_t i_end = -1, bool after_force = false);
 cudaError_t launch_fx_finish(lj_ctx *c, double *v, double4_16a *f);
-// Rebuild cell_of, start and perm from the last slotted binning.
+// Rebuild cell_of, start and perm from the last binning if it was a slotted one.
 cudaError_t launch_slots_to_lists(lj_ctx *c);
 cudaError_t launch_force_n3(lj_ctx *c, void *f, bool energy);

@@ -284,27 +284,36 @@ __device__ __forceinline__ int slot_index(const void *pos, int64_t s)
     return __float_as_int(reinterpret_cast<const float4 *>(pos)[s].w);
 }
 
+// The count buffers and which of them the last force launch read; its value
+// -1: the sorted lists are newer and stay as they are.
+struct SlotLast {
+    const int2 *cellq[2];
+    const int *last;
+};
+
 // Counts of every cell (the extra one included) for the scan of
 // launch_slots_to_lists; cell_of starts as the extra cell everywhere.
-__global__ void k_slot_counts(const int2 *__restrict__ cellq, int ncell1, int32_t *__restrict__ count, int n,
-                              int32_t *__restrict__ cell_of)
+__global__ void k_slot_counts(SlotLast l, int ncell1, const int32_t *__restrict__ start, int32_t *__restrict__ count,
+                              int n, int32_t *__restrict__ cell_of)
 {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < ncell1) count[t] = cellq[t].x;
-    if (t < n) cell_of[t] = ncell1 - 1;
+    const int q = *l.last;
+    if (t < ncell1) count[t] = q < 0 ? start[t + 1] - start[t] : l.cellq[q][t].x;
+    if (q >= 0 && t < n) cell_of[t] = ncell1 - 1;
 }
 
 // perm and cell_of of the particles in slots and overflow lists, one thread
 // per cell.
 template <bool FX>
-__global__ void k_slot_lists(const int2 *__restrict__ cellq, const void *__restrict__ pos,
+__global__ void k_slot_lists(SlotLast l, const void *__restrict__ pos,
                              const int32_t *__restrict__ onext, int ncell, int cap, int nslots,
                              const int32_t *__restrict__ start, int32_t *__restrict__ perm,
                              int32_t *__restrict__ cell_of)
 {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= ncell) return;
-    const int2 q = cellq[c];
+    const int p = *l.last;
+    if (c >= ncell || p < 0) return;
+    const int2 q = l.cellq[p][c];
     const int s = start[c];
     int r = 0;
     for (; r < min(q.x, cap); r++) {
@@ -312,7 +321,7 @@ __global__ void k_slot_lists(const int2 *__restrict__ cellq, const void *__restr
         perm[s + r] = i;
         cell_of[i] = c;
     }
-    for (int o = q.y; o > 0; o = onext[o - 1], r++) {
+    for (int o = q.y; o > 0 && r < q.x; o = onext[o - 1], r++) {
         const int i = slot_index<FX>(pos, (int64_t)nslots + o - 1);
         perm[s + r] = i;
         cell_of[i] = c;
@@ -321,11 +330,11 @@ __global__ void k_slot_lists(const int2 *__restrict__ cellq, const void *__restr
 
 // The particles left in the extra cell (non-finite positions), listed after
 // the grid's; count[ncell] is the cursor, zero before and after (last block).
-__global__ void k_slot_extra(const int32_t *__restrict__ cell_of, int n, int ncell, const int32_t *__restrict__ start,
+__global__ void k_slot_extra(SlotLast l, const int32_t *__restrict__ cell_of, int n, int ncell, const int32_t *__restrict__ start,
                              int32_t *__restrict__ perm, int32_t *__restrict__ cursor)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n && cell_of[i] == ncell) perm[start[ncell] + atomicAdd(cursor, 1)] = i;
+    if (*l.last >= 0 && i < n && cell_of[i] == ncell) perm[start[ncell] + atomicAdd(cursor, 1)] = i;
 }
 
 inline unsigned blocks_for(int64_t n, int threads) { return (unsigned)((n + threads - 1) / threads); }
@@ -351,6 +360,7 @@ SlotBin slot_bin_of(const lj_ctx *c)
     b.ncell = (int)c->ncell;
     b.cap = c->scap;
     b.nslots = c->nslots;
+    b.nover = (int)c->p.n;
     b.cell0 = 0;
     b.S = c->p.precision == LJ_PREC_FP64 ? fx_shift(c) : 0;
     return b;
@@ -395,7 +405,8 @@ cudaError_t slots_setup(lj_ctx *c)
     cudaError_t e = cudaSuccess;
     const size_t qb = (size_t)(c->ncell + 1) * sizeof(int2);
     for (int k = 0; k < 2 && e == cudaSuccess; k++) e = cudaMalloc(&c->cellq[k], qb);
-    if (e == cudaSuccess) e = cudaMalloc(&c->octr, 2 * sizeof(unsigned));
+    if (e == cudaSuccess) e = cudaMalloc(&c->octr, 4 * sizeof(unsigned));
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->octr, 0xff, 4 * sizeof(unsigned), c->stream);
     if (e == cudaSuccess)
         e = cudaMalloc(&c->spos, (size_t)(nslots + c->p.n) * (fp64 ? sizeof(longlong4_16a) : sizeof(float4)));
     if (e == cudaSuccess && fp64) e = cudaMalloc(&c->fx_acc, (size_t)c->p.n * 4 * sizeof(long long));
@@ -480,7 +491,19 @@ cudaError_t slots_begin(lj_ctx *c, int64_t i_begin)
 {
     if (i_begin > 0) return cudaSuccess;
     cudaError_t e = cudaSuccess;
-    if (c->slots_open) {   // first use, or a binning that no kernel consumed
+    bool zero = c->slots_open != 0;   // first use, or a binning that no kernel consumed
+    if (!c->own_capture) {
+        const unsigned long long id = capture_id(c->stream);
+        if (id) {   // recorded: replays start from buffers in any state
+            zero = zero || id != c->cap_id;
+            c->cap_id = id;
+            c->captured = 1;
+        } else if (c->captured && c->new_call) {   // a replay may have come since the last call
+            zero = true;
+        }
+        c->new_call = 0;
+    }
+    if (zero) {
         const size_t qb = (size_t)(c->ncell + 1) * sizeof(int2);
         e = cudaMemsetAsync(c->cellq[0], 0, qb, c->stream);
         if (e == cudaSuccess) e = cudaMemsetAsync(c->cellq[1], 0, qb, c->stream);
@@ -488,6 +511,15 @@ cudaError_t slots_begin(lj_ctx *c, int64_t i_begin)
     }
     c->slots_open = 1;
     return e;
+}
+
+cudaError_t lists_begin(lj_ctx *c)
+{
+    c->slots_last = 0;
+    if (c->scap == 0 || c->own_capture) return cudaSuccess;
+    if (!c->captured && !capture_id(c->stream)) return cudaSuccess;
+    c->captured = 1;
+    return cudaMemsetAsync(c->octr + 2, 0xff, sizeof(unsigned), c->stream);
 }
 
 void slots_consumed(lj_ctx *c)
@@ -549,10 +581,13 @@ cudaError_t launch_host_out(lj_ctx *c, const double *x, const double *v, const f
 
 cudaError_t launch_slots_to_lists(lj_ctx *c)
 {
+    if (c->scap == 0) return cudaSuccess;
+    if (capture_id(c->stream)) c->captured = 1;   // recorded, not run
+    if (!c->slots_last && !c->captured) return cudaSuccess;
     const int n = (int)c->p.n, ncell = (int)c->ncell;
-    const int2 *q = c->cellq[c->slot_par ^ 1];
-    k_slot_counts<<<blocks_for(n > ncell + 1 ? n : ncell + 1, 256), 256, 0, c->stream>>>(q, ncell + 1, c->count, n,
-                                                                                         c->cell_of);
+    const SlotLast q = {{c->cellq[0], c->cellq[1]}, reinterpret_cast<const int *>(c->octr + 2)};
+    k_slot_counts<<<blocks_for(n > ncell + 1 ? n : ncell + 1, 256), 256, 0, c->stream>>>(q, ncell + 1, c->start,
+                                                                                         c->count, n, c->cell_of);
     c->kernel_launches++;
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = launch_scan(c);   // start from the counts, which it zeroes
@@ -563,7 +598,7 @@ cudaError_t launch_slots_to_lists(lj_ctx *c)
     else
         k_slot_lists<false><<<blocks_for(ncell, 256), 256, 0, c->stream>>>(q, c->spos, c->onext, ncell, c->scap,
                                                                            c->nslots, c->start, c->perm, c->cell_of);
-    k_slot_extra<<<blocks_for(n, 256), 256, 0, c->stream>>>(c->cell_of, n, ncell, c->start, c->perm, c->count + ncell);
+    k_slot_extra<<<blocks_for(n, 256), 256, 0, c->stream>>>(q, c->cell_of, n, ncell, c->start, c->perm, c->count + ncell);
     c->kernel_launches += 2;
     e = cudaMemsetAsync(c->count + ncell, 0, sizeof(int32_t), c->stream);
     if (e != cudaSuccess) return e;

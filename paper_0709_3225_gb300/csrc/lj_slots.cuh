@@ -14,7 +14,8 @@
 //
 // The counts must be zero when a binning starts.  They are held twice; the
 // force (or VJP) kernel that reads one buffer zeroes the other for the
-// next binning.
+// next binning.  Which buffer is next is the host's knowledge; calls that a
+// caller records into a graph zero both first (slots_begin).
 #pragma once
 
 #include "lj_internal.cuh"
@@ -29,6 +30,7 @@ struct SlotBin {
     double L, whi, wlo, s;
     float sf;               // (float)s
     int nc, ncell, cap, nslots, S;   // S: scale of the fixed-point coordinates (FP64)
+    int nover;              // entries of the overflow region
     int cell0;              // id of the grid's first cell (a batch's replica; else 0); ncell counts all grids' cells
 };
 
@@ -70,6 +72,10 @@ __device__ __forceinline__ int slot_place(const SlotBin &b, bool valid, int i, d
     int slot = c * b.cap + r;
     if (r >= b.cap) {   // overflow: the next free entry, pushed on the cell's list
         const int k = (int)atomicAdd(b.octr, 1u);
+        if (k >= b.nover) {   // never with counts that were zero
+            atomicOr(err, LJ_ERRBIT_OVERFLOW);
+            return -1;
+        }
         slot = b.nslots + k;
         b.onext[k] = atomicExch(&b.cellq[c].y, k + 1);
     }

@@ -47,7 +47,8 @@ struct VjpN3Coef {
     int scap, nslots;
     const int2 *cellq;
     int2 *cellq_next;
-    unsigned *octr_next;
+    unsigned *octr_next, *last_par;
+    unsigned par;
     const int32_t *onext;
 };
 
@@ -371,8 +372,8 @@ __device__ void vn3_plain(const VjpN3Coef &k, const float4 *__restrict__ pos, co
         int si = s_home + (vi ? i : 0);
         if (SLOTS && vi && i >= k.scap) {
             int o = __ldg(&k.cellq[c].y);
-            for (int m = k.scap; m < i; m++) o = __ldg(k.onext + o - 1);
-            si = k.nslots + o - 1;
+            for (int m = k.scap; m < i && o > 0; m++) o = __ldg(k.onext + o - 1);
+            if (o > 0) si = k.nslots + o - 1;
         }
         const float4 pi = __ldg(pos + si);
         const float4 gi = __ldg(g4 + si);
@@ -386,6 +387,7 @@ __device__ void vn3_plain(const VjpN3Coef &k, const float4 *__restrict__ pos, co
                 int sj = s + j;
                 if (SLOTS && j >= k.scap) {
                     o = j == k.scap ? __ldg(&k.cellq[half_cell(c, kk, k.nc, k.inv_nc)].y) : __ldg(k.onext + o - 1);
+                    if (o <= 0) break;
                     sj = k.nslots + o - 1;
                 }
                 const float4 q = __ldg(pos + sj);
@@ -435,6 +437,7 @@ __global__ void __launch_bounds__(kVn3Threads, 4) k_vjp_n3(VjpN3Coef k, const fl
         if (blockIdx.x == 0 && threadIdx.x == 0) {
             k.cellq_next[k.ncell] = make_int2(0, 0);
             *k.octr_next = 0u;
+            *k.last_par = k.par;
         }
     }
     auto load = [&](int c) { return half_load<true, SLOTS>(start, c, k.nc, k.inv_nc, 0, k.scap); };
@@ -624,6 +627,8 @@ cudaError_t launch_vjp_n3(lj_ctx *c, const double *coef, double scale, double *d
     k.cellq = c->cellq[c->slot_par];
     k.cellq_next = c->cellq[c->slot_par ^ 1];
     k.octr_next = slots ? c->octr + (c->slot_par ^ 1) : nullptr;
+    k.last_par = slots ? c->octr + 2 : nullptr;
+    k.par = (unsigned)c->slot_par;
     k.onext = c->onext;
     k.nc = c->nc;
     k.cap = cap;
