@@ -18,13 +18,28 @@
 //  * r^2: the upper 64 bits of the squares, 2^-57 relative at r = 0.4 rc.
 //  * u = sigma^2 / r^2: a float reciprocal of the normalised r^2 (error e <
 //    2^-22, formed exactly in integers) and the series 1 + e + e^2 (e^3 <
-//    2^-66), then u^2, u^3, u^4 by high products; F(r) / r = 24 eps / sigma^2
-//    u^4 (2 u^3 - 1), in units of 2^-56, and its products with d.
+//    2^-66), then u^2, u^3, u^4 by high products and |F(r)| / r = 24 eps /
+//    sigma^2 u^4 |2 u^3 - 1|.
 //  * The sums are 64-bit integers, added by integer atomics: exact, so they
-//    do not depend on the order (the forces repeat from run to run).  Their
-//    unit, 2^-52 24 eps / sigma at most, leaves a range of 300 times the
-//    largest pair force taken here, for the net force of a particle (sums
-//    that leave the range on the way come back): eight cells' slots hold 256.
+//    do not depend on the order (the forces repeat from run to run).  One
+//    unit cannot hold them all: a pair at 2.45 sigma is 1/3,300 of the
+//    largest one taken here, and in that one's unit it had 43 bits.  So there
+//    are three sums per component, of units q = 2^-52 24 eps / sigma at
+//    sigma = 1 (fx_tsh), q / 32 and q / 256, for the repulsive pairs, the
+//    attractive ones and those beyond 1.8 sigma, the products rounded to
+//    nearest in magnitude.  With |F| <= 6.35, 0.1 and 0.0155 of 24 eps /
+//    sigma in the three, their ranges hold 320, 590 and 480 pairs that all
+//    pull one way, more than cells of 32 slots can place so; sums that leave
+//    the range on the way come back.  A home particle's partial sums become
+//    one number in units of q / 256, which is added as its upper bits, to the
+//    first sum, and its lowest 8, which the three components share a word
+//    for: four atomics, not nine.
+//    Emulated in exact integers for single pairs, RMS error relative to the
+//    force (FP64 coordinates and term: L = 7.6, 13, 27, 54; one unit for all
+//    pairs): r = 1.0 2.5e-16 (1e-15 to 2e-14), 1.2 5e-17 (3e-16 to 6e-15; one
+//    unit 2.4e-15), 1.7 1.6e-16 (4e-16 to 5e-15; 9e-15), 2.45 2.4e-16 (4e-16
+//    to 5e-15; 1.1e-13), 2.65 4.0e-16 (4.2e-16 at L = 9); 2.9 7.7e-16
+//    (4.1e-16): hence rc <= 2.6 sigma in uses_fx.
 //  * Pairs closer than sqrt(0.8) sigma, where u > 1.25 and the force has no
 //    bound, and cells that take the plain path are evaluated in FP64 as
 //    before (pair64_nf) and added to f itself; the readers of the sums add
@@ -61,7 +76,7 @@ struct FxParams {
     const double *centre;
     int S, kappa_e, tsh;                        // u = K / 2^63 2^kappa_e 2^lz RI 2^-62
     long long Lfix;
-    unsigned long long K, r2c, r2min;
+    unsigned long long K, r2c, r2min, r2far;
     // FP64 pairs
     double to_d;                           // 2^-S
     double rc2, a12, b6;
@@ -101,22 +116,23 @@ __device__ __forceinline__ void fx_add64(double4_16a *f, int i, double x, double
     atomicAdd(&f[i].z, z);
 }
 
-__device__ __forceinline__ void fx_add(long long *acc, int i, long long x, long long y, long long z)
+__device__ __forceinline__ void fx_red(unsigned long long *o, long long v) { atomicAdd(o, (unsigned long long)v); }
+
+// A home particle's partial sums (of at most 32 pairs): r, m, f in units of q,
+// q / 32, q / 256.  v = 8 m + f: |m| < 2^59, |f| < 2^59.
+__device__ __forceinline__ long long fx_split(long long r, long long m, long long f, int sh, unsigned long long &lo)
 {
-    unsigned long long *o = reinterpret_cast<unsigned long long *>(acc) + 4 * (int64_t)i;
-    atomicAdd(o, (unsigned long long)x);
-    atomicAdd(o + 1, (unsigned long long)y);
-    atomicAdd(o + 2, (unsigned long long)z);
+    const long long v = (m << 3) + f;
+    lo += (unsigned long long)(v & 255) << sh;
+    return r + (v >> 8);
 }
 
-__device__ __forceinline__ unsigned long long fx_sq(long long d)
-{
-    const unsigned long long a = (unsigned long long)(d < 0 ? -d : d);
-    return __umul64hi(a, a);
-}
+__device__ __forceinline__ unsigned long long fx_abs(long long d) { return (unsigned long long)(d < 0 ? -d : d); }
 
-// F(r) / r in units of 24 eps / sigma^2 2^-56 for r2min <= R2 < r2c.
-__device__ __forceinline__ long long fx_term(unsigned long long R2, const FxParams &k)
+// |F(r)| / r in units of 24 eps / sigma^2 2^-(58 + 4 cls) for r2min <= R2 <
+// r2c; cls: 0 repulsive, 1 attractive, 2 beyond 1.8 sigma.  u^2 is shifted up
+// by 2 cls bits (u^2 < 1.5, 0.631, 0.096), so that u^4 and the result keep 58 bits.
+__device__ __forceinline__ unsigned long long fx_term(unsigned long long R2, const FxParams &k, int &cls)
 {
     const int lz = __clzll((long long)R2);
     const unsigned long long M = R2 << lz;   // m = M 2^-64 in [1/2, 1)
@@ -135,17 +151,18 @@ __device__ __forceinline__ long long fx_term(unsigned long long R2, const FxPara
     const unsigned long long U = s >= 0 ? h << s : (s > -64 ? h >> -s : 0ull);   // u 2^63
     const unsigned long long U2 = __umul64hi(U, U);                              // 2^62
     const unsigned long long U3 = __umul64hi(U2, U);                             // 2^61
-    const unsigned long long U4 = __umul64hi(U2, U2);                            // 2^60
     const long long T = (long long)U3 - (1ll << 60);                             // (2 u^3 - 1) 2^60
-    return __mul64hi((long long)U4, T);
+    cls = R2 >= k.r2far ? 2 : T < 0 ? 1 : 0;
+    const unsigned long long V2 = U2 << (2 * cls);                               // 2^(62 + 2 cls)
+    const unsigned long long V4 = __umul64hi(V2, V2);                            // u^4 2^(60 + 4 cls)
+    return __umul64hi(V4, fx_abs(T)) << 2;
 }
 
-// The product's upper 64 bits, rounded towards zero: the same magnitude for d
-// and -d, so that a pair's force does not depend on which of the two is home.
-__device__ __forceinline__ long long fx_mul(long long t, long long d)
+// t a 2^-64, rounded to nearest at bit sh >= 1: in magnitude, so that a pair's
+// force does not depend on which of the two is home.
+__device__ __forceinline__ long long fx_mul(unsigned long long t, unsigned long long a, int sh)
 {
-    const long long h = __mul64hi(t, d);
-    return h + (long long)((unsigned long long)h >> 63);
+    return (long long)((__umul64hi(t, a) + (1ull << (sh - 1))) >> sh);
 }
 
 // Plain path: lanes own home particles, FP64 over the half stencil's slots
@@ -289,10 +306,18 @@ __device__ __forceinline__ void fx_pairs(const FxParams &k, long long *__restric
             if (q + step < P && off[q + step] <= lo) q += step;
         int nxt = off[q + 1];
         long long xp = X64[pb + q], yp = Y64[pb + q], zp = Z64[pb + q];
-        long long ax = 0, ay = 0, az = 0;
+        long long sx[3] = {0, 0, 0}, sy[3] = {0, 0, 0}, sz[3] = {0, 0, 0};   // per class
+        auto flush = [&](int i) {
+            unsigned long long *o = reinterpret_cast<unsigned long long *>(acc) + kFxAcc * (int64_t)i;
+            unsigned long long lo = 0;
+            fx_red(o, fx_split(sx[0], sx[1], sx[2], 0, lo));
+            fx_red(o + 1, fx_split(sy[0], sy[1], sy[2], kFxLow, lo));
+            fx_red(o + 2, fx_split(sz[0], sz[1], sz[2], 2 * kFxLow, lo));
+            fx_red(o + 9, (long long)lo);
+        };
         for (int e = lo; e < hi; e++) {
             if (e == nxt) {
-                fx_add(acc, iw[pb + q], ax, ay, az);
+                flush(iw[pb + q]);
                 do {
                     q++;
                     nxt = off[q + 1];
@@ -300,11 +325,13 @@ __device__ __forceinline__ void fx_pairs(const FxParams &k, long long *__restric
                 xp = X64[pb + q];
                 yp = Y64[pb + q];
                 zp = Z64[pb + q];
-                ax = ay = az = 0;
+#pragma unroll
+                for (int u = 0; u < 3; u++) sx[u] = sy[u] = sz[u] = 0;
             }
             const int j = list[e];
             const long long dx = xp - X64[j], dy = yp - Y64[j], dz = zp - Z64[j];
-            const unsigned long long R2 = fx_sq(dx) + fx_sq(dy) + fx_sq(dz);
+            const unsigned long long bx = fx_abs(dx), by = fx_abs(dy), bz = fx_abs(dz);
+            const unsigned long long R2 = __umul64hi(bx, bx) + __umul64hi(by, by) + __umul64hi(bz, bz);
             if (R2 >= k.r2c) continue;
             if (R2 < k.r2min) {   // too close for the fixed-point range
                 const double ex = (double)dx * k.to_d, ey = (double)dy * k.to_d, ez = (double)dz * k.to_d;
@@ -313,14 +340,28 @@ __device__ __forceinline__ void fx_pairs(const FxParams &k, long long *__restric
                 fx_add64(f, iw[j], nf * ex, nf * ey, nf * ez);
                 continue;
             }
-            const long long t = fx_term(R2, k) >> k.tsh;
-            const long long gx = fx_mul(t, dx), gy = fx_mul(t, dy), gz = fx_mul(t, dz);
-            ax += gx;
-            ay += gy;
-            az += gz;
-            fx_add(acc, iw[j], -gx, -gy, -gz);
+            int cls;
+            const unsigned long long t = fx_term(R2, k, cls);
+            const int sh = k.tsh + (cls == 1 ? 1 : 2);
+            long long gx = fx_mul(t, bx, sh), gy = fx_mul(t, by, sh), gz = fx_mul(t, bz, sh);
+            const long long at = cls == 0 ? 0 : -1;   // attractive: F against d
+            const long long mx = (dx >> 63) ^ at, my = (dy >> 63) ^ at, mz = (dz >> 63) ^ at;
+            gx = (gx ^ mx) - mx;
+            gy = (gy ^ my) - my;
+            gz = (gz ^ mz) - mz;
+            unsigned long long *o = reinterpret_cast<unsigned long long *>(acc) + (kFxAcc * (int64_t)iw[j] + 3 * cls);
+            fx_red(o, -gx);
+            fx_red(o + 1, -gy);
+            fx_red(o + 2, -gz);
+#pragma unroll
+            for (int u = 0; u < 3; u++)
+                if (cls == u) {
+                    sx[u] += gx;
+                    sy[u] += gy;
+                    sz[u] += gz;
+                }
         }
-        fx_add(acc, iw[pb + q], ax, ay, az);
+        flush(iw[pb + q]);
     }
     __syncwarp();   // list and off are rewritten by the next batch
 }
@@ -422,11 +463,13 @@ __global__ void __launch_bounds__(kFxThreads) k_force_fx(FxParams k, const longl
 
 int fx_shift(const lj_ctx *c) { return (int)floor(62.95 - log2(1.5 * c->cw)); }
 
-// acc counts 24 eps / sigma^2 2^-(S - 8 - tsh); tsh makes that 2^-52 / sigma
-// or more (the file header's range).
+// The first sums' unit is 24 eps / sigma^2 2^-(S - 8 - tsh); tsh makes that
+// 2^-52 24 eps / sigma at sigma = 1, and elsewhere so much that the range is
+// 2,040 to 4,080 of 24 eps / sigma (with rc <= 2.6 sigma S - 8 - tsh is never
+// below it: cells are less than 4/3 rc wide).
 static int fx_tsh(const lj_ctx *c)
 {
-    const int fb = (int)floor(63.0 - log2(1900.0 * c->p.sigma));
+    const int fb = (int)floor(63.0 - log2(2040.0 * c->p.sigma));
     const int t = fx_shift(c) - 8 - fb;
     return t > 0 ? t : 0;
 }
@@ -486,12 +529,14 @@ cudaError_t launch_force_fx(lj_ctx *c, double4_16a *f)
     k.tsh = fx_tsh(c);
     k.Lfix = lj_fix64(c->p.box, S);
     int ex = 0;
-    const double mant = frexp(sg * sg, &ex);
-    k.K = (unsigned long long)ldexp(mant, 64);
+    const double s2 = sg * sg, mant = frexp(s2, &ex);   // sigma^2 to 64 bits: the product and its rounding error
+    k.K = (unsigned long long)ldexp(mant, 64) + (unsigned long long)(long long)ldexp(fma(sg, sg, -s2), 64 - ex);
     k.kappa_e = ex + 2 * S - 129;
     k.r2c = (unsigned long long)ldexp(rc * rc, 2 * S - 64);
     const double rmin = ldexp(0.8 * sg * sg, 2 * S - 64);
     k.r2min = rmin < (double)k.r2c ? (unsigned long long)rmin : k.r2c;
+    const double rfar = ldexp(3.24 * sg * sg, 2 * S - 64);   // none beyond it if rc is not
+    k.r2far = rfar < (double)k.r2c ? (unsigned long long)rfar : ~0ull;
     k.to_d = ldexp(1.0, -S);
     const double s6 = sg * sg * sg * sg * sg * sg;
     k.rc2 = rc * rc;

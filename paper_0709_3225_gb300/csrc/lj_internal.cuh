@@ -136,7 +136,7 @@ struct lj_ctx {
     float4 *sg4;             // cotangents (lazily allocated)
     int32_t *onext;          // overflow lists: index + 1 of the next, 0 = end
     // FP64 contexts (lj_force_fx.cu): spos holds longlong4 (fixed-point
-    // coordinates, particle index), fx_acc the force sums, int64[4] per particle
+    // coordinates, particle index), fx_acc the force sums, int64[kFxAcc] per particle
     long long *fx_acc;
     int fx_cap, fx_smem, fx_grid;
     int slot_par;            // buffer of the next binning
@@ -172,6 +172,10 @@ struct lj_ctx {
     int64_t force_launches;
     int64_t kernel_launches;
 };
+
+// fx_acc's words per particle: x, y, z in units of q, of q / 32 and of q / 256,
+// then the home sums' lowest parts, in fields of kFxLow bits (units of q / 256).
+constexpr int kFxAcc = 10, kFxLow = 21;
 
 // x 2^S mod 2^64 for x >= 0, truncated (exact when x >= 2^(53-S)).
 __host__ __device__ __forceinline__ long long lj_fix64(double x, int S)
@@ -529,7 +533,7 @@ cudaError_t slots_begin(lj_ctx *c, int64_t i_begin);   // before a slotted binni
 cudaError_t lists_begin(lj_ctx *c);                    // before a binning into the sorted lists
 void slots_consumed(lj_ctx *c);                        // after the launch that reads it
 // FP64 contexts: the fixed-point kernel (lj_force_fx.cu) over slotted cells.
-// Its forces are f (the pairs taken in FP64) plus fx_scale times fx_acc:
+// Its forces are f (the pairs taken in FP64) plus fx_acc (fx_scale is q):
 // launch_kick_drift_fx reads both (with_acc) or f alone and zeroes them,
 // launch_fx_finish leaves the sum in f and with v adds the half kick.
 bool uses_fx(const lj_ctx *c);

@@ -180,16 +180,27 @@ __global__ void __launch_bounds__(kHostThreads) k_host_out(const double *__restr
 }
 
 // The FP64 forms (lj_force_fx.cu): fixed-point coordinates; f holds the
-// forces of the pairs taken in FP64 and acc, in units of 1 / scale, those of
-// all others.
-__device__ __forceinline__ void fx_force(const double4_16a *f, const longlong2 *acc, int i, double scale, double &fx,
+// forces of the pairs taken in FP64 and acc those of all others.  Their three
+// sums and the low part make one integer in units of q / 256, exactly, which
+// is then rounded once.
+__device__ __forceinline__ double fx_sum(long long r, long long m, long long f, unsigned long long lo, double q)
+{
+    const __int128 t = ((__int128)r << 8) + ((__int128)m << 3) + f + (long long)(lo & ((1ull << kFxLow) - 1));
+    const long long v = (long long)t;
+    if (t == v) return (double)v * (q * 0x1p-8);
+    return (double)(long long)(t >> 8) * q;
+}
+
+__device__ __forceinline__ void fx_force(const double4_16a *f, const longlong2 *acc, int i, double q, double &fx,
                                          double &fy, double &fz)
 {
-    const double4_16a q = f[i];
-    const longlong2 a = acc[2 * (int64_t)i], b = acc[2 * (int64_t)i + 1];
-    fx = fma((double)a.x, scale, q.x);
-    fy = fma((double)a.y, scale, q.y);
-    fz = fma((double)b.x, scale, q.z);
+    const double4_16a p = f[i];
+    const longlong2 *o = acc + kFxAcc / 2 * (int64_t)i;
+    const longlong2 a = o[0], b = o[1], c = o[2], d = o[3], e = o[4];
+    const unsigned long long lo = (unsigned long long)e.y;
+    fx = fx_sum(a.x, b.y, d.x, lo, q) + p.x;
+    fy = fx_sum(a.y, c.x, d.y, lo >> kFxLow, q) + p.y;
+    fz = fx_sum(b.x, c.y, e.x, lo >> (2 * kFxLow), q) + p.z;
 }
 
 __device__ __forceinline__ void fx_zero(double4_16a *f, longlong2 *acc, int i)
@@ -197,7 +208,8 @@ __device__ __forceinline__ void fx_zero(double4_16a *f, longlong2 *acc, int i)
     double4_16a z;
     z.x = z.y = z.z = z.w = 0.0;
     f[i] = z;
-    acc[2 * (int64_t)i] = acc[2 * (int64_t)i + 1] = make_longlong2(0, 0);
+#pragma unroll
+    for (int u = 0; u < kFxAcc / 2; u++) acc[kFxAcc / 2 * (int64_t)i + u] = make_longlong2(0, 0);
 }
 
 __global__ void __launch_bounds__(256) k_bin_fx(SlotBin b, const double *__restrict__ x, int n, double4_16a *__restrict__ f,
@@ -409,7 +421,7 @@ cudaError_t slots_setup(lj_ctx *c)
     if (e == cudaSuccess) e = cudaMemsetAsync(c->octr, 0xff, 4 * sizeof(unsigned), c->stream);
     if (e == cudaSuccess)
         e = cudaMalloc(&c->spos, (size_t)(nslots + c->p.n) * (fp64 ? sizeof(longlong4_16a) : sizeof(float4)));
-    if (e == cudaSuccess && fp64) e = cudaMalloc(&c->fx_acc, (size_t)c->p.n * 4 * sizeof(long long));
+    if (e == cudaSuccess && fp64) e = cudaMalloc(&c->fx_acc, (size_t)c->p.n * kFxAcc * sizeof(long long));
     if (e == cudaSuccess) e = cudaMalloc(&c->onext, (size_t)c->p.n * sizeof(int32_t));
     if (e == cudaErrorMemoryAllocation) {   // the sorted lists need less
         cudaGetLastError();
@@ -439,14 +451,12 @@ bool uses_slots(const lj_ctx *c)
     return c->scap > 0 && c->skin <= 0.0 && !c->fuse_update && uses_force_n3(c) && slots_suit(c);
 }
 
-// The fixed-point term's error is below FP64's while rc <= 5 sigma (measured
-// against 113 bits: 2.7e-15 against 1.4e-14, in units of 24 eps / sigma^2, at
-// 2.5 and 3, 1.1e-14 against 1.3e-14 at 5, 4.2e-14 against 1.2e-14 at 10:
-// r^2 is held in units of rc^2 2^-60).
+// The fixed-point forces are the more exact ones, pair by pair, while rc <=
+// 2.6 sigma (the file header of lj_force_fx.cu has the errors).
 bool uses_fx(const lj_ctx *c)
 {
-    return c->scap > 0 && c->p.rc <= 4.0 * c->p.sigma && c->skin <= 0.0 && c->p.precision == LJ_PREC_FP64 && c->n3 && !c->deterministic &&
-           !c->use_run_kernel && !c->use_aop && slots_suit(c);
+    return c->scap > 0 && c->p.rc <= 2.6 * c->p.sigma && c->skin <= 0.0 && c->p.precision == LJ_PREC_FP64 && c->n3 &&
+           !c->deterministic && !c->use_run_kernel && !c->use_aop && slots_suit(c);
 }
 
 cudaError_t launch_bin_fx(lj_ctx *c, const double *x, double4_16a *f)
