@@ -413,9 +413,9 @@ struct BatchSlots {
 // Bound by HBM and the latency of the replica's fields: 48 registers, for 5
 // blocks per SM (56 and 4 without the bound: a step 319 -> 316 us).
 template <int OP>
-__global__ void __launch_bounds__(256, 5) k_batch_slots(BatchSlots a, double *__restrict__ x, double *__restrict__ v,
-                                                     float4 *__restrict__ f, int n, double hk, double dt,
-                                                     int32_t *__restrict__ err)
+__global__ void __launch_bounds__(256, 5) k_batch_slots(BatchSlots a, double *x, double *v,
+                                                     float4 *f, int n, double hk, double dt,
+                                                     int32_t *err)
 {
     pdl_wait();
     const int i = (gridDim.x - 1 - blockIdx.x) * blockDim.x + threadIdx.x;   // as k_kick_drift_slots
@@ -473,7 +473,7 @@ __global__ void __launch_bounds__(256, 5) k_batch_slots(BatchSlots a, double *__
 // k_force_n3 with each cell's replica looked up (one cell ahead, as the
 // cell's own table loads).  The energies go to f.w alone.
 template <int MODE, bool ENERGY>
-__global__ void __launch_bounds__(kN3Threads, ENERGY ? 4 : 6) k_batch_force_n3(WarpParams k, BatchSlots a, float4 *__restrict__ f)
+__global__ void __launch_bounds__(kN3Threads, ENERGY ? 4 : 6) k_batch_force_n3(WarpParams k, BatchSlots a, float4 *f)
 {
     extern __shared__ __align__(16) float nsmem[];
     const int lane = threadIdx.x & 31;
@@ -519,7 +519,7 @@ __global__ void __launch_bounds__(kN3Threads, ENERGY ? 4 : 6) k_batch_force_n3(W
             const Cell cur = nxt;
             if (c + 1 < c1) nxt = load(c + 1);
             if (lane == 31) k.cellq_next[c] = make_int2(0, 0);
-            n3_cell<MODE, ENERGY, true, true, false>(k, pos, f, cur.t, c - cur.cell0, cur.cell0,
+            n3_cell<MODE, ENERGY, false, true, false>(k, pos, f, cur.t, c - cur.cell0, cur.cell0,
                                                      __float_as_int(cur.g.w), cur.g.y, 0, 0, cur.g.x, S, stab, spre, H,
                                                      eacc, wacc);
         }
@@ -539,7 +539,7 @@ void *batch_slots_kernel(int mode, bool energy)
 }
 
 // Closing half kick of the last step: v += h f.
-__global__ void k_batch_kick(double *__restrict__ v, const float4 *__restrict__ f, int64_t n, double h)
+__global__ void k_batch_kick(double *v, const float4 *f, int64_t n, double h)
 {
     pdl_wait();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;

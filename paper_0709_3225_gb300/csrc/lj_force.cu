@@ -348,8 +348,8 @@ __global__ void k_wait_selftest(int32_t *err)
 // result is for the host: out and host_err are pinned memory, written here in
 // place of two copies and the synchronization between them (an energy call at
 // 2,048 particles 41 -> 25 us).
-__global__ void k_reduce_pairs(const double *__restrict__ partial, int n, double *__restrict__ out,
-                               const int32_t *__restrict__ err, int32_t *__restrict__ host_err)
+__global__ void k_reduce_pairs(const double *partial, int n, double *out,
+                               const int32_t *err, int32_t *host_err)
 {
     pdl_wait();
     __shared__ double se[kReduceThreads], sw[kReduceThreads];

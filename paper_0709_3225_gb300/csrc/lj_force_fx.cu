@@ -167,7 +167,7 @@ __device__ __forceinline__ long long fx_mul(unsigned long long t, unsigned long 
 
 // Plain path: lanes own home particles, FP64 over the half stencil's slots
 // and overflow lists.
-__device__ void fx_plain(const FxParams &k, const longlong4_16a *__restrict__ pos, double4_16a *__restrict__ f,
+__device__ void fx_plain(const FxParams &k, const longlong4_16a *pos, double4_16a *f,
                          const long long *sh, const int *st, const int *spre, int c, int n_home)
 {
     const int lane = threadIdx.x & 31;
@@ -176,8 +176,8 @@ __device__ void fx_plain(const FxParams &k, const longlong4_16a *__restrict__ po
         const bool vi = i < n_home;
         int si = st[0] + (vi ? i : 0);
         if (vi && i >= k.scap) {
-            int o = __ldg(&k.cellq[c].y);
-            for (int m = k.scap; m < i && o > 0; m++) o = __ldg(k.onext + o - 1);
+            int o = k.cellq[c].y;
+            for (int m = k.scap; m < i && o > 0; m++) o = k.onext[o - 1];
             if (o > 0) si = k.nslots + o - 1;
         }
         const longlong4_16a pi = pos[si];
@@ -191,7 +191,7 @@ __device__ void fx_plain(const FxParams &k, const longlong4_16a *__restrict__ po
             for (int j = 0; j < nn; j++) {
                 int sj = st[kk] + j;
                 if (j >= k.scap) {
-                    o = j == k.scap ? __ldg(&k.cellq[half_cell(c, kk, k.nc, k.inv_nc)].y) : __ldg(k.onext + o - 1);
+                    o = j == k.scap ? k.cellq[half_cell(c, kk, k.nc, k.inv_nc)].y : k.onext[o - 1];
                     if (o <= 0) break;
                     sj = k.nslots + o - 1;
                 }
@@ -215,7 +215,7 @@ __device__ void fx_plain(const FxParams &k, const longlong4_16a *__restrict__ po
 // Staging: the half stencil's candidates within rc of the home box, home
 // particles first; returns their number, or -1 when they and 64 entries of
 // padding would not fit.
-__device__ __forceinline__ int fx_stage(const FxParams &k, const longlong4_16a *__restrict__ pos, long long *X64,
+__device__ __forceinline__ int fx_stage(const FxParams &k, const longlong4_16a *pos, long long *X64,
                                         float *X, int *iw, const long long *sh, const int *st, const int *spre, int tot,
                                         int n_home)
 {
@@ -245,8 +245,8 @@ __device__ __forceinline__ int fx_stage(const FxParams &k, const longlong4_16a *
             const int kb = __shfl_sync(0xffffffffu, s_e, kc);
             kcs[u] = kc;
             const longlong2 *p = reinterpret_cast<const longlong2 *>(pos + min(st[kc] + (t - kb), k.last));
-            qa[u] = __ldg(p);
-            qb[u] = __ldg(p + 1);
+            qa[u] = p[0];
+            qb[u] = p[1];
         }
 #pragma unroll
         for (int u = 0; u < kB; u++) {
@@ -292,7 +292,7 @@ __device__ __forceinline__ int fx_stage(const FxParams &k, const longlong4_16a *
 
 // Phase B over one batch: the entries [0, E) of the list, home particles pb
 // .. pb + P - 1; every lane takes an equal contiguous range.
-__device__ __forceinline__ void fx_pairs(const FxParams &k, long long *__restrict__ acc, double4_16a *__restrict__ f,
+__device__ __forceinline__ void fx_pairs(const FxParams &k, long long *acc, double4_16a *f,
                                          const long long *X64, const int *iw, const uint16_t *list, const int *off,
                                          int E, int P, int pb)
 {
@@ -366,8 +366,8 @@ __device__ __forceinline__ void fx_pairs(const FxParams &k, long long *__restric
     __syncwarp();   // list and off are rewritten by the next batch
 }
 
-__global__ void __launch_bounds__(kFxThreads) k_force_fx(FxParams k, const longlong4_16a *__restrict__ pos,
-                                                         long long *__restrict__ acc, double4_16a *__restrict__ f)
+__global__ void __launch_bounds__(kFxThreads) k_force_fx(FxParams k, const longlong4_16a *pos,
+                                                         long long *acc, double4_16a *f)
 {
     extern __shared__ __align__(16) unsigned char fxsmem[];
     const int lane = threadIdx.x & 31;

@@ -9,9 +9,9 @@ namespace {
 // SLOTS: slotted cells (start unused); the launch also zeroes the next
 // binning's counts.  SPLIT: each cell is 2^k.lgw items.
 template <int MODE, bool ENERGY, bool SLOTS, bool SPLIT>
-__global__ void __launch_bounds__(kN3Threads, ENERGY ? 4 : 6) k_force_n3(WarpParams k, const float4 *__restrict__ pos,
-                                                         const int32_t *__restrict__ start, float4 *__restrict__ fout,
-                                                         double *__restrict__ partial)
+__global__ void __launch_bounds__(kN3Threads, ENERGY ? 4 : 6) k_force_n3(WarpParams k, const float4 *pos,
+                                                         const int32_t *start, float4 *fout,
+                                                         double *partial)
 {
     extern __shared__ __align__(16) float nsmem[];
     const int lane = threadIdx.x & 31;
@@ -34,7 +34,7 @@ __global__ void __launch_bounds__(kN3Threads, ENERGY ? 4 : 6) k_force_n3(WarpPar
     auto load = [&](int c) { return half_load<true, SLOTS>(start, c, nc, k.inv_nc, 0, k.scap); };
     auto one_cell = [&](HalfLoad tl, int c, int part) {
         if (SLOTS && lane == 31 && part == 0) k.cellq_next[c] = make_int2(0, 0);
-        n3_cell<MODE, ENERGY, true, SLOTS, SPLIT>(k, pos, fout, tl, c, 0, nc, k.inv_nc, part, k.lgw, k.cw, S, stab, spre, H,
+        n3_cell<MODE, ENERGY, !SLOTS, SLOTS, SPLIT>(k, pos, fout, tl, c, 0, nc, k.inv_nc, part, k.lgw, k.cw, S, stab, spre, H,
                                                   eacc, wacc);
     };
     if constexpr (SPLIT) {

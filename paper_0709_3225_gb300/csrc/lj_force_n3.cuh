@@ -111,7 +111,7 @@ __device__ __forceinline__ int half_cell(int c, int e, int nc, float inv_nc)
 }
 
 template <bool NC, bool SLOTS = false>
-__device__ __forceinline__ HalfLoad half_load(const int32_t *__restrict__ start, int c, int nc, float inv_nc,
+__device__ __forceinline__ HalfLoad half_load(const int32_t *start, int c, int nc, float inv_nc,
                                               int cell_base = 0, int scap = 0)
 {
     const int lane = threadIdx.x & 31;
@@ -120,7 +120,7 @@ __device__ __forceinline__ HalfLoad half_load(const int32_t *__restrict__ start,
         const int cn = cell_base + half_cell(c, lane, nc, inv_nc);
         if constexpr (SLOTS) {
             t.s = cn * scap;
-            t.e = t.s + __ldg(reinterpret_cast<const int2 *>(start) + cn).x;
+            t.e = t.s + (reinterpret_cast<const int2 *>(start) + cn)->x;
         } else if constexpr (NC) {
             t.s = __ldg(start + cn);
             t.e = __ldg(start + cn + 1);
@@ -266,7 +266,7 @@ __device__ __forceinline__ float4 n3_ld4(const float4 *p)
 // pairs (0, 1) and (2, 3), one float4 each, then a float4 of padding so
 // that the groups' simultaneous reads fall in different banks.
 template <int NH, int LGB, int MODE, bool ENERGY, bool SELF>
-__device__ __forceinline__ void n3_block1(const WarpParams &k, float4 *__restrict__ fout, const float4 *S, int T, int j0,
+__device__ __forceinline__ void n3_block1(const WarpParams &k, float4 *fout, const float4 *S, int T, int j0,
                                           int a, int b, int A, const float4 *H, float2 *fx, float2 *fy, float2 *fz,
                                           float2 *fe, float2 &fw)
 {
@@ -302,7 +302,7 @@ __device__ __forceinline__ void n3_block1(const WarpParams &k, float4 *__restric
 }
 
 template <int NH, int LGB, int MODE, bool ENERGY>
-__device__ __forceinline__ void n3_blocks(const WarpParams &k, float4 *__restrict__ fout, const float4 *S, int T,
+__device__ __forceinline__ void n3_blocks(const WarpParams &k, float4 *fout, const float4 *S, int T,
                                           int jbeg, int n_home, int a, int b, int A, const float4 *H, float2 *fx, float2 *fy,
                                           float2 *fz, float2 *fe, float2 &fw)
 {
@@ -325,7 +325,7 @@ __device__ __forceinline__ void n3_blocks(const WarpParams &k, float4 *__restric
 // reuses S once the candidate blocks are done (S holds >= kN3Home * 32).
 // jbeg: the first candidate, 0, or n_home for a part without the home pairs.
 template <int MODE, bool ENERGY>
-__device__ __forceinline__ void n3_compute(const WarpParams &k, float4 *__restrict__ fout, float4 *S, float4 *H,
+__device__ __forceinline__ void n3_compute(const WarpParams &k, float4 *fout, float4 *S, float4 *H,
                                            int T, int jbeg, int n_home, double &eacc, double &wacc)
 {
     const int lane = threadIdx.x & 31;
@@ -411,7 +411,7 @@ __device__ __forceinline__ void n3_compute(const WarpParams &k, float4 *__restri
 // too, first).  n_home <= 32.  Returns false, having computed nothing, when
 // the kept candidates would not fit the slice.  SPLIT: ta may be above 0.
 template <bool NC, bool SPLIT>
-__device__ __forceinline__ bool n3_stage(const WarpParams &k, const float4 *__restrict__ pos, float4 *S,
+__device__ __forceinline__ bool n3_stage(const WarpParams &k, const float4 *pos, float4 *S,
                                          const float4 *stab, const int *spre, int ta, int tb_end, int s_home,
                                          int n_home, int &T_out)
 {
@@ -510,7 +510,7 @@ __device__ __forceinline__ bool n3_stage(const WarpParams &k, const float4 *__re
 // memory (all lanes the same one; the slots, then the cell's overflow list),
 // reactions summed over the warp.
 template <int MODE, bool ENERGY, bool NC, bool SLOTS, bool SPLIT>
-__device__ void n3_plain(const WarpParams &k, const float4 *__restrict__ pos, float4 *__restrict__ fout,
+__device__ void n3_plain(const WarpParams &k, const float4 *pos, float4 *fout,
                          const float4 *stab, const int *spre, int c, int cell0, int nc, float inv_nc, int ta,
                          int tb_end, int s_home, int n_home, double &eacc, double &wacc)
 {
@@ -520,8 +520,8 @@ __device__ void n3_plain(const WarpParams &k, const float4 *__restrict__ pos, fl
         const bool vi = i < n_home;
         int si = s_home + (vi ? i : 0);
         if (SLOTS && vi && i >= k.scap) {   // the (i - scap)-th of the home cell's overflow list
-            int o = __ldg(&k.cellq[cell0 + c].y);
-            for (int m = k.scap; m < i && o > 0; m++) o = __ldg(k.onext + o - 1);
+            int o = k.cellq[cell0 + c].y;
+            for (int m = k.scap; m < i && o > 0; m++) o = k.onext[o - 1];
             if (o > 0) si = k.nslots + o - 1;   // (a list shorter than its count: only with its error latched)
         }
         const float4 pi = load_pos<NC>(pos + si);
@@ -535,7 +535,7 @@ __device__ void n3_plain(const WarpParams &k, const float4 *__restrict__ pos, fl
             for (int j = (kk == 0 && !SLOTS ? p0 + 1 : 0); j < nn; j++) {
                 int sj = s + j;
                 if (SLOTS && j >= k.scap) {
-                    o = j == k.scap ? __ldg(&k.cellq[cell0 + half_cell(c, kk, nc, inv_nc)].y) : __ldg(k.onext + o - 1);
+                    o = j == k.scap ? k.cellq[cell0 + half_cell(c, kk, nc, inv_nc)].y : k.onext[o - 1];
                     if (o <= 0) break;
                     sj = k.nslots + o - 1;
                 }
@@ -592,14 +592,15 @@ __device__ void n3_plain(const WarpParams &k, const float4 *__restrict__ pos, fl
 // particles or whose pruned half stencil does not fit the slice (S, stab,
 // spre, H: the warp's slice).  cw: the
 // cell side of the cell's grid.  NC: read-only loads of the sorted
-// positions (not when an earlier phase of the same launch writes them).
+// positions (not when an earlier phase of the same launch writes them, nor in
+// a dependent launch, pdl_wait).
 // SLOTS: slotted cells; c: the cell's id in its grid of nc^3 cells, whose ids
 // start at cell0.  part of 2^lgw: the cell's
 // candidates are split evenly over 2^lgw warps (0 of 1: the whole cell),
 // part 0 with the home pairs; every part stages the home particles and adds
 // its share of their forces (SPLIT; otherwise whole cells only).
 template <int MODE, bool ENERGY, bool NC, bool SLOTS, bool SPLIT>
-__device__ __forceinline__ void n3_cell(const WarpParams &k, const float4 *__restrict__ pos, float4 *__restrict__ fout,
+__device__ __forceinline__ void n3_cell(const WarpParams &k, const float4 *pos, float4 *fout,
                                         HalfLoad tl, int c, int cell0, int nc, float inv_nc, int part, int lgw,
                                         float cw, float4 *S, float4 *stab, int *spre, float4 *H, double &eacc,
                                         double &wacc)

@@ -8,7 +8,7 @@
 namespace {
 
 template <typename F4>
-__device__ __forceinline__ void load_f(const F4 *__restrict__ f, int i, double &fx, double &fy, double &fz)
+__device__ __forceinline__ void load_f(const F4 *f, int i, double &fx, double &fy, double &fz)
 {
     F4 q = f[i];
     if constexpr (sizeof(q.x) == 4) {
@@ -157,7 +157,7 @@ __global__ void k_skin_decide(int32_t *flags, long long *counts, float thr2, int
 }
 
 template <typename F4>
-__global__ void k_kick(double *__restrict__ v, const F4 *__restrict__ f, int n, double h)
+__global__ void k_kick(double *v, const F4 *f, int n, double h)
 {
     pdl_wait();
     int i = blockIdx.x * blockDim.x + threadIdx.x;

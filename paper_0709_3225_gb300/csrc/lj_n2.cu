@@ -271,8 +271,8 @@ __device__ __forceinline__ float2 n2_r2(float2 xi, float2 yi, float2 zi, float2 
 // -> 27 us, 120 -> 40 at 16,000); where the order is random the boxes fill the
 // system and the test's cost does not show (46 us).
 template <int MODE, bool ENERGY>
-__global__ void __launch_bounds__(kN2Threads) k_n2_force_f32(N2Params p, int npad, int tile, const float *__restrict__ soa,
-                                                             float4 *__restrict__ part, double *__restrict__ epart,
+__global__ void __launch_bounds__(kN2Threads) k_n2_force_f32(N2Params p, int npad, int tile, const float *soa,
+                                                             float4 *part, double *epart,
                                                              int32_t *err)
 {
     __shared__ __align__(128) float sm[2][3][kN2TileF];
@@ -398,8 +398,8 @@ __global__ void __launch_bounds__(kN2Threads) k_n2_force_f32(N2Params p, int npa
 constexpr int kN2SumThreads = 64;
 
 template <typename T>
-__global__ void __launch_bounds__(kN2SumThreads) k_n2_sum(const typename Vec4<T>::type *__restrict__ part, int nsplit, int n,
-                         typename Vec4<T>::type *__restrict__ f)
+__global__ void __launch_bounds__(kN2SumThreads) k_n2_sum(const typename Vec4<T>::type *part, int nsplit, int n,
+                         typename Vec4<T>::type *f)
 {
     pdl_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;

@@ -118,7 +118,7 @@ __global__ void __launch_bounds__(kR48Threads) k_r48_gen(uint64_t *__restrict__ 
 }
 
 // state_i -> state_i after all R rounds, (A, C) being their map.
-__global__ void __launch_bounds__(kR48Threads) k_r48_advance(uint64_t *__restrict__ state, int64_t S, uint64_t A,
+__global__ void __launch_bounds__(kR48Threads) k_r48_advance(uint64_t *state, int64_t S, uint64_t A,
                                                              uint64_t C)
 {
     pdl_wait();
@@ -156,9 +156,9 @@ __device__ __forceinline__ void box_muller(uint64_t a, uint64_t b, T &z0, T &z1)
 // One BAOAB update of particle i, random numbers included: x, v and the
 // stream advance, the wrapped position is returned in p.
 template <typename F4, typename T>
-__device__ __forceinline__ void baoab(double *__restrict__ x, double *__restrict__ v, F4 q, int i, double hk, double hdt,
+__device__ __forceinline__ void baoab(double *x, double *v, F4 q, int i, double hk, double hdt,
                                       double c1, double c2s, double L, double whi, double wlo,
-                                      uint64_t *__restrict__ state, uint64_t A, uint64_t C, double *p)
+                                      uint64_t *state, uint64_t A, uint64_t C, double *p)
 {
     // four series elements of this particle for this step
     const uint64_t u0 = state[i];
@@ -234,10 +234,10 @@ __global__ void k_langevin_bin(double *__restrict__ x, double *__restrict__ v, c
 
 // The same update with the slotted binning (lj_slots.cuh); f is zeroed for
 // the force kernel, which adds into it.
-__global__ void __launch_bounds__(256) k_langevin_slots(SlotBin b, double *__restrict__ x, double *__restrict__ v,
-                                                        float4 *__restrict__ f, int n, double hk, double hdt, double c1,
-                                                        double c2s, uint64_t *__restrict__ state, uint64_t A, uint64_t C,
-                                                        int32_t *__restrict__ err)
+__global__ void __launch_bounds__(256) k_langevin_slots(SlotBin b, double *x, double *v,
+                                                        float4 *f, int n, double hk, double hdt, double c1,
+                                                        double c2s, uint64_t *state, uint64_t A, uint64_t C,
+                                                        int32_t *err)
 {
     pdl_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;

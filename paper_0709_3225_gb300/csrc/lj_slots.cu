@@ -46,8 +46,8 @@ __global__ void __launch_bounds__(256) k_bin_slots(SlotBin b, const double *__re
 // 4M, 57 -> 40 at 131,072, 26 -> 16.5 at 2,048.
 // xo: where the new positions go, x itself or the next state of a trajectory.
 __global__ void __launch_bounds__(256) k_kick_drift_slots(SlotBin b, const double *x, double *xo,
-                                                          double *__restrict__ v, float4 *__restrict__ f, int i_begin,
-                                                          int n, double hk, double dt, int32_t *__restrict__ err)
+                                                          double *v, float4 *f, int i_begin,
+                                                          int n, double hk, double dt, int32_t *err)
 {
     pdl_wait();
     // the last particles first: what this kernel wrote last, and the force
@@ -151,11 +151,11 @@ __global__ void __launch_bounds__(kHostThreads) k_host_in(SlotBin b, const doubl
 
 // The closing half kick v += h f into the host arrays, with f (and x, if hx)
 // and the latched errors.
-__global__ void __launch_bounds__(kHostThreads) k_host_out(const double *__restrict__ x, const double *__restrict__ v,
-                                                           const float4 *__restrict__ f, int n, double h,
-                                                           double *__restrict__ hx, double *__restrict__ hv,
-                                                           float4 *__restrict__ hf, const int32_t *__restrict__ err,
-                                                           int32_t *__restrict__ host_err)
+__global__ void __launch_bounds__(kHostThreads) k_host_out(const double *x, const double *v,
+                                                           const float4 *f, int n, double h,
+                                                           double *hx, double *hv,
+                                                           float4 *hf, const int32_t *err,
+                                                           int32_t *host_err)
 {
     __shared__ double2 s[3 * kHostThreads / 2];
     pdl_wait();
@@ -230,10 +230,10 @@ __global__ void __launch_bounds__(256) k_bin_fx(SlotBin b, const double *__restr
 }
 
 // k_kick_drift_slots in FP64; with_acc: f alone is not yet the force.
-__global__ void __launch_bounds__(256) k_kick_drift_fx(SlotBin b, double *__restrict__ x, double *__restrict__ v,
-                                                       double4_16a *__restrict__ f, longlong2 *__restrict__ acc,
+__global__ void __launch_bounds__(256) k_kick_drift_fx(SlotBin b, double *x, double *v,
+                                                       double4_16a *f, longlong2 *acc,
                                                        int with_acc, double scale, int i_begin, int n, double hk,
-                                                       double dt, int32_t *__restrict__ err)
+                                                       double dt, int32_t *err)
 {
     pdl_wait();
     const int t = (gridDim.x - 1 - blockIdx.x) * blockDim.x + threadIdx.x;
@@ -270,8 +270,8 @@ __global__ void __launch_bounds__(256) k_kick_drift_fx(SlotBin b, double *__rest
 }
 
 // f := the force; with v also the closing half kick v += h f.
-__global__ void __launch_bounds__(256) k_fx_finish(double *__restrict__ v, double4_16a *__restrict__ f,
-                                                   const longlong2 *__restrict__ acc, int n, double scale, double h)
+__global__ void __launch_bounds__(256) k_fx_finish(double *v, double4_16a *f,
+                                                   const longlong2 *acc, int n, double scale, double h)
 {
     pdl_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;

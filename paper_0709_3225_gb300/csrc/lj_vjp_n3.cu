@@ -60,8 +60,8 @@ __host__ __device__ constexpr int vn3_slice_words(int cap) { return 8 * cap + 4 
 // Staging as n3_stage (lj_force_n3.cuh) with the cotangents copied along,
 // and the slice checked per round.  Returns false when the kept candidates
 // would not fit.
-__device__ __forceinline__ bool vn3_stage(const VjpN3Coef &k, const float4 *__restrict__ pos,
-                                          const float4 *__restrict__ g4, float4 *S, float4 *SG, const float4 *stab,
+__device__ __forceinline__ bool vn3_stage(const VjpN3Coef &k, const float4 *pos,
+                                          const float4 *g4, float4 *S, float4 *SG, const float4 *stab,
                                           const int *spre, int Ttot, int n_home, int &T_out)
 {
     const int lane = threadIdx.x & 31;
@@ -93,8 +93,8 @@ __device__ __forceinline__ bool vn3_stage(const VjpN3Coef &k, const float4 *__re
             const int kb = __shfl_sync(0xffffffffu, s_e, kc);
             sh[u] = stab[kc];
             const int idx = min(__float_as_int(sh[u].w) + (t - kb), last);
-            q[u] = __ldg(pos + idx);
-            qg[u] = __ldg(g4 + idx);
+            q[u] = pos[idx];
+            qg[u] = g4[idx];
         }
         if (t0 == 0) {   // the home particles are candidates 0 .. n_home-1 of the first round
             if (lane < n_home) {
@@ -220,7 +220,7 @@ __device__ __forceinline__ void vn3_pair2(float2 hx, float2 hy, float2 hz, float
 // the z of pairs (0, 1) and (2, 3), then the same for the cotangents, and a
 // float4 of padding.
 template <int NH, int LGB, int MODE, bool SELF>
-__device__ __forceinline__ void vn3_block(const VjpN3Coef &k, float4 *__restrict__ acc, const float4 *S,
+__device__ __forceinline__ void vn3_block(const VjpN3Coef &k, float4 *acc, const float4 *S,
                                           const float4 *SG, int T, int blk, int a, int b, int A, const float4 *H,
                                           float2 *ax, float2 *ay, float2 *az, float2 &te, float2 &ts)
 {
@@ -263,7 +263,7 @@ __device__ __forceinline__ void vn3_block(const VjpN3Coef &k, float4 *__restrict
 }
 
 template <int NH, int LGB, int MODE>
-__device__ __forceinline__ void vn3_blocks(const VjpN3Coef &k, float4 *__restrict__ acc, const float4 *S,
+__device__ __forceinline__ void vn3_blocks(const VjpN3Coef &k, float4 *acc, const float4 *S,
                                            const float4 *SG, int T, int n_home, int a, int b, int A, const float4 *H,
                                            float2 *ax, float2 *ay, float2 *az, float2 &te, float2 &ts)
 {
@@ -278,7 +278,7 @@ __device__ __forceinline__ void vn3_blocks(const VjpN3Coef &k, float4 *__restric
 // Compute phase of a staged cell of n_home <= 32 home particles (S holds at
 // least kN3Home * 32 slots, reused for the transpose of the home sums).
 template <int MODE>
-__device__ __forceinline__ void vn3_compute(const VjpN3Coef &k, float4 *__restrict__ acc, float4 *S,
+__device__ __forceinline__ void vn3_compute(const VjpN3Coef &k, float4 *acc, float4 *S,
                                             const float4 *SG, float4 *H, int T, int n_home, double &acc_e,
                                             double &acc_s)
 {
@@ -361,8 +361,8 @@ __device__ __forceinline__ void vn3_compute(const VjpN3Coef &k, float4 *__restri
 // from global memory (all lanes the same one; with SLOTS the slots, then the
 // cell's overflow list, as n3_plain), reactions summed over the warp.
 template <int MODE, bool SLOTS>
-__device__ void vn3_plain(const VjpN3Coef &k, const float4 *__restrict__ pos, const float4 *__restrict__ g4,
-                          float4 *__restrict__ acc, const float4 *stab, const int *spre, int c, int s_home, int n_home,
+__device__ void vn3_plain(const VjpN3Coef &k, const float4 *pos, const float4 *g4,
+                          float4 *acc, const float4 *stab, const int *spre, int c, int s_home, int n_home,
                           double &acc_e, double &acc_s)
 {
     const int lane = threadIdx.x & 31;
@@ -371,12 +371,12 @@ __device__ void vn3_plain(const VjpN3Coef &k, const float4 *__restrict__ pos, co
         const bool vi = i < n_home;
         int si = s_home + (vi ? i : 0);
         if (SLOTS && vi && i >= k.scap) {
-            int o = __ldg(&k.cellq[c].y);
-            for (int m = k.scap; m < i && o > 0; m++) o = __ldg(k.onext + o - 1);
+            int o = k.cellq[c].y;
+            for (int m = k.scap; m < i && o > 0; m++) o = k.onext[o - 1];
             if (o > 0) si = k.nslots + o - 1;
         }
-        const float4 pi = __ldg(pos + si);
-        const float4 gi = __ldg(g4 + si);
+        const float4 pi = pos[si];
+        const float4 gi = g4[si];
         float2 ax = f2(0.f), ay = f2(0.f), az = f2(0.f), te = f2(0.f), ts = f2(0.f);
         for (int kk = 0; kk < kN3Half; kk++) {
             const float4 sh = stab[kk];
@@ -386,12 +386,12 @@ __device__ void vn3_plain(const VjpN3Coef &k, const float4 *__restrict__ pos, co
             for (int j = (kk == 0 && !SLOTS ? p0 + 1 : 0); j < nn; j++) {
                 int sj = s + j;
                 if (SLOTS && j >= k.scap) {
-                    o = j == k.scap ? __ldg(&k.cellq[half_cell(c, kk, k.nc, k.inv_nc)].y) : __ldg(k.onext + o - 1);
+                    o = j == k.scap ? k.cellq[half_cell(c, kk, k.nc, k.inv_nc)].y : k.onext[o - 1];
                     if (o <= 0) break;
                     sj = k.nslots + o - 1;
                 }
-                const float4 q = __ldg(pos + sj);
-                const float4 h = __ldg(g4 + sj);
+                const float4 q = pos[sj];
+                const float4 h = g4[sj];
                 float2 rx = f2(0.f), ry = f2(0.f), rz = f2(0.f);
                 // slot y is a far dummy; home pairs count for j > i only
                 vn3_pair2<MODE, true>(make_float2(pi.x, -kFar), make_float2(pi.y, -kFar), make_float2(pi.z, -kFar),
@@ -417,10 +417,10 @@ __device__ void vn3_plain(const VjpN3Coef &k, const float4 *__restrict__ pos, co
 }
 
 template <int MODE, bool SLOTS>
-__global__ void __launch_bounds__(kVn3Threads, 4) k_vjp_n3(VjpN3Coef k, const float4 *__restrict__ pos,
-                                                         const float4 *__restrict__ g4,
-                                                         const int32_t *__restrict__ start, float4 *__restrict__ acc,
-                                                         double *__restrict__ partial)
+__global__ void __launch_bounds__(kVn3Threads, 4) k_vjp_n3(VjpN3Coef k, const float4 *pos,
+                                                         const float4 *g4,
+                                                         const int32_t *start, float4 *acc,
+                                                         double *partial)
 {
     extern __shared__ __align__(16) float vsm[];
     const int lane = threadIdx.x & 31;
@@ -497,12 +497,12 @@ __global__ void __launch_bounds__(kVn3Threads, 4) k_vjp_n3(VjpN3Coef k, const fl
 // for what were three: at 32,000 particles each took 3 to 6 us.  BIN: the
 // binning of x, for the VJP of lam that follows (k_bin_slots), as well.
 template <bool BIN>
-__global__ void __launch_bounds__(kReduceThreads) k_vjp_finish(float4 *__restrict__ acc, int n, double scale,
-                                                               double *__restrict__ dx, double *__restrict__ lam,
-                                                               double a, const double *__restrict__ partial, int np,
-                                                               double *__restrict__ dparam, SlotBin b,
-                                                               const double *__restrict__ x, float4 *__restrict__ g4,
-                                                               int32_t *__restrict__ err)
+__global__ void __launch_bounds__(kReduceThreads) k_vjp_finish(float4 *acc, int n, double scale,
+                                                               double *dx, double *lam,
+                                                               double a, const double *partial, int np,
+                                                               double *dparam, SlotBin b,
+                                                               const double *x, float4 *g4,
+                                                               int32_t *err)
 {
     pdl_wait();
     if (blockIdx.x == 0) {
