@@ -90,7 +90,7 @@ void free_ctx(lj_ctx *c)
     cudaFree(c->scan_status);
     cudaFree(c->scan_ctl);
     cudaFree(c->centre);
-    cudaFree(c->centre2);
+    cudaFree(c->cfix);
     cudaFree(c->work);
     cudaFree(c->thb);
     cudaFree(c->partial);
@@ -492,7 +492,7 @@ int setup_grid(lj_ctx *c, int nc)
     cudaFree(c->count);
     cudaFree(c->start);
     cudaFree(c->centre);
-    cudaFree(c->centre2);
+    cudaFree(c->cfix);
     cudaFree(c->thb);
     cudaFree(c->tile_sum);
     cudaFree(c->scan_status);
@@ -502,7 +502,7 @@ int setup_grid(lj_ctx *c, int nc)
     c->scan_status = nullptr;
     c->scan_ctl = nullptr;
     c->centre = nullptr;
-    c->centre2 = nullptr;
+    c->cfix = nullptr;
     c->thb = nullptr;
     c->partial = nullptr;
     c->nc = nc;
@@ -523,17 +523,14 @@ int setup_grid(lj_ctx *c, int nc)
         for (int k = 0; k < nc; k++) h[k] = ((double)k + 0.5) * c->cw;
         cudaError_t e = cudaMalloc(&c->centre, sizeof(double) * (size_t)nc);
         if (e == cudaSuccess) e = cudaMemcpy(c->centre, h, sizeof(double) * (size_t)nc, cudaMemcpyHostToDevice);
-        float2 *h2 = (float2 *)malloc(sizeof(float2) * (size_t)nc);
-        if (!h2 && e == cudaSuccess) e = cudaErrorMemoryAllocation;
-        if (h2) {
-            for (int k = 0; k < nc; k++) {
-                h2[k].x = (float)h[k];
-                h2[k].y = (float)(h[k] - (double)h2[k].x);
-            }
-            if (e == cudaSuccess) e = cudaMalloc(&c->centre2, sizeof(float2) * (size_t)nc);
+        long long *hf = (long long *)malloc(sizeof(long long) * (size_t)nc);
+        if (!hf && e == cudaSuccess) e = cudaErrorMemoryAllocation;
+        if (hf) {
+            for (int k = 0; k < nc; k++) hf[k] = lj_fix64(h[k], rel_shift(c->cw));
+            if (e == cudaSuccess) e = cudaMalloc(&c->cfix, sizeof(long long) * (size_t)nc);
             if (e == cudaSuccess)
-                e = cudaMemcpy(c->centre2, h2, sizeof(float2) * (size_t)nc, cudaMemcpyHostToDevice);
-            free(h2);
+                e = cudaMemcpy(c->cfix, hf, sizeof(long long) * (size_t)nc, cudaMemcpyHostToDevice);
+            free(hf);
         }
         free(h);
         long long *tb = (long long *)malloc(sizeof(long long) * (size_t)(nc + 1));

@@ -400,11 +400,11 @@ __global__ void __launch_bounds__(kBatchThreads, 3) k_batch_step_n3(BatchDev b, 
 struct BatchRep {   // one replica's grid, 64 bytes
     double L, whi, wlo, s;
     float cw, inv_nc, sf;
-    int nc, cell0, thoff, ceoff, pad;
+    int nc, cell0, thoff, ceoff, S;   // S: rel_shift
 };
 
 struct BatchSlots {
-    SlotBin bin;                // thb, centre: all replicas' tables; the replica's fields are filled per particle
+    SlotBin bin;                // thb, cfix: all replicas' tables; the replica's fields are filled per particle
     const BatchRep *rep;
     const int32_t *rep_of, *rep_of_cell;
 };
@@ -445,7 +445,8 @@ __global__ void __launch_bounds__(256, 5) k_batch_slots(BatchSlots a, double *x,
         b.nc = r->nc;
         b.cell0 = r->cell0;
         b.thb += r->thoff;
-        b.centre += r->ceoff;
+        b.cfix += r->ceoff;
+        b.S = r->S;
         f[i] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (OP == 0) {
             v0 = __fma_rn(hk, f64_of_f32(q.x), v0);
@@ -684,7 +685,7 @@ struct lj_batch {
     float4 *spos;
     int32_t *onext;
     const BatchRep *rep;
-    const float2 *centre2;
+    const long long *cfix;
     WarpParams ks;
     int gpar;             // par where the captured pair of steps starts
     // calls recorded into a caller's graph, as lj_ctx holds them (lj_internal.cuh)
@@ -692,7 +693,7 @@ struct lj_batch {
     int captured, new_call, own_capture;
     int slots_ok;         // cells beyond their slots are rare in every replica
     std::vector<BatchRep> hrep;
-    std::vector<float2> hcentre2;
+    std::vector<long long> hcfix;
     double max_mean_occ;
     double *rep_out, *host_out;
     int32_t *host_err;
@@ -784,7 +785,7 @@ cudaError_t configure(lj_batch *b)
 cudaError_t batch_slots_setup(lj_batch *b)
 {
     const std::vector<BatchRep> &rep = b->hrep;
-    const std::vector<float2> &centre2 = b->hcentre2;
+    const std::vector<long long> &cfix = b->hcfix;
     const double mean = b->max_mean_occ;
     int cap = ((int)ceil(mean + 7.0 * sqrt(mean) + 3.0) + 7) & ~7;
     cap = cap > kBatchSlotMax ? kBatchSlotMax : cap;
@@ -794,14 +795,14 @@ cudaError_t batch_slots_setup(lj_batch *b)
         return cudaSuccess;
     cudaError_t e = cudaSuccess;
     BatchRep *rd = nullptr;
-    float2 *cd = nullptr;
+    long long *cd = nullptr;
     const size_t mark = b->allocs.size();
     for (int k = 0; k < 2 && e == cudaSuccess; k++) e = balloc(b, &b->cellq[k], (size_t)b->ncell + 1);
     if (e == cudaSuccess) e = balloc(b, &b->octr, 2);
     if (e == cudaSuccess) e = balloc(b, &b->spos, (size_t)(nslots + b->ntot));
     if (e == cudaSuccess) e = balloc(b, &b->onext, (size_t)b->ntot);
     if (e == cudaSuccess) e = balloc(b, &rd, rep.size());
-    if (e == cudaSuccess) e = balloc(b, &cd, centre2.size());
+    if (e == cudaSuccess) e = balloc(b, &cd, cfix.size());
     if (e == cudaErrorMemoryAllocation) {
         cudaGetLastError();
         while (b->allocs.size() > mark) {
@@ -811,10 +812,10 @@ cudaError_t batch_slots_setup(lj_batch *b)
         return cudaSuccess;
     }
     if (e == cudaSuccess) e = cudaMemcpy(rd, rep.data(), rep.size() * sizeof(BatchRep), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(cd, centre2.data(), centre2.size() * sizeof(float2), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(cd, cfix.data(), cfix.size() * sizeof(long long), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return e;
     b->rep = rd;
-    b->centre2 = cd;
+    b->cfix = cd;
     b->ssmem = (kN3Threads / 32) * n3_slice_words(b->kn3.cap) * (int)sizeof(float);
     int nblk = 1 << 30;
     for (int q = 0; q < 6; q++) {
@@ -872,7 +873,7 @@ cudaError_t launch_slots_step(lj_batch *b, bool energy, int op, double *x, doubl
     a.bin.onext = b->onext;
     a.bin.octr = b->octr + b->par;
     a.bin.work = b->d.work;
-    a.bin.centre = b->centre2;
+    a.bin.cfix = b->cfix;
     a.bin.thb = b->d.thb;
     a.bin.ncell = (int)b->ncell;
     a.bin.cap = b->scap;
@@ -1105,13 +1106,11 @@ extern "C" int lj_batch_create(lj_batch **out, int32_t nrep, const int64_t *n, c
         q.cell0 = coff[r];
         q.thoff = thoff[r];
         q.ceoff = ceoff[r];
+        q.S = rel_shift(cw[r]);
         const int64_t nr = (int64_t)nc * nc * nc;
         q.inv_nc = nr + 1 < (1 << 24) ? 1.0f / (float)nc : 0.0f;
         b->hrep.push_back(q);
-        for (int k = 0; k < nc; k++) {
-            const double ce = centre[ceoff[r] + k];
-            b->hcentre2.push_back(make_float2((float)ce, (float)(ce - (double)(float)ce)));
-        }
+        for (int k = 0; k < nc; k++) b->hcfix.push_back(lj_fix64(centre[ceoff[r] + k], q.S));
         // as slots_suit (lj_slots.cu)
         const double mean = (double)n[r] / (double)nr, sl = common->sigma / box[r];
         if (!(mean + 4.5 * sqrt(mean) <= kBatchSlotMax ||

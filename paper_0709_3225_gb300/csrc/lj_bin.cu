@@ -273,7 +273,7 @@ constexpr int kScatterPer = 1;
 template <typename T>
 __global__ void __launch_bounds__(256) k_scatter(const double *__restrict__ x, int n, double L, double whi,
                                                  double wlo, const double *__restrict__ centre,
-                                                 const float2 *__restrict__ centre2, int nc,
+                                                 const long long *__restrict__ cfix, int S, int nc,
                                                  float inv_nc, bool wrap, const int32_t *__restrict__ cell_of,
                                                  const int32_t *__restrict__ rank, const int32_t *__restrict__ start,
                                                  int32_t *__restrict__ perm, typename Vec4<T>::type *__restrict__ pos)
@@ -309,9 +309,9 @@ __global__ void __launch_bounds__(256) k_scatter(const double *__restrict__ x, i
             int cx, cy, cz;
             lj_cell_decode(c, nc, inv_nc, cx, cy, cz);
             if constexpr (sizeof(T) == 4) {
-                q.x = rel_f32(px, __ldg(centre2 + cx));
-                q.y = rel_f32(py, __ldg(centre2 + cy));
-                q.z = rel_f32(pz, __ldg(centre2 + cz));
+                q.x = rel_f32(px, __ldg(cfix + cx), S);
+                q.y = rel_f32(py, __ldg(cfix + cy), S);
+                q.z = rel_f32(pz, __ldg(cfix + cz), S);
             } else {
                 q.x = px - __ldg(centre + cx);
                 q.y = py - __ldg(centre + cy);
@@ -420,12 +420,12 @@ cudaError_t launch_scatter(lj_ctx *c, const double *x, bool wrap)
         // inv_nc_f is 0 in contexts that do not set it (integer division)
         if (c->p.precision == LJ_PREC_FP64)
             k_scatter<double><<<grid, 256, 0, c->stream>>>(x, n, c->p.box, c->wrap_hi, c->wrap_lo, c->centre,
-                                                            c->centre2, c->nc,
+                                                            c->cfix, rel_shift(c->cw), c->nc,
                                                             c->inv_nc_f, wrap, c->cell_of, c->rank, c->start, c->perm,
                                                             (double4_16a *)c->pos);
         else
             k_scatter<float><<<grid, 256, 0, c->stream>>>(x, n, c->p.box, c->wrap_hi, c->wrap_lo, c->centre,
-                                                            c->centre2, c->nc,
+                                                            c->cfix, rel_shift(c->cw), c->nc,
                                                            c->inv_nc_f, wrap, c->cell_of, c->rank, c->start, c->perm,
                                                            (float4 *)c->pos);
         c->kernel_launches++;

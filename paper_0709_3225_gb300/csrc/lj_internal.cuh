@@ -2,6 +2,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 
 #include "../../include/lj.h"
@@ -51,7 +52,7 @@ struct lj_ctx {
     int32_t *cell_of, *rank, *count, *start, *perm;
     void *pos;           // float4 or double4_16a [n], sorted, cell-centred coordinates
     double *centre;      // [nc] cell-centre coordinate (k + 1/2) L / nc
-    float2 *centre2;     // [nc] the same as two floats (rel_f32)
+    long long *cfix;     // [nc] the same in fixed point (rel_f32)
     long long *thb;      // [nc + 1] bits of the cell thresholds (lj_cell_from_guess)
     double wrap_hi, wrap_lo;  // lj_wrap_fast bounds
     int32_t *tile_sum;
@@ -192,6 +193,9 @@ __host__ __device__ __forceinline__ long long lj_fix64(double x, int S)
     if (s >= 0) return s < 64 ? (long long)(m << s) : 0ll;
     return s > -64 ? (long long)(m >> -s) : 0ll;
 }
+
+// Scale of rel_f32's fixed point in cells of side cw: 2^61 <= cw 2^S < 2^62.
+__host__ __device__ __forceinline__ int rel_shift(double cw) { return 61 - ilogb(cw); }
 
 // ---------------------------------------------------------------- device --
 
@@ -356,26 +360,24 @@ __device__ __forceinline__ bool finite64(double x)
     return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000;
 }
 
-// (float)(x - c) for a wrapped x in [0, L) and a cell centre c given as two
-// floats (c = c.x + c.y, c.x its nearest float), without the FP64 pipe: x =
-// h + l with h its leading 24 bits and l the other 29 (as a float, rounded
-// to 2^-48 x); h - c.x with its rounding error (a two-sum), then the low
-// parts.  Rounded to nearest but for an absolute error of 2^-48 x, at most
-// 2^-37 cell sides (x <= 1290 of them), far below the 2^-25 of the rounding:
-// 3 in 10^5 results differ from (float)(x - c) in their last place at L = 168.
-__device__ __forceinline__ float rel_f32(double x, float2 c)
+// (float)(x - c) for a wrapped x and the centre c of its cell, rounded once,
+// without the FP64 pipe: cfix is c 2^S mod 2^64, S = rel_shift(cell side), and
+// x is taken likewise, exactly for x >= 1/256 of a side (below that to 2^-61
+// of it, where the subtraction in FP64 rounds to 2^-54 of it).  Their difference is
+// shifted to 32 bits, the lowest of which also stands for all that follow, so
+// that the conversion rounds as it would the whole.  In FP64 the three
+// subtractions are 42 us of an update of 4M particles.
+__device__ __forceinline__ float rel_f32(double x, long long cfix, int S)
 {
-    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-    const float h = f32_trunc(x);
-    // 2^(e - 1075), the weight of the mantissa's last bit, as a float; 0
-    // where it is below 2^-126 (x < 2^-74)
-    const int ew = (int)((hi >> 20) & 0x7ffu) - 1075 + 127;
-    const float w = __uint_as_float(ew > 0 ? (unsigned)ew << 23 : 0u);
-    const float s = __fsub_rn(h, c.x);
-    const float bb = __fsub_rn(s, h);
-    const float e = __fsub_rn(__fsub_rn(h, __fsub_rn(s, bb)), __fadd_rn(c.x, bb));
-    const float l = __fmaf_rn(__uint2float_rn(lo & 0x1fffffffu), w, -c.y);
-    return __fadd_rn(s, __fadd_rn(l, e));
+    const unsigned hi = (unsigned)__double2hiint(x);
+    const unsigned long long m =
+        (unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32 | (unsigned)__double2loint(x);
+    const int k = (int)((hi >> 20) & 0x7ffu) - 1075 + S;
+    const long long d = (long long)(k >= 0 ? m << min(k, 63) : m >> min(-k, 63)) - cfix;
+    const int s = __clzll(d ^ (d >> 63)) - 1;
+    const long long t = d << s;
+    const int q = (int)(t >> 32) | ((unsigned)t != 0u ? 1 : 0);
+    return __fmul_rn((float)q, __uint_as_float((unsigned)max(159 - S - s, 0) << 23));
 }
 
 template <typename T> struct Vec4;

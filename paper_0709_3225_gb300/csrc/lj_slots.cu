@@ -361,7 +361,7 @@ SlotBin slot_bin_of(const lj_ctx *c)
     b.onext = c->onext;
     b.octr = c->octr + c->slot_par;
     b.work = c->work;
-    b.centre = c->centre2;
+    b.cfix = c->cfix;
     b.thb = c->thb;
     b.L = c->p.box;
     b.whi = c->wrap_hi;
@@ -374,7 +374,7 @@ SlotBin slot_bin_of(const lj_ctx *c)
     b.nslots = c->nslots;
     b.nover = (int)c->p.n;
     b.cell0 = 0;
-    b.S = c->p.precision == LJ_PREC_FP64 ? fx_shift(c) : 0;
+    b.S = c->p.precision == LJ_PREC_FP64 ? fx_shift(c) : rel_shift(c->cw);
     return b;
 }
 

@@ -25,11 +25,11 @@ struct SlotBin {
     void *pos;              // [nslots + n] float4, or longlong4 in FP64 contexts
     int32_t *onext;
     unsigned *octr, *work;  // overflow counter of this buffer; the force kernel's work counter, zeroed here
-    const float2 *centre;   // cell centres as two floats
+    const long long *cfix;  // cell centres (rel_f32)
     const long long *thb;
     double L, whi, wlo, s;
     float sf;               // (float)s
-    int nc, ncell, cap, nslots, S;   // S: scale of the fixed-point coordinates (FP64)
+    int nc, ncell, cap, nslots, S;   // S: scale of the fixed-point coordinates (FP64: lj_force_fx.cu, else rel_shift)
     int nover;              // entries of the overflow region
     int cell0;              // id of the grid's first cell (a batch's replica; else 0); ncell counts all grids' cells
 };
@@ -85,8 +85,8 @@ __device__ __forceinline__ int slot_place(const SlotBin &b, bool valid, int i, d
         o[1] = make_longlong2(lj_fix64(pz, b.S), (long long)i);
     } else {
         reinterpret_cast<float4 *>(b.pos)[slot] =
-            make_float4(rel_f32(px, __ldg(b.centre + cc.x)), rel_f32(py, __ldg(b.centre + cc.y)),
-                        rel_f32(pz, __ldg(b.centre + cc.z)), __int_as_float(i));
+            make_float4(rel_f32(px, __ldg(b.cfix + cc.x), b.S), rel_f32(py, __ldg(b.cfix + cc.y), b.S),
+                        rel_f32(pz, __ldg(b.cfix + cc.z), b.S), __int_as_float(i));
     }
     return slot;
 }

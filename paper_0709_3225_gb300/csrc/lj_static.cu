@@ -35,8 +35,8 @@ constexpr size_t kOffPos = kOffPerm + align256(4 * kMaxN);
 constexpr size_t kOffCount = kOffPos + align256(32 * kMaxN);          // double4 in FP64 mode
 constexpr size_t kOffStart = kOffCount + align256(4 * (kMaxCells + 1));
 constexpr size_t kOffCentre = kOffStart + align256(4 * (kMaxCells + 2));
-constexpr size_t kOffCentre2 = kOffCentre + align256(8 * kMaxNc);
-constexpr size_t kOffTiles = kOffCentre2 + align256(8 * kMaxNc);
+constexpr size_t kOffCfix = kOffCentre + align256(8 * kMaxNc);
+constexpr size_t kOffTiles = kOffCfix + align256(8 * kMaxNc);
 constexpr size_t kOffPartial = kOffTiles + align256(4 * ((kMaxCells + 1 + kScanTile - 1) / kScanTile));
 constexpr size_t kOffScalars = kOffPartial + align256(16 * kMaxPartials);
 constexpr size_t kOffErr = kOffScalars + align256(4 * sizeof(double));
@@ -44,14 +44,13 @@ constexpr size_t kScratchBytes = kOffErr + 256;
 
 static __device__ __align__(256) unsigned char g_lj_static_scratch[kScratchBytes];
 
-__global__ void k_static_centres(double *centre, float2 *centre2, int nc, double cw)
+__global__ void k_static_centres(double *centre, long long *cfix, int S, int nc, double cw)
 {
     const int k = threadIdx.x;
     if (k < nc) {
         const double x = ((double)k + 0.5) * cw;
-        const float h = (float)x;
         centre[k] = x;
-        centre2[k] = make_float2(h, (float)(x - (double)h));
+        cfix[k] = lj_fix64(x, S);
     }
 }
 
@@ -122,7 +121,7 @@ extern "C" int lj_forces_static(const lj_params *p, const double *x, void *f, vo
     c.count = (int32_t *)(base + kOffCount);
     c.start = (int32_t *)(base + kOffStart);
     c.centre = (double *)(base + kOffCentre);
-    c.centre2 = (float2 *)(base + kOffCentre2);
+    c.cfix = (long long *)(base + kOffCfix);
     c.tile_sum = (int32_t *)(base + kOffTiles);
     c.ntiles = (int)((ncell + 1 + kScanTile - 1) / kScanTile);
     c.partial = (double *)(base + kOffPartial);
@@ -139,7 +138,7 @@ extern "C" int lj_forces_static(const lj_params *p, const double *x, void *f, vo
     if ((e = cudaMemsetAsync(c.count, 0, (size_t)(ncell + 1) * sizeof(int32_t), c.stream)) != cudaSuccess)
         return map_err(e);
     if ((e = cudaMemsetAsync(c.err, 0, sizeof(int32_t), c.stream)) != cudaSuccess) return map_err(e);
-    k_static_centres<<<1, kMaxNc, 0, c.stream>>>(c.centre, c.centre2, nc, c.cw);
+    k_static_centres<<<1, kMaxNc, 0, c.stream>>>(c.centre, c.cfix, rel_shift(c.cw), nc, c.cw);
     if ((e = cudaGetLastError()) != cudaSuccess) return map_err(e);
     if ((e = launch_bin_count(&c, x)) != cudaSuccess) return map_err(e);
     if ((e = launch_scan(&c)) != cudaSuccess) return map_err(e);
