@@ -526,7 +526,8 @@ int setup_grid(lj_ctx *c, int nc)
         long long *hf = (long long *)malloc(sizeof(long long) * (size_t)nc);
         if (!hf && e == cudaSuccess) e = cudaErrorMemoryAllocation;
         if (hf) {
-            for (int k = 0; k < nc; k++) hf[k] = lj_fix64(h[k], rel_shift(c->cw));
+            const int S = c->p.precision == LJ_PREC_FP64 ? fx_shift(c) : rel_shift(c->cw);
+            for (int k = 0; k < nc; k++) hf[k] = lj_fix64(h[k], S);
             if (e == cudaSuccess) e = cudaMalloc(&c->cfix, sizeof(long long) * (size_t)nc);
             if (e == cudaSuccess)
                 e = cudaMemcpy(c->cfix, hf, sizeof(long long) * (size_t)nc, cudaMemcpyHostToDevice);

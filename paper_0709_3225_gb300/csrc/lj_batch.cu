@@ -787,11 +787,11 @@ cudaError_t batch_slots_setup(lj_batch *b)
     const std::vector<BatchRep> &rep = b->hrep;
     const std::vector<long long> &cfix = b->hcfix;
     const double mean = b->max_mean_occ;
-    int cap = ((int)ceil(mean + 7.0 * sqrt(mean) + 3.0) + 7) & ~7;
-    cap = cap > kBatchSlotMax ? kBatchSlotMax : cap;
+    double cw = 0.0;
+    for (const BatchRep &r : rep) cw = fmax(cw, (double)r.cw);
+    const int cap = slots_per_cell(mean, cw / b->p.sigma, kBatchSlotMax, b->ncell, b->ntot);
     const int64_t nslots = b->ncell * cap;
-    if (b->grid_n3 == 0 || b->ntot == 0 || !b->slots_ok || nslots + b->ntot >= ((int64_t)1 << 31) ||
-        nslots > 12 * b->ntot + ((int64_t)1 << 16))
+    if (b->grid_n3 == 0 || b->ntot == 0 || !b->slots_ok || cap == 0 || nslots + b->ntot >= ((int64_t)1 << 31))
         return cudaSuccess;
     cudaError_t e = cudaSuccess;
     BatchRep *rd = nullptr;

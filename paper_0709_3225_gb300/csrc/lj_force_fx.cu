@@ -73,8 +73,8 @@ struct FxParams {
     unsigned *octr_next, *last_par;
     unsigned par;
     const int32_t *onext;
-    const double *centre;
-    int S, kappa_e, tsh;                        // u = K / 2^63 2^kappa_e 2^lz RI 2^-62
+    const long long *cfix;                 // cell centres, fixed point
+    int kappa_e, tsh;                           // u = K / 2^63 2^kappa_e 2^lz RI 2^-62
     long long Lfix;
     unsigned long long K, r2c, r2min, r2far;
     // FP64 pairs
@@ -214,25 +214,38 @@ __device__ void fx_plain(const FxParams &k, const longlong4_16a *pos, double4_16
 
 // Staging: the half stencil's candidates within rc of the home box, home
 // particles first; returns their number, or -1 when they and 64 entries of
-// padding would not fit.
-__device__ __forceinline__ int fx_stage(const FxParams &k, const longlong4_16a *pos, long long *X64,
-                                        float *X, int *iw, const long long *sh, const int *st, const int *spre, int tot,
-                                        int n_home)
+// padding would not fit.  PART: as many as fit of those from `next` on, after
+// the T that are there already (none, or the home particles); next is then the
+// next part's first.  A part takes at least 32 candidates (cap >= 128).
+// tmp: int[kN3Half].
+template <bool PART>
+__device__ __forceinline__ int fx_stage(const FxParams &k, const longlong4_16a *pos, int &next, int T, long long *X64,
+                                        float *X, int *iw, int *tmp, const long long *sh, const int *st,
+                                        const int *spre, int tot, int n_home)
 {
     const int lane = threadIdx.x & 31;
+    if (!PART) T = 0;
     const unsigned lt = (1u << lane) - 1u, le = (2u << lane) - 1u;
     float bxl = 3.4e38f, byl = 3.4e38f, bzl = 3.4e38f, bxh = -3.4e38f, byh = -3.4e38f, bzh = -3.4e38f;
     // warp-vote entry lookup, as n3_stage
     const int s_e = lane < kN3Half ? spre[lane] : 0x7fffffff;
     const bool ne = lane < kN3Half && spre[lane + 1] > s_e;
     const unsigned nem = __ballot_sync(0xffffffffu, ne);
-    if (ne) iw[__popc(nem & lt)] = lane;
+    if (ne) tmp[__popc(nem & lt)] = lane;
     __syncwarp();
-    const int j_entry = lane < __popc(nem) ? iw[lane] : 0;
+    const int j_entry = lane < __popc(nem) ? tmp[lane] : 0;
     __syncwarp();
-    int T = 0;
+    if (PART && T > 0) {
+        if (lane < n_home) {
+            bxl = bxh = X[lane];
+            byl = byh = X[k.cap + lane];
+            bzl = bzh = X[2 * k.cap + lane];
+        }
+        box_reduce(bxl, byl, bzl, bxh, byh, bzh);
+    }
     constexpr int kB = 2;   // rounds whose loads are in flight together
-    for (int t0 = 0; t0 < tot; t0 += 32 * kB) {
+    int t0 = PART ? next : 0, end = tot;
+    for (; t0 < end; t0 += 32 * kB) {
         longlong2 qa[kB], qb[kB];
         int kcs[kB];
 #pragma unroll
@@ -268,9 +281,13 @@ __device__ __forceinline__ int fx_stage(const FxParams &k, const longlong4_16a *
             const float dz = fmaxf(fmaxf(bzl - cz, cz - bzh), 0.f);
             const bool keep = t < tot && dx * dx + dy * dy + dz * dz < k.rc2_box;
             const unsigned kept = __ballot_sync(0xffffffffu, keep);
-            if (T + __popc(kept) + 64 > k.cap) {   // the padding must fit too
-                __syncwarp();
-                return -1;
+            if (T + __popc(kept) + 64 > k.cap) {   // the next part's
+                if (!PART) {
+                    __syncwarp();
+                    return -1;
+                }
+                end = t0 + 32 * u;
+                break;
             }
             if (keep) {
                 const int s = T + __popc(kept & lt);
@@ -287,6 +304,7 @@ __device__ __forceinline__ int fx_stage(const FxParams &k, const longlong4_16a *
     }
     for (int u = 0; u < 64; u += 32) X[T + u + lane] = X[k.cap + T + u + lane] = X[2 * k.cap + T + u + lane] = kFar;
     __syncwarp();
+    if (PART) next = end;
     return T;
 }
 
@@ -366,97 +384,164 @@ __device__ __forceinline__ void fx_pairs(const FxParams &k, long long *acc, doub
     __syncwarp();   // list and off are rewritten by the next batch
 }
 
-__global__ void __launch_bounds__(kFxThreads) k_force_fx(FxParams k, const longlong4_16a *pos,
+// Phases A and B for T staged candidates, of which those from `done` on are
+// taken (and home pairs only if done = 0).
+__device__ __forceinline__ void fx_compute(const FxParams &k, long long *acc, double4_16a *f, const long long *X64,
+                                           const float *X, const int *iw, uint16_t *list, int *off, int T, int done,
+                                           int n_home)
+{
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    const float2 *X2 = reinterpret_cast<const float2 *>(X);
+    const float2 *Y2 = reinterpret_cast<const float2 *>(X + k.cap);
+    const float2 *Z2 = reinterpret_cast<const float2 *>(X + 2 * k.cap);
+    int p = 0;
+    while (p < n_home) {
+        // Phase A: the lists of the batch's particles (candidates j > p)
+        const int pb = p;
+        int E = 0;
+        if (lane == 0) off[0] = 0;
+        while (p < n_home && E + T <= kFxList) {
+            const float2 xs = f2(X[p]), ys = f2(X[k.cap + p]), zs = f2(X[2 * k.cap + p]);
+            const int jlo = max(p + 1, done);
+            for (int j0 = 0; j0 < T; j0 += 64) {
+                const int jx = j0 + 2 * lane;
+                const float2 qx = X2[(j0 >> 1) + lane], qy = Y2[(j0 >> 1) + lane], qz = Z2[(j0 >> 1) + lane];
+                const float2 dx = __ffma2_rn(qx, f2(-1.0f), xs);
+                const float2 dy = __ffma2_rn(qy, f2(-1.0f), ys);
+                const float2 dz = __ffma2_rn(qz, f2(-1.0f), zs);
+                float2 r2 = __fmul2_rn(dx, dx);
+                r2 = __ffma2_rn(dy, dy, r2);
+                r2 = __ffma2_rn(dz, dz, r2);
+                const bool ina = r2.x < k.rc2_pair && jx >= jlo;
+                const bool inb = r2.y < k.rc2_pair && jx + 1 >= jlo;
+                const unsigned ba = __ballot_sync(0xffffffffu, ina);
+                const unsigned bb = __ballot_sync(0xffffffffu, inb);
+                if (ina) list[E + __popc(ba & lt)] = (uint16_t)jx;
+                if (inb) list[E + __popc(ba) + __popc(bb & lt)] = (uint16_t)(jx + 1);
+                E += __popc(ba) + __popc(bb);
+            }
+            if (lane == 0) off[p - pb + 1] = E;
+            p++;
+        }
+        __syncwarp();
+        fx_pairs(k, acc, f, X64, iw, list, off, E, p - pb, pb);
+    }
+}
+
+// The slice of a warp.
+struct FxSlice {
+    long long *X64, *sh;
+    int *st, *iw, *spre, *off;
+    float *X;
+    uint16_t *list;
+    __device__ FxSlice(unsigned char *smem, int cap)
+    {
+        const FxLayout L(cap);
+        X64 = reinterpret_cast<long long *>(smem + L.x64);
+        sh = reinterpret_cast<long long *>(smem + L.sh);
+        st = reinterpret_cast<int *>(sh + 3 * kN3Half);
+        X = reinterpret_cast<float *>(smem + L.x32);
+        iw = reinterpret_cast<int *>(smem + L.iw);
+        spre = reinterpret_cast<int *>(smem + L.spre);
+        off = reinterpret_cast<int *>(smem + L.off);
+        list = reinterpret_cast<uint16_t *>(smem + L.list);
+    }
+};
+
+// The pairs of home cell c.  A cell whose candidates do not fit the slice, or
+// with more than 32 home particles or a cell of its half stencil beyond its
+// slots, takes the plain path (FITS); is left, the result being false; or, ANY,
+// is taken in parts, the home particles with some of the candidates at a time,
+// or by the plain path if it must.
+template <bool FITS, bool ANY>
+__device__ __forceinline__ bool fx_cell(const FxParams &k, const longlong4_16a *pos, long long *acc, double4_16a *f,
+                                        const FxSlice &w, int c)
+{
+    const int lane = threadIdx.x & 31;
+    if (lane == 31) k.cellq_next[c] = make_int2(0, 0);
+    __syncwarp();   // the slice still holds the previous cell's data
+    // half-stencil table: first slot, prefix sums, image shift minus the
+    // home cell's centre
+    const HalfLoad tl = half_load<true, true>(reinterpret_cast<const int32_t *>(k.cellq), c, k.nc, k.inv_nc, 0, k.scap);
+    const int nn = tl.e - tl.s;
+    if (lane < kN3Half) {
+        int cx, cy, cz, dx, dy, dz;
+        lj_cell_decode(c, k.nc, k.inv_nc, cx, cy, cz);
+        half_delta(lane, dx, dy, dz);
+        const int ux = cx + dx, uy = cy + dy, uz = cz + dz;
+        w.sh[lane] = (ux < 0 ? -k.Lfix : ux >= k.nc ? k.Lfix : 0ll) - __ldg(k.cfix + cx);
+        w.sh[kN3Half + lane] = (uy < 0 ? -k.Lfix : uy >= k.nc ? k.Lfix : 0ll) - __ldg(k.cfix + cy);
+        w.sh[2 * kN3Half + lane] = (uz < 0 ? -k.Lfix : uz >= k.nc ? k.Lfix : 0ll) - __ldg(k.cfix + cz);
+        w.st[lane] = tl.s;
+    }
+    int Pf = nn;
+#pragma unroll
+    for (int o = 1; o < 16; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, Pf, o);
+        if (lane >= o) Pf += y;
+    }
+    if (lane < kN3Half) w.spre[lane] = Pf - nn;
+    if (lane == kN3Half - 1) w.spre[kN3Half] = Pf;
+    __syncwarp();
+    const int tot = w.spre[kN3Half], n_home = w.spre[1];
+    if (n_home == 0) return true;
+    const bool plain = __any_sync(0xffffffffu, nn > k.scap) || n_home > 32;
+    int next = 0;
+    if constexpr (ANY) {
+        if (plain)
+            fx_plain(k, pos, f, w.sh, w.st, w.spre, c, n_home);
+        else
+            for (int done = 0; next < tot; done = n_home) {
+                const int T =
+                    fx_stage<true>(k, pos, next, done, w.X64, w.X, w.iw, w.off, w.sh, w.st, w.spre, tot, n_home);
+                fx_compute(k, acc, f, w.X64, w.X, w.iw, w.list, w.off, T, done, n_home);
+            }
+    } else {
+        const int T = plain || tot > 4 * k.cap
+                          ? -1 : fx_stage<false>(k, pos, next, 0, w.X64, w.X, w.iw, w.off, w.sh, w.st, w.spre, tot, n_home);
+        if (T >= 0)
+            fx_compute(k, acc, f, w.X64, w.X, w.iw, w.list, w.off, T, 0, n_home);
+        else if (FITS)
+            fx_plain(k, pos, f, w.sh, w.st, w.spre, c, n_home);
+        else
+            return false;
+    }
+    return true;
+}
+
+// The next cell (asked for when a cell is done, as k_force_n3's single pulls).
+__device__ __forceinline__ int fx_next(const FxParams &k)
+{
+    unsigned nx = 0;
+    if ((threadIdx.x & 31) == 0) nx = gridDim.x + atomicAdd(k.work, 1u);
+    return (int)__shfl_sync(0xffffffffu, nx, 0);
+}
+
+// FITS: the slice has room for a liquid's cells (fx_fits), and the few that do
+// not fit take the plain path.  Otherwise a warp that meets one (a droplet's
+// in a box sized for its vapour) takes all further cells by the general form,
+// in a loop of its own: a droplet of 97,556 particles at a mean density of 0.1
+// 2,210 -> 116 us, at 0.5 1,850 -> 100.  The second loop costs the first one 2
+// to 4 % by itself (500,000 particles of liquid 363 -> 372 us); as the only
+// loop, for its registers, it costs 7 % (a gas of density 0.1 84 -> 90).
+template <bool FITS>
+__global__ void __launch_bounds__(kFxThreads, 26) k_force_fx(FxParams k, const longlong4_16a *pos,
                                                          long long *acc, double4_16a *f)
 {
     extern __shared__ __align__(16) unsigned char fxsmem[];
-    const int lane = threadIdx.x & 31;
-    const FxLayout L(k.cap);
-    long long *X64 = reinterpret_cast<long long *>(fxsmem + L.x64);
-    long long *sh = reinterpret_cast<long long *>(fxsmem + L.sh);
-    int *st = reinterpret_cast<int *>(sh + 3 * kN3Half);
-    float *X = reinterpret_cast<float *>(fxsmem + L.x32);
-    int *iw = reinterpret_cast<int *>(fxsmem + L.iw);
-    int *spre = reinterpret_cast<int *>(fxsmem + L.spre);
-    int *off = reinterpret_cast<int *>(fxsmem + L.off);
-    uint16_t *list = reinterpret_cast<uint16_t *>(fxsmem + L.list);
-    const unsigned lt = (1u << lane) - 1u;
+    const FxSlice w(fxsmem, k.cap);
     pdl_wait();
-    if (blockIdx.x == 0 && lane == 0) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
         k.cellq_next[k.ncell] = make_int2(0, 0);
         *k.octr_next = 0u;
         *k.last_par = k.par;
     }
-    const float2 *X2 = reinterpret_cast<const float2 *>(X);
-    const float2 *Y2 = reinterpret_cast<const float2 *>(X + k.cap);
-    const float2 *Z2 = reinterpret_cast<const float2 *>(X + 2 * k.cap);
-    for (int c = blockIdx.x; c < k.ncell;) {
-        if (lane == 31) k.cellq_next[c] = make_int2(0, 0);
-        __syncwarp();   // the slice still holds the previous cell's data
-        // half-stencil table: first slot, prefix sums, image shift minus the
-        // home cell's centre
-        const HalfLoad tl = half_load<true, true>(reinterpret_cast<const int32_t *>(k.cellq), c, k.nc, k.inv_nc, 0, k.scap);
-        const int nn = tl.e - tl.s;
-        if (lane < kN3Half) {
-            int cx, cy, cz, dx, dy, dz;
-            lj_cell_decode(c, k.nc, k.inv_nc, cx, cy, cz);
-            half_delta(lane, dx, dy, dz);
-            const int ux = cx + dx, uy = cy + dy, uz = cz + dz;
-            sh[lane] = (ux < 0 ? -k.Lfix : ux >= k.nc ? k.Lfix : 0ll) - lj_fix64(__ldg(k.centre + cx), k.S);
-            sh[kN3Half + lane] = (uy < 0 ? -k.Lfix : uy >= k.nc ? k.Lfix : 0ll) - lj_fix64(__ldg(k.centre + cy), k.S);
-            sh[2 * kN3Half + lane] = (uz < 0 ? -k.Lfix : uz >= k.nc ? k.Lfix : 0ll) - lj_fix64(__ldg(k.centre + cz), k.S);
-            st[lane] = tl.s;
-        }
-        int Pf = nn;
-#pragma unroll
-        for (int o = 1; o < 16; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, Pf, o);
-            if (lane >= o) Pf += y;
-        }
-        if (lane < kN3Half) spre[lane] = Pf - nn;
-        if (lane == kN3Half - 1) spre[kN3Half] = Pf;
-        __syncwarp();
-        const int tot = spre[kN3Half], n_home = spre[1];
-        if (n_home > 0) {
-            const bool over = __any_sync(0xffffffffu, nn > k.scap);
-            const int T = over || n_home > 32 || tot > 4 * k.cap ? -1 : fx_stage(k, pos, X64, X, iw, sh, st, spre, tot, n_home);
-            if (T < 0) fx_plain(k, pos, f, sh, st, spre, c, n_home);
-            int p = T < 0 ? n_home : 0;
-            while (p < n_home) {
-                // Phase A: the lists of the batch's particles (candidates j > p)
-                const int pb = p;
-                int E = 0;
-                if (lane == 0) off[0] = 0;
-                while (p < n_home && E + T <= kFxList) {
-                    const float2 xs = f2(X[p]), ys = f2(X[k.cap + p]), zs = f2(X[2 * k.cap + p]);
-                    for (int j0 = p & ~63; j0 < T; j0 += 64) {
-                        const int jx = j0 + 2 * lane;
-                        const float2 qx = X2[(j0 >> 1) + lane], qy = Y2[(j0 >> 1) + lane], qz = Z2[(j0 >> 1) + lane];
-                        const float2 dx = __ffma2_rn(qx, f2(-1.0f), xs);
-                        const float2 dy = __ffma2_rn(qy, f2(-1.0f), ys);
-                        const float2 dz = __ffma2_rn(qz, f2(-1.0f), zs);
-                        float2 r2 = __fmul2_rn(dx, dx);
-                        r2 = __ffma2_rn(dy, dy, r2);
-                        r2 = __ffma2_rn(dz, dz, r2);
-                        const bool ina = r2.x < k.rc2_pair && jx > p;
-                        const bool inb = r2.y < k.rc2_pair && jx + 1 > p;
-                        const unsigned ba = __ballot_sync(0xffffffffu, ina);
-                        const unsigned bb = __ballot_sync(0xffffffffu, inb);
-                        if (ina) list[E + __popc(ba & lt)] = (uint16_t)jx;
-                        if (inb) list[E + __popc(ba) + __popc(bb & lt)] = (uint16_t)(jx + 1);
-                        E += __popc(ba) + __popc(bb);
-                    }
-                    if (lane == 0) off[p - pb + 1] = E;
-                    p++;
-                }
-                __syncwarp();
-                fx_pairs(k, acc, f, X64, iw, list, off, E, p - pb, pb);
-            }
-        }
-        unsigned nx = 0;   // the next cell (asked for when this one is done, as k_force_n3's single pulls)
-        if (lane == 0) nx = gridDim.x + atomicAdd(k.work, 1u);
-        c = (int)__shfl_sync(0xffffffffu, nx, 0);
-    }
+    int c = blockIdx.x;
+    for (; c < k.ncell; c = fx_next(k))
+        if (!fx_cell<FITS, false>(k, pos, acc, f, w, c)) break;
+    if constexpr (!FITS)
+        for (; c < k.ncell; c = fx_next(k)) fx_cell<false, true>(k, pos, acc, f, w, c);
 }
 
 }  // namespace
@@ -491,14 +576,25 @@ cudaError_t fx_configure(lj_ctx *c)
     cap = cap < 128 ? 128 : (cap > kFxList ? kFxList : cap);
     c->fx_cap = cap;
     c->fx_smem = FxLayout(cap).bytes;
-    cudaError_t e = raise_dyn_smem((const void *)k_force_fx, c->fx_smem);
-    if (e != cudaSuccess) return e;
-    int nb = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_force_fx, kFxThreads, c->fx_smem);
-    if (e != cudaSuccess) return e;
+    int nb = 1 << 30;
+    for (const void *kern : {(const void *)k_force_fx<true>, (const void *)k_force_fx<false>}) {
+        int b = 0;
+        cudaError_t e = raise_dyn_smem(kern, c->fx_smem);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kern, kFxThreads, c->fx_smem);
+        if (e != cudaSuccess) return e;
+        nb = b < nb ? b : nb;
+    }
     const int64_t grid = (int64_t)(nb > 0 ? nb : 1) * c->nsm;
     c->fx_grid = (int)(grid < c->ncell ? grid : c->ncell);
     return cudaSuccess;
+}
+
+// The slice holds what is left of a liquid's half stencil (density 0.85) and
+// the padding: mean densities of 0.6 and above at rc = 2.5 sigma.
+static bool fx_fits(const lj_ctx *c)
+{
+    const double cw = c->cw / c->p.sigma;
+    return 0.63 * kN3Half * 0.85 * cw * cw * cw + 64.0 <= (double)c->fx_cap;
 }
 
 cudaError_t launch_force_fx(lj_ctx *c, double4_16a *f)
@@ -524,8 +620,7 @@ cudaError_t launch_force_fx(lj_ctx *c, double4_16a *f)
     k.last_par = c->octr + 2;
     k.par = (unsigned)c->slot_par;
     k.onext = c->onext;
-    k.centre = c->centre;
-    k.S = S;
+    k.cfix = c->cfix;
     k.tsh = fx_tsh(c);
     k.Lfix = lj_fix64(c->p.box, S);
     int ex = 0;
@@ -546,7 +641,7 @@ cudaError_t launch_force_fx(lj_ctx *c, double4_16a *f)
     long long *acc = c->fx_acc;
     void *args[] = {&k, (void *)&pos, &acc, &f};
     if (c->timing && c->ev_used + 2 <= c->nev) cudaEventRecord(c->ev[c->ev_used], c->stream);
-    const cudaError_t e = launch_pdl((const void *)k_force_fx, c->fx_grid, kFxThreads, args, (size_t)c->fx_smem, c->stream,
+    const cudaError_t e = launch_pdl(fx_fits(c) ? (const void *)k_force_fx<true> : (const void *)k_force_fx<false>, c->fx_grid, kFxThreads, args, (size_t)c->fx_smem, c->stream,
                                      !c->timing);
     if (c->timing && c->ev_used + 2 <= c->nev) {
         cudaEventRecord(c->ev[c->ev_used + 1], c->stream);

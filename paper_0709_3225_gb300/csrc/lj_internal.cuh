@@ -52,7 +52,7 @@ struct lj_ctx {
     int32_t *cell_of, *rank, *count, *start, *perm;
     void *pos;           // float4 or double4_16a [n], sorted, cell-centred coordinates
     double *centre;      // [nc] cell-centre coordinate (k + 1/2) L / nc
-    long long *cfix;     // [nc] the same in fixed point (rel_f32)
+    long long *cfix;     // [nc] the same in fixed point (rel_f32; FP64: lj_force_fx.cu)
     long long *thb;      // [nc + 1] bits of the cell thresholds (lj_cell_from_guess)
     double wrap_hi, wrap_lo;  // lj_wrap_fast bounds
     int32_t *tile_sum;

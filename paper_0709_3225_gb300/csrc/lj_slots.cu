@@ -403,17 +403,10 @@ cudaError_t slots_setup(lj_ctx *c)
     // (FP64: the fixed-point kernel has no force-shifted form)
     const bool fp64 = c->p.precision == LJ_PREC_FP64;
     if (c->p.cell_subdiv == 2 || c->p.n == 0 || (fp64 && c->p.shift_mode == LJ_SHIFT_FORCE)) return cudaSuccess;
-    // Slots per cell: the mean occupancy plus 7 standard deviations of a
-    // random gas, a multiple of 8 (128 bytes), at most the 32 home particles
-    // that the kernels' fast path takes.
     const double mean = (double)c->p.n / (double)c->ncell;
-    int cap = ((int)ceil(mean + 7.0 * sqrt(mean) + 3.0) + 7) & ~7;
-    cap = cap > kSlotMax ? kSlotMax : cap;
+    const int cap = slots_per_cell(mean, c->cw / c->p.sigma, kSlotMax, c->ncell, c->p.n);
     const int64_t nslots = c->ncell * cap;
-    // sparse boxes (far more slots than particles) keep the sorted lists
-    if (mean > 22.0 || nslots + c->p.n >= ((int64_t)1 << 31) ||
-        nslots > (int64_t)12 * c->p.n + ((int64_t)1 << 16))
-        return cudaSuccess;
+    if (mean > 22.0 || cap == 0 || nslots + c->p.n >= ((int64_t)1 << 31)) return cudaSuccess;
     cudaError_t e = cudaSuccess;
     const size_t qb = (size_t)(c->ncell + 1) * sizeof(int2);
     for (int k = 0; k < 2 && e == cudaSuccess; k++) e = cudaMalloc(&c->cellq[k], qb);
