@@ -129,12 +129,14 @@ struct lj_ctx {
     // two buffers: the binning fills slot_par's, which is zero by then, and
     // the force (VJP) kernel after it zeroes the other one.
     int scap, nslots;        // nslots = ncell * scap; spos holds nslots + n
+    void *slot_mem;          // holds the following
     int2 *cellq[2];
     // [0], [1] overflow particles per buffer; [2] the buffer of the last
     // force (VJP) launch, -1 (as int) when the sorted lists are newer
     unsigned *octr;
     void *spos;              // slotted positions: float4 (FP64: longlong4)
-    float4 *sg4;             // cotangents (lazily allocated)
+    float4 *sg4;             // cotangents (slots)
+    int sg4_inside;          // in slot_mem
     int32_t *onext;          // overflow lists: index + 1 of the next, 0 = end
     // FP64 contexts (lj_force_fx.cu): spos holds longlong4 (fixed-point
     // coordinates, particle index), fx_acc the force sums, int64[kFxAcc] per particle

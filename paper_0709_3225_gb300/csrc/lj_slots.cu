@@ -6,6 +6,7 @@
 
 namespace {
 
+constexpr size_t kSlotsTogether = (size_t)16 << 20;
 constexpr int kSlotMax = 32;   // the pair-once kernels' limit on home particles
 
 // Bin given positions (wrapped here), zero the array the force (VJP) kernel
@@ -380,17 +381,14 @@ SlotBin slot_bin_of(const lj_ctx *c)
 
 void slots_free(lj_ctx *c)
 {
-    cudaFree(c->cellq[0]);
-    cudaFree(c->cellq[1]);
-    cudaFree(c->octr);
-    cudaFree(c->spos);
-    cudaFree(c->sg4);
-    cudaFree(c->onext);
-    cudaFree(c->fx_acc);
+    cudaFree(c->slot_mem);
+    if (!c->sg4_inside) cudaFree(c->sg4);
+    c->slot_mem = nullptr;
     c->cellq[0] = c->cellq[1] = nullptr;
     c->octr = nullptr;
     c->spos = nullptr;
     c->sg4 = nullptr;
+    c->sg4_inside = 0;
     c->onext = nullptr;
     c->fx_acc = nullptr;
     c->scap = c->nslots = 0;
@@ -407,20 +405,39 @@ cudaError_t slots_setup(lj_ctx *c)
     const int cap = slots_per_cell(mean, c->cw / c->p.sigma, kSlotMax, c->ncell, c->p.n);
     const int64_t nslots = c->ncell * cap;
     if (mean > 22.0 || cap == 0 || nslots + c->p.n >= ((int64_t)1 << 31)) return cudaSuccess;
-    cudaError_t e = cudaSuccess;
+    // One allocation: each costs a context's creation about 10 us, and one
+    // above 1 MB some 90.  Small contexts get the cotangents' slots with it
+    // (32,000 particles: the first gradient 143 us when it allocated them, now
+    // 61); large ones with their first gradient (ensure_vjp_buffers), if any.
+    const size_t m = (size_t)(nslots + c->p.n), n = (size_t)c->p.n;
+    const size_t sb = m * (fp64 ? sizeof(longlong4_16a) : sizeof(float4));
+    c->sg4_inside = !fp64 && sb <= kSlotsTogether;
     const size_t qb = (size_t)(c->ncell + 1) * sizeof(int2);
-    for (int k = 0; k < 2 && e == cudaSuccess; k++) e = cudaMalloc(&c->cellq[k], qb);
-    if (e == cudaSuccess) e = cudaMalloc(&c->octr, 4 * sizeof(unsigned));
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->octr, 0xff, 4 * sizeof(unsigned), c->stream);
-    if (e == cudaSuccess)
-        e = cudaMalloc(&c->spos, (size_t)(nslots + c->p.n) * (fp64 ? sizeof(longlong4_16a) : sizeof(float4)));
-    if (e == cudaSuccess && fp64) e = cudaMalloc(&c->fx_acc, (size_t)c->p.n * kFxAcc * sizeof(long long));
-    if (e == cudaSuccess) e = cudaMalloc(&c->onext, (size_t)c->p.n * sizeof(int32_t));
+    const size_t part[7] = {sb, c->sg4_inside ? sb : 0, fp64 ? n * kFxAcc * sizeof(long long) : 0,
+                            qb, qb, n * sizeof(int32_t), 4 * sizeof(unsigned)};
+    char *at[7];
+    size_t bytes = 0;
+    for (size_t p : part) bytes += (p + 255) & ~(size_t)255;
+    cudaError_t e = cudaMalloc(&c->slot_mem, bytes);
     if (e == cudaErrorMemoryAllocation) {   // the sorted lists need less
         cudaGetLastError();
         slots_free(c);
         return cudaSuccess;
     }
+    if (e != cudaSuccess) return e;
+    bytes = 0;
+    for (int k = 0; k < 7; k++) {
+        at[k] = (char *)c->slot_mem + bytes;
+        bytes += (part[k] + 255) & ~(size_t)255;
+    }
+    c->spos = at[0];
+    c->sg4 = c->sg4_inside ? (float4 *)at[1] : nullptr;
+    c->fx_acc = fp64 ? (long long *)at[2] : nullptr;
+    c->cellq[0] = (int2 *)at[3];
+    c->cellq[1] = (int2 *)at[4];
+    c->onext = (int32_t *)at[5];
+    c->octr = (unsigned *)at[6];
+    e = cudaMemsetAsync(c->octr, 0xff, part[6], c->stream);
     if (e != cudaSuccess) return e;
     c->scap = cap;
     c->nslots = (int)nslots;
