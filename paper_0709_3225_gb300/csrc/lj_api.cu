@@ -1,5 +1,6 @@
 // C ABI of liblj.so (declared in include/lj.h): context management,
 // argument checking and the sequencing of the kernels of one MD step.
+#include <cuda.h>
 #include <math.h>
 #include <stdlib.h>
 #include <string.h>
@@ -373,28 +374,47 @@ int persistent_steps(lj_ctx *c, double *x, double *v, void *f, int nsteps, cudaE
 
 constexpr int kHostChunks = 4;   // parts of lj_step_host's copies in
 
+}  // namespace
+
 // Pinned host memory from p on, readable and writable by kernels in 16-byte
-// accesses.
-bool mapped_host(const void *p, size_t bytes)
+// accesses: all of it in the one allocation or registration that p is in (the
+// bytes between two registrations need not be pinned).
+extern "C" int lj_mapped_host(const void *p, size_t bytes)
 {
-    if (((uintptr_t)p) % 16 != 0) return false;
-    const char *ends[2] = {(const char *)p, (const char *)p + bytes - 1};
-    for (const char *q : ends) {
-        cudaPointerAttributes a;
-        unsigned flags = 0;
-        if (cudaPointerGetAttributes(&a, q) != cudaSuccess) {
+    using Get = CUresult (*)(void *, CUpointer_attribute, CUdeviceptr);
+    static const Get get = [] {
+        void *fn = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttribute", &fn, 4000, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess) {
             cudaGetLastError();
-            return false;
+            fn = nullptr;
         }
-        if (a.type != cudaMemoryTypeHost || a.devicePointer != (void *)q) return false;
-        if (cudaHostGetFlags(&flags, (void *)q) != cudaSuccess) {
-            cudaGetLastError();
-            return false;
-        }
-        if (flags & cudaHostRegisterReadOnly) return false;
+        return (Get)fn;
+    }();
+    if (!get || ((uintptr_t)p) % 16 != 0) return 0;
+    cudaPointerAttributes a;
+    unsigned flags = 0;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
     }
-    return true;
+    if (a.type != cudaMemoryTypeHost || a.devicePointer != p) return 0;
+    if (cudaHostGetFlags(&flags, (void *)p) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    if (flags & cudaHostRegisterReadOnly) return 0;
+    CUdeviceptr start = 0;
+    size_t size = 0;
+    if (get(&start, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, (CUdeviceptr)p) != CUDA_SUCCESS ||
+        get(&size, CU_POINTER_ATTRIBUTE_RANGE_SIZE, (CUdeviceptr)p) != CUDA_SUCCESS)
+        return 0;
+    const size_t off = (size_t)((CUdeviceptr)p - start);
+    return (CUdeviceptr)p >= start && off <= size && bytes <= size - off;
 }
+
+namespace {
 
 constexpr int kHostSmall = 32768;   // below it x goes back in k_host_out too: 4 us of the link, less than a copy's set-up
 
@@ -832,8 +852,8 @@ extern "C" int lj_step_host(lj_ctx *c, double *x, double *v, void *f, int32_t ns
     if (!c->ev_entry) LJ_CK(cudaEventCreateWithFlags(&c->ev_entry, cudaEventDisableTiming));
     for (int k = 0; k < kHostChunks; k++)
         if (!c->ev_chunk[k]) LJ_CK(cudaEventCreateWithFlags(&c->ev_chunk[k], cudaEventDisableTiming));
-    if (n > 0 && nsteps > 0 && uses_slots(c) && !persistent_mode(c) && mapped_host(x, bx) && mapped_host(v, bx) &&
-        mapped_host(f, bf)) {
+    if (n > 0 && nsteps > 0 && uses_slots(c) && !persistent_mode(c) && lj_mapped_host(x, bx) &&
+        lj_mapped_host(v, bx) && lj_mapped_host(f, bf)) {
         const bool copy_x = n > kHostSmall;
         LJ_CK(launch_host_in(c, x, v, (const float4 *)f, c->xs, c->vs, (float4 *)c->fs));
         c->kdb_done = 1;
