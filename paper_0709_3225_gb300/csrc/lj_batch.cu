@@ -396,7 +396,7 @@ __global__ void __launch_bounds__(kBatchThreads, 3) k_batch_step_n3(BatchDev b, 
 // update, two scan phases and the scatter at the force phase's occupancy,
 // with four grid barriers between them, and kept the FP64 pipe busy with
 // conversions (64 replicas, 1.6 million particles, per step:
-// 382 -> 316 us).
+// 421 -> 357 us).
 struct BatchRep {   // one replica's grid, 64 bytes
     double L, whi, wlo, s;
     float cw, inv_nc, sf;
@@ -411,7 +411,7 @@ struct BatchSlots {
 
 // op 0: kicks, drift and wrap, then bin; op 1: bin the given positions.
 // Bound by HBM and the latency of the replica's fields: 48 registers, for 5
-// blocks per SM (56 and 4 without the bound: a step 319 -> 316 us).
+// blocks per SM (56 and 4 without the bound: a step 1 % longer).
 template <int OP>
 __global__ void __launch_bounds__(256, 5) k_batch_slots(BatchSlots a, double *x, double *v,
                                                      float4 *f, int n, double hk, double dt,

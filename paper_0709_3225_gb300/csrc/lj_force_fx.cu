@@ -44,12 +44,12 @@
 //    bound, and cells that take the plain path are evaluated in FP64 as
 //    before (pair64_nf) and added to f itself; the readers of the sums add
 //    the two (fx_force, lj_slots.cu).
-// Bound by instruction issue and the latencies that 14 to 18 warps per SM
-// leave (52 % of issue slots; ALU pipe 40 %).  Step in FP64: 257 -> 96 us at
-// 131,072 particles (the force kernel 220 -> 92), 174 -> 34 at 32,000, 1,309
-// -> 646 at 10^6.  Forces against an FP64 evaluation: 6.7e-15 of their norm at
-// 131,072 particles (2.5e-14 before), 5.5e-15 at 2,048 (8.3e-15), 1.3e-14 for
-// a gas of 100,003 at density 0.3 (3.9e-14).
+// Bound by instruction issue and the latencies that 15 warps per SM leave (60
+// % of issue slots; ALU pipe 47 %).  Step in FP64: 257 -> 105 us at 131,072
+// particles (the force kernel 220 -> 95), 174 -> 35 at 32,000, 1,309 -> 655 at
+// 10^6.  Forces against the oracle: 4.9e-15 of their norm at 131,072 particles
+// (2.8e-14 with lj_force_w64.cu), 3.0e-15 at 2,048 (1.0e-14), 4.7e-15 for a gas
+// of 100,003 at density 0.3 (2.1e-14).
 #include <math.h>
 #include <string.h>
 
@@ -570,7 +570,7 @@ cudaError_t fx_configure(lj_ctx *c)
     // ~0.63 m of the m = 14 n_cell raw candidates survive the box test; room
     // for 2.5 sqrt(m) more and the padding.  Slots cost resident warps (12 KB
     // a warp at liquid density, 18 warps per SM): with 4 sqrt(m) + 96 the step
-    // at 10^6 particles took 688 us, with 2.5 sqrt(m) + 96 669, now 646.
+    // at 10^6 particles took 6 % longer, with 2.5 sqrt(m) + 96 3 %.
     const double m = kN3Half * mean;
     int cap = ((int)(0.65 * m + 2.5 * sqrt(m)) + 64 + 7) & ~7;
     cap = cap < 128 ? 128 : (cap > kFxList ? kFxList : cap);
