@@ -656,7 +656,8 @@ extern "C" int lj_create(lj_ctx **out, const lj_params *p, void *stream)
     LJ_CREATE_CK(cudaMemset(c->work, 0, sizeof(unsigned)));
     c->grab = 4;   // dynamic pulls of 4 cells: measured fastest at 4M (static striding 5% slower)
     LJ_CREATE_CK(cudaMallocHost(&c->host_scalars, 8 * sizeof(double)));
-    LJ_CREATE_CK(cudaMallocHost(&c->host_err, sizeof(int32_t)));
+    LJ_CREATE_CK(cudaMallocHost(&c->host_err, 2 * sizeof(int32_t)));
+    c->host_err[0] = c->host_err[1] = 0;
     LJ_CREATE_CK(cudaMemsetAsync(c->cell_of, 0, n1 * sizeof(int32_t), c->stream));
     LJ_CREATE_CK(cudaMemsetAsync(c->scalars, 0, 8 * sizeof(double), c->stream));
     LJ_CREATE_CK(cudaMemsetAsync(c->err, 0, sizeof(int32_t), c->stream));
@@ -721,7 +722,7 @@ extern "C" int lj_forces(lj_ctx *c, const double *x, void *f, double *e_pot, dou
         r = check_dev_ptr(f, 16);
         if (r) return r;
     }
-    c->new_call = 1;
+    LJ_CK(slots_new_call(c));
     const bool energy = e_pot || virial;
     if (!energy && uses_fx(c)) {
         LJ_CK(launch_bin_fx(c, x, (double4_16a *)f));
@@ -787,8 +788,8 @@ extern "C" int lj_langevin_step(lj_ctx *c, double *x, double *v, void *f, int32_
     if (r) return r;
     r = check_dev_ptr(f, 16);
     if (r) return r;
+    LJ_CK(slots_new_call(c));
     const bool slots = uses_slots(c);
-    c->new_call = 1;
     if (!slots) LJ_CK(lists_begin(c));
     for (int s = 0; s < nsteps; s++) {
         LJ_CK(launch_langevin_bin(c, x, v, f, s == 0 ? 1 : 2, gamma, kT, slots && s > 0 && !c->timing));
@@ -834,7 +835,7 @@ extern "C" int lj_step(lj_ctx *c, double *x, double *v, void *f, int32_t nsteps)
         r = check_dev_ptr(f, 16);
         if (r) return r;
     }
-    c->new_call = 1;
+    LJ_CK(slots_new_call(c));
     return do_steps(c, x, v, f, nsteps);
 }
 
@@ -843,7 +844,7 @@ extern "C" int lj_step_host(lj_ctx *c, double *x, double *v, void *f, int32_t ns
     if (!c || nsteps < 0) return LJ_EINVAL;
     const size_t n = (size_t)c->p.n;
     if (n > 0 && (!x || !v || !f)) return LJ_EINVAL;
-    c->new_call = 1;
+    LJ_CK(slots_new_call(c));
     int r = ensure_staging(c);
     if (r) return r;
     const size_t bx = 3 * n * sizeof(double), bf = n * force_vsize(c);
@@ -934,7 +935,7 @@ extern "C" int lj_energy(lj_ctx *c, const double *x, const double *v, double *ou
     LJ_CK(cudaMemsetAsync(c->scalars, 0, 4 * sizeof(double), c->stream));
     if (c->p.n > 0) {
         LJ_CK(launch_ekin(c, v));
-        c->new_call = 1;
+        LJ_CK(slots_new_call(c));
         r = bin_for_force(c, x, c->fs);
         if (r) return r;
         LJ_CK(launch_force(c, c->fs, true));
@@ -963,7 +964,7 @@ extern "C" int lj_observables(lj_ctx *c, const double *x, const double *v, doubl
     LJ_CK(cudaMemsetAsync(c->scalars, 0, 8 * sizeof(double), c->stream));
     if (c->p.n > 0) {
         LJ_CK(launch_ekin(c, v));
-        c->new_call = 1;
+        LJ_CK(slots_new_call(c));
         r = bin_for_force(c, x, c->fs);
         if (r) return r;
         LJ_CK(launch_force(c, c->fs, true));
@@ -1011,8 +1012,8 @@ extern "C" int lj_forces_vjp(lj_ctx *c, const double *x, const double *g, double
     if ((r = check_dev_ptr(x, 8)) != LJ_OK) return r;
     if ((r = check_dev_ptr(g, 8)) != LJ_OK) return r;
     if ((r = check_dev_ptr(dx, 8)) != LJ_OK) return r;
+    LJ_CK(slots_new_call(c));
     if ((r = ensure_vjp_buffers(c)) != LJ_OK) return r;
-    c->new_call = 1;
     if ((r = bin_for_vjp(c, x, g)) != LJ_OK) return r;
     LJ_CK(launch_vjp(c, g, scale, dx, dparam));
     return LJ_OK;
@@ -1029,9 +1030,9 @@ extern "C" int lj_vv_adjoint_step(lj_ctx *c, const double *x_n, const double *x_
     if ((r = check_dev_ptr(x_n1, 8)) != LJ_OK) return r;
     if ((r = check_dev_ptr(lam_x, 8)) != LJ_OK) return r;
     if ((r = check_dev_ptr(lam_v, 8)) != LJ_OK) return r;
+    LJ_CK(slots_new_call(c));
     if ((r = ensure_vjp_buffers(c)) != LJ_OK) return r;
     const double h = 0.5 * c->p.dt / c->p.mass;
-    c->new_call = 1;
     // v_{n+1} = v_half + h F(x_{n+1})
     // and x_{n+1} = x_n + dt v_half
     if ((r = bin_for_vjp(c, x_n1, lam_v)) != LJ_OK) return r;
@@ -1051,7 +1052,7 @@ extern "C" int lj_step_record(lj_ctx *c, double *traj, double *v, void *f, int32
     if ((r = check_dev_ptr(v, 8)) != LJ_OK) return r;
     if ((r = check_dev_ptr(f, 16)) != LJ_OK) return r;
     const size_t m = 3 * (size_t)c->p.n;
-    c->new_call = 1;
+    LJ_CK(slots_new_call(c));
     if (!uses_slots(c) || persistent_mode(c)) {
         for (int s = 0; s < nsteps; s++) {
             LJ_CK(cudaMemcpyAsync(traj + (s + 1) * m, traj + s * m, m * sizeof(double), cudaMemcpyDeviceToDevice,
@@ -1084,10 +1085,10 @@ extern "C" int lj_vv_adjoint_segment(lj_ctx *c, const double *traj, int32_t nste
     if ((r = check_dev_ptr(traj, 8)) != LJ_OK) return r;
     if ((r = check_dev_ptr(lam_x, 8)) != LJ_OK) return r;
     if ((r = check_dev_ptr(lam_v, 8)) != LJ_OK) return r;
+    LJ_CK(slots_new_call(c));
     if ((r = ensure_vjp_buffers(c)) != LJ_OK) return r;
     const double h = 0.5 * c->p.dt / c->p.mass;
     const size_t m = 3 * (size_t)c->p.n;
-    c->new_call = 1;
     const bool slots = uses_slots(c);   // then each VJP's last kernel bins the next state
     for (int s = nsteps; s >= 0; s--) {
         if (s == nsteps || !slots)

@@ -714,6 +714,18 @@ cudaError_t balloc(lj_batch *b, T **p, size_t count)
     return e;
 }
 
+template <typename T>
+void bfree(lj_batch *b, T *&p)
+{
+    for (size_t k = 0; k < b->allocs.size(); k++)
+        if (b->allocs[k] == (const void *)p) {
+            cudaFree(b->allocs[k]);
+            b->allocs.erase(b->allocs.begin() + (long)k);
+            break;
+        }
+    p = nullptr;
+}
+
 void batch_free(lj_batch *b)
 {
     if (!b) return;
@@ -782,14 +794,14 @@ cudaError_t configure(lj_batch *b)
 // cells of (4/3 rc)^3, beyond the 32 home particles of the kernel's fast path,
 // and as neighbours they still need their slots.  Set up when kernel 7 is
 // chosen; without them (sparse boxes, no memory) the cooperative launch serves.
-cudaError_t batch_slots_setup(lj_batch *b)
+cudaError_t batch_slots_setup(lj_batch *b, bool wide = false)
 {
     const std::vector<BatchRep> &rep = b->hrep;
     const std::vector<long long> &cfix = b->hcfix;
     const double mean = b->max_mean_occ;
     double cw = 0.0;
     for (const BatchRep &r : rep) cw = fmax(cw, (double)r.cw);
-    const int cap = slots_per_cell(mean, cw / b->p.sigma, kBatchSlotMax, b->ncell, b->ntot);
+    const int cap = slots_per_cell(mean, cw / b->p.sigma, kBatchSlotMax, b->ncell, b->ntot, sizeof(float4), wide);
     const int64_t nslots = b->ncell * cap;
     if (b->grid_n3 == 0 || b->ntot == 0 || !b->slots_ok || cap == 0 || nslots + b->ntot >= ((int64_t)1 << 31))
         return cudaSuccess;
@@ -843,6 +855,29 @@ cudaError_t batch_slots_setup(lj_batch *b)
 
 bool batch_slots(const lj_batch *b) { return b->n3 && b->scap > 0; }
 
+// At the start of a call that bins, as slots_new_call (lj_slots.cu).
+cudaError_t batch_new_call(lj_batch *b)
+{
+    b->new_call = 1;
+    if (b->scap == 0 || *(volatile int32_t *)(b->host_err + 1) == 0) return cudaSuccess;
+    if (b->captured || capture_id(b->stream)) return cudaSuccess;
+    cudaError_t e = cudaStreamSynchronize(b->stream);
+    b->host_err[1] = 0;
+    if (e != cudaSuccess) return e;
+    if (b->gexec) cudaGraphExecDestroy(b->gexec);
+    b->gexec = nullptr;
+    bfree(b, b->cellq[0]);
+    bfree(b, b->cellq[1]);
+    bfree(b, b->octr);
+    bfree(b, b->spos);
+    bfree(b, b->onext);
+    bfree(b, b->rep);
+    bfree(b, b->cfix);
+    b->scap = b->par = 0;
+    e = batch_slots_setup(b, true);
+    return e == cudaSuccess && b->scap == 0 ? batch_slots_setup(b) : e;
+}
+
 // One evaluation on slotted cells.  nkick: half kicks of the update (op 0);
 // after: the launch before it in the stream is this batch's force kernel.
 cudaError_t launch_slots_step(lj_batch *b, bool energy, int op, double *x, double *v, float4 *f, int nkick, bool after)
@@ -879,6 +914,8 @@ cudaError_t launch_slots_step(lj_batch *b, bool energy, int op, double *x, doubl
     a.bin.cap = b->scap;
     a.bin.nslots = b->nslots;
     a.bin.nover = (int)b->ntot;
+    a.bin.grow_at = slots_grow_at(b->scap, kBatchSlotMax, b->ntot);
+    a.bin.grow = b->host_err + 1;
     a.rep = b->rep;
     a.rep_of = b->d.rep_of;
     a.rep_of_cell = b->d.rep_of_cell;
@@ -1187,7 +1224,8 @@ extern "C" int lj_batch_create(lj_batch **out, int32_t nrep, const int64_t *n, c
     LJ_BCK(balloc(b, &d.first, 16));
     LJ_BCK(balloc(b, &b->rep_out, 3 * (size_t)nrep));
     LJ_BCK(cudaMallocHost(&b->host_out, sizeof(double) * 3 * (size_t)nrep));
-    LJ_BCK(cudaMallocHost(&b->host_err, sizeof(int32_t)));
+    LJ_BCK(cudaMallocHost(&b->host_err, 2 * sizeof(int32_t)));   // [1]: wider slots are asked for
+    b->host_err[0] = b->host_err[1] = 0;
     LJ_BCK(cudaMemset(d.count, 0, sizeof(int32_t) * ((size_t)ncell + 1)));
     LJ_BCK(cudaMemset(d.cell_of, 0, sizeof(int32_t) * n1));
     LJ_BCK(cudaMemset(d.err, 0, sizeof(int32_t)));
@@ -1279,8 +1317,9 @@ extern "C" int lj_batch_forces(lj_batch *b, const double *x, void *f, int32_t en
     int r;
     if ((r = check_ptr(x, 8)) != LJ_OK) return r;
     if ((r = check_ptr(f, 16)) != LJ_OK) return r;
-    b->new_call = 1;
-    cudaError_t e = launch_step_kernel(b, energy != 0, 1, (double *)x, nullptr, (float4 *)f);
+    cudaError_t e = batch_new_call(b);
+    if (e != cudaSuccess) return map_err(e);
+    e = launch_step_kernel(b, energy != 0, 1, (double *)x, nullptr, (float4 *)f);
     return e == cudaSuccess ? LJ_OK : map_err(e);
 }
 
@@ -1292,7 +1331,10 @@ extern "C" int lj_batch_step(lj_batch *b, double *x, double *v, void *f, int32_t
     if ((r = check_ptr(x, 8)) != LJ_OK) return r;
     if ((r = check_ptr(v, 8)) != LJ_OK) return r;
     if ((r = check_ptr(f, 16)) != LJ_OK) return r;
-    b->new_call = 1;
+    {
+        const cudaError_t en = batch_new_call(b);
+        if (en != cudaSuccess) return map_err(en);
+    }
     if (batch_slots(b)) {
         const cudaError_t es = slots_steps(b, x, v, (float4 *)f, nsteps);
         return es == cudaSuccess ? LJ_OK : map_err(es);
@@ -1362,8 +1404,9 @@ extern "C" int lj_batch_energy(lj_batch *b, const double *x, const double *v, vo
         if ((r = check_ptr(x, 8)) != LJ_OK) return r;
         if ((r = check_ptr(v, 8)) != LJ_OK) return r;
         if ((r = check_ptr(f, 16)) != LJ_OK) return r;
-        b->new_call = 1;
-        cudaError_t e = launch_step_kernel(b, true, 1, (double *)x, nullptr, (float4 *)f);
+        cudaError_t e = batch_new_call(b);
+        if (e != cudaSuccess) return map_err(e);
+        e = launch_step_kernel(b, true, 1, (double *)x, nullptr, (float4 *)f);
         if (e != cudaSuccess) return map_err(e);
     }
     k_batch_energy<<<b->nrep, kReduceThreads, 0, b->stream>>>(v, (const float4 *)f, b->d.poff, b->p.mass,
@@ -1385,7 +1428,10 @@ extern "C" int lj_batch_relax(lj_batch *b, double *x, void *f, int32_t nsteps, d
     int r;
     if ((r = check_ptr(x, 8)) != LJ_OK) return r;
     if ((r = check_ptr(f, 16)) != LJ_OK) return r;
-    b->new_call = 1;
+    {
+        const cudaError_t en = batch_new_call(b);
+        if (en != cudaSuccess) return map_err(en);
+    }
     for (int s = 0; s < nsteps; s++) {
         cudaError_t e = launch_step_kernel(b, false, 1, x, nullptr, (float4 *)f);
         if (e != cudaSuccess) return map_err(e);

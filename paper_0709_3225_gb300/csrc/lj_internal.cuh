@@ -66,7 +66,7 @@ struct lj_ctx {
     double *scalars;     // 8 doubles: [0] = E_pot, [1] = virial, [2] = E_kin, [3] = E_tot, [4] = T, [5] = P
     int32_t *err;
     double *host_scalars;   // pinned, 8 doubles
-    int32_t *host_err;      // pinned
+    int32_t *host_err;      // pinned; [1]: wider slots are asked for (slot_place)
 
     // force kernel configuration: run-staged kernel (lj_force.cu) ...
     int run_len, runs, nitems, cap, force_grid, force_smem, use_tma, use_run_kernel;
@@ -520,7 +520,9 @@ cudaError_t launch_vjp_n3(lj_ctx *c, const double *coef, double scale, double *d
 // where they do not apply), whether force evaluations take them, and the
 // binning: bin x (any coordinates), zero `zero` (float4 [n]), and with g
 // copy the cotangents beside the positions.
-cudaError_t slots_setup(lj_ctx *c);
+cudaError_t slots_setup(lj_ctx *c, bool wide = false);
+// At the start of a call that bins (new_call); widens the slots if asked for.
+cudaError_t slots_new_call(lj_ctx *c);
 void slots_free(lj_ctx *c);
 bool uses_slots(const lj_ctx *c);
 cudaError_t launch_bin_slots(lj_ctx *c, const double *x, float4 *zero, const double *g);

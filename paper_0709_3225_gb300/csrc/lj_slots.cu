@@ -374,6 +374,8 @@ SlotBin slot_bin_of(const lj_ctx *c)
     b.cap = c->scap;
     b.nslots = c->nslots;
     b.nover = (int)c->p.n;
+    b.grow_at = slots_grow_at(c->scap, kSlotMax, c->p.n);
+    b.grow = c->host_err + 1;
     b.cell0 = 0;
     b.S = c->p.precision == LJ_PREC_FP64 ? fx_shift(c) : rel_shift(c->cw);
     return b;
@@ -395,14 +397,15 @@ void slots_free(lj_ctx *c)
     c->slot_par = c->slots_open = c->slots_last = 0;
 }
 
-cudaError_t slots_setup(lj_ctx *c)
+cudaError_t slots_setup(lj_ctx *c, bool wide)
 {
     slots_free(c);
     // (FP64: the fixed-point kernel has no force-shifted form)
     const bool fp64 = c->p.precision == LJ_PREC_FP64;
     if (c->p.cell_subdiv == 2 || c->p.n == 0 || (fp64 && c->p.shift_mode == LJ_SHIFT_FORCE)) return cudaSuccess;
     const double mean = (double)c->p.n / (double)c->ncell;
-    const int cap = slots_per_cell(mean, c->cw / c->p.sigma, kSlotMax, c->ncell, c->p.n);
+    const size_t bytes = fp64 ? sizeof(longlong4_16a) : sizeof(float4);
+    const int cap = slots_per_cell(mean, c->cw / c->p.sigma, kSlotMax, c->ncell, c->p.n, bytes, wide);
     const int64_t nslots = c->ncell * cap;
     if (mean > 22.0 || cap == 0 || nslots + c->p.n >= ((int64_t)1 << 31)) return cudaSuccess;
     // One allocation: each costs a context's creation about 10 us, and one
@@ -410,25 +413,25 @@ cudaError_t slots_setup(lj_ctx *c)
     // (32,000 particles: the first gradient 143 us when it allocated them, now
     // 61); large ones with their first gradient (ensure_vjp_buffers), if any.
     const size_t m = (size_t)(nslots + c->p.n), n = (size_t)c->p.n;
-    const size_t sb = m * (fp64 ? sizeof(longlong4_16a) : sizeof(float4));
+    const size_t sb = m * bytes;
     c->sg4_inside = !fp64 && sb <= kSlotsTogether;
     const size_t qb = (size_t)(c->ncell + 1) * sizeof(int2);
     const size_t part[7] = {sb, c->sg4_inside ? sb : 0, fp64 ? n * kFxAcc * sizeof(long long) : 0,
                             qb, qb, n * sizeof(int32_t), 4 * sizeof(unsigned)};
     char *at[7];
-    size_t bytes = 0;
-    for (size_t p : part) bytes += (p + 255) & ~(size_t)255;
-    cudaError_t e = cudaMalloc(&c->slot_mem, bytes);
+    size_t total = 0;
+    for (size_t p : part) total += (p + 255) & ~(size_t)255;
+    cudaError_t e = cudaMalloc(&c->slot_mem, total);
     if (e == cudaErrorMemoryAllocation) {   // the sorted lists need less
         cudaGetLastError();
         slots_free(c);
         return cudaSuccess;
     }
     if (e != cudaSuccess) return e;
-    bytes = 0;
+    total = 0;
     for (int k = 0; k < 7; k++) {
-        at[k] = (char *)c->slot_mem + bytes;
-        bytes += (part[k] + 255) & ~(size_t)255;
+        at[k] = (char *)c->slot_mem + total;
+        total += (part[k] + 255) & ~(size_t)255;
     }
     c->spos = at[0];
     c->sg4 = c->sg4_inside ? (float4 *)at[1] : nullptr;
@@ -443,6 +446,20 @@ cudaError_t slots_setup(lj_ctx *c)
     c->nslots = (int)nslots;
     c->slots_open = 2;
     return fp64 ? fx_configure(c) : cudaSuccess;
+}
+
+// Not while a caller's graph holds the old buffers, and not inside a capture.
+cudaError_t slots_new_call(lj_ctx *c)
+{
+    c->new_call = 1;
+    if (c->scap == 0 || *(volatile int32_t *)(c->host_err + 1) == 0) return cudaSuccess;
+    if (c->captured || capture_id(c->stream)) return cudaSuccess;
+    cudaError_t e = cudaStreamSynchronize(c->stream);
+    c->host_err[1] = 0;
+    if (e != cudaSuccess) return e;
+    c->gen++;   // captured steps hold the old buffers
+    e = slots_setup(c, true);
+    return e == cudaSuccess && c->scap == 0 ? slots_setup(c, false) : e;   // (no memory for the wide ones)
 }
 
 // Force evaluations take the slotted cells where the pair-once kernel runs

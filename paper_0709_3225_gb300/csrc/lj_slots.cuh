@@ -33,25 +33,37 @@ struct SlotBin {
     float sf;               // (float)s
     int nc, ncell, cap, nslots, S;   // S: scale of the fixed-point coordinates (FP64: lj_force_fx.cu, else rel_shift)
     int nover;              // entries of the overflow region
+    int grow_at;            // overflow particles that set *grow (pinned host memory)
+    int32_t *grow;
     int cell0;              // id of the grid's first cell (a batch's replica; else 0); ncell counts all grids' cells
 };
 
-// Slots per cell of `cw` sigma a side in ncell cells of n particles, a multiple
-// of 8 (128 bytes) up to limit; 0: the box is too sparse (far more slots than
-// particles) and keeps the sorted lists.  The mean occupancy plus 7 standard
-// deviations of a random gas, and, where 24 slots a particle allow it, room
-// for a liquid or crystal (0.9 particles per sigma^3 and 16 more: at 2.5 sigma a
-// lattice can put 4 of its planes in a cell, 32 particles): a vapour may condense,
-// a box hold both, and a cell beyond its slots takes all cells around it to
-// the plain path.  A droplet of 97,556 particles at a mean density of 0.1, 16
-// slots by the gas alone: forces 288 us, VJP 383.
-inline int slots_per_cell(double mean, double cw, int limit, int64_t ncell, int64_t n)
+// Slots per cell of `cw` sigma a side in ncell cells of n particles, `bytes`
+// each, a multiple of 8 (128 bytes) up to limit; 0: the box is too sparse (far
+// more slots than particles) and keeps the sorted lists.  The mean occupancy
+// plus 7 standard deviations of a random gas; and, where that makes up to 24
+// MB of slots, room for a liquid or crystal (0.9 particles per sigma^3 and 16
+// more: at 2.5 sigma a lattice can put 4 of its planes in a cell, 32
+// particles).  A vapour may condense, a box hold both, and a cell beyond its
+// slots takes all cells around it to the plain path (a droplet of 97,556
+// particles at a mean density of 0.1, 16 slots by the gas alone: forces 288 us,
+// VJP 383).  Larger boxes get the wide slots (limit) when they are seen to need
+// them (slot_place, slots_new_call): 32 slots in place of 16 cost a gas of 10^6
+// particles, whose positions then lie further apart in memory, 1 to 5 %.
+inline int slots_per_cell(double mean, double cw, int limit, int64_t ncell, int64_t n, size_t bytes, bool wide)
 {
     auto up8 = [limit](double m) { return m < (double)limit ? ((int)ceil(m) + 7) & ~7 : limit; };
     const int gas = up8(mean + 7.0 * sqrt(mean) + 3.0), liquid = up8(0.9 * cw * cw * cw + 16.0);
-    const int64_t free_slots = (int64_t)1 << 16;
-    if (liquid > gas && ncell * liquid <= 24 * n + free_slots) return liquid;
-    return ncell * gas <= 12 * n + free_slots ? gas : 0;
+    if (ncell * gas > 12 * n + ((int64_t)1 << 16)) return 0;
+    if (wide) return limit;
+    return liquid > gas && (size_t)(ncell * liquid) * bytes <= ((size_t)24 << 20) ? liquid : gas;
+}
+
+// The wide slots are asked for when a binning has so many particles beyond
+// their cells' slots.
+inline int slots_grow_at(int cap, int limit, int64_t n)
+{
+    return cap < limit ? 32 + (int)(n / 2048) : 0x7fffffff;
 }
 
 #ifdef __CUDACC__
@@ -92,6 +104,7 @@ __device__ __forceinline__ int slot_place(const SlotBin &b, bool valid, int i, d
     int slot = c * b.cap + r;
     if (r >= b.cap) {   // overflow: the next free entry, pushed on the cell's list
         const int k = (int)atomicAdd(b.octr, 1u);
+        if (k == b.grow_at) *b.grow = 1;
         if (k >= b.nover) {   // never with counts that were zero
             atomicOr(err, LJ_ERRBIT_OVERFLOW);
             return -1;
