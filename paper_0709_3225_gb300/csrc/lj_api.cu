@@ -463,7 +463,10 @@ int ensure_vjp_buffers(lj_ctx *c)
     if (!c->g4 && !uses_slots(c)) LJ_CK(cudaMalloc(&c->g4, (size_t)c->p.n * force_vsize(c)));
     if (c->p.precision == LJ_PREC_MIXED && uses_vjp_n3(c) && !c->f_sorted)
         LJ_CK(cudaMalloc(&c->f_sorted, (size_t)c->p.n * sizeof(float4)));
-    if (uses_slots(c) && !c->sg4) LJ_CK(cudaMalloc(&c->sg4, ((size_t)c->nslots + (size_t)c->p.n) * sizeof(float4)));
+    if (uses_slots(c) && !c->sg4) {   // the first time, and after the slots were widened
+        RelaxedCapture relaxed;
+        LJ_CK(cudaMalloc(&c->sg4, ((size_t)c->nslots + (size_t)c->p.n) * sizeof(float4)));
+    }
     return LJ_OK;
 }
 

@@ -861,6 +861,7 @@ cudaError_t batch_new_call(lj_batch *b)
     b->new_call = 1;
     if (b->scap == 0 || *(volatile int32_t *)(b->host_err + 1) == 0) return cudaSuccess;
     if (b->captured || capture_id(b->stream)) return cudaSuccess;
+    RelaxedCapture relaxed;
     cudaError_t e = cudaStreamSynchronize(b->stream);
     b->host_err[1] = 0;
     if (e != cudaSuccess) return e;

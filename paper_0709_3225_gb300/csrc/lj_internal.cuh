@@ -431,6 +431,14 @@ inline unsigned long long capture_id(cudaStream_t s)
     return st == cudaStreamCaptureStatusActive ? id : 0;
 }
 
+// While it lives, allocations and synchronizations of this thread leave a
+// capture that is going on in another stream alone.
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 // Kernel launchers (each returns cudaGetLastError()).
 // gated: skin mode, run only when the device-side rebuild flag is set
 cudaError_t launch_bin_count(lj_ctx *c, const double *x, bool gated = false);

@@ -454,6 +454,7 @@ cudaError_t slots_new_call(lj_ctx *c)
     c->new_call = 1;
     if (c->scap == 0 || *(volatile int32_t *)(c->host_err + 1) == 0) return cudaSuccess;
     if (c->captured || capture_id(c->stream)) return cudaSuccess;
+    RelaxedCapture relaxed;
     cudaError_t e = cudaStreamSynchronize(c->stream);
     c->host_err[1] = 0;
     if (e != cudaSuccess) return e;

@@ -190,3 +190,28 @@ def test_a_recorded_context_keeps_its_slots(oracle_mod):
                 assert rel_rms(s.f.double().cpu().numpy()[:, :3], fo) <= 5e-6
         s.check()
         s.close()
+
+
+def test_widening_leaves_another_streams_capture_alone(oracle_mod):
+    import torch
+    from paper_0709_3225_gb300 import lj
+    x, L = _droplet(29, 0.1, 35)
+    fo = oracle_mod.forces_cells(x, L, mode=1)[0]
+    st, other = torch.cuda.Stream(), torch.cuda.Stream()
+    s = lj.System(x, None, L, shift_mode=1, stream=st)
+    torch.cuda.synchronize()
+    s.forces()                                # asks for wider slots
+    torch.cuda.synchronize()
+    a = torch.ones(8, device="cuda")
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=other):
+        a.mul_(2.0)
+        s.forces()                            # not part of the capture: widens
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(a, torch.full_like(a, 2.0))
+    s.forces()
+    torch.cuda.synchronize()
+    s.check()
+    assert rel_rms(s.f.double().cpu().numpy()[:, :3], fo) <= 5e-6
+    s.close()
